@@ -111,13 +111,13 @@ def _tokens(case, g):
     return base.repeat(1, 1, frames, 1)[:, :, :n] + 0.1 * torch.randn(B, H, n, d, generator=g, device="cuda")
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """Everything random about a case's state, drawn in one order for prepare() and exact()."""
     g = torch.Generator(device="cuda")
     g.manual_seed(int(seed))
     dt = _dtype(case)
     B, H, n, n_q, d, m, T = (case[k] for k in ("B", "H", "n", "n_q", "d", "m", "T"))
-    ctx = binding.Csat(n, m, d, H, 0, B=B, n_q=n_q, dtype=case["dtype"], T=T, lam=case["lam"])
-    s = {"case": case, "ctx": ctx}
+    s = {}
     if case["pass"] == "layer":
         dm = H * d
         s["X"] = torch.randn(B, n, dm, generator=g, device="cuda").to(dt)
@@ -132,23 +132,37 @@ def prepare(case, seed):
         beta = torch.randn(B, H, n, d, generator=g, device="cuda")
         beta *= keys < 0.25
         s["V"] = (beta @ psi.t()).to(dt)
-        ctx.set_dictionary(psi.to(dt))
+        s["psi"] = psi.to(dt)
     else:
         s["V"] = _tokens(case, g).to(dt)
     if case["pass"] in ("train", "learned"):
         s["Q"] *= math.sqrt(m / n)          # rows of K~ = Phi K are sqrt(n / m) times as long as those of K
         s["dOut"] = torch.randn(B, H, n_q, d, generator=g, device="cuda").to(dt)
+    if case["pass"] == "learned":
+        # weights some way into training: the derived ones, moved a little, each layer by itself
+        moved = 0.02 / math.sqrt(d)
+        s["dS"] = moved * torch.randn(T, H, d, d, generator=g, device="cuda")
+        s["dBm"] = moved * torch.randn(T, H, d, d, generator=g, device="cuda")
+        s["dtheta"] = 0.5 + torch.rand(T, H, generator=g, device="cuda")
+        s["phi"] = (torch.randn(H, m, n, generator=g, device="cuda") / math.sqrt(m)).to(dt)
+    return s
+
+
+def prepare(case, seed):
+    B, H, n, n_q, d, m, T = (case[k] for k in ("B", "H", "n", "n_q", "d", "m", "T"))
+    ctx = binding.Csat(n, m, d, H, 0, B=B, n_q=n_q, dtype=case["dtype"], T=T, lam=case["lam"])
+    s = dict(_inputs(case, seed), case=case, ctx=ctx)
+    if case["psi"]:
+        ctx.set_dictionary(s["psi"])
+    if case["pass"] in ("train", "learned"):
         for k in "QKV":
             s[k].requires_grad_(True)
     if case["pass"] == "learned":
-        # weights some way into training: the derived ones, moved a little, each layer by itself
         binding.csat_set_i64(ctx.h, binding.CSAT_WEIGHT_GRADS, 1)
         S, Bm, theta, _ = ctx.get_decoder()
-        moved = 0.02 / math.sqrt(d)
-        s["S"] = (S + moved * torch.randn(T, H, d, d, generator=g, device="cuda")).to(dt)
-        s["Bm"] = (Bm + moved * torch.randn(T, H, d, d, generator=g, device="cuda")).to(dt)
-        s["theta"] = theta * (0.5 + torch.rand(T, H, generator=g, device="cuda"))
-        s["phi"] = (torch.randn(H, m, n, generator=g, device="cuda") / math.sqrt(m)).to(dt)
+        s["S"] = (S + s.pop("dS")).to(_dtype(case))
+        s["Bm"] = (Bm + s.pop("dBm")).to(_dtype(case))
+        s["theta"] = theta * s.pop("dtheta")
     return s
 
 
@@ -206,3 +220,76 @@ def tolerance(case):
     if case["dtype"] == "fp32":
         return {"rel": 5e-3, "max": 0.6} if train else {"rel": 5e-6, "max": 5e-5}
     return {"rel": 0.02, "max": 0.9} if train else {"rel": 0.025, "max": 0.5}
+
+
+def _phi(m, n, h, dt):
+    """Measurement matrix of head h for seed 0: Philox4x32-10, four Gaussians of a block by Box-Muller on 23-bit
+    uniforms, divided by sqrt(m) and held in the storage type; as float64."""
+    lo32 = 0xFFFFFFFF
+    q = torch.arange(h * m * n // 4, ((h + 1) * m * n + 3) // 4, device="cuda")
+    c = [q & lo32, q >> 32, torch.zeros_like(q), torch.zeros_like(q)]
+    k = [0, 0]
+    for _ in range(10):
+        p0, p1 = c[0] * 0xD2511F53, c[2] * 0xCD9E8D57                 # modulo 2^64
+        c = [((p1 >> 32) & lo32) ^ c[1] ^ k[0], p1 & lo32, ((p0 >> 32) & lo32) ^ c[3] ^ k[1], p0 & lo32]
+        k = [(k[0] + 0x9E3779B9) & lo32, (k[1] + 0xBB67AE85) & lo32]
+    u = [((w >> 9).double() + 0.5) * 2.0 ** -23 for w in c]
+    g = []
+    for a, b in ((u[0], u[1]), (u[2], u[3])):
+        r = torch.sqrt(-2.0 * torch.log(a))
+        g += [r * torch.cos(2 * math.pi * b), r * torch.sin(2 * math.pi * b)]
+    first = h * m * n % 4
+    g = torch.stack(g, 1).flatten()[first:first + m * n] / math.sqrt(m)
+    return g.to(torch.float32).to(dt).double().view(m, n)
+
+
+def exact(case, seed):
+    """The paper's equations in 64 bits on the same inputs: K~ = Phi K, V~ = Phi V, Z = softmax(Q K~^T / sqrt(d)) V~,
+    alpha <- eta_theta(alpha S + Z B) with S = I - mu M^T M, B = mu M, M = Phi[:d, :d] Psi, 1 / mu the largest absolute
+    row sum of M^T M and theta = mu lambda, out = alpha Psi^T; gradients by torch's autograd."""
+    s = _inputs(case, seed)
+    dt, f64 = _dtype(case), torch.float64
+    B, H, n, n_q, d, m, T = (case[k] for k in ("B", "H", "n", "n_q", "d", "m", "T"))
+    kind = case["pass"]
+    if kind == "layer":
+        QKV = (s["X"].double().view(B * n, -1) @ s["W"].double()).view(B, n, 3, H, d).permute(2, 0, 3, 1, 4)
+        s["Q"], s["K"], s["V"] = QKV[0], QKV[1], QKV[2]
+    eye = torch.eye(d, dtype=f64, device="cuda")
+    psi = s["psi"].double() if case["psi"] else eye
+    grad = kind in ("train", "learned")
+    out = torch.empty(B, H, n_q, d, dtype=f64, device="cuda")
+    res = {k: torch.empty(s[k].shape, dtype=f64, device="cuda") for k in "QKV"} if grad else {}
+    if kind == "learned":
+        res.update(S=torch.zeros(T, H, d, d, dtype=f64, device="cuda"), B=torch.zeros(T, H, d, d, dtype=f64, device="cuda"),
+                   phi=torch.zeros(H, m, n, dtype=f64, device="cuda"))
+    for h in range(H):
+        phi = _phi(m, n, h, dt)
+        M = phi[:d, :d] @ psi
+        G = M.t() @ M
+        mu = 1.0 / G.abs().sum(1).max()
+        Ss, Bs, thetas = (eye - mu * G).expand(T, d, d), (mu * M).expand(T, d, d), (mu * case["lam"]).expand(T)
+        if kind == "learned":
+            Ss, Bs = ((x.float() + s[k][:, h]).to(dt).double().requires_grad_(True) for x, k in ((Ss, "dS"), (Bs, "dBm")))
+            thetas = thetas * s["dtheta"][:, h].double()
+            phi = s["phi"][h].double().requires_grad_(True)
+        for b in range(B):
+            q, k, v = (s[x][b, h].detach().double().requires_grad_(grad) for x in "QKV")
+            with torch.set_grad_enabled(grad):
+                z = torch.softmax(q @ (phi @ k).t() / math.sqrt(d), 1) @ (phi @ v)
+                c = z @ Bs[0]
+                alpha = torch.zeros_like(z)
+                for t in range(T):
+                    x = (z @ Bs[t] if kind == "learned" else c) + (alpha @ Ss[t] if t else 0.0)
+                    alpha = x - torch.clamp(x, -thetas[t], thetas[t])
+                o = alpha @ psi.t()
+            out[b, h] = o.detach()
+            if grad:
+                of = (q, k, v) + ((Ss, Bs, phi) if kind == "learned" else ())
+                gr = torch.autograd.grad(o, of, s["dOut"][b, h].double())
+                for x, y in zip("QKV", gr):
+                    res[x][b, h] = y
+                if kind == "learned":
+                    res["S"][:, h] += gr[3]
+                    res["B"][:, h] += gr[4]
+                    res["phi"][h] += gr[5]
+    return (out,) + tuple(res.values()) if grad else out
