@@ -188,6 +188,17 @@ cudaError_t launch_decoder_setup(csat_ctx* c, cudaStream_t s, int* launches);
 // (phi_j0, n_len, partial): token-sharded use, see compress_sm100.cu; defaults = the whole sequence into the workspace
 cudaError_t launch_simt_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int* launches,
                                  int64_t phi_j0 = 0, int64_t n_len = 0, float* partial = nullptr);
+// ffma_forward.cu : the same two stages for d <= kFfmaMaxD, where the launchers above send them
+constexpr int64_t kFfmaMaxD = 128;
+struct FfmaAttend {                       // layer t of head h: S + t * layer_stride + h d d, theta[t * theta_stride + h]
+  const float *S, *B, *theta, *psi;       // psi: null = identity
+  int64_t layer_stride, nq, m, BH;
+  int theta_stride, d, H, T, device, sms;
+  float scale;
+};
+cudaError_t launch_ffma_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
+                                 float* partial);
+cudaError_t launch_ffma_attend(const FfmaAttend& a, int dtype, const void* Q, const void* kv, void* out, cudaStream_t s);
 // workspace := sum over r < R of partials[r] (float32 [B,H,m,2d] each), added in the order r = 0, 1, ..., rounded
 // once to the context's storage type
 cudaError_t launch_reduce_partials(csat_ctx* c, const float* partials, int R, cudaStream_t s, int* launches);

@@ -1,0 +1,368 @@
+// The float32 forward for head sizes up to 128 (float32 contexts, and bf16 storage with head sizes that have no
+// tensor-core kernel): K~ = Phi K, V~ = Phi V, then A~ = softmax(Q K~^T / sqrt(d_k)), Z = A~ V~ and the unrolled recovery
+// alpha^{t+1} = eta_theta(S alpha^t + B Z_i), C^_i = Psi alpha^_i, all sums and iterates in float32.
+//
+// Bound: the FMA pipe (128 multiply-adds per clock and SM; ~100 reachable, see ffma_tile.cuh) for large jobs, the chain of
+// waits of one warp for small ones.  Measured against kernels with one warp per query row and one lane per column (one
+// B200, us): one head of 256 x 64, m = 64, T = 10 in float32: compression 58.6 -> 3.2, attention and recovery 57.9 -> 13.6;
+// 32 heads of 1024 x 96 in bf16, m = 128, T = 10: 384 -> 46 and 1573 -> 192 (1573: 5 TFLOP/s; 192: 41 of 74).
+#include "csat_internal.h"
+#include "ffma_tile.cuh"
+
+namespace csat {
+namespace {
+
+using namespace ffma;
+
+// ---------------------------------------------------------------------------------------------
+// K~|V~[b,h,r,:] = sum_j Phi[h,r,j] [K|V][b,h,j,:]
+// A CTA owns 4 TR measurements x 32 TCQ columns of K~ or of V~; its warps share out the tokens in chunks of 16 (each
+// warp stages and multiplies its own chunks: no block-wide barrier until the end) and their partial sums are added in
+// warp order.  The work is a few hundred multiply-adds per thread and the wait for memory, so the split over the tokens
+// is what fills the SMs at small batches.
+// ---------------------------------------------------------------------------------------------
+constexpr int kCmpWarps = 8, kCmpK = 16, kCmpLdA = kCmpK + 4;
+
+template <typename T, typename TO, int TR, int TCQ>
+__global__ void __launch_bounds__(kCmpWarps * 32) ffma_compress_kernel(TO* __restrict__ kv, const T* __restrict__ phi,
+                                                                       const T* __restrict__ K, const T* __restrict__ V,
+                                                                       int64_t n, int64_t n_pad, int64_t m, int d, int H,
+                                                                       int phi_v_head0, int64_t phi_j0, int col_blocks) {
+  constexpr int kRows = 4 * TR, kCols = 32 * TCQ, kN = Vec<T>::kN;
+  constexpr int kStage = kRows * kCmpLdA + kCmpK * kCols;                    // floats per warp
+  extern __shared__ __align__(16) float cmp_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+  const int bh = blockIdx.y, h = bh % H;
+  const int is_v = blockIdx.z >= col_blocks, c0 = (blockIdx.z - (is_v ? col_blocks : 0)) * kCols;
+  const int64_t r0 = (int64_t)blockIdx.x * kRows;
+  const T* ph = phi + (int64_t)((is_v ? phi_v_head0 : 0) + h) * m * n_pad + phi_j0;
+  const T* src = (is_v ? V : K) + (int64_t)bh * n * d;
+  float* As = cmp_smem + warp * kStage;
+  float* Bs = As + kRows * kCmpLdA;
+  float2 acc[TR][2 * TCQ];
+  clear(acc);
+
+  constexpr int kAVecs = kRows * (kCmpK / kN) / 32 > 0 ? kRows * (kCmpK / kN) / 32 : 1;
+  constexpr int kBVecs = kCmpK * (kCols / kN) / 32;
+  constexpr int kVpa = kCmpK / kN, kVpb = kCols / kN;                       // 16-byte pieces per row
+  uint4 va[kAVecs], vb[kBVecs];
+  auto fetch = [&](int64_t j0) {
+#pragma unroll
+    for (int u = 0; u < kAVecs; ++u) {
+      const int i = lane + 32 * u, r = i / kVpa, k = (i % kVpa) * kN;
+      va[u] = make_uint4(0, 0, 0, 0);
+      // a piece that starts inside the tokens may end beyond them: Phi's rows are padded, and the matching rows of
+      // the other operand are zero (a shard's neighbour columns are finite or zero weights never reach the sum)
+      if (r < kRows && r0 + r < m && j0 + k < n) va[u] = *reinterpret_cast<const uint4*>(ph + (r0 + r) * n_pad + j0 + k);
+    }
+#pragma unroll
+    for (int u = 0; u < kBVecs; ++u) {
+      const int i = lane + 32 * u, k = i / kVpb, c = c0 + (i % kVpb) * kN;
+      vb[u] = make_uint4(0, 0, 0, 0);
+      if (j0 + k < n && c < d) vb[u] = *reinterpret_cast<const uint4*>(src + (j0 + k) * d + c);
+    }
+  };
+  int64_t j0 = (int64_t)warp * kCmpK;
+  if (j0 < n) fetch(j0);
+  for (; j0 < n; j0 += kCmpWarps * kCmpK) {
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < kAVecs; ++u) {
+      const int i = lane + 32 * u, r = i / kVpa, k = (i % kVpa) * kN;
+      float f[kN];
+      Vec<T>::to_float(va[u], f);
+      if (r < kRows)
+#pragma unroll
+        for (int w = 0; w < kN; w += 4) {
+          // tokens beyond n (another shard's columns of Phi, or padding) are cleared
+          float4 x = make_float4(f[w], f[w + 1], f[w + 2], f[w + 3]);
+          if (j0 + k + w + 4 > n) {
+            if (j0 + k + w >= n) x.x = 0.f;
+            if (j0 + k + w + 1 >= n) x.y = 0.f;
+            if (j0 + k + w + 2 >= n) x.z = 0.f;
+            if (j0 + k + w + 3 >= n) x.w = 0.f;
+          }
+          *reinterpret_cast<float4*>(As + r * kCmpLdA + k + w) = x;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kBVecs; ++u) {
+      const int i = lane + 32 * u, k = i / kVpb, c = (i % kVpb) * kN;
+      float f[kN];
+      Vec<T>::to_float(vb[u], f);
+#pragma unroll
+      for (int w = 0; w < kN; w += 4)
+        *reinterpret_cast<float4*>(Bs + k * kCols + c + w) = make_float4(f[w], f[w + 1], f[w + 2], f[w + 3]);
+    }
+    __syncwarp();
+    if (j0 + kCmpWarps * kCmpK < n) fetch(j0 + kCmpWarps * kCmpK);
+    gemm_t<TR, TCQ>(acc, As + ty * kCmpLdA, kCmpLdA, Bs + 4 * tx, kCols, kCmpK);
+  }
+  // partial sums of the warps, added in warp order
+  __syncthreads();
+  constexpr int kTile = kRows * kCols;
+#pragma unroll
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int q = 0; q < TCQ; ++q)
+      *reinterpret_cast<float4*>(cmp_smem + warp * kTile + (ty + 4 * i) * kCols + 4 * tx + 32 * q) =
+          make_float4(acc[i][2 * q].x, acc[i][2 * q].y, acc[i][2 * q + 1].x, acc[i][2 * q + 1].y);
+  __syncthreads();
+  for (int i = threadIdx.x * 4; i < kTile; i += kCmpWarps * 32 * 4) {
+    const int r = i / kCols, c = c0 + i % kCols;
+    if (r0 + r >= m || c >= d) continue;
+    float4 s = *reinterpret_cast<const float4*>(cmp_smem + i);
+#pragma unroll
+    for (int w = 1; w < kCmpWarps; ++w) {
+      const float4 x = *reinterpret_cast<const float4*>(cmp_smem + w * kTile + i);
+      s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+    }
+    store4(kv + ((int64_t)bh * m + r0 + r) * 2 * d + (is_v ? d : 0) + c, s.x, s.y, s.z, s.w);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Attention over the measurements and recovery, 16 TR queries per CTA (4 TR per warp)
+// ---------------------------------------------------------------------------------------------
+template <int DP, int TR> struct AttendSmem {               // in floats
+  static constexpr int kRows = kWarps * 4 * TR;
+  // Ks | Vs; later the rows of B, a block at a time, then (DP <= 64) the rows' c = z B
+  static constexpr int kC = DP <= 64 ? kRows * Ld<DP>::kA : 0;
+  static constexpr int kChunks = 2 * kChunk * Ld<DP>::kB > kC ? 2 * kChunk * Ld<DP>::kB : kC;
+  static constexpr int kS = kChunks;                         // [DP][DP + 4]
+  static constexpr int kA = kS + DP * Ld<DP>::kB;            // [kRows][DP + 8]
+  static constexpr int kP = kA + kRows * Ld<DP>::kA;         // [kRows][40]
+  static constexpr int kZ = kP + kRows * kPLd;               // [kRows][DP + 8], per-layer weights only
+  static constexpr int kFloats = kZ, kFloatsUntied = kZ + kRows * Ld<DP>::kA;
+};
+
+template <typename T, int DP, int TR>
+__global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ out, const T* __restrict__ Q, const T* __restrict__ kv,
+                                                               const FfmaAttend p) {
+  using L = AttendSmem<DP, TR>;
+  constexpr int kLdA = Ld<DP>::kA, kLdB = Ld<DP>::kB, kTCQ = DP / 32, kRW = 4 * TR;
+  extern __shared__ __align__(16) float att_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+  const int bh = blockIdx.y, h = bh % p.H, d = p.d;
+  const int64_t row0 = (int64_t)blockIdx.x * L::kRows + warp * kRW;          // of the warp
+  float* Ks = att_smem;
+  float* Vs = att_smem + kChunk * kLdB;
+  float* Ss = att_smem + L::kS;
+  float* Arows = att_smem + L::kA + warp * kRW * kLdA;
+  float* Aw = Arows + ty * kLdA;
+  float* Pw = att_smem + L::kP + (warp * kRW + ty) * kPLd;
+  const bool untied = p.layer_stride != 0;
+  float* Zw = untied ? att_smem + L::kZ + (warp * kRW + ty) * kLdA : Aw;
+  const int64_t hdd = (int64_t)h * d * d;
+
+  if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
+  load_own_rows<T>(Arows, kLdA, Q + (int64_t)bh * p.nq * d, row0, p.nq, d, kRW, lane, d);
+  __syncwarp();
+
+  float2 a[TR][2 * kTCQ];                                   // Z, then the iterate
+  {
+    float mx[TR], sum[TR];
+    softmax_rows<T, DP, TR>(a, mx, sum, Ks, Vs, Aw, Pw, kv + (int64_t)bh * p.m * 2 * d, p.m, d, p.scale);
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+      const float inv = 1.f / sum[i];
+#pragma unroll
+      for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = __fmul2_rn(a[i][j], dup(inv));
+    }
+  }
+  if (p.T > 0) {
+    __syncwarp();
+    store_rows<TR, kTCQ>(Zw, kLdA, tx, a);                  // z as an operand
+    float2 c[TR][2 * kTCQ];
+    // c = z B_t; the rows of B pass through the chunk buffers
+    auto times_B = [&](int t) {
+      constexpr int kFit = 2 * kChunk;
+      clear(c);
+      for (int k0 = 0; k0 < d; k0 += kFit) {
+        const int rows = d - k0 < kFit ? d - k0 : kFit;
+        __syncthreads();
+        stage_matrix_async(Ks, kLdB, p.B + t * p.layer_stride + hdd, d, k0, rows);
+        cp_async_wait_all();
+        __syncthreads();
+        gemm_t<TR, kTCQ>(c, Zw + k0, kLdA, Ks + 4 * tx, kLdB, rows);
+      }
+    };
+    times_B(0);
+    float th = p.theta[h];
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = shrink(c[i][j], th);       // alpha^1 = eta(0 S + z B)
+    if (DP <= 64 && !untied && p.T > 1) {
+      // One S for all layers: every warp keeps it in registers and takes its rows four at a time.  c waits in shared memory
+      // (its place: the warp's probabilities, then its Z rows), the lane's columns are those of RegMatrix.
+      constexpr int kDR = DP <= 64 ? DP : 64;               // (not instantiated beyond 64)
+      constexpr int kNC = RegMatrix<kDR>::NC;
+      RegMatrix<kDR> S;
+      S.load(Ss, kLdB, d, tx, ty);
+      float* Crows = att_smem + warp * kRW * kLdA;          // the chunk buffers are free: [kRows][DP + 8] there
+      __syncthreads();
+      store_rows<TR, kTCQ>(Crows + ty * kLdA, kLdA, tx, c);
+      store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
+      const int col = RegMatrix<kDR>::col(tx, ty);
+      constexpr int kN = 4;
+      for (int it = 1; it < p.T; ++it) {
+        th = p.theta[(int64_t)it * p.theta_stride + h];
+        __syncwarp();
+#pragma unroll 1
+        for (int r = 0; r < kRW; r += kN) {
+          float y[kN][kNC];
+          S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+#pragma unroll
+          for (int u = 0; u < kN; ++u)
+#pragma unroll
+            for (int j = 0; j < kNC; ++j)
+              Arows[(r + u) * kLdA + col + 8 * j] = shrink(y[u][j] + Crows[(r + u) * kLdA + col + 8 * j], th);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int q = 0; q < kTCQ; ++q) {
+          const float4 x = *reinterpret_cast<const float4*>(Aw + 4 * i * kLdA + 4 * tx + 32 * q);
+          a[i][2 * q] = make_float2(x.x, x.y);
+          a[i][2 * q + 1] = make_float2(x.z, x.w);
+        }
+    } else
+    for (int it = 1; it < p.T; ++it) {
+      th = p.theta[(int64_t)it * p.theta_stride + h];
+      if (untied) {
+        times_B(it);
+        stage_matrix_async(Ss, kLdB, p.S + it * p.layer_stride + hdd, d, 0, d);
+        cp_async_wait_all();
+        __syncthreads();
+      } else {
+        __syncwarp();                                       // the operand rows have been read
+      }
+      store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = c[i][j];
+      gemm_t<TR, kTCQ>(a, Aw, kLdA, Ss + 4 * tx, kLdB, d);
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = shrink(a[i][j], th);
+      if (untied) __syncwarp();
+    }
+    if (p.psi) {                                            // out_c = sum_k alpha_k Psi[c][k]
+      __syncthreads();
+      stage_matrix_async(Ss, kLdB, p.psi + hdd, d, 0, d);
+      store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
+      cp_async_wait_all();
+      __syncthreads();
+      for (int c0 = 0; c0 < d; c0 += 32) {
+        float2 o2[TR][4];
+        clear(o2);
+        gemm_n<TR, 4>(o2, Aw, kLdA, Ss + (c0 + tx) * kLdB, kLdB, d);
+#pragma unroll
+        for (int i = 0; i < TR; ++i) {
+          const int64_t row = row0 + ty + 4 * i;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (row < p.nq && c0 + tx + 8 * j < d)
+              store1(out + ((int64_t)bh * p.nq + row) * d + c0 + tx + 8 * j, o2[i][j].x + o2[i][j].y);
+        }
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < TR; ++i) {
+    const int64_t row = row0 + ty + 4 * i;
+#pragma unroll
+    for (int q = 0; q < kTCQ; ++q)
+      if (row < p.nq && 4 * tx + 32 * q < d)
+        store4(out + ((int64_t)bh * p.nq + row) * d + 4 * tx + 32 * q, a[i][2 * q].x, a[i][2 * q].y, a[i][2 * q + 1].x,
+               a[i][2 * q + 1].y);
+  }
+}
+
+template <typename T, typename TO, int TR, int TCQ>
+cudaError_t launch_compress(csat_ctx* c, TO* dst, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len) {
+  const Params& p = c->p;
+  constexpr int kRows = 4 * TR, kCols = 32 * TCQ;
+  constexpr int kStage = kCmpWarps * (kRows * kCmpLdA + kCmpK * kCols), kTile = kCmpWarps * kRows * kCols;
+  constexpr int kBytes = (kStage > kTile ? kStage : kTile) * 4;
+  static DeviceFlags opt_in;
+  cudaError_t e = ensure_dynamic_smem(ffma_compress_kernel<T, TO, TR, TCQ>, kBytes, c->device, opt_in);
+  if (e != cudaSuccess) return e;
+  const int cb = (int)((p.d + kCols - 1) / kCols);
+  const dim3 grid((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(p.B * p.H), (unsigned)(2 * cb));
+  ffma_compress_kernel<T, TO, TR, TCQ><<<grid, kCmpWarps * 32, kBytes, s>>>(
+      dst, (const T*)c->phi, (const T*)K, (const T*)V, n_len, p.n_pad, p.m, (int)p.d, (int)p.H, p.separate_phi ? (int)p.H : 0,
+      phi_j0, cb);
+  return cudaGetLastError();
+}
+
+// The tile: 32 measurements x all columns of K~ or V~ up to 96 (the operand reads of 8 rows per lane keep up with the
+// arithmetic) where that gives most SMs a CTA, otherwise 16 x 32, and 8 x 32 where even that fills less than one wave.
+// Measured (float32, d = 64, m = 96, n = 512; 8 x 32 / 16 x 32 / 32 x 64): 2 heads 4.7 / 5.3 / 10.7 us, 8 heads 9.9 / 8.6
+// / 10.9, 16 heads 17.6 / 12.2 / 11.1, 64 heads 55.6 / 38.3 / 30.7 us.
+template <typename T, typename TO>
+cudaError_t compress_t(csat_ctx* c, TO* dst, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len) {
+  const Params& p = c->p;
+  const int tcq = p.d <= 32 ? 1 : p.d <= 64 ? 2 : p.d <= 96 ? 3 : 2;          // 128 columns: two blocks of 64
+  const int64_t bh = p.B * p.H, sms = c->sms;
+  const int64_t big = (p.m + 31) / 32 * bh * 2 * ((p.d + 32 * tcq - 1) / (32 * tcq));
+  if (5 * big >= (tcq == 1 ? 10 : 3) * sms) switch (tcq) {
+    case 1: return launch_compress<T, TO, 8, 1>(c, dst, K, V, s, phi_j0, n_len);
+    case 2: return launch_compress<T, TO, 8, 2>(c, dst, K, V, s, phi_j0, n_len);
+    default: return launch_compress<T, TO, 8, 3>(c, dst, K, V, s, phi_j0, n_len);
+  }
+  if ((p.m + 7) / 8 * bh * 2 * ((p.d + 31) / 32) <= sms) return launch_compress<T, TO, 2, 1>(c, dst, K, V, s, phi_j0, n_len);
+  return launch_compress<T, TO, 4, 1>(c, dst, K, V, s, phi_j0, n_len);
+}
+
+template <typename T, int DP, int TR>
+cudaError_t launch_attend(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
+  using L = AttendSmem<DP, TR>;
+  static DeviceFlags opt_in;
+  cudaError_t e = ensure_dynamic_smem(ffma_attend_kernel<T, DP, TR>, L::kFloatsUntied * 4, a.device, opt_in);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)a.BH);
+  ffma_attend_kernel<T, DP, TR><<<grid, kThreads, (a.layer_stride ? L::kFloatsUntied : L::kFloats) * 4, s>>>((T*)out, (const T*)Q,
+                                                                                                           (const T*)kv, a);
+  return cudaGetLastError();
+}
+
+template <typename T, int DP>
+cudaError_t attend_rows(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
+  // the smallest tile that still gives every SM a CTA of its own: measured (d = 64, m = 96, T = 10; 16 / 32 / 64 rows per
+  // CTA) at 1024 rows 15.9 / 21.2 / 31.9 us, at 4096 rows 25.2 / 22.3 / 32.9 us, at 16384 rows 80.9 / 65.9 / 55.0 us
+  if ((a.nq + 15) / 16 * a.BH <= a.sms) return launch_attend<T, DP, 1>(a, Q, kv, out, s);
+  if ((a.nq + 31) / 32 * a.BH <= a.sms) return launch_attend<T, DP, 2>(a, Q, kv, out, s);
+  return launch_attend<T, DP, 4>(a, Q, kv, out, s);
+}
+
+template <typename T>
+cudaError_t attend_t(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
+  if (a.d <= 32) return attend_rows<T, 32>(a, Q, kv, out, s);
+  if (a.d <= 64) return attend_rows<T, 64>(a, Q, kv, out, s);
+  if (a.d <= 96) return attend_rows<T, 96>(a, Q, kv, out, s);
+  return attend_rows<T, 128>(a, Q, kv, out, s);
+}
+
+}  // namespace
+
+cudaError_t launch_ffma_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
+                                 float* partial) {
+  if (c->p.dtype == CSAT_DTYPE_FP32)
+    return compress_t<float, float>(c, partial ? partial : (float*)c->kv, K, V, s, phi_j0, n_len);
+  return partial ? compress_t<__nv_bfloat16, float>(c, partial, K, V, s, phi_j0, n_len)
+                 : compress_t<__nv_bfloat16, __nv_bfloat16>(c, (__nv_bfloat16*)c->kv, K, V, s, phi_j0, n_len);
+}
+
+cudaError_t launch_ffma_attend(const FfmaAttend& a, int dtype, const void* Q, const void* kv, void* out, cudaStream_t s) {
+  return dtype == CSAT_DTYPE_FP32 ? attend_t<float>(a, Q, kv, out, s) : attend_t<__nv_bfloat16>(a, Q, kv, out, s);
+}
+
+}  // namespace csat

@@ -1,5 +1,5 @@
-// Plain FFMA kernels for the CSAT forward: the float32 path (and bf16 storage with head sizes the
-// tensor-core kernels do not cover).  Accumulation, softmax and the recovery iterates are float32.
+// Plain FFMA kernels for the CSAT forward at head sizes above 128 (smaller ones: ffma_forward.cu), the float32 stages'
+// launchers, and the entry point that allocates nothing.  Accumulation, softmax and the recovery iterates are float32.
 //
 // Paper equations, in order: K~ = Phi K, V~ = Phi V (compress_kernel); A~ = softmax(Q K~^T / sqrt(d_k)),
 // Z = A~ V~, alpha^{t+1} = eta_theta(S alpha^t + B Z_i), C^_i = Psi alpha^_i (attend_recover_kernel).
@@ -283,7 +283,6 @@ cudaError_t compress_t(csat_ctx* c, const void* K, const void* V, cudaStream_t s
   const int d = (int)p.d;
   const dim3 grid((unsigned)((p.m + kCmpRows - 1) / kCmpRows), (unsigned)(p.B * p.H));
   const size_t sm = (size_t)(2 * kCmpRows * (kCmpChunk + 1) + kCmpChunk * 2 * d) * sizeof(float);
-  const int kc = (2 * d + 31) / 32;
 #define CSAT_CMP(KC)                                                                                                  \
   do {                                                                                                                \
     if (partial)                                                                                                      \
@@ -295,9 +294,7 @@ cudaError_t compress_t(csat_ctx* c, const void* K, const void* V, cudaStream_t s
                                                       p.n_pad, p.m, d, (int)p.H, p.separate_phi ? (int)p.H : 0,      \
                                                       phi_j0);                                                        \
   } while (0)
-  if (kc <= 4) CSAT_CMP(4);
-  else if (kc <= 8) CSAT_CMP(8);
-  else CSAT_CMP(16);
+  CSAT_CMP(16);
 #undef CSAT_CMP
   return cudaGetLastError();
 }
@@ -309,7 +306,19 @@ cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
   const dim3 grid((unsigned)((p.nq + kAttWarps - 1) / kAttWarps), (unsigned)(p.B * p.H));
   const size_t sm = (size_t)(32 * (2 * d + 1) + kAttWarps * d) * sizeof(float);
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)d));
-  const int dc = (d + 31) / 32;
+  if (d <= kFfmaMaxD) {
+    FfmaAttend a;
+    a.S = c->w_untied ? c->Sl_dec : c->S_dec;
+    a.B = c->w_untied ? c->Bl_dec : c->B_dec;
+    a.theta = c->thr();
+    a.psi = c->psi ? c->psi_f32 : nullptr;
+    a.layer_stride = c->w_untied ? p.H * p.d * p.d : 0;
+    a.nq = p.nq; a.m = p.m; a.BH = p.B * p.H;
+    a.theta_stride = c->thr_stride();
+    a.d = d; a.H = (int)p.H; a.T = p.T; a.device = c->device; a.sms = c->sms;
+    a.scale = scale;
+    return launch_ffma_attend(a, p.dtype, Q, c->kv, out, s);
+  }
   cudaError_t e = cudaSuccess;
 #define CSAT_ATT(DC)                                                                                              \
   do {                                                                                                            \
@@ -323,9 +332,7 @@ cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
           c->psi ? c->psi_f32 : nullptr,                                                                         \
           p.nq, p.m, d, (int)p.H, p.T, scale);                                                                    \
   } while (0)
-  if (dc <= 2) CSAT_ATT(2);
-  else if (dc <= 4) CSAT_ATT(4);
-  else CSAT_ATT(8);
+  CSAT_ATT(8);
 #undef CSAT_ATT
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -336,6 +343,7 @@ cudaError_t launch_simt_compress(csat_ctx* c, const void* K, const void* V, cuda
                                  int64_t phi_j0, int64_t n_len, float* partial) {
   *launches += 1;
   if (n_len <= 0) n_len = c->p.n;
+  if (c->p.d <= kFfmaMaxD) return launch_ffma_compress(c, K, V, s, phi_j0, n_len, partial);
   return c->p.dtype == CSAT_DTYPE_FP32 ? compress_t<float>(c, K, V, s, phi_j0, n_len, partial)
                                        : compress_t<__nv_bfloat16>(c, K, V, s, phi_j0, n_len, partial);
 }
@@ -380,6 +388,7 @@ cudaError_t launch_split_kv(const csat_ctx* c, void* kt, void* vt, cudaStream_t 
 // workspace.  See include/csat.h for who needs this and for the rules of use.
 // =============================================================================================
 #include <mutex>
+#include <type_traits>
 
 namespace csat {
 namespace {
@@ -423,9 +432,19 @@ int attend_noalloc_t(const void* Q, const void* K, const void* V, const void* ph
                                                           d, (int)H, total);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (d <= kFfmaMaxD) {
+      FfmaAttend a = {};
+      a.nq = nq; a.m = m; a.BH = B * H;
+      a.d = d; a.H = (int)H; a.device = dev; a.sms = sms;
+      a.scale = scale;
+      if (e == cudaSuccess)
+        e = launch_ffma_attend(a, std::is_same<T, float>::value ? CSAT_DTYPE_FP32 : CSAT_DTYPE_BF16, Q, scratch, out, s);
+    } else {
     const dim3 grid((unsigned)((nq + kAttWarps - 1) / kAttWarps), (unsigned)(B * H));
     const size_t sm = (size_t)(32 * (2 * d + 1) + kAttWarps * d) * sizeof(float);
-    const int dc = (d + 31) / 32;
 #define CSAT_NOALLOC_ATT(DC)                                                                                        \
   do {                                                                                                              \
     if (sm > 48 * 1024)                                                                                             \
@@ -436,10 +455,9 @@ int attend_noalloc_t(const void* Q, const void* K, const void* V, const void* ph
                                                                     nullptr, nq, m, d,                              \
                                                                     (int)H, /*T_iters=*/0, scale);                  \
   } while (0)
-    if (dc <= 2) CSAT_NOALLOC_ATT(2);
-    else if (dc <= 4) CSAT_NOALLOC_ATT(4);
-    else CSAT_NOALLOC_ATT(8);
+    CSAT_NOALLOC_ATT(8);
 #undef CSAT_NOALLOC_ATT
+    }
     if (e == cudaSuccess) e = cudaGetLastError();
   }
   if (e != cudaSuccess) {

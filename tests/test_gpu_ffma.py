@@ -1,0 +1,64 @@
+"""The float32 kernels at the edges of their tiles, against the float64 oracle: every padded head size (32, 64, 96, 128 and
+beyond), every number of rows per CTA (by the number of queries), every tile of the compression (by batch and heads), ragged
+measurement and token counts, with and without a dictionary, one decoder for all layers and one per layer."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import csat_oracle as orc
+from paper_2507_02957_b200 import workloads as wl
+from gpu_util import TOL, device_inputs, make_ctx, rel_err, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+# Sums of at most n + m + T d < 2000 terms in float32 (2^-24 each): a few 1e-6 of the result for random signs (the forward's
+# common bar is 1e-4).  bf16 storage: the common bar.
+BAR = {"fp32": 2e-5, "bf16": TOL["bf16"]}
+
+#         B  H   n    n_q   m    d
+SHAPES = [(1, 1, 65, 1, 33, 8),
+          (2, 3, 130, 77, 32, 32),       # 16 rows per CTA, 8 x 32 tiles of the compression
+          (2, 8, 197, 150, 64, 40),      # 32 rows
+          (2, 8, 200, 257, 97, 64),      # 64 rows, a lone row in the last CTA
+          (3, 16, 150, 65, 96, 32),
+          (4, 16, 143, 129, 101, 64),    # 32 x 64 tiles of the compression
+          (4, 8, 160, 130, 96, 72),
+          (2, 12, 111, 100, 100, 96),
+          (1, 2, 300, 33, 131, 104),
+          (4, 8, 129, 90, 128, 128),
+          (1, 2, 150, 40, 140, 136)]     # beyond the tiled kernels
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "B%dH%d_n%d_nq%d_m%d_d%d" % s)
+def test_forward_at_the_edges_of_the_tiles(shape, dtype):
+    B, H, n, nq, m, d = shape
+    w = wl.Workload("edges", B, H, n, nq, d, m, dtype, 4, 0.01, "iid", 900 + d)
+    inp = wl.make_inputs(w)
+    Q, K, V, _ = device_inputs(w, inp)
+    ctx = make_ctx(w)
+    ctx.set(force_simt=1)                                   # bf16 with d in {64, 128} on these kernels as well
+    phi = to_np(ctx.get_phi())
+    r = np.random.default_rng(7)
+    Psi = wl.round_to_storage((np.eye(d) + 0.3 * r.standard_normal((d, d)) / np.sqrt(d)).astype(np.float32), dtype)
+    S = wl.round_to_storage((0.6 * np.eye(d) + 0.4 * r.standard_normal((4, H, d, d)) / np.sqrt(d)).astype(np.float32), dtype)
+    Bm = wl.round_to_storage((r.standard_normal((4, H, d, d)) / np.sqrt(d)).astype(np.float32), dtype)
+    th = np.full((4, H), 0.02, np.float32) * r.uniform(0.5, 1.5, size=(4, H)).astype(np.float32)
+
+    def check(**kw):
+        ref = orc.csat_forward(inp["Q"], inp["K"], inp["V"], phi, **kw)
+        out = to_np(ctx.forward(Q, K, V))
+        assert np.isfinite(out).all() and np.abs(ref).max() > 0
+        assert rel_err(out, ref) <= BAR[dtype], (shape, kw.keys(), rel_err(out, ref))
+
+    ctx.set(T=0)
+    check(T=0, lam=0.0)
+    for T in (1, 4):
+        ctx.set(T=T, lam=0.001)
+        check(T=T, lam=0.001)
+    ctx.set_dictionary(to_dev(Psi, dtype))
+    check(T=4, lam=0.001, Psi=Psi.astype(np.float64))
+    ctx.set_lista_layer_weights(to_dev(S, dtype), to_dev(Bm, dtype), torch.from_numpy(th).cuda())
+    check(T=4, lam=0.0, Psi=Psi.astype(np.float64),
+          weights=(S.astype(np.float64), Bm.astype(np.float64), list(th.astype(np.float64))))
+    ctx.close()
