@@ -4,8 +4,8 @@
 // V~ = Phi V).  The paper trains through the unrolled decoder but prints no backward pass; eta_theta has derivative
 // 1 where |x| > theta and 0 elsewhere.
 //
-// First CUDA version: plain FFMA kernels, float32 arithmetic, nothing stored by the forward.  After the
-// compression (the forward's own kernel) three kernels run:
+// launch_backward picks the kernels: the tensor-core stages (bf16, d in {64, 128}), ffma_backward.cu (d <= 128), or the
+// plain FFMA kernels below (larger d; float32 arithmetic, nothing stored by the forward):
 //   transpose_kernel: float32 transposes of the decoder matrices S_t, B_t, so that every product below reads its
 //                     matrix row by row (coalesced).
 //   bwd_rows_kernel : one warp per query row.  Recomputes the row's scores, softmax statistics and Z, runs the
@@ -15,10 +15,8 @@
 //                     Stores dZ, L = log sum exp of the row's scores and D = <dZ, Z>, then sweeps K~|V~ again:
 //                     p = exp(s - L), dS = p (dZ . V~_r - D), dQ = scale sum_r dS_r K~_r.
 //   bwd_cols_kernel : one warp per measurement r, all query rows in turn (deterministic, no atomics):
-//                     dK~_r = scale sum_i dS_ir Q_i,  dV~_r = sum_i p_ir dZ_i  (bf16 contexts with d in {64, 128}
-//                     run this stage on the tensor cores instead: bwd_cols_sm100.cu).
-//   bwd_phiT_kernel : dK = Phi^T dK~, dV = Phi_V^T dV~  (bf16 contexts with d in {64, 128} run this product on the
-//                     tensor cores instead: phiT_sm100.cu, from a bf16 copy of dK~|dV~).
+//                     dK~_r = scale sum_i dS_ir Q_i,  dV~_r = sum_i p_ir dZ_i.
+//   bwd_phiT_kernel : dK = Phi^T dK~, dV = Phi_V^T dV~.
 #include "csat_internal.h"
 
 namespace csat {
@@ -96,7 +94,7 @@ __global__ void expand_masks_kernel(uint32_t* __restrict__ out, const uint32_t* 
 
 template <typename T, int DC>   // DC = ceil(d / 32)
 __global__ void __launch_bounds__(kRowWarps * 32) bwd_rows_kernel(
-    T* __restrict__ dQ, float* __restrict__ ws_dZ, __nv_bfloat16* __restrict__ ws_dZ16, float* __restrict__ ws_LD,
+    T* __restrict__ dQ, float* __restrict__ ws_dZ, float* __restrict__ ws_LD,
     const T* __restrict__ Q,
     const T* __restrict__ G, const T* __restrict__ kv, const float* __restrict__ S_dec, const float* __restrict__ B_dec,
     const float* __restrict__ S_decT, const float* __restrict__ B_decT, int64_t layer_stride, const float* __restrict__ theta, int theta_stride, const float* __restrict__ psi_f32,
@@ -227,10 +225,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) bwd_rows_kernel(
     const int col = lane + 32 * j;
     if (col < d) {
       dzr[col] = dz[j];
-      if (live) {
-        ws_dZ[grow * d + col] = dz[j];
-        if (ws_dZ16) ws_dZ16[grow * d + col] = __float2bfloat16_rn(dz[j]);     // operand of the tensor-core stage
-      }
+      if (live) ws_dZ[grow * d + col] = dz[j];
     }
   }
   if (live && lane == 0) { ws_LD[grow * 2] = L; ws_LD[grow * 2 + 1] = Dr; }
@@ -400,7 +395,7 @@ __global__ void __launch_bounds__(256) bwd_phiT_kernel(T* __restrict__ dK, T* __
 template <typename T>
 cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s, int* launches) {
   const Params& p = c->p;
-  const int d = (int)p.d, dc = (d + 31) / 32;
+  const int d = (int)p.d;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)d));
   const unsigned BH = (unsigned)(p.B * p.H);
   const float* Sd = c->w_untied ? c->Sl_dec : c->S_dec;
@@ -431,6 +426,7 @@ cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, v
     if ((e = launch_sm100_bwd_cols(c, Q, s, launches)) != cudaSuccess) return e;
     return launch_sm100_phiT(c, c->bw_dKV16, dK, dV, s, launches);
   }
+  if (p.d <= kFfmaMaxD) return launch_ffma_backward(c, Q, G, dQ, dK, dV, s, launches);
   const int64_t mats = (c->w_untied ? c->w_layers : 1) * p.H;
   float* SdT = c->bw_WT;
   float* BdT = c->bw_WT + mats * d * d;
@@ -451,22 +447,13 @@ cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, v
       e = cudaFuncSetAttribute(bwd_rows_kernel<T, DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);        \
     if (e == cudaSuccess)                                                                                            \
       bwd_rows_kernel<T, DC><<<grid, kRowWarps * 32, sm, s>>>(                                                       \
-          (T*)dQ, c->bw_dZ, tc_stages ? c->bw_dZ16 : nullptr, c->bw_LD, (const T*)Q, (const T*)G, (const T*)c->kv, Sd, Bd, SdT, BdT, lstride, c->thr(), \
+          (T*)dQ, c->bw_dZ, c->bw_LD, (const T*)Q, (const T*)G, (const T*)c->kv, Sd, Bd, SdT, BdT, lstride, c->thr(), \
           c->thr_stride(), c->psi ? c->psi_f32 : nullptr, p.nq, p.m, d, (int)p.H, p.T, scale, c->bw_masks);          \
   } while (0)
-    if (dc <= 2) CSAT_BWD_ROWS(2);
-    else if (dc <= 4) CSAT_BWD_ROWS(4);
-    else CSAT_BWD_ROWS(8);
+    CSAT_BWD_ROWS(8);
 #undef CSAT_BWD_ROWS
     if (e != cudaSuccess) return e;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (tc_stages) {
-    // dK~, dV~ and dK, dV on the tensor cores
-    if ((e = launch_sm100_bwd_cols(c, Q, s, launches)) != cudaSuccess) return e;
-    if ((e = launch_sm100_phiT(c, c->bw_dKV16, dK, dV, s, launches)) != cudaSuccess) return e;
-    *launches += 1;
-    return cudaSuccess;
   }
   {
     const dim3 grid((unsigned)((p.m + kColWarps - 1) / kColWarps), BH);
@@ -474,9 +461,7 @@ cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, v
 #define CSAT_BWD_COLS(DC)                                                                                            \
   bwd_cols_kernel<T, DC><<<grid, kColWarps * 32, sm, s>>>(c->bw_dKV, (const T*)Q, (const T*)c->kv, c->bw_dZ, c->bw_LD, \
                                                          p.nq, p.m, d, scale)
-    if (dc <= 2) CSAT_BWD_COLS(2);
-    else if (dc <= 4) CSAT_BWD_COLS(4);
-    else CSAT_BWD_COLS(8);
+    CSAT_BWD_COLS(8);
 #undef CSAT_BWD_COLS
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -243,6 +243,10 @@ cudaError_t launch_project(csat_ctx* c, const void* X, const void* W, int64_t n_
 cudaError_t launch_backward(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s,
                             int* launches);
 
+// ffma_backward.cu : the float32 stages of the same for d <= kFfmaMaxD (launch_backward sends them there)
+cudaError_t launch_ffma_backward(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s,
+                                 int* launches);
+
 // bwd_cols_sm100.cu : dK~ = scale dS^T Q, dV~ = P^T dZ on the tensor cores (bf16, d in {64, 128}); reads bw_dZ16,
 // bw_LD and the K~|V~ workspace, writes bw_dKV and bw_dKV16
 cudaError_t launch_sm100_bwd_cols(csat_ctx* c, const void* Q, cudaStream_t s, int* launches);

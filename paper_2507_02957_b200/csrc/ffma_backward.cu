@@ -1,0 +1,607 @@
+// The float32 backward for head sizes up to 128 (float32 contexts, and bf16 storage with head sizes that have no
+// tensor-core kernel): the chain rule through the forward's equations, last to first, all sums in float32.
+//   ffma_bwd_rows : a few query rows per warp.  Scores, softmax statistics and Z again, the recurrence forward with one
+//                   decision bit per layer and column, then backward: d alpha_T = G Psi, dx_t = d alpha_{t+1} o mask_t,
+//                   d alpha_t = dx_t S_t^T, dZ = sum_t dx_t B_t^T; L = log sum exp, D = <dZ, Z>; then over the
+//                   measurements again dS = p (dZ V~_r - D), dQ = scale dS K~.
+//   ffma_bwd_cols : a few measurements per CTA, the queries shared out between its warps (a fixed order, no atomics):
+//                   dK~ = scale dS^T Q, dV~ = P^T dZ.
+//   ffma_phiT     : dK = Phi^T dK~, dV = Phi_V^T dV~.
+// Bound: shared-memory reads and the FMA pipe (ffma_tile.cuh); for small jobs the chain of waits of one warp.  Measured
+// against kernels with one warp per row (one B200, 16 heads of 512 x 64, m = 96, T = 10, float32): rows 344 -> 73,
+// columns 158 -> 33, Phi^T 16.6 -> 8.0 us.
+#include "csat_internal.h"
+#include "ffma_tile.cuh"
+
+namespace csat {
+namespace {
+
+using namespace ffma;
+
+struct RowsArgs {
+  const float *S, *B, *theta, *psi;
+  int64_t layer_stride, nq, m;
+  int theta_stride, d, H, T;
+  float scale;
+  float *dZ, *LD;
+  uint32_t* masks;                        // may be null
+};
+
+template <int DP, int TR> struct RowsSmem {                 // in floats
+  static constexpr int kRows = kWarps * 4 * TR, kBuf = kRows * Ld<DP>::kA;
+  static constexpr int kS = 2 * kChunk * Ld<DP>::kB;         // after Ks | Vs (and the blocks of the decoder matrices)
+  static constexpr int kQ = kS + DP * Ld<DP>::kB;
+  static constexpr int kA = kQ + kBuf;                       // the operand of the products: alpha, dx
+  static constexpr int kZ = kA + kBuf;
+  static constexpr int kD = kZ + kBuf;                       // c = z B, then the sum of dx (one B) or dZ (one B per layer)
+  static constexpr int kP = kD + kBuf;
+  static constexpr int kM = kP + kRows * kPLd;               // decisions (DP <= 64)
+  static constexpr int kFloats = kM + (DP <= 64 ? kBuf : 0);
+};
+
+template <typename T, int DP, int TR>
+__global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__ dQ, const T* __restrict__ Q, const T* __restrict__ G,
+                                                                 const T* __restrict__ kv, const RowsArgs p) {
+  using L = RowsSmem<DP, TR>;
+  constexpr int kLdA = Ld<DP>::kA, kLdB = Ld<DP>::kB, kTCQ = DP / 32, kRW = 4 * TR, kTC = kChunk / 8;
+  extern __shared__ __align__(16) float rows_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+  const int bh = blockIdx.y, h = bh % p.H, d = p.d;
+  const int64_t row0 = (int64_t)blockIdx.x * L::kRows + warp * kRW;
+  float* Ks = rows_smem;
+  float* Vs = rows_smem + kChunk * kLdB;
+  float* Ss = rows_smem + L::kS;
+  const int own = warp * kRW * kLdA;                        // the warp's rows in every row buffer
+  float *Arows = rows_smem + L::kA + own, *Drows = rows_smem + L::kD + own;
+  float *Qw = rows_smem + L::kQ + own + ty * kLdA, *Aw = Arows + ty * kLdA;
+  float *Zw = rows_smem + L::kZ + own + ty * kLdA, *Dw = Drows + ty * kLdA;
+  float* Pw = rows_smem + L::kP + (warp * kRW + ty) * kPLd;
+  const T* kvb = kv + (int64_t)bh * p.m * 2 * d;
+  const bool untied = p.layer_stride != 0;
+  const int64_t hdd = (int64_t)h * d * d;
+
+  if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
+  load_own_rows<T>(rows_smem + L::kQ + own, kLdA, Q + (int64_t)bh * p.nq * d, row0, p.nq, d, kRW, lane, d);
+  __syncwarp();
+
+  float2 a[TR][2 * kTCQ];
+  float lse[TR];
+  {
+    float mx[TR], sum[TR];
+    softmax_rows<T, DP, TR>(a, mx, sum, Ks, Vs, Qw, Pw, kvb, p.m, d, p.scale);
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+      const float inv = 1.f / sum[i];
+#pragma unroll
+      for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = __fmul2_rn(a[i][j], dup(inv));
+      lse[i] = mx[i] + logf(sum[i]);                        // log sum exp of the row's scaled scores
+    }
+  }
+  store_rows<TR, kTCQ>(Zw, kLdA, tx, a);
+  __syncwarp();
+
+  // ---- recurrence forward (decisions), then backward; dZ ends in the rows at dz ----
+  float* dz = Aw;
+  auto load_G = [&]() { load_own_rows<T>(Arows, kLdA, G + (int64_t)bh * p.nq * d, row0, p.nq, d, kRW, lane, d); };
+  if (p.T == 0) {
+    load_G();
+  } else {
+    float2 c[TR][2 * kTCQ];
+    clear(c);
+    times_matrix<TR, kTCQ>(c, Zw, kLdA, p.B + hdd, d, Ks, kLdB, tx);
+    clear_beyond<TR, kTCQ>(c, d, tx);                       // RegMatrix reads whole rows
+    float th = p.theta[h];
+    // d alpha_T = G Psi into the operand rows
+    auto start_backward = [&]() {
+      __syncwarp();
+      load_G();
+      __syncwarp();
+      if (p.psi) {
+        clear(c);
+        times_matrix<TR, kTCQ>(c, Aw, kLdA, p.psi + hdd, d, Ks, kLdB, tx);
+        clear_beyond<TR, kTCQ>(c, d, tx);
+        __syncwarp();
+        store_rows<TR, kTCQ>(Aw, kLdA, tx, c);
+        __syncwarp();
+      }
+    };
+    if (DP <= 64 && !untied) {
+      // one S for all layers, in registers; the rows' state (operand, c or the sum of dx, decisions) in shared memory, the
+      // lane's columns those of RegMatrix
+      constexpr int kDR = DP <= 64 ? DP : 64, kNC = RegMatrix<kDR>::NC, kN = 4;
+      uint32_t* Mrows = reinterpret_cast<uint32_t*>(rows_smem + (DP <= 64 ? L::kM : 0)) + own;
+      const int col = RegMatrix<kDR>::col(tx, ty);
+      store_rows<TR, kTCQ>(Dw, kLdA, tx, c);
+      __syncwarp();
+      for (int r = 0; r < kRW; ++r)
+#pragma unroll
+        for (int j = 0; j < kNC; ++j) {
+          const int at = r * kLdA + col + 8 * j;
+          const float x = Drows[at];
+          Mrows[at] = fabsf(x) > th ? 1u : 0u;
+          Arows[at] = shrink(x, th);
+        }
+      {
+        RegMatrix<kDR> S;
+        if (p.T > 1) S.load(Ss, kLdB, d, tx, ty);
+        for (int it = 1; it < p.T; ++it) {
+          th = p.theta[(int64_t)it * p.theta_stride + h];
+          __syncwarp();
+#pragma unroll 1
+          for (int r = 0; r < kRW; r += kN) {
+            float y[kN][kNC];
+            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+#pragma unroll
+            for (int u = 0; u < kN; ++u)
+#pragma unroll
+              for (int j = 0; j < kNC; ++j) {
+                const int at = (r + u) * kLdA + col + 8 * j;
+                const float x = y[u][j] + Drows[at];
+                if (fabsf(x) > th) Mrows[at] |= 1u << it;
+                Arows[at] = shrink(x, th);
+              }
+          }
+        }
+      }
+      start_backward();
+      for (int r = 0; r < kRW; ++r)
+#pragma unroll
+        for (int j = 0; j < kNC; ++j) {
+          const int at = r * kLdA + col + 8 * j;
+          const uint32_t mk = Mrows[at];
+          const float dx = (mk >> (p.T - 1)) & 1u ? Arows[at] : 0.f;
+          Drows[at] = dx;
+          Arows[at] = dx;
+          if (p.masks && row0 + r < p.nq && col + 8 * j < d)
+            p.masks[((int64_t)bh * p.nq + row0 + r) * d + col + 8 * j] = mk;     // bit t: |x_t| > theta_t
+        }
+      {
+        RegMatrix<kDR> S;
+        if (p.T > 1) S.load_transposed(Ss, kLdB, d, tx, ty);
+        for (int it = p.T - 2; it >= 0; --it) {
+          __syncwarp();
+#pragma unroll 1
+          for (int r = 0; r < kRW; r += kN) {
+            float y[kN][kNC];
+            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+#pragma unroll
+            for (int u = 0; u < kN; ++u)
+#pragma unroll
+              for (int j = 0; j < kNC; ++j) {
+                const int at = (r + u) * kLdA + col + 8 * j;
+                const float dx = (Mrows[at] >> it) & 1u ? y[u][j] : 0.f;
+                Drows[at] += dx;
+                Arows[at] = dx;
+              }
+          }
+        }
+      }
+      __syncwarp();
+      times_transposed<TR>(Aw, Dw, kLdA, p.B + hdd, d, Ks, kLdB, tx, false);       // dZ = (sum_t dx_t) B^T
+    } else {
+      uint32_t mask[TR][4 * kTCQ];
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < 2 * kTCQ; ++j) {
+          mask[i][2 * j] = fabsf(c[i][j].x) > th ? 1u : 0u;
+          mask[i][2 * j + 1] = fabsf(c[i][j].y) > th ? 1u : 0u;
+          a[i][j] = shrink(c[i][j], th);
+        }
+      for (int it = 1; it < p.T; ++it) {
+        th = p.theta[(int64_t)it * p.theta_stride + h];
+        if (untied) {
+          clear(c);
+          times_matrix<TR, kTCQ>(c, Zw, kLdA, p.B + it * p.layer_stride + hdd, d, Ks, kLdB, tx);
+          stage_matrix_async(Ss, kLdB, p.S + it * p.layer_stride + hdd, d, 0, d);
+          cp_async_wait_all();
+          __syncthreads();
+        }
+        __syncwarp();
+        store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int j = 0; j < 2 * kTCQ; ++j) a[i][j] = c[i][j];
+        gemm_t<TR, kTCQ>(a, Aw, kLdA, Ss + 4 * tx, kLdB, d);
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int j = 0; j < 2 * kTCQ; ++j) {
+            if (fabsf(a[i][j].x) > th) mask[i][2 * j] |= 1u << it;
+            if (fabsf(a[i][j].y) > th) mask[i][2 * j + 1] |= 1u << it;
+            a[i][j] = shrink(a[i][j], th);
+          }
+      }
+      if (p.masks)
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int q = 0; q < kTCQ; ++q)
+            if (row0 + ty + 4 * i < p.nq && 4 * tx + 32 * q < d)
+              *reinterpret_cast<uint4*>(p.masks + ((int64_t)bh * p.nq + row0 + ty + 4 * i) * d + 4 * tx + 32 * q) =
+                  make_uint4(mask[i][4 * q], mask[i][4 * q + 1], mask[i][4 * q + 2], mask[i][4 * q + 3]);
+      start_backward();
+      float2 sum[TR][2 * kTCQ];
+      clear(sum);
+      for (int it = p.T - 1; it >= 0; --it) {
+        // the operand rows hold d alpha_{it + 1}
+        load_rows<TR, kTCQ>(a, Aw, kLdA, tx);
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int j = 0; j < 2 * kTCQ; ++j) {
+            a[i][j].x = (mask[i][2 * j] >> it) & 1u ? a[i][j].x : 0.f;
+            a[i][j].y = (mask[i][2 * j + 1] >> it) & 1u ? a[i][j].y : 0.f;
+            sum[i][j] = __fadd2_rn(sum[i][j], a[i][j]);
+          }
+        __syncwarp();
+        store_rows<TR, kTCQ>(Aw, kLdA, tx, a);              // dx
+        __syncwarp();
+        if (untied) times_transposed<TR>(Dw, Aw, kLdA, p.B + it * p.layer_stride + hdd, d, Ks, kLdB, tx, it != p.T - 1);
+        if (it > 0) {
+          if (untied) {
+            __syncthreads();
+            stage_matrix_async(Ss, kLdB, p.S + it * p.layer_stride + hdd, d, 0, d);
+            cp_async_wait_all();
+            __syncthreads();
+          }
+          float2 y[TR][DP / 8];
+          clear(y);
+          gemm_n<TR, DP / 8>(y, Aw, kLdA, Ss + tx * kLdB, kLdB, d);     // d alpha_it = dx S^T
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < TR; ++i)
+#pragma unroll
+            for (int j = 0; j < DP / 8; ++j) Aw[4 * i * kLdA + tx + 8 * j] = y[i][j].x + y[i][j].y;
+          __syncwarp();
+        }
+      }
+      if (untied) {
+        dz = Dw;
+      } else {
+        store_rows<TR, kTCQ>(Dw, kLdA, tx, sum);
+        __syncwarp();
+        times_transposed<TR>(Aw, Dw, kLdA, p.B + hdd, d, Ks, kLdB, tx, false);
+      }
+    }
+  }
+  __syncwarp();
+  float Dr[TR];
+#pragma unroll
+  for (int i = 0; i < TR; ++i) {
+    const int64_t row = row0 + ty + 4 * i;
+    float part = 0.f;
+#pragma unroll
+    for (int q = 0; q < kTCQ; ++q)
+      if (4 * tx + 32 * q < d) {
+        const float4 x = *reinterpret_cast<const float4*>(dz + 4 * i * kLdA + 4 * tx + 32 * q);
+        const float4 z = *reinterpret_cast<const float4*>(Zw + 4 * i * kLdA + 4 * tx + 32 * q);
+        part = fmaf(x.x, z.x, fmaf(x.y, z.y, fmaf(x.z, z.z, fmaf(x.w, z.w, part))));
+        if (row < p.nq) *reinterpret_cast<float4*>(p.dZ + ((int64_t)bh * p.nq + row) * d + 4 * tx + 32 * q) = x;
+      }
+    Dr[i] = sum8(part);                                     // <dZ, Z> = rowsum(dA o A)
+    if (tx == 0 && row < p.nq) *reinterpret_cast<float2*>(p.LD + ((int64_t)bh * p.nq + row) * 2) = make_float2(lse[i], Dr[i]);
+  }
+
+  // ---- dS, dQ ----
+  clear(a);
+  PairChunk<T, DP> ch;
+  ch.fetch(kvb, kvb + d, 2 * d, 0, p.m, d);
+  for (int64_t r0 = 0; r0 < p.m; r0 += kChunk) {
+    __syncthreads();
+    ch.put(Ks, Vs, kLdB, d);
+    __syncthreads();
+    if (r0 + kChunk < p.m) ch.fetch(kvb, kvb + d, 2 * d, r0 + kChunk, p.m, d);
+    float2 s2[TR][kTC], v2[TR][kTC];
+    clear(s2);
+    clear(v2);
+    gemm_n<TR, kTC>(s2, Qw, kLdA, Ks + tx * kLdB, kLdB, d);
+    gemm_n<TR, kTC>(v2, dz, kLdA, Vs + tx * kLdB, kLdB, d);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int j = 0; j < kTC; ++j) {
+        const float pr = r0 + tx + 8 * j < p.m ? expf((s2[i][j].x + s2[i][j].y) * p.scale - lse[i]) : 0.f;
+        Pw[4 * i * kPLd + tx + 8 * j] = pr * ((v2[i][j].x + v2[i][j].y) - Dr[i]);
+      }
+    __syncwarp();
+    gemm_t<TR, kTCQ>(a, Pw, kPLd, Ks + 4 * tx, kLdB, kChunk);
+  }
+#pragma unroll
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int q = 0; q < kTCQ; ++q)
+      if (row0 + ty + 4 * i < p.nq && 4 * tx + 32 * q < d)
+        store4(dQ + ((int64_t)bh * p.nq + row0 + ty + 4 * i) * d + 4 * tx + 32 * q, a[i][2 * q].x * p.scale, a[i][2 * q].y * p.scale,
+               a[i][2 * q + 1].x * p.scale, a[i][2 * q + 1].y * p.scale);
+}
+
+// dK~ = scale dS^T Q, dV~ = P^T dZ.  The four warps of a CTA hold the same 4 TR measurements and share out the queries in
+// chunks of CQ: a chunk's operand reads then serve 4 TR measurements instead of TR (with rows of their own and chunks in
+// common 16 heads of 512 x 64, m = 96, took 58 us, bound by the shared-memory reads).  Each warp stages its own chunks one
+// ahead of the arithmetic; the warps' sums are added in warp order.
+template <int DP, int TR, int CQ> struct ColsSmem {          // in floats
+  static constexpr int kRows = 4 * TR, kPLdQ = CQ + 8;
+  static constexpr int kStage = 2 * CQ * Ld<DP>::kB + 2 * CQ;                // Q | dZ | (L, D) of a chunk
+  static constexpr int kWarp = 2 * kStage + 2 * kRows * kPLdQ;              // two chunks, P, dS
+  static constexpr int kK = kWarps * kWarp, kV = kK + kRows * Ld<DP>::kA;
+  static constexpr int kFloats = kV + kRows * Ld<DP>::kA;
+  static_assert(2 * kRows * DP <= kWarp, "a warp's sums fit where its chunks were");
+};
+
+template <typename T> struct StageRows {                    // rows x d values to shared memory by one warp
+  static __device__ __forceinline__ void run(float* dst, int ld, const T* src, int rows, int have, int d, int lane) {
+    constexpr int kN = Vec<T>::kN;
+    const int vpr = d / kN;
+    for (int i = lane; i < rows * vpr; i += 32) {
+      const int r = i / vpr, c = (i - r * vpr) * kN;
+      float f[kN];
+      Vec<T>::to_float(r < have ? *reinterpret_cast<const uint4*>(src + (int64_t)r * d + c) : make_uint4(0, 0, 0, 0), f);
+#pragma unroll
+      for (int u = 0; u < kN; u += 4) *reinterpret_cast<float4*>(dst + r * ld + c + u) = make_float4(f[u], f[u + 1], f[u + 2], f[u + 3]);
+    }
+  }
+};
+template <> struct StageRows<float> {
+  static __device__ __forceinline__ void run(float* dst, int ld, const float* src, int rows, int have, int d, int lane) {
+    const int vpr = d / 4;
+    for (int i = lane; i < rows * vpr; i += 32) {
+      const int r = i / vpr, c = (i - r * vpr) * 4;
+      if (r < have) cp_async16(dst + r * ld + c, src + (int64_t)r * d + c);
+      else *reinterpret_cast<float4*>(dst + r * ld + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+};
+
+template <typename T, int DP, int TR, int CQ>
+__global__ void __launch_bounds__(kThreads) ffma_bwd_cols_kernel(float* __restrict__ dKV, const T* __restrict__ Q, const T* __restrict__ kv,
+                                                                 const float* __restrict__ dZ, const float* __restrict__ LD, int64_t nq,
+                                                                 int64_t m, int d, float scale) {
+  using L = ColsSmem<DP, TR, CQ>;
+  constexpr int kLdA = Ld<DP>::kA, kLdB = Ld<DP>::kB, kTCQ = DP / 32, kTC = CQ / 8;
+  extern __shared__ __align__(16) float cols_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+  const int bh = blockIdx.y;
+  const int64_t r0 = (int64_t)blockIdx.x * L::kRows;        // first measurement
+  float* mine = cols_smem + warp * L::kWarp;
+  float *Pw = mine + 2 * L::kStage + ty * L::kPLdQ, *Sw = Pw + L::kRows * L::kPLdQ;
+  float *Kw = cols_smem + L::kK + ty * kLdA, *Vw = cols_smem + L::kV + ty * kLdA;
+  const T* kvb = kv + (int64_t)bh * m * 2 * d;
+  const T* Qb = Q + (int64_t)bh * nq * d;
+  const float* Gb = dZ + (int64_t)bh * nq * d;
+  const float* LDb = LD + (int64_t)bh * nq * 2;
+  auto stage = [&](int64_t i0, int st) {
+    float* dst = mine + st * L::kStage;
+    const int have = (int)(nq - i0 < CQ ? nq - i0 : CQ);
+    StageRows<T>::run(dst, kLdB, Qb + i0 * d, CQ, have, d, lane);
+    StageRows<float>::run(dst + CQ * kLdB, kLdB, Gb + i0 * d, CQ, have, d, lane);
+    for (int i = lane; i < 2 * CQ; i += 32) dst[2 * CQ * kLdB + i] = (i >> 1) < have ? LDb[i0 * 2 + i] : 0.f;
+  };
+  int64_t i0 = (int64_t)warp * CQ;
+  if (i0 < nq) stage(i0, 0);
+  if (warp == 0) load_own_rows<T>(cols_smem + L::kK, kLdA, kvb, r0, m, d, L::kRows, lane, 2 * d);
+  if (warp == 1) load_own_rows<T>(cols_smem + L::kV, kLdA, kvb + d, r0, m, d, L::kRows, lane, 2 * d);
+  __syncthreads();
+
+  float2 dk[TR][2 * kTCQ], dv[TR][2 * kTCQ];
+  clear(dk);
+  clear(dv);
+  for (int st = 0; i0 < nq; i0 += kWarps * CQ, st ^= 1) {
+    cp_async_wait_all();
+    __syncwarp();
+    if (i0 + kWarps * CQ < nq) stage(i0 + kWarps * CQ, st ^ 1);
+    const float *Qs = mine + st * L::kStage, *Gs = Qs + CQ * kLdB, *ld = Gs + CQ * kLdB;
+    float2 s2[TR][kTC];
+    clear(s2);
+    gemm_n<TR, kTC>(s2, Kw, kLdA, Qs + tx * kLdB, kLdB, d);
+#pragma unroll
+    for (int j = 0; j < kTC; ++j)
+#pragma unroll
+      for (int i = 0; i < TR; ++i) {
+        // a query beyond the end contributes nothing
+        const int q = tx + 8 * j;
+        s2[i][j].x = i0 + q < nq ? expf((s2[i][j].x + s2[i][j].y) * scale - ld[2 * q]) : 0.f;
+        Pw[4 * i * L::kPLdQ + q] = s2[i][j].x;
+      }
+    float2 v2[TR][kTC];
+    clear(v2);
+    gemm_n<TR, kTC>(v2, Vw, kLdA, Gs + tx * kLdB, kLdB, d);
+#pragma unroll
+    for (int j = 0; j < kTC; ++j)
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+        Sw[4 * i * L::kPLdQ + tx + 8 * j] = s2[i][j].x * ((v2[i][j].x + v2[i][j].y) - ld[2 * (tx + 8 * j) + 1]);
+    __syncwarp();
+    gemm_t<TR, kTCQ>(dv, Pw, L::kPLdQ, Gs + 4 * tx, kLdB, CQ);
+    gemm_t<TR, kTCQ>(dk, Sw, L::kPLdQ, Qs + 4 * tx, kLdB, CQ);
+    __syncwarp();
+  }
+  // each warp's sums over its own chunks' place, then all of them in warp order
+  store_rows<TR, kTCQ>(mine + ty * DP, DP, tx, dk);
+  store_rows<TR, kTCQ>(mine + (L::kRows + ty) * DP, DP, tx, dv);
+  __syncthreads();
+  for (int i = threadIdx.x * 4; i < 2 * L::kRows * DP; i += kThreads * 4) {
+    const int is_v = i >= L::kRows * DP, r = i / DP - (is_v ? L::kRows : 0), c = i % DP;
+    if (r0 + r >= m || c >= d) continue;
+    float4 x = *reinterpret_cast<const float4*>(cols_smem + i);
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      const float4 y = *reinterpret_cast<const float4*>(cols_smem + w * L::kWarp + i);
+      x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+    }
+    const float f = is_v ? 1.f : scale;
+    store4(dKV + ((int64_t)bh * m + r0 + r) * 2 * d + (is_v ? d : 0) + c, x.x * f, x.y * f, x.z * f, x.w * f);
+  }
+}
+
+// dK[j][c] = sum_r Phi_K[r][j] dK~[r][c], dV likewise: 128 tokens x 32 TCQ columns per CTA, 32 tokens per warp; Phi's rows
+// run along the tokens, so both operands are read as rows of one k.
+constexpr int kPtTok = 128, kPtK = 16;
+template <typename T, int TCQ>
+__global__ void __launch_bounds__(kThreads) ffma_phiT_kernel(T* __restrict__ dK, T* __restrict__ dV, const T* __restrict__ phi,
+                                                             const float* __restrict__ dKV, int64_t n, int64_t n_pad, int64_t m, int d,
+                                                             int H, int phi_v_head0, int col_blocks) {
+  constexpr int kN = Vec<T>::kN, kCols = 32 * TCQ;
+  __shared__ __align__(16) float As[kPtK][kPtTok], Bs[kPtK][kCols];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+  const int bh = blockIdx.y, h = bh % H, is_v = blockIdx.z >= col_blocks;
+  const int c0 = (blockIdx.z - (is_v ? col_blocks : 0)) * kCols;
+  const int64_t j0 = (int64_t)blockIdx.x * kPtTok;
+  const T* ph = phi + (int64_t)((is_v ? phi_v_head0 : 0) + h) * m * n_pad;
+  const float* g = dKV + (int64_t)bh * m * 2 * d + (is_v ? d : 0);
+  constexpr int kAV = kPtK * kPtTok / kN / kThreads, kBV = kPtK * kCols / 4 / kThreads;
+  uint4 va[kAV];
+  float4 vb[kBV];
+  auto fetch = [&](int64_t r0) {
+#pragma unroll
+    for (int u = 0; u < kAV; ++u) {
+      const int i = threadIdx.x + kThreads * u, r = i / (kPtTok / kN), j = (i % (kPtTok / kN)) * kN;
+      va[u] = make_uint4(0, 0, 0, 0);
+      if (r0 + r < m && j0 + j < n_pad) va[u] = *reinterpret_cast<const uint4*>(ph + (r0 + r) * n_pad + j0 + j);
+    }
+#pragma unroll
+    for (int u = 0; u < kBV; ++u) {
+      const int i = threadIdx.x + kThreads * u, r = i / (kCols / 4), c = c0 + (i % (kCols / 4)) * 4;
+      vb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r0 + r < m && c < d) vb[u] = *reinterpret_cast<const float4*>(g + (r0 + r) * 2 * d + c);
+    }
+  };
+  float2 acc[8][2 * TCQ];                                   // tokens 4 ty + {0..3} and 16 + 4 ty + {0..3} of the warp's 32
+  clear(acc);
+  fetch(0);
+  for (int64_t r0 = 0; r0 < m; r0 += kPtK) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kAV; ++u) {
+      const int i = threadIdx.x + kThreads * u, r = i / (kPtTok / kN), j = (i % (kPtTok / kN)) * kN;
+      float f[kN];
+      Vec<T>::to_float(va[u], f);
+#pragma unroll
+      for (int w = 0; w < kN; w += 4) *reinterpret_cast<float4*>(&As[r][j + w]) = make_float4(f[w], f[w + 1], f[w + 2], f[w + 3]);
+    }
+#pragma unroll
+    for (int u = 0; u < kBV; ++u) {
+      const int i = threadIdx.x + kThreads * u;
+      *reinterpret_cast<float4*>(&Bs[i / (kCols / 4)][(i % (kCols / 4)) * 4]) = vb[u];
+    }
+    __syncthreads();
+    if (r0 + kPtK < m) fetch(r0 + kPtK);
+#pragma unroll 4
+    for (int k = 0; k < kPtK; ++k) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[k][warp * 32 + 4 * ty]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[k][warp * 32 + 16 + 4 * ty]);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+      for (int q = 0; q < TCQ; ++q) {
+        const float4 b = *reinterpret_cast<const float4*>(&Bs[k][4 * tx + 32 * q]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          acc[i][2 * q] = __ffma2_rn(dup(av[i]), make_float2(b.x, b.y), acc[i][2 * q]);
+          acc[i][2 * q + 1] = __ffma2_rn(dup(av[i]), make_float2(b.z, b.w), acc[i][2 * q + 1]);
+        }
+      }
+    }
+  }
+  T* dst = is_v ? dV : dK;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int64_t j = j0 + warp * 32 + 4 * ty + (i & 3) + (i >> 2) * 16;
+#pragma unroll
+    for (int q = 0; q < TCQ; ++q) {
+      const int c = c0 + 4 * tx + 32 * q;
+      if (j < n && c < d)
+        store4(dst + ((int64_t)bh * n + j) * d + c, acc[i][2 * q].x, acc[i][2 * q].y, acc[i][2 * q + 1].x, acc[i][2 * q + 1].y);
+    }
+  }
+}
+
+template <typename T, int DP, int TR>
+cudaError_t launch_rows(csat_ctx* c, const void* Q, const void* G, void* dQ, cudaStream_t s, const RowsArgs& a) {
+  using L = RowsSmem<DP, TR>;
+  static_assert(L::kFloats * 4 <= 227 * 1024, "shared memory budget");
+  static DeviceFlags opt_in;
+  cudaError_t e = ensure_dynamic_smem(ffma_bwd_rows_kernel<T, DP, TR>, L::kFloats * 4, c->device, opt_in);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)(c->p.B * c->p.H));
+  ffma_bwd_rows_kernel<T, DP, TR><<<grid, kThreads, L::kFloats * 4, s>>>((T*)dQ, (const T*)Q, (const T*)G, (const T*)c->kv, a);
+  return cudaGetLastError();
+}
+
+template <typename T, int DP, int TR>
+cudaError_t launch_cols(csat_ctx* c, const void* Q, cudaStream_t s, float scale) {
+  constexpr int CQ = DP <= 64 ? 32 : 16;
+  using L = ColsSmem<DP, TR, CQ>;
+  static_assert(L::kFloats * 4 <= 227 * 1024, "shared memory budget");
+  const Params& p = c->p;
+  static DeviceFlags opt_in;
+  cudaError_t e = ensure_dynamic_smem(ffma_bwd_cols_kernel<T, DP, TR, CQ>, L::kFloats * 4, c->device, opt_in);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((p.m + L::kRows - 1) / L::kRows), (unsigned)(p.B * p.H));
+  ffma_bwd_cols_kernel<T, DP, TR, CQ><<<grid, kThreads, L::kFloats * 4, s>>>(c->bw_dKV, (const T*)Q, (const T*)c->kv, c->bw_dZ, c->bw_LD,
+                                                                           p.nq, p.m, (int)p.d, scale);
+  return cudaGetLastError();
+}
+
+template <typename T, int TCQ>
+cudaError_t launch_phiT(csat_ctx* c, void* dK, void* dV, cudaStream_t s) {
+  const Params& p = c->p;
+  const int cb = (int)((p.d + 32 * TCQ - 1) / (32 * TCQ));
+  const dim3 grid((unsigned)((p.n + kPtTok - 1) / kPtTok), (unsigned)(p.B * p.H), (unsigned)(2 * cb));
+  ffma_phiT_kernel<T, TCQ><<<grid, kThreads, 0, s>>>((T*)dK, (T*)dV, (const T*)c->phi, c->bw_dKV, p.n, p.n_pad, p.m, (int)p.d, (int)p.H,
+                                                    p.separate_phi ? (int)p.H : 0, cb);
+  return cudaGetLastError();
+}
+
+template <typename T, int DP>
+cudaError_t run_d(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s, const RowsArgs& a) {
+  const Params& p = c->p;
+  const int64_t bh = p.B * p.H, sms = c->sms;
+  cudaError_t e;
+  // rows per CTA: 16 where that fills no more than one wave, else 32 (d = 64, T = 10, us: 1024 rows 33 / 50, 4096 rows 52 / 51,
+  // 8192 rows 98 / 73, 32768 rows 330 / 249; with 64 rows 78 / 78 / 79 / 311: two CTAs no longer fit an SM)
+  if ((p.nq + 15) / 16 * bh <= sms) e = launch_rows<T, DP, 1>(c, Q, G, dQ, s, a);
+  else e = launch_rows<T, DP, 2>(c, Q, G, dQ, s, a);
+  if (e != cudaSuccess) return e;
+  // measurements per CTA: the fewest of 4, 8 that fill no more than one wave, else 16 (d = 64, 512 queries, us with 4 / 8 /
+  // 16: 192 measurements in all 25 / 26 / 32, 768 49 / 27 / 33, 1536 73 / 51 / 33, 3072 142 / 76 / 64)
+  if ((p.m + 3) / 4 * bh <= sms) e = launch_cols<T, DP, 1>(c, Q, s, a.scale);
+  else if ((p.m + 7) / 8 * bh <= sms) e = launch_cols<T, DP, 2>(c, Q, s, a.scale);
+  else e = launch_cols<T, DP, 4>(c, Q, s, a.scale);
+  if (e != cudaSuccess) return e;
+  if (p.d <= 32) return launch_phiT<T, 1>(c, dK, dV, s);
+  if (p.d > 64 && p.d <= 96) return launch_phiT<T, 3>(c, dK, dV, s);
+  return launch_phiT<T, 2>(c, dK, dV, s);
+}
+
+template <typename T>
+cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s) {
+  const Params& p = c->p;
+  RowsArgs a;
+  a.S = c->w_untied ? c->Sl_dec : c->S_dec;
+  a.B = c->w_untied ? c->Bl_dec : c->B_dec;
+  a.theta = c->thr();
+  a.psi = c->psi ? c->psi_f32 : nullptr;
+  a.layer_stride = c->w_untied ? p.H * p.d * p.d : 0;
+  a.nq = p.nq; a.m = p.m;
+  a.theta_stride = c->thr_stride();
+  a.d = (int)p.d; a.H = (int)p.H; a.T = p.T;
+  a.scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)p.d));
+  a.dZ = c->bw_dZ; a.LD = c->bw_LD; a.masks = c->bw_masks;
+  if (p.d <= 32) return run_d<T, 32>(c, Q, G, dQ, dK, dV, s, a);
+  if (p.d <= 64) return run_d<T, 64>(c, Q, G, dQ, dK, dV, s, a);
+  if (p.d <= 96) return run_d<T, 96>(c, Q, G, dQ, dK, dV, s, a);
+  return run_d<T, 128>(c, Q, G, dQ, dK, dV, s, a);
+}
+
+}  // namespace
+
+cudaError_t launch_ffma_backward(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, void* dV, cudaStream_t s,
+                                 int* launches) {
+  *launches += 3;
+  return c->p.dtype == CSAT_DTYPE_FP32 ? run<float>(c, Q, G, dQ, dK, dV, s) : run<__nv_bfloat16>(c, Q, G, dQ, dK, dV, s);
+}
+
+}  // namespace csat

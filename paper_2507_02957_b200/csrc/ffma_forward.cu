@@ -174,20 +174,12 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
     __syncwarp();
     store_rows<TR, kTCQ>(Zw, kLdA, tx, a);                  // z as an operand
     float2 c[TR][2 * kTCQ];
-    // c = z B_t; the rows of B pass through the chunk buffers
-    auto times_B = [&](int t) {
-      constexpr int kFit = 2 * kChunk;
+    auto times_B = [&](int t) {                             // c = z B_t
       clear(c);
-      for (int k0 = 0; k0 < d; k0 += kFit) {
-        const int rows = d - k0 < kFit ? d - k0 : kFit;
-        __syncthreads();
-        stage_matrix_async(Ks, kLdB, p.B + t * p.layer_stride + hdd, d, k0, rows);
-        cp_async_wait_all();
-        __syncthreads();
-        gemm_t<TR, kTCQ>(c, Zw + k0, kLdA, Ks + 4 * tx, kLdB, rows);
-      }
+      times_matrix<TR, kTCQ>(c, Zw, kLdA, p.B + t * p.layer_stride + hdd, d, Ks, kLdB, tx);
     };
     times_B(0);
+    if (DP <= 64) clear_beyond<TR, kTCQ>(c, d, tx);         // RegMatrix reads whole rows
     float th = p.theta[h];
 #pragma unroll
     for (int i = 0; i < TR; ++i)
@@ -221,14 +213,7 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
         }
       }
       __syncwarp();
-#pragma unroll
-      for (int i = 0; i < TR; ++i)
-#pragma unroll
-        for (int q = 0; q < kTCQ; ++q) {
-          const float4 x = *reinterpret_cast<const float4*>(Aw + 4 * i * kLdA + 4 * tx + 32 * q);
-          a[i][2 * q] = make_float2(x.x, x.y);
-          a[i][2 * q + 1] = make_float2(x.z, x.w);
-        }
+      load_rows<TR, kTCQ>(a, Aw, kLdA, tx);
     } else
     for (int it = 1; it < p.T; ++it) {
       th = p.theta[(int64_t)it * p.theta_stride + h];

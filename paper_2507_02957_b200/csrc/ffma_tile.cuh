@@ -148,7 +148,8 @@ __device__ __forceinline__ void gemm_n(float2 (&acc)[TR][TC], const float* A, in
 // A DP x DP matrix W (DP <= 64) in the registers of one warp, for products x W with many rows x, one row at a time.
 // Lane (ty, tx) holds W[k][col] for k = 8 u + 2 ty + {0, 1} and col = tx + 8 j, as pairs over k, so that x is read from
 // shared memory as it lies (8 bytes per 2 NJ multiply-adds and lane) and no scalar is duplicated; the four ty add up their
-// shares by a reduce-scatter, after which the lane holds NC = DP / 32 columns tx + 8 (NC ty' + {0 ..}).
+// shares by a reduce-scatter, after which the lane holds NC = DP / 32 columns tx + 8 (NC ty' + {0 ..}).  x has to be zero
+// (at least finite) in the columns beyond d.
 template <int DP> struct RegMatrix {
   static constexpr int NJ = DP / 8, NU = DP / 8, NC = DP / 32;
   float2 w[NU][NJ];
@@ -161,6 +162,16 @@ template <int DP> struct RegMatrix {
         const int k = 8 * u + 2 * ty, c = tx + 8 * j;
         const bool in = k < d && c < d;                    // d is a multiple of 8: k + 1 < d as well
         w[u][j] = in ? make_float2(W[k * ld + c], W[(k + 1) * ld + c]) : make_float2(0.f, 0.f);
+      }
+  }
+  // W = the transpose of the matrix in shared memory
+  __device__ __forceinline__ void load_transposed(const float* W, int ld, int d, int tx, int ty) {
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int k = 8 * u + 2 * ty, c = tx + 8 * j;
+        w[u][j] = k < d && c < d ? *reinterpret_cast<const float2*>(W + c * ld + k) : make_float2(0.f, 0.f);
       }
   }
   // the lane's first column after a product
@@ -259,18 +270,70 @@ __device__ __forceinline__ void stage_matrix_async(float* dst, int ld, const flo
     cp_async16(dst + r * ld + c, W + (int64_t)(k0 + r) * d + c);
   }
 }
-// dst[b][a] = W[a][b]: lanes walk the rows a, so that the scattered stores hit different banks
-__device__ __forceinline__ void stage_matrix_transposed(float* dst, int ld, const float* W, int d) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int a0 = 0; a0 < d; a0 += 32)
-    for (int b = warp * 4; b < d; b += kWarps * 4)
-      if (a0 + lane < d) {
-        const float4 v = *reinterpret_cast<const float4*>(W + (int64_t)(a0 + lane) * d + b);
-        dst[b * ld + a0 + lane] = v.x;
-        dst[(b + 1) * ld + a0 + lane] = v.y;
-        dst[(b + 2) * ld + a0 + lane] = v.z;
-        dst[(b + 3) * ld + a0 + lane] = v.w;
-      }
+// zeroes the columns beyond d (what the products leave there comes from unwritten shared memory)
+template <int TR, int TCQ> __device__ __forceinline__ void clear_beyond(float2 (&v)[TR][2 * TCQ], int d, int tx) {
+#pragma unroll
+  for (int q = 0; q < TCQ; ++q)
+    if (4 * tx + 32 * q >= d)
+#pragma unroll
+      for (int i = 0; i < TR; ++i) v[i][2 * q] = v[i][2 * q + 1] = make_float2(0.f, 0.f);
+}
+
+// the lane's columns of its rows from a buffer (A points at row ty)
+template <int TR, int TCQ>
+__device__ __forceinline__ void load_rows(float2 (&v)[TR][2 * TCQ], const float* A, int lda, int tx) {
+#pragma unroll
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int q = 0; q < TCQ; ++q) {
+      const float4 x = *reinterpret_cast<const float4*>(A + 4 * i * lda + 4 * tx + 32 * q);
+      v[i][2 * q] = make_float2(x.x, x.y);
+      v[i][2 * q + 1] = make_float2(x.z, x.w);
+    }
+}
+
+// acc += (the rows at A) W for a d x d matrix W in global memory, by all warps of the CTA: W's rows pass through `buf`
+// (room for 2 kChunk rows of pitch ldb) a block at a time.  A points at row ty.
+template <int TR, int TCQ>
+__device__ __forceinline__ void times_matrix(float2 (&acc)[TR][2 * TCQ], const float* A, int lda, const float* W, int d, float* buf, int ldb,
+                                             int tx) {
+  for (int k0 = 0; k0 < d; k0 += 2 * kChunk) {
+    const int rows = d - k0 < 2 * kChunk ? d - k0 : 2 * kChunk;
+    __syncthreads();
+    stage_matrix_async(buf, ldb, W, d, k0, rows);
+    cp_async_wait_all();
+    __syncthreads();
+    gemm_t<TR, TCQ>(acc, A + k0, lda, buf + 4 * tx, ldb, rows);
+  }
+}
+// dst row r, column a (+)= <the row at A, row a of W>, i.e. (the rows at A) W^T; dst and A point at row ty, and differ
+template <int TR>
+__device__ __forceinline__ void times_transposed(float* dst, const float* A, int lda, const float* W, int d, float* buf, int ldb, int tx,
+                                                 bool add) {
+  for (int k0 = 0; k0 < d; k0 += 2 * kChunk) {
+    const int rows = d - k0 < 2 * kChunk ? d - k0 : 2 * kChunk;
+    __syncthreads();
+    stage_matrix_async(buf, ldb, W, d, k0, rows);
+    cp_async_wait_all();
+    __syncthreads();
+    for (int c0 = 0; c0 < rows; c0 += 32) {
+      float2 o[TR][4];
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o[i][j] = make_float2(0.f, 0.f);
+      gemm_n<TR, 4>(o, A, lda, buf + (c0 + tx) * ldb, ldb, d);
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (c0 + tx + 8 * j < rows) {
+            float* p = dst + 4 * i * lda + k0 + c0 + tx + 8 * j;
+            *p = (add ? *p : 0.f) + (o[i][j].x + o[i][j].y);
+          }
+    }
+  }
+  __syncwarp();
 }
 
 // A chunk of 32 rows of a matrix pair (two halves of `d` columns each; row r of half u at src[u] + r * pitch) on its way

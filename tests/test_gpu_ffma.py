@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import csat_oracle as orc
-from paper_2507_02957_b200 import workloads as wl
+from paper_2507_02957_b200 import binding, workloads as wl
 from gpu_util import TOL, device_inputs, make_ctx, rel_err, to_dev, to_np
 
 pytestmark = pytest.mark.gpu
@@ -61,4 +61,45 @@ def test_forward_at_the_edges_of_the_tiles(shape, dtype):
     ctx.set_lista_layer_weights(to_dev(S, dtype), to_dev(Bm, dtype), torch.from_numpy(th).cuda())
     check(T=4, lam=0.0, Psi=Psi.astype(np.float64),
           weights=(S.astype(np.float64), Bm.astype(np.float64), list(th.astype(np.float64))))
+    ctx.close()
+
+
+@pytest.mark.parametrize("untied", [False, True], ids=["one_decoder", "per_layer"])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "B%dH%d_n%d_nq%d_m%d_d%d" % s)
+def test_backward_at_the_edges_of_the_tiles(shape, untied):
+    """Gradients of float32 contexts, with the library's own decisions handed to the oracle (the derivative of the
+    shrinkage is discontinuous); the bar is the backward's common one, 2e-5."""
+    B, H, n, nq, m, d = shape
+    T = 4
+    w = wl.Workload("edges", B, H, n, nq, d, m, "fp32", T, 0.001, "iid", 950 + d)
+    inp = wl.make_inputs(w)
+    Q, K, V, _ = device_inputs(w, inp)
+    ctx = make_ctx(w)
+    binding.csat_set_i64(ctx.h, binding.CSAT_KEEP_MASKS, 1)
+    phi = to_np(ctx.get_phi())
+    r = np.random.default_rng(11)
+    kw = dict(T=T, lam=w.lam)
+    Psi = (np.eye(d) + 0.3 * r.standard_normal((d, d)) / np.sqrt(d)).astype(np.float32)
+    if untied or H % 2 == 0:                                # the dictionary in every per-layer and some of the other cases
+        ctx.set_dictionary(to_dev(Psi, "fp32"))
+        kw.update(Psi=Psi.astype(np.float64))
+    if untied:
+        S = (0.6 * np.eye(d) + 0.4 * r.standard_normal((T, H, d, d)) / np.sqrt(d)).astype(np.float32)
+        Bm = (r.standard_normal((T, H, d, d)) / np.sqrt(d)).astype(np.float32)
+        th = (0.02 * r.uniform(0.5, 1.5, size=(T, H))).astype(np.float32)
+        ctx.set_lista_layer_weights(to_dev(S, "fp32"), to_dev(Bm, "fp32"), torch.from_numpy(th).cuda())
+        kw.update(lam=0.0, weights=(S.astype(np.float64), Bm.astype(np.float64), list(th.astype(np.float64))))
+    G = r.standard_normal(inp["Q"].shape).astype(np.float32)
+    got = ctx.backward(Q, K, V, to_dev(G, "fp32"))
+    words = ctx.backward_masks().cpu().numpy().astype(np.uint32)
+    masks = np.stack([(words >> t) & 1 for t in range(T)], axis=2).astype(bool)
+    stages = []
+    orc.csat_backward(inp["Q"], inp["K"], inp["V"], phi, G, stages=stages, **kw)
+    own = np.stack([s["masks"] for s in stages]).reshape(masks.shape)
+    assert (masks != own).mean() <= 1e-4
+    ref = orc.csat_backward(inp["Q"], inp["K"], inp["V"], phi, G, masks=masks, **kw)
+    for nm, g, rf in zip(("dQ", "dK", "dV"), got, ref):
+        g = to_np(g)
+        assert np.isfinite(g).all() and np.abs(rf).max() > 0
+        assert rel_err(g, rf) <= 2e-5, (shape, nm, rel_err(g, rf))
     ctx.close()
