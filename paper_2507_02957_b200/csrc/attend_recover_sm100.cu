@@ -1241,6 +1241,7 @@ cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, c
   // with untied layers and T > 0 the per-layer kernel; the set-up has then built its operands for exactly T layers
   if (c->w_S && c->w_untied && c->p.T > 0)
     return c->p.d == 64 ? launch<64, true>(c, Q, out, s, c->p.T, nullptr, 0) : launch<128, true>(c, Q, out, s, c->p.T, nullptr, 0);
+  if (warp_attend_better(c)) return launch_warp_attend(c, Q, out, s);
   // Long jobs with the ISTA-derived decoder (one S, B and one positive threshold for all layers) fold B into the
   // values first: one more small launch, which only pays where the attention kernel walks several items per SM
   // (measured: from ~2 tiles of 128 queries per SM at d = 128, where a layer's hand-over chain is long, from ~8 at
@@ -1270,6 +1271,7 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
     if (untied) return d64 ? CSAT_REC_LAUNCH(64, true, 2) : CSAT_REC_LAUNCH(128, true, 2);
     return d64 ? CSAT_REC_LAUNCH(64, false, 2) : CSAT_REC_LAUNCH(128, false, 2);
   }
+  if (!untied && warp_attend_better(c)) return launch_warp_attend_recording(c, Q, out, s, lse_out, lse_stride, z_out, mask_out);
   if (untied) return d64 ? CSAT_REC_LAUNCH(64, true, 1) : CSAT_REC_LAUNCH(128, true, 1);
   return d64 ? CSAT_REC_LAUNCH(64, false, 1) : CSAT_REC_LAUNCH(128, false, 1);
 #undef CSAT_REC_LAUNCH

@@ -223,6 +223,12 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
                                              int lse_stride, uint32_t* mask_out, __nv_bfloat16* alpha_out,
                                              cudaStream_t s, int* launches, void* out = nullptr);
 
+// warp_attend.cu : the same two for d = 64 with 16 queries per warp (one S, B for all layers; no iterates)
+bool warp_attend_better(const csat_ctx* c);      // by the context's shape alone
+cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s);
+cudaError_t launch_warp_attend_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
+                                         __nv_bfloat16* z, uint32_t* masks);
+
 // wgrad_sm100.cu : gradients of the decoder's parameters from the stored iterates and dx_t (bf16, d in {64, 128}, one
 // S, B for all layers) into bw_wgrad; wgrad_splits = CTAs per head of its contraction kernel
 int wgrad_splits(const csat_ctx* c);

@@ -1,0 +1,382 @@
+// Compressed attention and recovery with 16 queries per warp (bf16, d = 64, one S, B for all layers): the whole chain of a
+// row block, softmax(Q K~^T / sqrt(d_k)) V~ and the unrolled recurrence alpha^{t+1} = eta_theta(S alpha^t + B Z_i), runs in
+// the registers of one warp (warp_mma.cuh), with -mu G held there as operand fragments.
+//
+// Why beside attend_recover_sm100.cu, which has four times the matrix rate: at d = 64 a layer of that kernel is a chain
+// thread -> MMA issuer -> tensor pipe -> thread of ~1500 cycles for 256 queries, and its tiles of 128 (pairs: 256) queries
+// leave SMs idle or rows empty at the sizes of single images and short query lists.  Here a layer takes 32 matrix
+// instructions (272 cycles) and ~80 others per 16 queries, 370 cycles in all: matrix and float32 instructions of different
+// warps do not overlap on a sub-core (one warp per sub-core 0.20 us per layer, two 0.38, three 0.575), which is why the
+// kernel stops paying off at one warp per sub-core, i.e. one CTA of 64 queries per SM (see warp_attend_better).
+//
+// The arithmetic is that kernel's: bf16 P and increments, float32 accumulators, statistics and iterates; the plain forward
+// with one positive threshold in units of 2 theta, otherwise the accumulator biased by the first threshold.
+#include "csat_internal.h"
+#include "sm100_ptx.cuh"
+#include "warp_mma.cuh"
+
+namespace csat {
+namespace {
+
+using namespace wmma16;
+
+constexpr int kD = 64, kWarps = 4, kRows = 16 * kWarps, kMC = 64;
+constexpr int kLd = kD + 8;                                   // bf16 row pitch: 8 rows of 16 bytes hit different banks
+constexpr int kTile = kMC * kLd;                              // K~ or V~ chunk, or a decoder matrix
+constexpr int kStages = 2;
+constexpr int kOffMats = kStages * 2 * kTile;                 // -mu G | B^T | Psi, each stored [output column][k]
+constexpr int kSmemBytes = 120 * 1024;                        // more than half an SM's, see launch()
+static_assert((kOffMats + 3 * kTile) * 2 <= kSmemBytes, "shared memory");
+
+struct Args {
+  __nv_bfloat16* out;
+  const __nv_bfloat16 *Q, *kv, *mats;
+  const float* theta;
+  int theta_stride, nq, m, H, T, has_psi, tiles, bh0;
+  float scale_log2;
+  // recording (the backward pass's forward), as in attend_recover_sm100.cu
+  float* lse;
+  int lse_stride;
+  __nv_bfloat16* z;
+  uint32_t* masks;
+};
+
+template <bool kRec>
+__global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args p) {
+  extern __shared__ __align__(16) __nv_bfloat16 smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int bh = p.bh0 + blockIdx.x / p.tiles, h = bh % p.H;
+  const int row0 = (blockIdx.x % p.tiles) * kRows + warp * 16;
+  const bool live = row0 < p.nq;                                // the warp has rows (it helps with the copies in any case)
+  const __nv_bfloat16* kvb = p.kv + (int64_t)bh * p.m * (2 * kD);
+  const int nchunks = (p.m + kMC - 1) / kMC;
+  __nv_bfloat16* mats = smem + kOffMats;
+
+  // decoder matrices (written before the compression kernel started) and this warp's queries
+  if (p.T > 0) {
+    const __nv_bfloat16* mh = p.mats + (int64_t)h * 3 * kD * kD;
+    for (int i = threadIdx.x; i < (p.has_psi ? 3 : 2) * kD * (kD / 8); i += kWarps * 32)
+      cp16(mats + (i >> 3) * kLd + (i & 7) * 8, mh + i * 8, true);
+  }
+  uint32_t q[kD / 16][4];
+  {
+    const __nv_bfloat16* Qb = p.Q + ((int64_t)bh * p.nq + row0) * kD + 2 * t;
+    const bool in0 = row0 + g < p.nq, in1 = row0 + g + 8 < p.nq;
+#pragma unroll
+    for (int k = 0; k < kD / 16; ++k)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        q[k][2 * u] = in0 ? *reinterpret_cast<const uint32_t*>(Qb + g * kD + 16 * k + 8 * u) : 0u;
+        q[k][2 * u + 1] = in1 ? *reinterpret_cast<const uint32_t*>(Qb + (g + 8) * kD + 16 * k + 8 * u) : 0u;
+      }
+  }
+  ptx::pdl_wait();                                              // K~|V~ come from the kernel before this one
+  auto stage = [&](int j) {
+    __nv_bfloat16* dst = smem + (j % kStages) * 2 * kTile;
+    for (int i = threadIdx.x; i < kMC * 16; i += kWarps * 32) {
+      const int r = i >> 4, c = i & 15;                         // 16 bytes c of row r: K~ (c < 8), then V~
+      cp16(dst + (c >> 3) * kTile + r * kLd + (c & 7) * 8, kvb + (int64_t)(j * kMC + r) * (2 * kD) + c * 8, j * kMC + r < p.m);
+    }
+    cp_commit();
+  };
+  stage(0);
+
+  float z[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) z[j][e] = 0.f;
+  float ref[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};   // log2 domain; this lane's columns
+  for (int c = 0; c < nchunks; ++c) {
+    if (c + 1 < nchunks) { stage(c + 1); cp_wait<1>(); } else cp_wait<0>();
+    __syncthreads();
+    if (live) {
+    const __nv_bfloat16* Ks = smem + (c % kStages) * 2 * kTile;
+    const __nv_bfloat16* Vs = Ks + kTile;
+    float s[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        uint32_t b[4];                                          // measurements 8 j .., columns 32 k .. 32 k + 31
+        ldsm4(b, Ks + (8 * j + (lane & 7)) * kLd + 32 * k + (lane >> 3) * 8);
+        mma(s[j], q[2 * k], b[0], b[1]);
+        mma(s[j], q[2 * k + 1], b[2], b[3]);
+      }
+    }
+    if ((c + 1) * kMC > p.m)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (c * kMC + 8 * j + 2 * t + (e & 1) >= p.m) s[j][e] = -INFINITY;
+    uint32_t pk[kMC / 16][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {                               // rows g, g + 8
+      float m0 = fmaxf(s[0][2 * u], s[0][2 * u + 1]), m1 = fmaxf(s[1][2 * u], s[1][2 * u + 1]);
+#pragma unroll
+      for (int j = 2; j < 8; j += 2) {
+        m0 = fmaxf(m0, fmaxf(s[j][2 * u], s[j][2 * u + 1]));
+        m1 = fmaxf(m1, fmaxf(s[j + 1][2 * u], s[j + 1][2 * u + 1]));
+      }
+      m0 = fmaxf(m0, m1);
+      m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1));
+      m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2));
+      const float nref = fmaxf(ref[u], m0 * p.scale_log2);       // finite: the chunk has a valid column
+      const float f = ex2(ref[u] - nref);                       // 0 on the first chunk
+      ref[u] = nref;
+      float ps = 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float p0 = ex2(fmaf(s[j][2 * u], p.scale_log2, -nref)), p1 = ex2(fmaf(s[j][2 * u + 1], p.scale_log2, -nref));
+        ps += p0 + p1;
+        pk[j >> 1][(j & 1) * 2 + u] = pack(p0, p1);
+        z[j][2 * u] *= f;
+        z[j][2 * u + 1] *= f;
+      }
+      sum[u] = fmaf(sum[u], f, ps);
+    }
+#pragma unroll
+    for (int k = 0; k < kMC / 16; ++k)
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        uint32_t b[4];                                          // measurements 16 k .., columns 8 j .. 8 j + 15
+        ldsm4t(b, Vs + (16 * k + ((lane >> 3) & 1) * 8 + (lane & 7)) * kLd + 8 * j + (lane >> 4) * 8);
+        mma(z[j], pk[k], b[0], b[1]);
+        mma(z[j + 1], pk[k], b[2], b[3]);
+      }
+    }
+    __syncthreads();                                            // the chunk's buffer may be overwritten
+  }
+  if (!live) return;
+  __nv_bfloat16* rows[2];                                       // where rows g, g + 8 go, null beyond n_q
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], 1);
+    sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], 2);
+    const float inv = 1.f / sum[u];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { z[j][2 * u] *= inv; z[j][2 * u + 1] *= inv; }
+    const int row = row0 + g + 8 * u;
+    if (kRec && p.lse && t == 0 && row < p.nq)
+      p.lse[((int64_t)bh * p.nq + row) * p.lse_stride] = (ref[u] + __log2f(sum[u])) * 0.69314718056f;
+    rows[u] = kRec && p.z && row < p.nq ? p.z + ((int64_t)bh * p.nq + row) * kD : nullptr;
+  }
+  if (kRec) store_rows<8>(rows, z, t);                          // Z as fed to the first product
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    rows[u] = p.out && row0 + g + 8 * u < p.nq ? p.out + ((int64_t)bh * p.nq + row0 + g + 8 * u) * kD : nullptr;
+
+  if (p.T > 0) {
+    // acc += (the operand rows) W, W's fragments read from shared memory
+    auto times = [&](float (&acc)[8][4], const uint32_t (&a)[4][4], const __nv_bfloat16* W) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          uint32_t b[4];
+          ldsm4(b, W + (8 * j + (lane & 7)) * kLd + 32 * k + (lane >> 3) * 8);
+          mma(acc[j], a[2 * k], b[0], b[1]);
+          mma(acc[j], a[2 * k + 1], b[2], b[3]);
+        }
+    };
+    uint32_t G[8][8];                                           // -mu G: tile j, steps k = 0..3 (two registers each)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        uint32_t b[4];
+        ldsm4(b, mats + (8 * j + (lane & 7)) * kLd + 32 * k + (lane >> 3) * 8);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) G[j][4 * k + e] = b[e];
+      }
+    auto times_G = [&](float (&acc)[8][4], const uint32_t (&a)[4][4]) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) mma(acc[j], a[k], G[j][2 * k], G[j][2 * k + 1]);
+    };
+    const float kappa = p.theta[h];
+    uint32_t a[4][4];
+    float r[8][4], v[8][4];                                     // accumulator; iterate
+    if (!kRec && p.theta_stride == 0 && kappa > 0.f) {
+      // v = alpha / (2 theta), r = 1/2 + (z B - a^ mu G) / (2 theta): s = sat(v + r), increment = r - s
+      const float i2 = 0.5f / kappa;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { z[j][e] *= i2; r[j][e] = 0.5f; v[j][e] = 0.f; }
+      to_operand<8>(a, z);
+      times(r, a, mats + kTile);
+      for (int it = 0; it + 1 < p.T; ++it) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float dn[4];
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const float2 s2 = make_float2(add_sat(v[j][e], r[j][e]), add_sat(v[j][e + 1], r[j][e + 1]));
+            const float2 d2 = __fadd2_rn(make_float2(r[j][e], r[j][e + 1]), make_float2(-s2.x, -s2.y));
+            const float2 v2 = __fadd2_rn(make_float2(v[j][e], v[j][e + 1]), d2);
+            dn[e] = d2.x; dn[e + 1] = d2.y;
+            v[j][e] = v2.x; v[j][e + 1] = v2.y;
+          }
+          a[j >> 1][(j & 1) * 2] = pack(dn[0], dn[1]);
+          a[j >> 1][(j & 1) * 2 + 1] = pack(dn[2], dn[3]);
+        }
+        times_G(r, a);
+      }
+      // exact shrinkage, back in the data's units: (u - 1/2) - (sat(u) - 1/2) is an exact zero for 0 <= u <= 1
+      const float tt = 2.f * kappa;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float u = v[j][e] + r[j][e];
+          v[j][e] = ((u - 0.5f) - (add_sat(u, 0.f) - 0.5f)) * tt;
+        }
+    } else {
+      // r = kappa + z B - a^ mu G, v = alpha - kappa (kappa: the first layer's threshold)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { r[j][e] = kappa; v[j][e] = -kappa; }
+      to_operand<8>(a, z);
+      times(r, a, mats + kTile);
+      // The layer's decisions: v8[2 u + w] collects a lane's 8 signs of theta - |x| of row g + 8 u, columns 32 w .. 32 w + 31
+      // (tile by tile, first column first).  A word has column c at bit 31 - c % 32: the four pairs of signs are spread to
+      // the word's bytes, shifted to the lane's place, and the four lanes of a row combine them so that lane t ends with
+      // word t.
+      uint32_t* mrow = nullptr;
+      if (kRec && p.masks && row0 + g + 8 * (t >> 1) < p.nq)
+        mrow = p.masks + ((int64_t)bh * p.T * p.nq + row0 + g + 8 * (t >> 1)) * 2 + (t & 1);
+      uint32_t v8[4];
+      auto store_masks = [&](int layer) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          uint32_t x = v8[i] & 0xffu;
+          x = (x | (x << 12)) & 0x000f000fu;
+          x = (x | (x << 6)) & 0x03030303u;
+          v8[i] = x << (6 - 2 * t);
+        }
+        const bool hi = t & 2, odd = t & 1;
+        const uint32_t g0 = __shfl_xor_sync(0xffffffffu, hi ? v8[0] : v8[2], 2), g1 = __shfl_xor_sync(0xffffffffu, hi ? v8[1] : v8[3], 2);
+        const uint32_t w0 = (hi ? v8[2] : v8[0]) | g0, w1 = (hi ? v8[3] : v8[1]) | g1;
+        const uint32_t g2 = __shfl_xor_sync(0xffffffffu, odd ? w0 : w1, 1);
+        if (mrow) mrow[(int64_t)layer * p.nq * 2] = (odd ? w1 : w0) | g2;
+      };
+      for (int it = 0; it + 1 < p.T; ++it) {
+        const float th = p.theta_stride ? p.theta[(int64_t)it * p.theta_stride + h] : kappa;
+        const float i2 = th > 0.f ? 0.5f / th : 0.f;            // theta = 0: sat(1/2) = 1/2 and eta(x) = x
+        const float2 m2 = make_float2(-2.f * th, -2.f * th), dk = make_float2(th - kappa, th - kappa);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float dn[4];
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const float2 r2 = make_float2(r[j][e], r[j][e + 1]);
+            const float2 x2 = __fadd2_rn(make_float2(v[j][e], v[j][e + 1]), r2);   // alpha^t S + z B
+            if (kRec) {
+              uint32_t& w = v8[e + (j >> 2)];
+              w = __funnelshift_l(__float_as_uint(th - fabsf(x2.x)), w, 1);
+              w = __funnelshift_l(__float_as_uint(th - fabsf(x2.y)), w, 1);
+            }
+            const float2 s2 = make_float2(fma_sat(x2.x, i2, 0.5f), fma_sat(x2.y, i2, 0.5f));
+            float2 bn = __ffma2_rn(s2, m2, x2), d2 = __ffma2_rn(s2, m2, r2);       // eta(x) - theta; the increment
+            if (p.theta_stride) { bn = __fadd2_rn(bn, dk); d2 = __fadd2_rn(d2, dk); }
+            v[j][e] = bn.x; v[j][e + 1] = bn.y;
+            dn[e] = d2.x; dn[e + 1] = d2.y;
+          }
+          a[j >> 1][(j & 1) * 2] = pack(dn[0], dn[1]);
+          a[j >> 1][(j & 1) * 2 + 1] = pack(dn[2], dn[3]);
+        }
+        times_G(r, a);
+        if (kRec) store_masks(it);
+      }
+      const float th = p.theta[(int64_t)(p.T - 1) * p.theta_stride + h];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float x = v[j][e] + r[j][e];
+          if (kRec) {
+            uint32_t& w = v8[(e & 2) + (j >> 2)];
+            w = __funnelshift_l(__float_as_uint(th - fabsf(x)), w, 1);
+          }
+          v[j][e] = x - fminf(fmaxf(x, -th), th);
+        }
+      if (kRec) store_masks(p.T - 1);
+    }
+    if (p.has_psi) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) r[j][e] = 0.f;
+      to_operand<8>(a, v);
+      times(r, a, mats + 2 * kTile);
+      store_rows<8>(rows, r, t);
+    } else {
+      store_rows<8>(rows, v, t);
+    }
+  } else {
+    store_rows<8>(rows, z, t);
+  }
+}
+
+template <bool kRec>
+cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride, __nv_bfloat16* z, uint32_t* masks) {
+  const Params& p = c->p;
+  static DeviceFlags opt_in;
+  cudaError_t e = ensure_dynamic_smem(warp_attend_kernel<kRec>, kSmemBytes, c->device, opt_in);
+  if (e != cudaSuccess) return e;
+  Args a;
+  a.out = (__nv_bfloat16*)out;
+  a.Q = (const __nv_bfloat16*)Q;
+  a.kv = (const __nv_bfloat16*)c->kv;
+  a.mats = c->mats_bf16;
+  a.theta = c->thr();
+  a.theta_stride = c->thr_stride();
+  a.nq = (int)p.nq; a.m = (int)p.m; a.H = (int)p.H; a.T = p.T;
+  a.has_psi = c->psi ? 1 : 0;
+  a.tiles = (int)((p.nq + kRows - 1) / kRows);
+  a.bh0 = (int)c->bh0;
+  a.scale_log2 = (float)((p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)kD)) * 1.4426950408889634);
+  a.lse = lse; a.lse_stride = lse_stride; a.z = z; a.masks = masks;
+  const int64_t grid = (int64_t)a.tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
+  if (grid > (int64_t)1 << 30) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kWarps * 32);
+  // one CTA per SM: without that, CTAs that start early would pile up on the SMs the compression leaves free
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;    // the prologue may run under the compression's tail
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, warp_attend_kernel<kRec>, a);
+}
+
+}  // namespace
+
+// As long as every SM has at most one CTA of 64 queries.  Measured with the compression in front (n = 1568, m = 256, T = 20,
+// us, this kernel / attend_recover_sm100): 1 CTA 16.2 / 21.3, 100 CTAs 17.2 / 25.0, 128 CTAs (heads of 64 queries) 22.5 /
+// 28.4, 256 CTAs 28.4 / 28.6 (queries in single tiles of 128) and 27.4 / 29.5 (pairs), 300 CTAs 28.9 / 25.3; one image of 12
+// heads of 197 tokens, m = 64, T = 10: 9.0 / 13.6.  The whole job counts, not the launch's range of (batch, head) pairs, so
+// that a forward cut into sub-range launches returns the same bits.
+bool warp_attend_better(const csat_ctx* c) {
+  const Params& p = c->p;
+  return p.d == kD && !(c->w_S && c->w_untied && p.T > 0) && (p.nq + kRows - 1) / kRows * p.B * p.H <= c->sms;
+}
+
+cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
+  return launch<false>(c, Q, out, s, nullptr, 0, nullptr, nullptr);
+}
+cudaError_t launch_warp_attend_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
+                                         __nv_bfloat16* z, uint32_t* masks) {
+  return launch<true>(c, Q, out, s, lse, lse_stride, z, masks);
+}
+
+}  // namespace csat
