@@ -199,6 +199,11 @@ struct FfmaAttend {                       // layer t of head h: S + t * layer_st
 cudaError_t launch_ffma_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
                                  float* partial);
 cudaError_t launch_ffma_attend(const FfmaAttend& a, int dtype, const void* Q, const void* kv, void* out, cudaStream_t s);
+// warp_split.cu : the same two stages for bf16 on the warp-level matrix instructions, float32 values in two bf16 parts;
+// where the launchers above send bf16 contexts with a head size that has no tcgen05 kernel
+cudaError_t launch_split_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
+                                  float* partial);
+cudaError_t launch_split_attend(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s);
 // workspace := sum over r < R of partials[r] (float32 [B,H,m,2d] each), added in the order r = 0, 1, ..., rounded
 // once to the context's storage type
 cudaError_t launch_reduce_partials(csat_ctx* c, const float* partials, int R, cudaStream_t s, int* launches);

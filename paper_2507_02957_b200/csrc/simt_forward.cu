@@ -299,6 +299,11 @@ cudaError_t compress_t(csat_ctx* c, const void* K, const void* V, cudaStream_t s
   return cudaGetLastError();
 }
 
+// bf16 with a head size that has no tcgen05 kernel (CSAT_FORCE_SIMT asks for the float32 kernels themselves)
+bool use_split(const csat_ctx* c) {
+  return c->p.dtype == CSAT_DTYPE_BF16 && c->p.d < 128 && c->p.d != 64 && c->force_simt == 0;
+}
+
 template <typename T>
 cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
   const Params& p = c->p;
@@ -317,6 +322,7 @@ cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
     a.theta_stride = c->thr_stride();
     a.d = d; a.H = (int)p.H; a.T = p.T; a.device = c->device; a.sms = c->sms;
     a.scale = scale;
+    if (use_split(c)) return launch_split_attend(a, Q, c->kv, out, s);
     return launch_ffma_attend(a, p.dtype, Q, c->kv, out, s);
   }
   cudaError_t e = cudaSuccess;
@@ -343,6 +349,7 @@ cudaError_t launch_simt_compress(csat_ctx* c, const void* K, const void* V, cuda
                                  int64_t phi_j0, int64_t n_len, float* partial) {
   *launches += 1;
   if (n_len <= 0) n_len = c->p.n;
+  if (use_split(c)) return launch_split_compress(c, K, V, s, phi_j0, n_len, partial);
   if (c->p.d <= kFfmaMaxD) return launch_ffma_compress(c, K, V, s, phi_j0, n_len, partial);
   return c->p.dtype == CSAT_DTYPE_FP32 ? compress_t<float>(c, K, V, s, phi_j0, n_len, partial)
                                        : compress_t<__nv_bfloat16>(c, K, V, s, phi_j0, n_len, partial);

@@ -29,15 +29,17 @@ SHAPES = [(1, 1, 65, 1, 33, 8),
           (1, 2, 150, 40, 140, 136)]     # beyond the tiled kernels
 
 
-@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("dtype, force", [("fp32", 0), ("bf16", 1), ("bf16", 0)], ids=["fp32", "bf16_ffma", "bf16"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "B%dH%d_n%d_nq%d_m%d_d%d" % s)
-def test_forward_at_the_edges_of_the_tiles(shape, dtype):
+def test_forward_at_the_edges_of_the_tiles(shape, dtype, force):
+    """bf16_ffma: bf16 storage on the float32 kernels; bf16: on the kernels the head size is served by (two bf16 parts per
+    float32 value on the matrix instructions where it is not 64 or 128)."""
     B, H, n, nq, m, d = shape
     w = wl.Workload("edges", B, H, n, nq, d, m, dtype, 4, 0.01, "iid", 900 + d)
     inp = wl.make_inputs(w)
     Q, K, V, _ = device_inputs(w, inp)
     ctx = make_ctx(w)
-    ctx.set(force_simt=1)                                   # bf16 with d in {64, 128} on these kernels as well
+    ctx.set(force_simt=force)
     phi = to_np(ctx.get_phi())
     r = np.random.default_rng(7)
     Psi = wl.round_to_storage((np.eye(d) + 0.3 * r.standard_normal((d, d)) / np.sqrt(d)).astype(np.float32), dtype)
