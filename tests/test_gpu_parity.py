@@ -744,3 +744,18 @@ def test_random_shapes_match_oracle(w):
     ctx.forward_host(Qh, Kh, Vh, oh)
     assert torch.equal(oh, ctx.forward(Q, K, V).cpu())
     ctx.close()
+
+
+@pytest.mark.parametrize("B, n, H", [(3, 130, 2), (5, 1000, 6), (4, 4096, 4)], ids=["pieces_only", "halves", "whole_and_quarters"])
+def test_project_qkv_tiles_across_batch_elements(B, n, H):
+    """Row tiles that straddle batch elements, and the tiles of the last, partial wave in whole, halved and quartered
+    pieces (148 SMs: 6, 40 x 5 and 128 x 3 tiles of 128 x 256)."""
+    r = np.random.default_rng(73)
+    d, dm = 64, 128
+    ctx = binding.Csat(n, 16, d, H, 3, B=B, T=0)
+    X = wl.round_to_storage(r.standard_normal((B, n, dm)).astype(np.float32), "bf16")
+    W = wl.round_to_storage((r.standard_normal((dm, 3 * H * d)) / np.sqrt(dm)).astype(np.float32), "bf16")
+    got = ctx.project_qkv(to_dev(X, "bf16"), to_dev(W, "bf16"))
+    for name, g, ref in zip("QKV", got, orc.project_qkv(X, W, H, d)):
+        assert rel_err(to_np(g), ref) <= 8e-3, name          # bf16: output rounding, 2^-8 of max
+    ctx.close()
