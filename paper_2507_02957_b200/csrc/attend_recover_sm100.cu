@@ -857,11 +857,11 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
           }
         }
       }
-      // One positive threshold for all layers (the ISTA-derived decoder), no decisions to record: the same recurrence
+      // One positive threshold for all layers (the ISTA-derived decoder), no iterates to record: the same recurrence
       // in units of 2 theta, which saves one instruction per pair of elements.  Registers c = alpha / (2 theta),
       // accumulator r' = 1/2 + (z B - a^ mu G) / (2 theta) (the threads store 1/2, z is published divided by 2 theta):
       //   s = sat(c + r') (= sat(x / (2 theta) + 1/2), one saturating add);  increment = r' - s;  c += increment.
-      const bool scaled_units = kFold || (!kUntied && !kMasks && T > 0 && theta_stride == 0 && kappa > 0.f);
+      const bool scaled_units = kFold || (!kUntied && !kKeep && T > 0 && theta_stride == 0 && kappa > 0.f);
       if (scaled_units) {
         const uint32_t op_addr = tbase + C::kColS;
         if (kFold) {
@@ -897,6 +897,13 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
 #pragma unroll
         for (int i = 0; i < D / 2; ++i) v2[i] = pack2(0.f, 0.f);      // alpha^0 = 0
         const F2 m1 = pack2(-1.f, -1.f);
+        // kMasks: |x| > theta where s is 0 or 1, i.e. where s (1 - s) vanishes; the sign bit of s (1 - s) - tiny says so
+        auto push_mask = [&](F2 s2, int c) {
+          float g0, g1;
+          unpack2(fma2(s2, fma2(s2, m1, pack2(1.f, 1.f)), pack2(-1e-30f, -1e-30f)), g0, g1);
+          mw[c >> 5] = __funnelshift_l(__float_as_uint(g0), mw[c >> 5], 1);
+          mw[c >> 5] = __funnelshift_l(__float_as_uint(g1), mw[c >> 5], 1);
+        };
         for (int it = 0; it + 1 < T; ++it) {
           if (!kFold || it > 0) { w.wait(&bars->r_full[t], phase & 1, 230); ++phase; }
           tc_fence_after();
@@ -907,6 +914,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
               float a0, a1;
               unpack2(v2[(c0 + e) >> 1], a0, a1);
               const F2 s2 = pack2(add_sat(a0, __uint_as_float(r[e])), add_sat(a1, __uint_as_float(r[e + 1])));
+              if (kMasks) push_mask(s2, c0 + e);
               const F2 dn = fma2(s2, m1, pack2u(r[e], r[e + 1]));     // (alpha^{t+1} - alpha^t) / (2 theta)
               v2[(c0 + e) >> 1] = add2(v2[(c0 + e) >> 1], dn);
               float d0, d1;
@@ -929,6 +937,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(&bars->a_full[t]);
+          if (kMasks) store_masks(it);
         }
         // last iteration, exact shrinkage, back in the data's units: alpha^T = 2 theta eta_{1/2}(c + r' - 1/2)
         w.wait(&bars->r_full[t], phase & 1, 231); ++phase;
@@ -945,6 +954,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
             float u0, u1;
             unpack2(u2, u0, u1);
             const F2 s2 = pack2(add_sat(u0, 0.f), add_sat(u1, 0.f));
+            if (kMasks) push_mask(s2, c0 + e);
             v2[(c0 + e) >> 1] = mul2(sub2(add2(u2, mh2), add2(s2, mh2)), tt2);
           }
         };
@@ -962,6 +972,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
             if (!has_psi && (c0 + 32) % 64 == 0) stage_box(c0 / 64);      // this box of the output is final
           }
           staged = !has_psi;
+          if (kMasks) store_masks(T - 1);
         }
         if (has_psi) {
           publish(0);
@@ -1057,7 +1068,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
             store_masks(it);
           }
         };
-        if (theta_stride != 0) iterate(std::true_type{}); else iterate(std::false_type{});
+        if (kRec == 1 || theta_stride != 0) iterate(std::true_type{}); else iterate(std::false_type{});
         const float th = theta[(int64_t)(T - 1) * theta_stride + h];
         // last iteration, exact shrinkage: alpha^T = eta_theta(x)
         w.wait(&bars->r_full[t], phase & 1, 231); ++phase;

@@ -1,0 +1,353 @@
+// The recurrence of the LISTA decoder run backwards (see bwd_rows_sm100.cu: the same step, operands, decisions and results)
+// for d = 128 and one S, B for all layers, two tiles of 128 queries per CTA.
+//
+// A tile's layer is a chain thread -> MMA issuer -> tensor pipe -> thread; with one tile per SM it takes ~2700 cycles, of
+// which the products dx_t (S - I)^T and dx_t B^T take 1084.  Two tiles alternate on the tensor pipe here.  What stood
+// against that was tensor memory (accumulator and dZ of two tiles fill it), so the operand dx_t goes through shared memory,
+// in two buffers per tile; and the matrix instructions are issued by a warp of their own per tile (issued from a compute
+// warp they delay its next pass by ~600 cycles).  16 heads of 8192 queries, T = 20: 203 -> @P@ us.
+//
+// CTA = 12 warps: 0-3 tile A, 4-7 tile B (one thread per query row, 224 registers), 8 and 10 issue tile A's and B's MMAs,
+// 9 loads G (into the operand buffers, whose layout it then has) and the matrices (S - I | B; with a dictionary Psi first, in
+// the place of S - I), 11 completes the warpgroup.  dZ leaves through an operand buffer and TMA stores: rows of 256 bytes
+// read and written by one thread each cost 20 us of the 203.
+#include "csat_internal.h"
+#include "sm100_ptx.cuh"
+#include "tma_host.h"
+
+namespace csat {
+namespace {
+
+using namespace ptx;
+
+constexpr int kD = 128, kRows = 128, kTiles = 2, kThreads = 384;
+constexpr int kBoxes = kD / 64;
+constexpr int kComputeRegs = 224, kControlRegs = 56;              // after setmaxnreg (checked on the host)
+constexpr uint32_t kMatBoxBytes = kD * 128, kMatBytes = kBoxes * kMatBoxBytes;
+constexpr uint32_t kOpBoxBytes = kRows * 128, kOpBytes = kBoxes * kOpBoxBytes;
+constexpr uint32_t kOffMat = 0;                                    // [S - I (Psi first) | B]
+constexpr uint32_t kOffOp = 2 * kMatBytes;                         // [tile][2]
+constexpr uint32_t kOffBar = kOffOp + kTiles * 2 * kOpBytes;
+constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024 /*alignment slack*/;
+constexpr uint32_t kTileCols = 2 * kD, kColAcc = 0, kColDz = kD;   // tensor memory, per tile
+static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+
+struct Bars {
+  uint64_t mats_full, psi_done, g_full[kTiles];
+  uint64_t a_full[kTiles], r_full[kTiles], op_free[kTiles][2];
+  uint32_t tmem_slot;
+  int abort;
+};
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&p);
+}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
+struct Waiter {
+  int* status;
+  int* cta_abort;
+  bool dead = false;
+  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, int code) {
+    if (dead) return;
+    if (!mbar_wait(bar, parity, status, code, cta_abort)) dead = true;
+  }
+};
+
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_recur_pair_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __grid_constant__ CUtensorMap tmap_g,
+                      const __grid_constant__ CUtensorMap tmap_dz, const __nv_bfloat16* __restrict__ Z16, float* __restrict__ ws_LD,
+                      const uint32_t* __restrict__ maskbits, int nq, int H, int T, int has_psi, int* status,
+                      __nv_bfloat16* __restrict__ dx_out, int64_t dx_slot) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bh = blockIdx.y, h = bh % H, row0 = blockIdx.x * (kTiles * kRows);
+  const int ntiles = nq - row0 > kRows ? 2 : 1;
+  Waiter w{status, &bars->abort};
+
+  if (threadIdx.x == 0) {
+    prefetch_tmap(&tmap_mats);
+    prefetch_tmap(&tmap_g);
+    prefetch_tmap(&tmap_dz);
+    mbar_init(&bars->mats_full, 1);
+    mbar_init(&bars->psi_done, ntiles);
+    for (int t = 0; t < kTiles; ++t) {
+      mbar_init(&bars->g_full[t], 1);
+      mbar_init(&bars->a_full[t], kRows);
+      mbar_init(&bars->r_full[t], 1);
+      mbar_init(&bars->op_free[t][0], 1);
+      mbar_init(&bars->op_free[t][1], 1);
+    }
+    bars->abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 8) {
+    tmem_alloc(&bars->tmem_slot, kTiles * kTileCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bars->tmem_slot;
+
+  // 2 x 128 x 224 + 128 x 56 = 64512 registers
+  if (warp >= 8) {
+    reg_dealloc<kControlRegs>();
+    if (warp == 9) {
+      if (elect_one()) {
+        auto load_mat = [&](int slot, int index) {
+          for (int gx = 0; gx < kBoxes; ++gx)
+            tma_load_3d(smem + kOffMat + slot * kMatBytes + gx * kMatBoxBytes, &tmap_mats, &bars->mats_full, gx * 64, 0, h * 3 + index);
+        };
+        for (int t = 0; t < ntiles; ++t) {                     // rows beyond n_q are zero-filled
+          mbar_arrive_expect_tx(&bars->g_full[t], kOpBytes);
+          for (int gx = 0; gx < kBoxes; ++gx)
+            tma_load_3d(smem + kOffOp + t * 2 * kOpBytes + gx * kOpBoxBytes, &tmap_g, &bars->g_full[t], gx * 64, row0 + t * kRows, bh);
+        }
+        mbar_arrive_expect_tx(&bars->mats_full, 2 * kMatBytes);
+        load_mat(0, has_psi ? 2 : 0);
+        load_mat(1, 1);
+        int loads = 1;
+        if (has_psi) {                                         // S - I once both tiles' products have read Psi
+          w.wait(&bars->psi_done, 0, 904);
+          if (!w.dead) {
+            mbar_arrive_expect_tx(&bars->mats_full, kMatBytes);
+            load_mat(0, 0);
+            loads = 2;
+          }
+        }
+        // the CTA stays until its copies have landed, whatever became of the waits
+        for (int t = 0; t < ntiles; ++t) mbar_wait_drain(&bars->g_full[t], 0);
+        mbar_wait_drain(&bars->mats_full, (loads - 1) & 1);
+      }
+    } else if (warp == 8 || warp == 10) {
+      const int t = warp == 8 ? 0 : 1;
+      if (t < ntiles && elect_one()) {
+        constexpr uint32_t idesc = make_idesc_bf16(kRows, kD, false, true);     // transposed product: B MN-major
+        const uint32_t acc = tmem + t * kTileCols + kColAcc, dz = tmem + t * kTileCols + kColDz;
+        const uint64_t op0 = make_smem_desc(smem_u32(smem + kOffOp + t * 2 * kOpBytes), 16, 1024);
+        const uint64_t mat0 = make_smem_desc(smem_u32(smem + kOffMat), kMatBoxBytes, 1024);
+        // A: K step k lies in 64-column box k / 4, 32 (k % 4) bytes into each row; B: 16 rows (2048 bytes) per K step
+        auto product = [&](uint32_t d_t, uint32_t n, int slot, uint32_t accumulate) {
+          const uint64_t ad = op0 + (uint64_t)((n & 1) * (kOpBytes >> 4)), bd = mat0 + (uint64_t)(slot * (kMatBytes >> 4));
+#pragma unroll
+          for (int k = 0; k < kD / 16; ++k)
+            mma_f16_ss(d_t, ad + (uint64_t)((k / 4) * (kOpBoxBytes >> 4) + (k % 4) * 2), bd + (uint64_t)(k * 128), idesc,
+                       k == 0 ? accumulate : 1u);
+        };
+        uint32_t n = 0;                                         // operands taken so far (buffer n & 1)
+        w.wait(&bars->mats_full, 0, 900);
+        if (has_psi) {                                         // d alpha_T = G Psi
+          w.wait(&bars->g_full[t], 0, 901);                    // G is the operand as it came
+          tc_fence_after();
+          product(acc, 0, 0, 0u);
+          mma_commit(&bars->r_full[t]);
+          mma_commit(&bars->op_free[t][0]);
+          mma_commit(&bars->psi_done);
+          n = 1;
+          w.wait(&bars->mats_full, 1, 902);
+        }
+        for (int l = T - 1; l >= 0; --l, ++n) {
+          w.wait(&bars->a_full[t], (T - 1 - l) & 1, 903);
+          tc_fence_after();
+          if (l > 0) {
+            product(acc, n, 0, 0u);                            // dx_l (S - I)^T
+            mma_commit(&bars->r_full[t]);
+          }
+          product(dz, n, 1, l == T - 1 ? 0u : 1u);             // dZ += dx_l B^T trails it
+          if (l == 0) mma_commit(&bars->r_full[t]);            // the last result the threads wait for is dZ itself
+          mma_commit(&bars->op_free[t][n & 1]);
+        }
+      }
+    }
+  } else {
+    reg_alloc<kComputeRegs>();
+    const int t = warp >> 2, row = (warp & 3) * 32 + lane, grow = row0 + t * kRows + row;
+    if (t < ntiles) {
+      const bool live = grow < nq;
+      const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + t * kTileCols;
+      const int64_t goff = ((int64_t)bh * nq + (live ? grow : 0)) * kD;
+      int phase = 0;
+      uint32_t n = 0;                                           // operands published so far (buffer n & 1)
+      float v[kD];                                              // d alpha_{t+1}, then dx_t
+      uint8_t* op_row = smem;                                   // this row in the operand buffer
+      auto begin = [&]() {
+        if (n >= 2) w.wait(&bars->op_free[t][n & 1], ((n >> 1) - 1) & 1, 913);
+        op_row = smem + kOffOp + (t * 2 + (n & 1)) * kOpBytes + row * 128;
+        ++n;
+      };
+      // 16 columns of v as bf16 into the operand (128-byte swizzle); with `keep` also to global memory (dx_t, for the
+      // gradients of the decoder's weights)
+      auto put16 = [&](int c0, __nv_bfloat16* keep) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) pk[e >> 1] = pack_bf16(v[c0 + e], v[c0 + e + 1]);
+        uint8_t* ob = op_row + (c0 / 64) * kOpBoxBytes;
+        const int ch = (c0 % 64) / 8;
+        *reinterpret_cast<uint4*>(ob + ((ch ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(ob + (((ch + 1) ^ (row & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+        if (keep != nullptr) {
+          uint4* kp = reinterpret_cast<uint4*>(keep + c0);
+          kp[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          kp[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+        }
+      };
+      auto end = [&]() {
+        fence_proxy_async();
+        tc_fence_before();
+        mbar_arrive(&bars->a_full[t]);
+      };
+      if (has_psi) {
+        n = 1;
+#pragma unroll
+        for (int c = 0; c < kD; ++c) v[c] = 0.f;                // d alpha_T is the product alone
+        w.wait(&bars->r_full[t], phase & 1, 911); ++phase;
+        tc_fence_after();
+      } else {                                                  // d alpha_T = G: this row of the first buffer
+        w.wait(&bars->g_full[t], 0, 910);
+        const uint8_t* g_row = smem + kOffOp + t * 2 * kOpBytes + row * 128;
+#pragma unroll
+        for (int c = 0; c < kD / 8; ++c) {
+          const uint4 q = *reinterpret_cast<const uint4*>(g_row + (c / 8) * kOpBoxBytes + (((c % 8) ^ (row & 7)) << 4));
+          v[8 * c + 0] = bf16_lo(q.x); v[8 * c + 1] = bf16_hi(q.x);
+          v[8 * c + 2] = bf16_lo(q.y); v[8 * c + 3] = bf16_hi(q.y);
+          v[8 * c + 4] = bf16_lo(q.z); v[8 * c + 5] = bf16_hi(q.z);
+          v[8 * c + 6] = bf16_lo(q.w); v[8 * c + 7] = bf16_hi(q.w);
+        }
+      }
+      // the forward's decisions of layer l: column c is bit 31 - c % 32 of word c / 32 (loaded one layer ahead)
+      uint32_t mw[kD / 32];
+      auto load_masks = [&](int l) {
+        uint4 q = make_uint4(0, 0, 0, 0);
+        if (live) q = *reinterpret_cast<const uint4*>(maskbits + (((int64_t)bh * T + l) * nq + grow) * (kD / 32));
+        mw[0] = q.x; mw[1] = q.y; mw[2] = q.z; mw[3] = q.w;
+      };
+      // dx = d alpha o mask for 16 columns, d alpha = v + r (r: the last product of these columns)
+      auto piece = [&](const uint32_t (&r)[16], int c0, __nv_bfloat16* keep) {
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+          const int c = c0 + e;
+          const float2 x = __fadd2_rn(make_float2(v[c], v[c + 1]), make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])));
+          v[c] = (mw[c >> 5] >> (31 - (c & 31))) & 1u ? x.x : 0.f;
+          v[c + 1] = (mw[c >> 5] >> (30 - (c & 31))) & 1u ? x.y : 0.f;
+        }
+        put16(c0, keep);
+      };
+      load_masks(T - 1);
+      auto pass = [&](int l) {                                  // dx_l from the last product (or G), handed over
+        __nv_bfloat16* keep = dx_out != nullptr && live && !w.dead ? dx_out + (int64_t)l * dx_slot + goff : nullptr;
+        begin();
+        // 16 columns at a time, the next piece's tensor-memory load in flight under this one's arithmetic
+        uint32_t r0[16], r1[16];
+        tmem_ld_32x32b_x16(tbase + kColAcc, r0);
+#pragma unroll
+        for (int c0 = 0; c0 < kD; c0 += 32) {
+          tmem_wait_ld();
+          tmem_ld_32x32b_x16(tbase + kColAcc + c0 + 16, r1);
+          piece(r0, c0, keep);
+          tmem_wait_ld();
+          if (c0 + 32 < kD) tmem_ld_32x32b_x16(tbase + kColAcc + c0 + 32, r0);
+          piece(r1, c0 + 16, keep);
+        }
+        end();
+      };
+      int l = T - 1;
+      if (!has_psi) {                                           // no product before the first layer
+        __nv_bfloat16* keep = dx_out != nullptr && live && !w.dead ? dx_out + (int64_t)l * dx_slot + goff : nullptr;
+        const uint32_t zero[16] = {};
+        begin();
+#pragma unroll
+        for (int c0 = 0; c0 < kD; c0 += 16) piece(zero, c0, keep);
+        end();
+        if (--l >= 0) {
+          load_masks(l);
+          w.wait(&bars->r_full[t], phase & 1, 912); ++phase;
+          tc_fence_after();
+        }
+      }
+      for (; l > 0; --l) {
+        pass(l);
+        load_masks(l - 1);
+        w.wait(&bars->r_full[t], phase & 1, 912); ++phase;
+        tc_fence_after();
+      }
+      if (l == 0) pass(0);
+      uint4 z[kD / 8];                                          // v is done with; Z travels under the last product
+      {
+        const uint4* zp = reinterpret_cast<const uint4*>(Z16 + goff);
+#pragma unroll
+        for (int c = 0; c < kD / 8; ++c) z[c] = live ? zp[c] : make_uint4(0, 0, 0, 0);
+      }
+      w.wait(&bars->r_full[t], phase & 1, 914); ++phase;
+      tc_fence_after();
+      // ---- dZ (the accumulated products) and D = <dZ, Z>; every product has finished: the operand buffers are free ----
+      float dsum = 0.f;
+      op_row = smem + kOffOp + t * 2 * kOpBytes + row * 128;
+#pragma unroll
+      for (int c0 = 0; c0 < kD; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld_32x32b_x16(tbase + kColDz + c0, r);
+        tmem_wait_ld();
+        const float* f = reinterpret_cast<const float*>(r);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const uint4 q = z[c0 / 8 + half];
+          dsum = fmaf(f[8 * half + 0], bf16_lo(q.x), dsum); dsum = fmaf(f[8 * half + 1], bf16_hi(q.x), dsum);
+          dsum = fmaf(f[8 * half + 2], bf16_lo(q.y), dsum); dsum = fmaf(f[8 * half + 3], bf16_hi(q.y), dsum);
+          dsum = fmaf(f[8 * half + 4], bf16_lo(q.z), dsum); dsum = fmaf(f[8 * half + 5], bf16_hi(q.z), dsum);
+          dsum = fmaf(f[8 * half + 6], bf16_lo(q.w), dsum); dsum = fmaf(f[8 * half + 7], bf16_hi(q.w), dsum);
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[c0 + e] = f[e];
+        put16(c0, nullptr);
+      }
+      fence_proxy_async();
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");              // the tile's rows are in shared memory
+      if ((threadIdx.x & 127) == 0) {
+        if (*(volatile int*)&bars->abort == 0 && !w.dead)                     // rows beyond n_q are clipped
+          for (int gx = 0; gx < kBoxes; ++gx)
+            tma_store_3d(&tmap_dz, smem + kOffOp + t * 2 * kOpBytes + gx * kOpBoxBytes, gx * 64, row0 + t * kRows, bh);
+        bulk_commit_group();
+        bulk_wait_group0();
+      }
+      if (live && !w.dead) ws_LD[((int64_t)bh * nq + grow) * 2 + 1] = dsum;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) tmem_dealloc(tmem, kTiles * kTileCols);
+}
+
+}  // namespace
+
+cudaError_t launch_sm100_bwd_recur_pair(csat_ctx* c, const void* G, cudaStream_t s) {
+  const Params& p = c->p;
+  static DeviceFlags opt_in;
+  cudaError_t e;
+  if (!opt_in.test(c->device)) {
+    // setmaxnreg moves registers inside the pool the CTA is launched with; a request it cannot satisfy waits forever
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, bwd_recur_pair_kernel)) != cudaSuccess) return e;
+    if ((int64_t)fa.numRegs * kThreads < (int64_t)kTiles * kRows * kComputeRegs + 128 * kControlRegs) return cudaErrorLaunchOutOfResources;
+  }
+  if ((e = ensure_dynamic_smem(bwd_recur_pair_kernel, (int)kSmemBytes, c->device, opt_in)) != cudaSuccess) return e;
+  CUtensorMap tg, tz;
+  const uint64_t qd[3] = {(uint64_t)kD, (uint64_t)p.nq, (uint64_t)(p.B * p.H)};
+  const uint64_t qs[2] = {(uint64_t)kD * 2, (uint64_t)p.nq * kD * 2};
+  const uint32_t qb[3] = {64, (uint32_t)kRows, 1};
+  if ((e = make_tmap_bf16_3d(&tg, G, qd, qs, qb)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16_3d(&tz, c->bw_dZ16, qd, qs, qb)) != cudaSuccess) return e;
+  const dim3 grid((unsigned)((p.nq + kTiles * kRows - 1) / (kTiles * kRows)), (unsigned)(p.B * p.H));
+  bwd_recur_pair_kernel<<<grid, kThreads, kSmemBytes, s>>>(
+      c->tmap_mats, tg, tz, c->bw_Z16, c->bw_LD, c->bw_maskbits, (int)p.nq, (int)p.H, p.T, c->psi ? 1 : 0,
+      c->status, c->weight_grads ? c->bw_dx16 : nullptr, (int64_t)(p.B * p.H * p.nq * p.d));
+  return cudaGetLastError();
+}
+
+}  // namespace csat

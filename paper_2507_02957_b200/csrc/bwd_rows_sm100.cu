@@ -556,7 +556,8 @@ cudaError_t launch_sm100_bwd_recur(csat_ctx* c, const void* G, cudaStream_t s, i
   *launches += 1;
   if (c->w_S && c->w_untied && c->p.T > 0)
     return c->p.d == 64 ? launch_recur<64, true>(c, G, s) : launch_recur<128, true>(c, G, s);
-  return c->p.d == 64 ? launch_recur<64, false>(c, G, s) : launch_recur<128, false>(c, G, s);
+  if (c->p.d == 64) return launch_recur<64, false>(c, G, s);
+  return c->p.T > 0 ? launch_sm100_bwd_recur_pair(c, G, s) : launch_recur<128, false>(c, G, s);
 }
 
 cudaError_t launch_sm100_bwd_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s, int* launches) {

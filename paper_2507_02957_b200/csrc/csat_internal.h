@@ -243,6 +243,8 @@ cudaError_t launch_sm100_wgrad(csat_ctx* c, const void* G, cudaStream_t s, int* 
 // for all layers).  recur: Z, G -> dZ (bf16 into bw_dZ16), D = <dZ, Z> (into bw_LD), optionally the masks;
 // dq: Q, dZ, L, D, K~|V~ -> dQ
 cudaError_t launch_sm100_bwd_recur(csat_ctx* c, const void* G, cudaStream_t s, int* launches);
+// bwd_recur_pair_sm100.cu : recur for d = 128, T > 0 and one S, B for all layers
+cudaError_t launch_sm100_bwd_recur_pair(csat_ctx* c, const void* G, cudaStream_t s);
 cudaError_t launch_sm100_bwd_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s, int* launches);
 
 // project_sm100.cu : input projections; one launch applies columns [col0, col0 + ncols) of W [dm, 3 H d] to
