@@ -24,7 +24,11 @@
 //   warps 2-9: TMEM lane = measurement; warps 2-5 take the tile's queries [0, 32), warps 6-9 the queries [32, 64):
 //              P = exp2(S^T scale log2 e - L log2 e), dS = scale P (dA^T - D) with the queries' L, D read from global
 //              memory (the same address in every lane), zero for queries beyond n_q.  At the end the same threads
-//              store the accumulators as float32 and as the bf16 operand of the product with Phi^T.
+//              put the accumulators into shared memory, from where all threads store them in whole lines as the bf16
+//              operand of the product with Phi^T.
+// A cluster of 2 (d = 64: or 4) CTAs shares out the queries of a block where that fills the SMs better (16 heads with m = 512 are 64
+// blocks); each CTA then adds up its share of the rows from all CTAs' shared memory, in rank order (bit-identical reruns).
+// 16 heads of 8192 x 128, m = 512: 131 -> 77 us; 96 heads of 1568 x 64, m = 256 (192 blocks, not shared out): 65 -> 61 us.
 #include "csat_internal.h"
 #include "sm100_ptx.cuh"
 #include "tma_host.h"
@@ -54,6 +58,9 @@ template <int D> struct Cfg {
   static constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024 /*alignment slack*/;
   // TMEM columns: set s at 128 s: S^T (64) | dA^T (64); then the accumulators
   static constexpr uint32_t kSetCols = 2 * kQT, kColA = kQT, kColV = 2 * kSetCols, kColK = kColV + D, kTmemCols = 512;
+  // at the end, over K~, V~ and the ring: the accumulators dK~ | dV~, four columns of row r at 16 (c4 kRedLd + r) bytes
+  static constexpr uint32_t kRedLd = kRows + 1;
+  static_assert((2 * D / 4) * kRedLd * 16 <= kOffBar, "accumulators in shared memory");
   static_assert(2 * kSetCols + 2 * D <= 512, "TMEM budget");
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
@@ -71,6 +78,15 @@ __device__ __forceinline__ float ex2f(float x) {
   return y;
 }
 
+__device__ __forceinline__ const float4* peer_smem(const float4* p, uint32_t rank) {   // the same place in a CTA of the cluster
+  uint64_t a;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+  return reinterpret_cast<const float4*>(a);
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // packed column (two bf16 per 32-bit column) of K step k (16 queries) inside S^T or dA^T: the warps of the first
 // half write over the first 16 columns of their own 32 scores, the second half over columns [32, 48)
 __device__ __forceinline__ constexpr uint32_t pcol(int k) { return (uint32_t)((k >> 1) * 32 + (k & 1) * 8); }
@@ -78,16 +94,18 @@ __device__ __forceinline__ constexpr uint32_t pcol(int k) { return (uint32_t)((k
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_z,
-                      const __grid_constant__ CUtensorMap tmap_kv, float* __restrict__ ws_dKV,
-                      __nv_bfloat16* __restrict__ ws_dKV16, const float* __restrict__ ws_LD, int nq, int m, float scale,
-                      int* status) {
+                      const __grid_constant__ CUtensorMap tmap_kv, __nv_bfloat16* __restrict__ ws_dKV16,
+                      const float* __restrict__ ws_LD, int nq, int m, float scale, int* status) {
   using C = Cfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Bars* bars = reinterpret_cast<Bars*>(smem + C::kOffBar);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mb = blockIdx.x, bh = blockIdx.y;
-  const int ntiles = (nq + kQT - 1) / kQT;
+  // this CTA's query tiles: [t0, t0 + ntiles)
+  const int rank = blockIdx.z, splits = gridDim.z, all_tiles = (nq + kQT - 1) / kQT;
+  const int per = (all_tiles + splits - 1) / splits, t0 = rank * per;
+  const int ntiles = all_tiles - t0 < per ? all_tiles - t0 : per;
 
   if (threadIdx.x == 0) {
     prefetch_tmap(&tmap_q);
@@ -133,11 +151,11 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         // (the copy may run up to 65 pairs past the rows of this (batch, head), into the next one's or into the slack
         // the buffer is allocated with; those queries are masked)
         bulk_load_1d(smem + C::kOffLd + (uint32_t)s * C::kLdStride,
-                     reinterpret_cast<const uint8_t*>((reinterpret_cast<uintptr_t>(LDg + i * kQT)) & ~uintptr_t(15)),
+                     reinterpret_cast<const uint8_t*>((reinterpret_cast<uintptr_t>(LDg + (t0 + i) * kQT)) & ~uintptr_t(15)),
                      C::kLdBytes, &bars->in_full[s]);
         for (int gx = 0; gx < C::kDBoxes; ++gx) {
-          tma_load_3d(qs + gx * C::kInBoxBytes, &tmap_q, &bars->in_full[s], gx * 64, i * kQT, bh);
-          tma_load_3d(qs + C::kInBytes + gx * C::kInBoxBytes, &tmap_z, &bars->in_full[s], gx * 64, i * kQT, bh);
+          tma_load_3d(qs + gx * C::kInBoxBytes, &tmap_q, &bars->in_full[s], gx * 64, (t0 + i) * kQT, bh);
+          tma_load_3d(qs + C::kInBytes + gx * C::kInBoxBytes, &tmap_z, &bars->in_full[s], gx * 64, (t0 + i) * kQT, bh);
         }
         ++issued;
       }
@@ -224,7 +242,7 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         float2 ld[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-          const int gq = i * kQT + c0 + e;
+          const int gq = (t0 + i) * kQT + c0 + e;
           ld[e] = gq < nq ? ldq[c0 + e] : make_float2(INFINITY, 0.f);         // beyond n_q: P = exp2(-inf) = 0
         }
         tmem_wait_ld();
@@ -250,33 +268,45 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     if (__all_sync(0xffffffffu, ok && mbar_wait(&bars->acc_done, 0, status, 506, &bars->abort) &&
                                     *(volatile int*)&bars->abort == 0)) {
       tc_fence_after();
-      const int r = mb * kRows + q * 32 + lane;   // measurement
-      // workspace row: dK~ | dV~; the first half of the warps stores dK~, the second dV~
+      // dK~ (the first half of the warps) and dV~ of the lane's measurement; every product has finished, so K~, V~ and the
+      // ring may be overwritten
       const uint32_t acc = tbase + (hf == 0 ? C::kColK : C::kColV);
-      float* o = ws_dKV + ((int64_t)bh * m + r) * 2 * D + hf * D;
-      __nv_bfloat16* o16 = ws_dKV16 + ((int64_t)bh * m + r) * 2 * D + hf * D;
+      float4* red = reinterpret_cast<float4*>(smem) + (hf * D / 4) * C::kRedLd + q * 32 + lane;
 #pragma unroll 1
       for (int c0 = 0; c0 < D; c0 += 16) {
         uint32_t v[16];
-        tmem_ld_32x32b_x16(acc + c0, v);          // the whole warp takes part in the load
+        tmem_ld_32x32b_x16(acc + c0, v);
         tmem_wait_ld();
-        if (r < m) {
 #pragma unroll
-          for (int e = 0; e < 16; e += 4)
-            *reinterpret_cast<float4*>(o + c0 + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]),
-                                                                 __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
-          uint32_t h[8];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
-            h[e >> 1] = *reinterpret_cast<uint32_t*>(&b2);
-          }
-          *reinterpret_cast<uint4*>(o16 + c0) = make_uint4(h[0], h[1], h[2], h[3]);
-          *reinterpret_cast<uint4*>(o16 + c0 + 8) = make_uint4(h[4], h[5], h[6], h[7]);
-        }
+        for (int e = 0; e < 16; e += 4)
+          red[((c0 + e) / 4) * C::kRedLd] = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]),
+                                                        __uint_as_float(v[e + 3]));
       }
     }
   }
+  tc_fence_before();
+  if (splits > 1) cluster_sync_all();
+  else __syncthreads();
+  if (*(volatile int*)&bars->abort == 0) {
+    // workspace row: dK~ | dV~; this CTA's rows, eight columns per thread
+    const int rows = kRows / splits;
+    for (int i = threadIdx.x; i < rows * (2 * D / 8); i += kThreads) {
+      const int r = rank * rows + i / (2 * D / 8), c8 = i % (2 * D / 8);
+      if (mb * kRows + r >= m) continue;
+      const float4* src = reinterpret_cast<const float4*>(smem) + 2 * c8 * C::kRedLd + r;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+      for (int k = 0; k < splits; ++k) {
+        const float4* p = splits > 1 ? peer_smem(src, k) : src;
+        const float4 u = p[0], w = p[C::kRedLd];
+        x.x += u.x; x.y += u.y; x.z += u.z; x.w += u.w;
+        y.x += w.x; y.y += w.y; y.z += w.z; y.w += w.w;
+      }
+      __nv_bfloat162 h[4] = {__floats2bfloat162_rn(x.x, x.y), __floats2bfloat162_rn(x.z, x.w), __floats2bfloat162_rn(y.x, y.y),
+                             __floats2bfloat162_rn(y.z, y.w)};
+      *reinterpret_cast<uint4*>(ws_dKV16 + ((int64_t)bh * m + mb * kRows + r) * 2 * D + 8 * c8) = *reinterpret_cast<uint4*>(h);
+    }
+  }
+  if (splits > 1) cluster_sync_all();             // nobody leaves while its shared memory is being read
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
@@ -296,10 +326,34 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   static DeviceFlags smem_opt_in;
   if ((e = ensure_dynamic_smem(bwd_cols_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
-  const dim3 grid((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  bwd_cols_sm100_kernel<D><<<grid, kThreads, C::kSmemBytes, s>>>(tq, tz, c->tmap_kv, c->bw_dKV, c->bw_dKV16, c->bw_LD,
-                                                                (int)p.nq, (int)p.m, scale, c->status);
-  return cudaGetLastError();
+  // Queries per block shared out between 1, 2 or (d = 64) 4 CTAs: the fewest rounds of CTAs (one per SM) weighted with their
+  // length, a CTA's start and end counted as kFixed query tiles.  Measured, us with 1 / 2 / 4: d = 64, 25 query tiles: 24
+  // blocks 31 / 22 / 17, 72 blocks 31 / 23 / 48, 192 blocks 61 / 65 / 98; d = 128: 64 blocks of 128 tiles 126 / 77 / 100, 16
+  // blocks of 32 tiles 38 / 31 / 54.
+  const int64_t blocks = (p.m + kRows - 1) / kRows * p.B * p.H, tiles = (p.nq + kQT - 1) / kQT;
+  constexpr int kFixed = 12;
+  int splits = 1;
+  int64_t best = 0;
+  for (int k = 1; k <= (D == 64 ? 4 : 2); k *= 2) {
+    const int64_t per = (tiles + k - 1) / k;
+    if (k > 1 && (k - 1) * per >= tiles) break;   // every CTA has a tile
+    const int64_t cost = (blocks * k + c->sms - 1) / c->sms * (per + kFixed);
+    if (k == 1 || cost < best) { best = cost; splits = k; }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(p.B * p.H), (unsigned)splits);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = (unsigned)splits;
+  cfg.attrs = attr;
+  cfg.numAttrs = splits > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, bwd_cols_sm100_kernel<D>, tq, tz, c->tmap_kv, c->bw_dKV16, (const float*)c->bw_LD, (int)p.nq, (int)p.m,
+                            scale, c->status);
 }
 
 }  // namespace
