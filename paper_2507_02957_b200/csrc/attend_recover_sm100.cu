@@ -189,7 +189,7 @@ struct Waiter {
 // Z (bf16, as fed to the first product), every row's log sum exp, and the decision |x_t| > theta_t of every layer,
 // one bit per column: word c / 32 of (layer, row), bit 31 - c % 32.  With alpha_out (the gradients of the decoder's
 // weights need them) also the iterates alpha^1 .. alpha^T as bf16: alpha^t of (b, h, row) at slot t of alpha_slot
-// elements each (slot 0, alpha^0 = 0, is the caller's to clear), and with sign_out the sign bit of every x_t in the
+// elements each (slot 0, alpha^0 = 0, is left alone), and with sign_out the sign bit of every x_t in the
 // layout of the decisions (the gradient of the thresholds is - sum sign(x_t) o dx_t).
 // kRec: 0 = the plain forward; 1 = also Z, log sum exp and the decisions (kMasks); 2 = also the iterates and the sign
 // bits of x_t (kKeep: only then are alpha_out / sign_out looked at, so that mode 1 carries none of their registers)
@@ -296,8 +296,12 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
           }
         }
         // K~|V~ come from the compression kernel before this one in the stream: with a programmatic dependent launch
-        // this kernel may have started (and loaded its first Q tiles) before that one finished
-        if (items_done == 0) pdl_wait();
+        // this kernel may have started (and loaded its first Q tiles) before that one finished.  (Every other role's global
+        // accesses follow from what this one loads.)
+        if (items_done == 0) {
+          pdl_wait();
+          pdl_launch_dependents();
+        }
         for (int j = 0; j < nchunks && !w.dead; ++j, ++g) {
           const int s = g % C::kStages;
           ring_wait_k(g, 201);

@@ -95,6 +95,8 @@ bwd_recur_pair_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   // 2 x 128 x 224 + 128 x 56 = 64512 registers
   if (warp >= 8) {
@@ -344,10 +346,9 @@ cudaError_t launch_sm100_bwd_recur_pair(csat_ctx* c, const void* G, cudaStream_t
   if ((e = make_tmap_bf16_3d(&tg, G, qd, qs, qb)) != cudaSuccess) return e;
   if ((e = make_tmap_bf16_3d(&tz, c->bw_dZ16, qd, qs, qb)) != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.nq + kTiles * kRows - 1) / (kTiles * kRows)), (unsigned)(p.B * p.H));
-  bwd_recur_pair_kernel<<<grid, kThreads, kSmemBytes, s>>>(
-      c->tmap_mats, tg, tz, c->bw_Z16, c->bw_LD, c->bw_maskbits, (int)p.nq, (int)p.H, p.T, c->psi ? 1 : 0,
+  return launch_pdl(
+      bwd_recur_pair_kernel, grid, kThreads, kSmemBytes, s, c->tmap_mats, tg, tz, c->bw_Z16, c->bw_LD, c->bw_maskbits, (int)p.nq, (int)p.H, p.T, c->psi ? 1 : 0,
       c->status, c->weight_grads ? c->bw_dx16 : nullptr, (int64_t)(p.B * p.H * p.nq * p.d));
-  return cudaGetLastError();
 }
 
 }  // namespace csat

@@ -120,6 +120,8 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 4) {
     if (T > 0 && elect_one()) {
@@ -388,6 +390,8 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 4) {
     if (elect_one()) {
@@ -524,10 +528,10 @@ cudaError_t launch_recur(csat_ctx* c, const void* G, cudaStream_t s) {
   cudaError_t e = ensure_dynamic_smem(bwd_recur_sm100_kernel<D, kUntied>, (int)C::kSmemBytes, c->device, smem_opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  bwd_recur_sm100_kernel<D, kUntied><<<grid, kRThreads, C::kSmemBytes, s>>>(
+  return launch_pdl(
+      bwd_recur_sm100_kernel<D, kUntied>, grid, kRThreads, C::kSmemBytes, s,
       kUntied ? c->tmap_lmats : c->tmap_mats, c->bw_Z16, (const __nv_bfloat16*)G, c->bw_dZ16, c->bw_LD, c->bw_maskbits, (int)p.nq, (int)p.H, p.T,
       c->psi ? 1 : 0, c->status, c->weight_grads ? c->bw_dx16 : nullptr, (int64_t)(p.B * p.H * p.nq * p.d));
-  return cudaGetLastError();
 }
 
 template <int D>
@@ -545,9 +549,8 @@ cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
   if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  bwd_dq_sm100_kernel<D><<<grid, kQThreads, C::kSmemBytes, s>>>(tq, tz, c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD, (int)p.nq,
-                                                              (int)p.m, scale, c->status);
-  return cudaGetLastError();
+  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD,
+                    (int)p.nq, (int)p.m, scale, c->status);
 }
 
 }  // namespace

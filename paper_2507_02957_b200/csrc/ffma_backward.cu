@@ -12,6 +12,7 @@
 // columns 158 -> 33, Phi^T 16.6 -> 8.0 us.
 #include "csat_internal.h"
 #include "ffma_tile.cuh"
+#include "sm100_ptx.cuh"
 
 namespace csat {
 namespace {
@@ -61,9 +62,10 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
   const int64_t hdd = (int64_t)h * d * d;
 
   if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
+  ptx::pdl_wait();                                          // K~|V~ come from the kernel before this one
+  ptx::pdl_launch_dependents();
   load_own_rows<T>(rows_smem + L::kQ + own, kLdA, Q + (int64_t)bh * p.nq * d, row0, p.nq, d, kRW, lane, d);
   __syncwarp();
-
   float2 a[TR][2 * kTCQ];
   float lse[TR];
   {
@@ -380,6 +382,8 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_cols_kernel(float* __restri
     StageRows<float>::run(dst + CQ * kLdB, kLdB, Gb + i0 * d, CQ, have, d, lane);
     for (int i = lane; i < 2 * CQ; i += 32) dst[2 * CQ * kLdB + i] = (i >> 1) < have ? LDb[i0 * 2 + i] : 0.f;
   };
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   int64_t i0 = (int64_t)warp * CQ;
   if (i0 < nq) stage(i0, 0);
   if (warp == 0) load_own_rows<T>(cols_smem + L::kK, kLdA, kvb, r0, m, d, L::kRows, lane, 2 * d);
@@ -471,6 +475,8 @@ __global__ void __launch_bounds__(kThreads) ffma_phiT_kernel(T* __restrict__ dK,
   };
   float2 acc[8][2 * TCQ];                                   // tokens 4 ty + {0..3} and 16 + 4 ty + {0..3} of the warp's 32
   clear(acc);
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   fetch(0);
   for (int64_t r0 = 0; r0 < m; r0 += kPtK) {
     __syncthreads();
@@ -526,8 +532,8 @@ cudaError_t launch_rows(csat_ctx* c, const void* Q, const void* G, void* dQ, cud
   cudaError_t e = ensure_dynamic_smem(ffma_bwd_rows_kernel<T, DP, TR>, L::kFloats * 4, c->device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)(c->p.B * c->p.H));
-  ffma_bwd_rows_kernel<T, DP, TR><<<grid, kThreads, L::kFloats * 4, s>>>((T*)dQ, (const T*)Q, (const T*)G, (const T*)c->kv, a);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_bwd_rows_kernel<T, DP, TR>, grid, kThreads, L::kFloats * 4, s, (T*)dQ, (const T*)Q, (const T*)G,
+                    (const T*)c->kv, a);
 }
 
 template <typename T, int DP, int TR>
@@ -540,9 +546,8 @@ cudaError_t launch_cols(csat_ctx* c, const void* Q, cudaStream_t s, float scale)
   cudaError_t e = ensure_dynamic_smem(ffma_bwd_cols_kernel<T, DP, TR, CQ>, L::kFloats * 4, c->device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.m + L::kRows - 1) / L::kRows), (unsigned)(p.B * p.H));
-  ffma_bwd_cols_kernel<T, DP, TR, CQ><<<grid, kThreads, L::kFloats * 4, s>>>(c->bw_dKV, (const T*)Q, (const T*)c->kv, c->bw_dZ, c->bw_LD,
-                                                                           p.nq, p.m, (int)p.d, scale);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_bwd_cols_kernel<T, DP, TR, CQ>, grid, kThreads, L::kFloats * 4, s, c->bw_dKV, (const T*)Q, (const T*)c->kv,
+                    c->bw_dZ, c->bw_LD, p.nq, p.m, (int)p.d, scale);
 }
 
 template <typename T, int TCQ>
@@ -550,9 +555,8 @@ cudaError_t launch_phiT(csat_ctx* c, void* dK, void* dV, cudaStream_t s) {
   const Params& p = c->p;
   const int cb = (int)((p.d + 32 * TCQ - 1) / (32 * TCQ));
   const dim3 grid((unsigned)((p.n + kPtTok - 1) / kPtTok), (unsigned)(p.B * p.H), (unsigned)(2 * cb));
-  ffma_phiT_kernel<T, TCQ><<<grid, kThreads, 0, s>>>((T*)dK, (T*)dV, (const T*)c->phi, c->bw_dKV, p.n, p.n_pad, p.m, (int)p.d, (int)p.H,
-                                                    p.separate_phi ? (int)p.H : 0, cb);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_phiT_kernel<T, TCQ>, grid, kThreads, 0, s, (T*)dK, (T*)dV, (const T*)c->phi, c->bw_dKV, p.n, p.n_pad, p.m,
+                    (int)p.d, (int)p.H, p.separate_phi ? (int)p.H : 0, cb);
 }
 
 template <typename T, int DP>

@@ -8,6 +8,7 @@
 // 32 heads of 1024 x 96 in bf16, m = 128, T = 10: 384 -> 46 and 1573 -> 192 (1573: 5 TFLOP/s; 192: 41 of 74).
 #include "csat_internal.h"
 #include "ffma_tile.cuh"
+#include "sm100_ptx.cuh"
 
 namespace csat {
 namespace {
@@ -62,6 +63,8 @@ __global__ void __launch_bounds__(kCmpWarps * 32) ffma_compress_kernel(TO* __res
       if (j0 + k < n && c < d) vb[u] = *reinterpret_cast<const uint4*>(src + (j0 + k) * d + c);
     }
   };
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   int64_t j0 = (int64_t)warp * kCmpK;
   if (j0 < n) fetch(j0);
   for (; j0 < n; j0 += kCmpWarps * kCmpK) {
@@ -156,9 +159,10 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
   const int64_t hdd = (int64_t)h * d * d;
 
   if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
+  ptx::pdl_wait();                                          // K~|V~ come from the kernel before this one
+  ptx::pdl_launch_dependents();
   load_own_rows<T>(Arows, kLdA, Q + (int64_t)bh * p.nq * d, row0, p.nq, d, kRW, lane, d);
   __syncwarp();
-
   float2 a[TR][2 * kTCQ];                                   // Z, then the iterate
   {
     float mx[TR], sum[TR];
@@ -282,10 +286,8 @@ cudaError_t launch_compress(csat_ctx* c, TO* dst, const void* K, const void* V, 
   if (e != cudaSuccess) return e;
   const int cb = (int)((p.d + kCols - 1) / kCols);
   const dim3 grid((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(p.B * p.H), (unsigned)(2 * cb));
-  ffma_compress_kernel<T, TO, TR, TCQ><<<grid, kCmpWarps * 32, kBytes, s>>>(
-      dst, (const T*)c->phi, (const T*)K, (const T*)V, n_len, p.n_pad, p.m, (int)p.d, (int)p.H, p.separate_phi ? (int)p.H : 0,
-      phi_j0, cb);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_compress_kernel<T, TO, TR, TCQ>, grid, kCmpWarps * 32, kBytes, s, dst, (const T*)c->phi, (const T*)K, (const T*)V,
+                    n_len, p.n_pad, p.m, (int)p.d, (int)p.H, p.separate_phi ? (int)p.H : 0, phi_j0, cb);
 }
 
 // The tile: 32 measurements x all columns of K~ or V~ up to 96 (the operand reads of 8 rows per lane keep up with the
@@ -314,9 +316,8 @@ cudaError_t launch_attend(const FfmaAttend& a, const void* Q, const void* kv, vo
   cudaError_t e = ensure_dynamic_smem(ffma_attend_kernel<T, DP, TR>, L::kFloatsUntied * 4, a.device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)a.BH);
-  ffma_attend_kernel<T, DP, TR><<<grid, kThreads, (a.layer_stride ? L::kFloatsUntied : L::kFloats) * 4, s>>>((T*)out, (const T*)Q,
-                                                                                                           (const T*)kv, a);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, a.sms), ffma_attend_kernel<T, DP, TR>, grid, kThreads, (a.layer_stride ? L::kFloatsUntied : L::kFloats) * 4, s, (T*)out,
+                    (const T*)Q, (const T*)kv, a);
 }
 
 template <typename T, int DP>

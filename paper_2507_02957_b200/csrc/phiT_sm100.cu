@@ -81,6 +81,8 @@ phiT_sm100_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -195,8 +197,7 @@ cudaError_t launch(csat_ctx* c, const void* g16, void* dK, void* dV, cudaStream_
   static DeviceFlags smem_opt_in;
   if ((e = ensure_dynamic_smem(phiT_sm100_kernel<D, SEP>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.n + kTileM - 1) / kTileM), (unsigned)(p.B * p.H));
-  phiT_sm100_kernel<D, SEP><<<grid, kThreads, C::kSmemBytes, s>>>(tphi, tg, tdk, tdv, (int)p.m, (int)p.n, (int)p.H, c->status);
-  return cudaGetLastError();
+  return launch_pdl(phiT_sm100_kernel<D, SEP>, grid, kThreads, C::kSmemBytes, s, tphi, tg, tdk, tdv, (int)p.m, (int)p.n, (int)p.H, c->status);
 }
 
 }  // namespace

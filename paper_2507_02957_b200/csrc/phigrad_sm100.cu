@@ -81,6 +81,8 @@ phigrad_sm100_kernel(const __grid_constant__ CUtensorMap tmap_g, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -206,8 +208,7 @@ cudaError_t launch_sm100_phigrad(csat_ctx* c, const void* K, const void* V, floa
   const unsigned grid = (unsigned)(n_tiles < c->sms ? n_tiles : c->sms);
   static DeviceFlags opt_in;
   if ((e = ensure_dynamic_smem(phigrad_sm100_kernel, (int)kSmemBytes, c->device, opt_in)) != cudaSuccess) return e;
-  phigrad_sm100_kernel<<<grid, kThreads, kSmemBytes, s>>>(tg, tk, tv, a, c->status);
-  return cudaGetLastError();
+  return launch_pdl(phigrad_sm100_kernel, dim3(grid), kThreads, kSmemBytes, s, tg, tk, tv, a, c->status);
 }
 
 }  // namespace csat

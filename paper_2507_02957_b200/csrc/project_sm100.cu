@@ -97,6 +97,8 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -279,13 +281,12 @@ cudaError_t launch_project(csat_ctx* c, const void* X, const void* W, int64_t n_
   if (p.d == 64) {
     static DeviceFlags opt_in64;
     if ((e = ensure_dynamic_smem(project_sm100_kernel<64>, (int)kSmemBytes, c->device, opt_in64)) != cudaSuccess) return e;
-    project_sm100_kernel<64><<<grid, kThreads, kSmemBytes, s>>>(tx, tw, a, c->status);
+    return launch_pdl(project_sm100_kernel<64>, dim3(grid), kThreads, kSmemBytes, s, tx, tw, a, c->status);
   } else {
     static DeviceFlags opt_in128;
     if ((e = ensure_dynamic_smem(project_sm100_kernel<128>, (int)kSmemBytes, c->device, opt_in128)) != cudaSuccess) return e;
-    project_sm100_kernel<128><<<grid, kThreads, kSmemBytes, s>>>(tx, tw, a, c->status);
+    return launch_pdl(project_sm100_kernel<128>, dim3(grid), kThreads, kSmemBytes, s, tx, tw, a, c->status);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace csat

@@ -69,11 +69,11 @@ vfold_sm100_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  pdl_wait();                     // V~ comes from the compression kernel before this one in the stream
   pdl_launch_dependents();        // the attention kernel's prologue may run under this kernel; it waits for this grid
 
   if (warp == 0) {
     if (elect_one()) {
-      pdl_wait();                 // V~ comes from the compression kernel before this one in the stream
       mbar_arrive_expect_tx(&bars->full, C::kTileBytes + C::kMatBytes);
       for (int gx = 0; gx < C::kDBoxes; ++gx)
         tma_load_3d(smem + C::kOffB + gx * C::kMatBoxBytes, &tmap_mats, &bars->full, gx * 64, 0, h * 3 + 1);

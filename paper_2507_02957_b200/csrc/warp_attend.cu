@@ -52,12 +52,14 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
   const int nchunks = (p.m + kMC - 1) / kMC;
   __nv_bfloat16* mats = smem + kOffMats;
 
-  // decoder matrices (written before the compression kernel started) and this warp's queries
+  // decoder matrices (not written by the kernel before this one)
   if (p.T > 0) {
     const __nv_bfloat16* mh = p.mats + (int64_t)h * 3 * kD * kD;
     for (int i = threadIdx.x; i < (p.has_psi ? 3 : 2) * kD * (kD / 8); i += kWarps * 32)
       cp16(mats + (i >> 3) * kLd + (i & 7) * 8, mh + i * 8, true);
   }
+  ptx::pdl_wait();                                              // K~|V~ come from the kernel before this one
+  ptx::pdl_launch_dependents();
   uint32_t q[kD / 16][4];
   {
     const __nv_bfloat16* Qb = p.Q + ((int64_t)bh * p.nq + row0) * kD + 2 * t;
@@ -70,7 +72,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
         q[k][2 * u + 1] = in1 ? *reinterpret_cast<const uint32_t*>(Qb + (g + 8) * kD + 16 * k + 8 * u) : 0u;
       }
   }
-  ptx::pdl_wait();                                              // K~|V~ come from the kernel before this one
   auto stage = [&](int j) {
     __nv_bfloat16* dst = smem + (j % kStages) * 2 * kTile;
     for (int i = threadIdx.x; i < kMC * 16; i += kWarps * 32) {

@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(kCW * 32) split_compress_kernel(TO* __restrict
     for (int j = 0; j < NT; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+  ptx::pdl_wait();
+  ptx::pdl_launch_dependents();
   int64_t j0 = (int64_t)warp * kCK;
   if (j0 < n) stage(j0, 0);
   for (int st = 0; j0 < n; j0 += kCW * kCK, st ^= 1) {
@@ -208,8 +210,10 @@ __global__ void __launch_bounds__(kW * 32) split_attend_kernel(__nv_bfloat16* __
     }
     cp_commit();
   };
-  stage(0);
   if (p.T > 0) build(p.B + hdd, d, 1, false);
+  ptx::pdl_wait();                                             // K~|V~ come from the kernel before this one
+  ptx::pdl_launch_dependents();
+  stage(0);
   uint32_t q[KS][4];
   {
     const __nv_bfloat16* Qb = Q + ((int64_t)bh * nq + row0) * d + 2 * t;
@@ -378,10 +382,9 @@ cudaError_t launch_compress(csat_ctx* c, TO* dst, const void* K, const void* V, 
   cudaError_t e = ensure_dynamic_smem(split_compress_kernel<TO, DP>, CmpSmem<DP>::kBytes, c->device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.m + kCRows - 1) / kCRows), (unsigned)(p.B * p.H), 2);
-  split_compress_kernel<TO, DP><<<grid, kCW * 32, CmpSmem<DP>::kBytes, s>>>(
-      dst, (const __nv_bfloat16*)c->phi, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, n_len, p.n_pad, p.m, (int)p.d, (int)p.H,
-      p.separate_phi ? (int)p.H : 0, phi_j0);
-  return cudaGetLastError();
+  return launch_maybe_pdl(small_grid(grid, c->sms), split_compress_kernel<TO, DP>, grid, kCW * 32, CmpSmem<DP>::kBytes, s, dst, (const __nv_bfloat16*)c->phi,
+                    (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, n_len, p.n_pad, p.m, (int)p.d, (int)p.H,
+                    p.separate_phi ? (int)p.H : 0, phi_j0);
 }
 
 template <typename TO>
@@ -398,9 +401,9 @@ template <int DP, bool kUntied> cudaError_t launch_attend(const FfmaAttend& a, c
   if (e != cudaSuccess) return e;
   const int64_t tiles = (a.nq + kRows - 1) / kRows;
   if (tiles * a.BH > (int64_t)1 << 30) return cudaErrorInvalidValue;
-  split_attend_kernel<DP, kUntied><<<(unsigned)(tiles * a.BH), kW * 32, AttSmem<DP>::kBytes, s>>>(
-      (__nv_bfloat16*)out, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)kv, a, (int)tiles);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)(tiles * a.BH));
+  return launch_maybe_pdl(small_grid(grid, a.sms), split_attend_kernel<DP, kUntied>, grid, kW * 32, AttSmem<DP>::kBytes, s,
+                    (__nv_bfloat16*)out, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)kv, a, (int)tiles);
 }
 template <int DP> cudaError_t attend_d(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
   return a.layer_stride != 0 ? launch_attend<DP, true>(a, Q, kv, out, s) : launch_attend<DP, false>(a, Q, kv, out, s);
