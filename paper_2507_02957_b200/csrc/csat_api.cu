@@ -672,8 +672,6 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
     // the iterates with CSAT_WEIGHT_GRADS) where csat_backward will look for them
     if (int rc = ensure_backward_scratch(c)) return rc;
     const bool wg = c->weight_grads && c->p.T > 0 && c->bw_alpha16 != nullptr;
-    if (wg && (e = cudaMemsetAsync(c->bw_alpha16, 0, (size_t)(c->p.B * c->p.H * c->p.nq * c->p.d) * 2, s)) != cudaSuccess)
-      return fail_cuda(c, e, "memset");
     e = csat::launch_sm100_attend_for_backward(c, Q, c->bw_Z16, c->bw_LD, 2, c->bw_maskbits, wg ? c->bw_alpha16 : nullptr, s,
                                                &launches, out);
     if (e == cudaSuccess) { c->saved_valid = true; c->saved_alpha = wg; }

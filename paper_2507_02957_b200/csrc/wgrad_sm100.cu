@@ -5,7 +5,7 @@
 //   dtheta_t = - sum  sign(x_t) o dx_t        (sign(x_t) = sign(alpha^{t+1}) wherever dx_t is not zero)
 //   dPsi   = G^T alpha^T
 // each summed over the queries and over the batch, per head (dPsi also over the heads: one dictionary).
-// The forward kernel (run for the backward pass) leaves the iterates alpha^0 .. alpha^T and the recurrence kernel the
+// The forward kernel (run for the backward pass) leaves the iterates alpha^1 .. alpha^T and the recurrence kernel the
 // dx_t, both bf16 [slot][B,H,n_q,d]; here they are only contracted:
 //
 // wgrad_gram_kernel: C = sum over a list of (slab pairs) of A1^T B and A2^T B, slabs = [n_q x d] bf16 matrices.
@@ -59,7 +59,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_a2,
                   const __grid_constant__ CUtensorMap tmap_b, SlabIndex ia1, SlabIndex ia2, SlabIndex ib,
-                  float* __restrict__ part, int nq, int H, int B, int nt, int units_per_cta, int* status,
+                  float* __restrict__ part, float* __restrict__ direct1, float* __restrict__ direct2, int zero_slot, int nq, int H, int B, int nt, int units_per_cta, int* status,
                   const uint32_t* __restrict__ signbits, float* __restrict__ thpart, int T) {
   using C = GCfg<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -90,6 +90,8 @@ wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 4) {
     if (elect_one()) {
@@ -104,7 +106,9 @@ wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
         uint8_t* st = smem + (uint32_t)s * C::kStageBytes;
         mbar_arrive_expect_tx(&bars->full[s], C::kStageBytes);
         for (int gx = 0; gx < C::kDBoxes; ++gx) {
-          tma_load_3d(st + gx * C::kBoxBytes, &tmap_a1, &bars->full[s], gx * 64, tile * kRows, ia1.off + t * ia1.tstride + bh);
+          // alpha^0 = 0 is not stored: a slab beyond the tensor reads as zeros
+          tma_load_3d(st + gx * C::kBoxBytes, &tmap_a1, &bars->full[s], gx * 64, tile * kRows,
+                      zero_slot > 0 && t == 0 ? zero_slot : ia1.off + t * ia1.tstride + bh);
           tma_load_3d(st + C::kTileBytes + gx * C::kBoxBytes, &tmap_a2, &bars->full[s], gx * 64, tile * kRows,
                       ia2.off + t * ia2.tstride + bh);
           tma_load_3d(st + 2 * C::kTileBytes + gx * C::kBoxBytes, &tmap_b, &bars->full[s], gx * 64, tile * kRows,
@@ -147,7 +151,10 @@ wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
     // epilogue: lane = row of C (d = 128: row i of A1^T B and of A2^T B; d = 64: rows 0-63 A1^T B, 64-127 A2^T B)
     const int row = warp * 32 + lane;
     const uint32_t tbase = tmem + ((uint32_t)(warp * 32) << 16);
-    float* p1 = part + ((int64_t)((blockIdx.z * gridDim.x + split) * H + h) * 2) * D * D;       // [2][D][D]
+    // the CTA's sums: partial [2][D][D] of its split, or (one split) the results themselves, matrix (layer, head) of each
+    float* p1 = direct1 != nullptr ? direct1 + (int64_t)(blockIdx.z * H + h) * D * D
+                                   : part + ((int64_t)((blockIdx.z * gridDim.x + split) * H + h) * 2) * D * D;
+    float* p2 = direct1 != nullptr ? direct2 + (int64_t)(blockIdx.z * H + h) * D * D : p1 + D * D;
     const bool have = steps > 0;
     bool ok = true;
     if (signbits != nullptr) {
@@ -215,7 +222,7 @@ wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
           for (int e = 0; e < 16; ++e) v[e] = 0u;   // a CTA without units contributes zeros
         }
         if (ok) {
-          float* o = (D == 64) ? p1 + ((int64_t)(row >> 6) * D + (row & 63)) * D + c0 : p1 + ((int64_t)a * D + row) * D + c0;
+          float* o = (D == 64) ? ((row >> 6) ? p2 : p1) + (row & 63) * D + c0 : (a ? p2 : p1) + row * D + c0;
 #pragma unroll
           for (int e = 0; e < 16; e += 4)
             *reinterpret_cast<float4*>(o + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]),
@@ -229,23 +236,27 @@ wgrad_gram_kernel(const __grid_constant__ CUtensorMap tmap_a1, const __grid_cons
   if (warp == 5) tmem_dealloc(tmem, C::kTmemCols);
 }
 
-// out[z][h][i] = sum over the splits, in order, of part[z][split][h][which][i]   (i over d*d; z = layer with one pair of
-// matrices per layer, else 0); all heads into out[i] with `over_heads` (the dictionary is shared by the heads)
-__global__ void wgrad_reduce_kernel(float* __restrict__ out, const float* __restrict__ part, int splits, int H, int Z,
-                                    int which, int64_t dd, int over_heads) {
-  const int64_t total = (over_heads ? 1 : (int64_t)Z * H) * dd;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i % dd;
-    float acc = 0.f;
-    if (over_heads) {
-      for (int h = 0; h < H; ++h)
-        for (int s = 0; s < splits; ++s) acc += part[(((int64_t)s * H + h) * 2 + which) * dd + e];
-    } else {
-      const int64_t zh = i / dd, z = zh / H, h = zh % H;
-      for (int s = 0; s < splits; ++s) acc += part[((((int64_t)z * splits + s) * H + h) * 2 + which) * dd + e];
-    }
-    out[i] = acc;
+// dS, dB [Z H][d d] = sums over the splits, in order, of part[z][split][h][2][d d]; grid (d d / 1024, Z H, 2)
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(float* __restrict__ dS, float* __restrict__ dB, const float* __restrict__ part,
+                                                           int splits, int H, int dd) {
+  const int e = (blockIdx.x * 256 + threadIdx.x) * 4, zh = blockIdx.y, z = zh / H, h = zh % H, which = blockIdx.z;
+  if (e >= dd) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s = 0; s < splits; ++s) {
+    const float4 x = *reinterpret_cast<const float4*>(part + ((((int64_t)z * splits + s) * H + h) * 2 + which) * dd + e);
+    acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
   }
+  *reinterpret_cast<float4*>((which ? dB : dS) + (int64_t)zh * dd + e) = acc;
+}
+
+// out [d d] = sum over the heads and splits, in order, of part[split][h][0] (the dictionary is shared by the heads)
+__global__ void wgrad_reduce_heads_kernel(float* __restrict__ out, const float* __restrict__ part, int splits, int H, int64_t dd) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= dd) return;
+  float acc = 0.f;
+  for (int h = 0; h < H; ++h)
+    for (int s = 0; s < splits; ++s) acc += part[(((int64_t)s * H + h) * 2) * dd + e];
+  out[e] = acc;
 }
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t b) { return __uint_as_float(b << 16); }
@@ -284,10 +295,11 @@ dtheta_partial_kernel(float* __restrict__ partial, const __nv_bfloat16* __restri
 }
 
 // out[t][h] = sum over the chunks, in order.  from_contraction: partial [chunk][H][T] holds + sum sign(x) o dx (the
-// gradient is its negative); else partial [chunk][T][H] already holds the negative
+// gradient is its negative); else partial [chunk][T][H] already holds the negative.  `zero` [nzero] is cleared on the side
 __global__ void dtheta_reduce_kernel(float* __restrict__ out, const float* __restrict__ partial, int chunks, int T, int H,
-                                     int from_contraction) {
+                                     int from_contraction, float* __restrict__ zero, int nzero) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int k = i; k < nzero; k += gridDim.x * blockDim.x) zero[k] = 0.f;
   if (i >= T * H) return;
   const int t = i / H, h = i % H;
   float acc = 0.f;
@@ -310,16 +322,15 @@ cudaError_t slab_map(CUtensorMap* m, const void* base, const Params& p, int64_t 
 template <int D>
 cudaError_t launch_gram(csat_ctx* c, const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b, SlabIndex ia1,
                         SlabIndex ia2, SlabIndex ib, int nt, int splits, int units_per_cta, cudaStream_t s, int layers_z = 1,
-                        const uint32_t* signbits = nullptr) {
+                        const uint32_t* signbits = nullptr, float* direct1 = nullptr, float* direct2 = nullptr, int zero_slot = 0) {
   using C = GCfg<D>;
   static DeviceFlags smem_opt_in;
   cudaError_t e = ensure_dynamic_smem(wgrad_gram_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in);
   if (e != cudaSuccess) return e;
   const Params& p = c->p;
-  wgrad_gram_kernel<D><<<dim3((unsigned)splits, (unsigned)p.H, (unsigned)layers_z), kThreads, C::kSmemBytes, s>>>(
-      a1, a2, b, ia1, ia2, ib, c->bw_wpart, (int)p.nq, (int)p.H, (int)p.B, nt, units_per_cta, c->status, signbits,
+  return launch_pdl(
+      wgrad_gram_kernel<D>, dim3((unsigned)splits, (unsigned)p.H, (unsigned)layers_z), kThreads, C::kSmemBytes, s, a1, a2, b, ia1, ia2, ib, c->bw_wpart, direct1, direct2, zero_slot, (int)p.nq, (int)p.H, (int)p.B, nt, units_per_cta, c->status, signbits,
       c->bw_thpart, p.T);
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -333,7 +344,7 @@ int wgrad_splits(const csat_ctx* c) {
   return (int)(s < 1 ? 1 : s);
 }
 
-// needs bw_alpha16 (slots 0 .. T, slot 0 cleared), bw_dx16 (slots 0 .. T-1), bw_Z16 and G; fills bw_wgrad:
+// needs bw_alpha16 (slots 1 .. T; slot 0, alpha^0 = 0, is never read), bw_dx16 (slots 0 .. T-1), bw_Z16 and G; fills bw_wgrad:
 // dS [H,d,d] | dB [H,d,d] | dPsi [d,d] | dtheta [T,H]
 cudaError_t launch_sm100_wgrad(csat_ctx* c, const void* G, cudaStream_t s, int* launches) {
   const Params& p = c->p;
@@ -353,39 +364,45 @@ cudaError_t launch_sm100_wgrad(csat_ctx* c, const void* G, cudaStream_t s, int* 
   float* dB = dS + (int64_t)Z * p.H * dd;
   float* dPsi = dB + (int64_t)Z * p.H * dd;
   float* dTh = dPsi + dd;
-  const unsigned rblocks = (unsigned)(((int64_t)Z * p.H * dd + 255) / 256);
   // dS = sum_t (alpha^t)^T dx_t, dB = sum_t Z^T dx_t (per layer: no sum over t, the layer is the grid's z index)
   const SlabIndex ia{0, (int)BH}, iz{0, 0}, ix{0, (int)BH};
   const int nt = Z > 1 ? 1 : p.T;
   // dtheta rides along where the per-layer sums fit the kernel's shared memory
   const bool fused_theta = c->bw_signbits != nullptr && nt <= kMaxFusedLayers;
   const uint32_t* sgn = fused_theta ? c->bw_signbits : nullptr;
-  e = p.d == 64 ? launch_gram<64>(c, ta, tz, tx, ia, iz, ix, nt, splits, upc, s, Z, sgn)
-                : launch_gram<128>(c, ta, tz, tx, ia, iz, ix, nt, splits, upc, s, Z, sgn);
+  // with one split (per-layer weights: every (head, layer) its own CTA) the kernel writes the results themselves
+  const bool direct = splits == 1;
+  const int zero_slot = (int)((p.T + 1) * BH);
+  float *d1 = direct ? dS : nullptr, *d2 = direct ? dB : nullptr;
+  e = p.d == 64 ? launch_gram<64>(c, ta, tz, tx, ia, iz, ix, nt, splits, upc, s, Z, sgn, d1, d2, zero_slot)
+                : launch_gram<128>(c, ta, tz, tx, ia, iz, ix, nt, splits, upc, s, Z, sgn, d1, d2, zero_slot);
   if (e != cudaSuccess) return e;
-  wgrad_reduce_kernel<<<rblocks, 256, 0, s>>>(dS, c->bw_wpart, splits, (int)p.H, Z, 0, dd, 0);
-  wgrad_reduce_kernel<<<rblocks, 256, 0, s>>>(dB, c->bw_wpart, splits, (int)p.H, Z, 1, dd, 0);
-  *launches += 3;
+  *launches += 1;
+  if (!direct) {
+    wgrad_reduce_kernel<<<dim3((unsigned)((dd + 1023) / 1024), (unsigned)(Z * p.H), 2), 256, 0, s>>>(dS, dB, c->bw_wpart, splits,
+                                                                                                  (int)p.H, (int)dd);
+    *launches += 1;
+  }
   if (c->psi) {
     // dPsi = G^T alpha^T: A1 = A2 = G, B = slot T of the iterates, one "layer"
     const SlabIndex ig{0, 0}, iaT{(int)(p.T * BH), 0};
     e = p.d == 64 ? launch_gram<64>(c, tg, tg, ta, ig, ig, iaT, 1, splits, upc, s)
                   : launch_gram<128>(c, tg, tg, ta, ig, ig, iaT, 1, splits, upc, s);
     if (e != cudaSuccess) return e;
-    wgrad_reduce_kernel<<<(unsigned)((dd + 255) / 256), 256, 0, s>>>(dPsi, c->bw_wpart, splits, (int)p.H, 1, 0, dd, 1);
+    wgrad_reduce_heads_kernel<<<(unsigned)((dd + 255) / 256), 256, 0, s>>>(dPsi, c->bw_wpart, splits, (int)p.H, dd);
     *launches += 2;
-  } else {
-    if ((e = cudaMemsetAsync(dPsi, 0, (size_t)dd * 4, s)) != cudaSuccess) return e;
   }
+  float* zero = c->psi ? nullptr : dPsi;                       // no dictionary: its gradient is zero
+  const int nzero = c->psi ? 0 : (int)dd;
   // dtheta [T,H]: the contraction kernel's partial sums [split][H][T], or the streaming kernel's [chunk][T][H]
   if (fused_theta) {
-    dtheta_reduce_kernel<<<(unsigned)((p.T * p.H + 255) / 256), 256, 0, s>>>(dTh, c->bw_thpart, splits, (int)p.T, (int)p.H, 1);
+    dtheta_reduce_kernel<<<(unsigned)((p.T * p.H + 255) / 256), 256, 0, s>>>(dTh, c->bw_thpart, splits, (int)p.T, (int)p.H, 1, zero, nzero);
     *launches += 1;
   } else {
     const int chunks = 64;
     dtheta_partial_kernel<<<dim3(chunks, (unsigned)p.H, (unsigned)p.T), kThThreads, 0, s>>>(
         c->bw_thpart, c->bw_alpha16, c->bw_dx16, BH * p.nq * p.d, p.nq * p.d, (int)p.B, (int)p.H, p.T);
-    dtheta_reduce_kernel<<<(unsigned)((p.T * p.H + 255) / 256), 256, 0, s>>>(dTh, c->bw_thpart, chunks, (int)p.T, (int)p.H, 0);
+    dtheta_reduce_kernel<<<(unsigned)((p.T * p.H + 255) / 256), 256, 0, s>>>(dTh, c->bw_thpart, chunks, (int)p.T, (int)p.H, 0, zero, nzero);
     *launches += 2;
   }
   return cudaGetLastError();
