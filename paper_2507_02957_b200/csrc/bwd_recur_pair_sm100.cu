@@ -5,7 +5,7 @@
 // which the products dx_t (S - I)^T and dx_t B^T take 1084.  Two tiles alternate on the tensor pipe here.  What stood
 // against that was tensor memory (accumulator and dZ of two tiles fill it), so the operand dx_t goes through shared memory,
 // in two buffers per tile; and the matrix instructions are issued by a warp of their own per tile (issued from a compute
-// warp they delay its next pass by ~600 cycles).  16 heads of 8192 queries, T = 20: 203 -> @P@ us.
+// warp they delay its next pass by ~600 cycles).  16 heads of 8192 queries, T = 20: 203 -> 149 us.
 //
 // CTA = 12 warps: 0-3 tile A, 4-7 tile B (one thread per query row, 224 registers), 8 and 10 issue tile A's and B's MMAs,
 // 9 loads G (into the operand buffers, whose layout it then has) and the matrices (S - I | B; with a dictionary Psi first, in
