@@ -206,7 +206,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
                             int has_psi, float scale_log2, int items_x, int n_items, int bh0, int* status,
                             float* __restrict__ lse_out, int lse_stride, __nv_bfloat16* __restrict__ z_out,
                             uint32_t* __restrict__ mask_out, __nv_bfloat16* __restrict__ alpha_out,
-                            int64_t alpha_slot, uint32_t* __restrict__ sign_out) {
+                            int64_t alpha_slot, uint32_t* __restrict__ sign_out, int wait_first) {
   using C = Cfg<D, kRec == 0>;
   constexpr bool kMasks = kRec >= 1, kKeep = kRec >= 2, kStaged = kRec == 0;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -261,6 +261,8 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  // A kernel before this one that is not this call's own compression or fold may still be writing Q, theta or the matrices
+  if (wait_first) pdl_wait();
 
   // 2 x 128 x 224 + 128 x 56 = 64512 registers; each branch below starts with its own setmaxnreg
   if (warp >= kMmaWarp) {
@@ -295,9 +297,10 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
             ++q_loads[t];
           }
         }
-        // K~|V~ come from the compression kernel before this one in the stream: with a programmatic dependent launch
-        // this kernel may have started (and loaded its first Q tiles) before that one finished.  (Every other role's global
-        // accesses follow from what this one loads.)
+        // K~|V~ come from the compression (or fold) kernel before this one in the stream: with a programmatic dependent
+        // launch this kernel may have started (and loaded its first Q tiles) before that one finished.  What else is read
+        // (Q, theta, the matrices) was complete before that kernel let this one start, unless wait_first says otherwise;
+        // every store follows from what is loaded below.
         if (items_done == 0) {
           pdl_wait();
           pdl_launch_dependents();
@@ -1166,7 +1169,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
 
 template <int D, bool kUntied, int kRec = 0, bool kFold = false>
 cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int T, float* lse_out, int lse_stride,
-                   __nv_bfloat16* z_out = nullptr, uint32_t* mask_out = nullptr, __nv_bfloat16* alpha_out = nullptr) {
+                   __nv_bfloat16* z_out = nullptr, uint32_t* mask_out = nullptr, __nv_bfloat16* alpha_out = nullptr, bool wait_first = false) {
   using C = Cfg<D, kRec == 0>;
   const Params& p = c->p;
   CUtensorMap tq;
@@ -1214,7 +1217,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int T,
                             kUntied ? c->tmap_lmats : c->tmap_mats, to, c->tmap_vb, (__nv_bfloat16*)out, c->thr(), c->thr_stride(),
                             (int)p.nq, (int)p.m, (int)p.H, T, c->psi ? 1 : 0, scale_log2, (int)items_x, (int)n_items,
                             (int)c->bh0, c->status, lse_out, lse_stride, z_out, mask_out, alpha_out,
-                            (int64_t)(p.B * p.H * p.nq * p.d), alpha_out != nullptr ? c->bw_signbits : nullptr);
+                            (int64_t)(p.B * p.H * p.nq * p.d), alpha_out != nullptr ? c->bw_signbits : nullptr, wait_first ? 1 : 0);
 }
 
 }  // namespace
@@ -1251,11 +1254,12 @@ cudaError_t make_layer_weights_tmap(csat_ctx* c) {
   return make_tmap_bf16_3d(&c->tmap_lmats, c->lmats_bf16, md, ms, mb);
 }
 
-cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches) {
+cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first) {
   *launches += 1;
+#define CSAT_ATTEND(DD, UU) launch<DD, UU>(c, Q, out, s, c->p.T, nullptr, 0, nullptr, nullptr, nullptr, wait_first)
   // with untied layers and T > 0 the per-layer kernel; the set-up has then built its operands for exactly T layers
   if (c->w_S && c->w_untied && c->p.T > 0)
-    return c->p.d == 64 ? launch<64, true>(c, Q, out, s, c->p.T, nullptr, 0) : launch<128, true>(c, Q, out, s, c->p.T, nullptr, 0);
+    return c->p.d == 64 ? CSAT_ATTEND(64, true) : CSAT_ATTEND(128, true);
   if (warp_attend_better(c)) return launch_warp_attend(c, Q, out, s);
   // Long jobs with the ISTA-derived decoder (one S, B and one positive threshold for all layers) fold B into the
   // values first: one more small launch, which only pays where the attention kernel walks several items per SM
@@ -1266,10 +1270,12 @@ cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, c
   if (!c->w_S && c->p.T >= 2 && c->p.lambda > 0.0 && tiles >= (c->p.d == 128 ? 2 : 8) * (int64_t)c->sms) {
     cudaError_t e = launch_sm100_vfold(c, s, launches);
     if (e != cudaSuccess) return e;
+    // the fold waits for whatever is before it: nothing to wait for but the fold itself
     return c->p.d == 64 ? launch<64, false, 0, true>(c, Q, out, s, c->p.T, nullptr, 0)
                         : launch<128, false, 0, true>(c, Q, out, s, c->p.T, nullptr, 0);
   }
-  return c->p.d == 64 ? launch<64, false>(c, Q, out, s, c->p.T, nullptr, 0) : launch<128, false>(c, Q, out, s, c->p.T, nullptr, 0);
+  return c->p.d == 64 ? CSAT_ATTEND(64, false) : CSAT_ATTEND(128, false);
+#undef CSAT_ATTEND
 }
 
 // The forward with what the backward pass needs as its only outputs: Z (bf16), the rows' log sum exp and the layers'

@@ -246,7 +246,8 @@ cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cud
 // attend_recover_sm100.cu : tcgen05 compressed attention + recovery (bf16, d in {64, 128})
 cudaError_t make_attend_tmaps(csat_ctx* c);
 cudaError_t make_layer_weights_tmap(csat_ctx* c);
-cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches);
+// wait_first: the kernel before it in the stream is not this call's own compression, so nothing is read before that has finished
+cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first = false);
 // the forward run for the backward pass: z_out [B,H,n_q,d] bf16 = Z, lse_out[row * lse_stride] = log sum exp of the
 // row's scores, mask_out [B,H,T,n_q,d/32] = the layers' decisions |x_t| > theta_t (column c: word c / 32, bit 31 - c % 32)
 // alpha_out (may be null): the iterates alpha^1 .. alpha^T as bf16 into slots 1 .. T of [T+1][B,H,n_q,d]
