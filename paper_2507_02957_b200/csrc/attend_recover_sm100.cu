@@ -1260,7 +1260,7 @@ cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, c
   // with untied layers and T > 0 the per-layer kernel; the set-up has then built its operands for exactly T layers
   if (c->w_S && c->w_untied && c->p.T > 0)
     return c->p.d == 64 ? CSAT_ATTEND(64, true) : CSAT_ATTEND(128, true);
-  if (warp_attend_better(c)) return launch_warp_attend(c, Q, out, s);
+  if (warp_attend_better(c)) return launch_warp_attend(c, Q, out, s, wait_first);
   // Long jobs with the ISTA-derived decoder (one S, B and one positive threshold for all layers) fold B into the
   // values first: one more small launch, which only pays where the attention kernel walks several items per SM
   // (measured: from ~2 tiles of 128 queries per SM at d = 128, where a layer's hand-over chain is long, from ~8 at

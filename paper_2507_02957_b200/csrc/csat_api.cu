@@ -760,7 +760,7 @@ int csat_attend(csat_ctx* c, const void* Q, void* out, void* stream) {
   const bool tc_attend = c->tmap_phi_valid && c->force_simt == 0;
   // whatever is in front in the stream (a projection, another attention, the decoder set-up) may be what writes Q or the decoder
   cudaError_t e = tc_attend ? csat::launch_sm100_attend_recover(c, Q, out, s, &launches, /*wait_first=*/true)
-                            : csat::launch_simt_attend_recover(c, Q, out, s, &launches);
+                            : csat::launch_simt_attend_recover(c, Q, out, s, &launches, /*wait_first=*/true);
   if (e != cudaSuccess) return fail_cuda(c, e, "csat_attend launch");
   c->last_launches = launches;
   return CSAT_OK;

@@ -222,6 +222,7 @@ struct FfmaAttend {                       // layer t of head h: S + t * layer_st
   int64_t layer_stride, nq, m, BH;
   int theta_stride, d, H, T, device, sms;
   float scale;
+  bool wait_first;                        // the kernel before it may write more than kv
 };
 cudaError_t launch_ffma_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
                                  float* partial);
@@ -234,7 +235,8 @@ cudaError_t launch_split_attend(const FfmaAttend& a, const void* Q, const void* 
 // workspace := sum over r < R of partials[r] (float32 [B,H,m,2d] each), added in the order r = 0, 1, ..., rounded
 // once to the context's storage type
 cudaError_t launch_reduce_partials(csat_ctx* c, const float* partials, int R, cudaStream_t s, int* launches);
-cudaError_t launch_simt_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches);
+// (wait_first: as at launch_sm100_attend_recover)
+cudaError_t launch_simt_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first = false);
 
 // compress_sm100.cu : tcgen05 / TMEM / TMA compression (bf16, d in {64, 128})
 cudaError_t make_phi_tmap(csat_ctx* c);
@@ -258,7 +260,7 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
 
 // warp_attend.cu : the same two for d = 64 with 16 queries per warp (one S, B for all layers; no iterates)
 bool warp_attend_better(const csat_ctx* c);      // by the context's shape alone
-cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s);
+cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool wait_first);
 cudaError_t launch_warp_attend_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
                                          __nv_bfloat16* z, uint32_t* masks);
 

@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
   const bool untied = p.layer_stride != 0;
   const int64_t hdd = (int64_t)h * d * d;
 
+  // (the kernel in front is this call's own compression: S was complete before that let this kernel start)
   if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
   ptx::pdl_wait();                                          // K~|V~ come from the kernel before this one
   ptx::pdl_launch_dependents();

@@ -158,6 +158,9 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
   float* Zw = untied ? att_smem + L::kZ + (warp * kRW + ty) * kLdA : Aw;
   const int64_t hdd = (int64_t)h * d * d;
 
+  // S was complete before this call's own compression started (it waits before it lets this kernel start); another kernel in
+  // front may be the decoder set-up that writes it
+  if (p.wait_first) ptx::pdl_wait();
   if (p.T > 1 && !untied) stage_matrix_async(Ss, kLdB, p.S + hdd, d, 0, d);   // lands during the attention
   ptx::pdl_wait();                                          // K~|V~ come from the kernel before this one
   ptx::pdl_launch_dependents();

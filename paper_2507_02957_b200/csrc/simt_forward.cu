@@ -305,7 +305,7 @@ bool use_split(const csat_ctx* c) {
 }
 
 template <typename T>
-cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
+cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool wait_first) {
   const Params& p = c->p;
   const int d = (int)p.d;
   const dim3 grid((unsigned)((p.nq + kAttWarps - 1) / kAttWarps), (unsigned)(p.B * p.H));
@@ -322,6 +322,7 @@ cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
     a.theta_stride = c->thr_stride();
     a.d = d; a.H = (int)p.H; a.T = p.T; a.device = c->device; a.sms = c->sms;
     a.scale = scale;
+    a.wait_first = wait_first;
     if (use_split(c)) return launch_split_attend(a, Q, c->kv, out, s);
     return launch_ffma_attend(a, p.dtype, Q, c->kv, out, s);
   }
@@ -368,9 +369,10 @@ cudaError_t launch_reduce_partials(csat_ctx* c, const float* partials, int R, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_simt_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches) {
+cudaError_t launch_simt_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first) {
   *launches += 1;
-  return c->p.dtype == CSAT_DTYPE_FP32 ? attend_t<float>(c, Q, out, s) : attend_t<__nv_bfloat16>(c, Q, out, s);
+  return c->p.dtype == CSAT_DTYPE_FP32 ? attend_t<float>(c, Q, out, s, wait_first)
+                                       : attend_t<__nv_bfloat16>(c, Q, out, s, wait_first);
 }
 
 cudaError_t launch_split_kv(const csat_ctx* c, void* kt, void* vt, cudaStream_t s) {

@@ -33,6 +33,7 @@ struct Args {
   const __nv_bfloat16 *Q, *kv, *mats;
   const float* theta;
   int theta_stride, nq, m, H, T, has_psi, tiles, bh0;
+  bool wait_first;
   float scale_log2;
   // recording (the backward pass's forward), as in attend_recover_sm100.cu
   float* lse;
@@ -52,7 +53,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
   const int nchunks = (p.m + kMC - 1) / kMC;
   __nv_bfloat16* mats = smem + kOffMats;
 
-  // decoder matrices (not written by the kernel before this one)
+  // decoder matrices: complete before this call's own compression started; another kernel in front may be the decoder set-up
+  // that writes them
+  if (p.wait_first) ptx::pdl_wait();
   if (p.T > 0) {
     const __nv_bfloat16* mh = p.mats + (int64_t)h * 3 * kD * kD;
     for (int i = threadIdx.x; i < (p.has_psi ? 3 : 2) * kD * (kD / 8); i += kWarps * 32)
@@ -326,7 +329,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
 }
 
 template <bool kRec>
-cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride, __nv_bfloat16* z, uint32_t* masks) {
+cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride, __nv_bfloat16* z, uint32_t* masks,
+                   bool wait_first) {
   const Params& p = c->p;
   static DeviceFlags opt_in;
   cudaError_t e = ensure_dynamic_smem(warp_attend_kernel<kRec>, kSmemBytes, c->device, opt_in);
@@ -342,6 +346,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   a.has_psi = c->psi ? 1 : 0;
   a.tiles = (int)((p.nq + kRows - 1) / kRows);
   a.bh0 = (int)c->bh0;
+  a.wait_first = wait_first;
   a.scale_log2 = (float)((p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)kD)) * 1.4426950408889634);
   a.lse = lse; a.lse_stride = lse_stride; a.z = z; a.masks = masks;
   const int64_t grid = (int64_t)a.tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
@@ -372,12 +377,12 @@ bool warp_attend_better(const csat_ctx* c) {
   return p.d == kD && !(c->w_S && c->w_untied && p.T > 0) && (p.nq + kRows - 1) / kRows * p.B * p.H <= c->sms;
 }
 
-cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s) {
-  return launch<false>(c, Q, out, s, nullptr, 0, nullptr, nullptr);
+cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool wait_first) {
+  return launch<false>(c, Q, out, s, nullptr, 0, nullptr, nullptr, wait_first);
 }
 cudaError_t launch_warp_attend_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
                                          __nv_bfloat16* z, uint32_t* masks) {
-  return launch<true>(c, Q, out, s, lse, lse_stride, z, masks);
+  return launch<true>(c, Q, out, s, lse, lse_stride, z, masks, false);
 }
 
 }  // namespace csat

@@ -210,6 +210,8 @@ __global__ void __launch_bounds__(kW * 32) split_attend_kernel(__nv_bfloat16* __
     }
     cp_commit();
   };
+  // B was complete before this call's own compression started; another kernel in front may be the decoder set-up that writes it
+  if (p.wait_first) ptx::pdl_wait();
   if (p.T > 0) build(p.B + hdd, d, 1, false);
   ptx::pdl_wait();                                             // K~|V~ come from the kernel before this one
   ptx::pdl_launch_dependents();

@@ -1,5 +1,5 @@
 """`csat_attend` directly behind a kernel of the library that may still be running: one that writes its queries (the input
-projection, another attention).  Attention kernels may start before the kernel in front has finished; every result has to
+projection, another attention), or one that writes its decoder (the set-up after a changed parameter).  Attention kernels may start before the kernel in front has finished; every result has to
 have the bits of the same call made after a synchronisation.  A buffer that could be read too early holds other finite values
 before the calls."""
 import pytest
@@ -69,3 +69,39 @@ def test_attend_behind_attend_and_forward(d, T, H, n):
     _check([lambda: first.forward(Q, K, V, out=mid), lambda: second.attend(mid, out=out)], [mid, out], others)
     first.close()
     second.close()
+
+
+@pytest.mark.parametrize("weights", [False, True], ids=["derived", "supplied"])
+@pytest.mark.parametrize("dtype, d, H, n", [("bf16", 64, 4, 1024), ("bf16", 64, 6, 1600), ("bf16", 128, 6, 1600), ("bf16", 96, 2, 300),
+                                            ("fp32", 64, 1, 300), ("fp32", 128, 1, 300)])
+def test_attend_behind_the_decoder_set_up(dtype, d, H, n, weights):
+    """A changed step size (S, B and the threshold depend on it), or other supplied weights, and at once an attention."""
+    ctx = _context(d, H, n, 10, dtype=dtype)
+    dt = ctx.torch_dtype
+    Q = _randn(31, 1, H, n, d, dtype=dt)
+    out = torch.empty_like(Q)
+    eye = torch.eye(d, device="cuda")
+    S = [(0.6 * eye + 0.3 * d ** -0.5 * _randn(40 + i, H, d, d, dtype=torch.float32)).to(dt) for i in (0, 1)]
+    Bm = [(_randn(50 + i, H, d, d, dtype=torch.float32) * d ** -0.5).to(dt) for i in (0, 1)]
+    th = [torch.full((1, H), x, device="cuda") for x in (0.01, 0.03)]
+
+    def change(i):
+        if weights:
+            ctx.set_lista_weights(S[i], Bm[i], th[i])
+        else:
+            ctx.set(step=(0.05, 0.1)[i])
+
+    want = []
+    for i in (0, 1):
+        change(i)
+        ctx.get_decoder()
+        torch.cuda.synchronize()
+        want.append(ctx.attend(Q).clone())
+        torch.cuda.synchronize()
+    assert not torch.equal(*want)
+    for k in range(10):
+        change(k % 2)
+        ctx.attend(Q, out=out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[k % 2])
+    ctx.close()
