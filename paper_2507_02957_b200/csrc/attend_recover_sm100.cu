@@ -206,7 +206,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
                             int has_psi, float scale_log2, int items_x, int n_items, int bh0, int* status,
                             float* __restrict__ lse_out, int lse_stride, __nv_bfloat16* __restrict__ z_out,
                             uint32_t* __restrict__ mask_out, __nv_bfloat16* __restrict__ alpha_out,
-                            int64_t alpha_slot, uint32_t* __restrict__ sign_out, int wait_first) {
+                            int64_t alpha_slot, uint32_t* __restrict__ sign_out, int wait_first, int contracting) {
   using C = Cfg<D, kRec == 0>;
   constexpr bool kMasks = kRec >= 1, kKeep = kRec >= 2, kStaged = kRec == 0;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -868,7 +868,20 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
       // in units of 2 theta, which saves one instruction per pair of elements.  Registers c = alpha / (2 theta),
       // accumulator r' = 1/2 + (z B - a^ mu G) / (2 theta) (the threads store 1/2, z is published divided by 2 theta):
       //   s = sat(c + r') (= sat(x / (2 theta) + 1/2), one saturating add);  increment = r' - s;  c += increment.
-      const bool scaled_units = kFold || (!kUntied && !kKeep && T > 0 && theta_stride == 0 && kappa > 0.f);
+      bool scaled_units = kFold || (!kUntied && !kKeep && T > 0 && theta_stride == 0 && kappa > 0.f);
+      if (kMasks && scaled_units) {
+        // The saturating add turns NaN into 0, which would be recorded as a decision like any other.  So a warp records in these
+        // units only where no iterate can leave the finite numbers: finite rows far from overflow, in a recurrence that does
+        // not grow.  The others keep the data's units below, where |NaN| > theta is false.  (64 packed multiply-adds per row
+        // against ~900 per layer.)
+        F2 q2 = pack2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < D / 2; ++i) q2 = fma2(v2[i], v2[i], q2);
+        float q0, q1;
+        unpack2(q2, q0, q1);
+        const float i2 = 0.5f / kappa;
+        scaled_units = __all_sync(0xffffffffu, contracting && (q0 + q1) * i2 * i2 < 1e30f);
+      }
       if (scaled_units) {
         const uint32_t op_addr = tbase + C::kColS;
         if (kFold) {
@@ -1217,7 +1230,9 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int T,
                             kUntied ? c->tmap_lmats : c->tmap_mats, to, c->tmap_vb, (__nv_bfloat16*)out, c->thr(), c->thr_stride(),
                             (int)p.nq, (int)p.m, (int)p.H, T, c->psi ? 1 : 0, scale_log2, (int)items_x, (int)n_items,
                             (int)c->bh0, c->status, lse_out, lse_stride, z_out, mask_out, alpha_out,
-                            (int64_t)(p.B * p.H * p.nq * p.d), alpha_out != nullptr ? c->bw_signbits : nullptr, wait_first ? 1 : 0);
+                            (int64_t)(p.B * p.H * p.nq * p.d), alpha_out != nullptr ? c->bw_signbits : nullptr, wait_first ? 1 : 0,
+                            // S = I - mu G with mu at most 1 over G's largest eigenvalue
+                            !c->w_S && p.step == 0.0 ? 1 : 0);
 }
 
 }  // namespace
