@@ -127,24 +127,26 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
       {
         RegMatrix<kDR> S;
         if (p.T > 1) S.load(Ss, kLdB, d, tx, ty);
-        for (int it = 1; it < p.T; ++it) {
-          th = p.theta[(int64_t)it * p.theta_stride + h];
-          __syncwarp();
+        run_whole<kDR>(d, [&](auto whole) {
+          for (int it = 1; it < p.T; ++it) {
+            th = p.theta[(int64_t)it * p.theta_stride + h];
+            __syncwarp();
 #pragma unroll 1
-          for (int r = 0; r < kRW; r += kN) {
-            float y[kN][kNC];
-            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+            for (int r = 0; r < kRW; r += kN) {
+              float y[kN][kNC];
+              S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-            for (int u = 0; u < kN; ++u)
+              for (int u = 0; u < kN; ++u)
 #pragma unroll
-              for (int j = 0; j < kNC; ++j) {
-                const int at = (r + u) * kLdA + col + 8 * j;
-                const float x = y[u][j] + Drows[at];
-                if (fabsf(x) > th) Mrows[at] |= 1u << it;
-                Arows[at] = shrink(x, th);
-              }
+                for (int j = 0; j < kNC; ++j) {
+                  const int at = (r + u) * kLdA + col + 8 * j;
+                  const float x = whole.value || col + 8 * j < d ? y[u][j] + Drows[at] : 0.f;
+                  if (fabsf(x) > th) Mrows[at] |= 1u << it;
+                  Arows[at] = shrink(x, th);
+                }
+            }
           }
-        }
+        });
       }
       start_backward();
       for (int r = 0; r < kRW; ++r)
@@ -161,23 +163,25 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
       {
         RegMatrix<kDR> S;
         if (p.T > 1) S.load_transposed(Ss, kLdB, d, tx, ty);
-        for (int it = p.T - 2; it >= 0; --it) {
-          __syncwarp();
+        run_whole<kDR>(d, [&](auto whole) {
+          for (int it = p.T - 2; it >= 0; --it) {
+            __syncwarp();
 #pragma unroll 1
-          for (int r = 0; r < kRW; r += kN) {
-            float y[kN][kNC];
-            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+            for (int r = 0; r < kRW; r += kN) {
+              float y[kN][kNC];
+              S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-            for (int u = 0; u < kN; ++u)
+              for (int u = 0; u < kN; ++u)
 #pragma unroll
-              for (int j = 0; j < kNC; ++j) {
-                const int at = (r + u) * kLdA + col + 8 * j;
-                const float dx = (Mrows[at] >> it) & 1u ? y[u][j] : 0.f;
-                Drows[at] += dx;
-                Arows[at] = dx;
-              }
+                for (int j = 0; j < kNC; ++j) {
+                  const int at = (r + u) * kLdA + col + 8 * j;
+                  const float dx = ((Mrows[at] >> it) & 1u) && (whole.value || col + 8 * j < d) ? y[u][j] : 0.f;
+                  Drows[at] += dx;
+                  Arows[at] = dx;
+                }
+            }
           }
-        }
+        });
       }
       __syncwarp();
       times_transposed<TR>(Aw, Dw, kLdA, p.B + hdd, d, Ks, kLdB, tx, false);       // dZ = (sum_t dx_t) B^T

@@ -205,20 +205,24 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
       store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
       const int col = RegMatrix<kDR>::col(tx, ty);
       constexpr int kN = 4;
-      for (int it = 1; it < p.T; ++it) {
-        th = p.theta[(int64_t)it * p.theta_stride + h];
-        __syncwarp();
+      run_whole<kDR>(d, [&](auto whole) {
+        for (int it = 1; it < p.T; ++it) {
+          th = p.theta[(int64_t)it * p.theta_stride + h];
+          __syncwarp();
 #pragma unroll 1
-        for (int r = 0; r < kRW; r += kN) {
-          float y[kN][kNC];
-          S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+          for (int r = 0; r < kRW; r += kN) {
+            float y[kN][kNC];
+            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-          for (int u = 0; u < kN; ++u)
+            for (int u = 0; u < kN; ++u)
 #pragma unroll
-            for (int j = 0; j < kNC; ++j)
-              Arows[(r + u) * kLdA + col + 8 * j] = shrink(y[u][j] + Crows[(r + u) * kLdA + col + 8 * j], th);
+              for (int j = 0; j < kNC; ++j) {
+                const float a1 = shrink(y[u][j] + Crows[(r + u) * kLdA + col + 8 * j], th);
+                Arows[(r + u) * kLdA + col + 8 * j] = whole.value || col + 8 * j < d ? a1 : 0.f;
+              }
+          }
         }
-      }
+      });
       __syncwarp();
       load_rows<TR, kTCQ>(a, Aw, kLdA, tx);
     } else

@@ -31,3 +31,41 @@ def test_decisions_of_rows_that_are_not_finite(d, H, n_q):
     for a, b in zip(dirty, clean):
         assert torch.equal(a[:, 1:], b[:, 1:])
     ctx.close()
+
+
+def _infinite_head(d, H, n_q, m, T, dtype, sign):
+    """Positive measurements and decoder matrices, and one infinity in the values of head 0: every sum of that head that meets
+    it is an infinity of its sign, no two of different signs meet."""
+    ctx = binding.Csat(200, m, d, H, 3, n_q=n_q, dtype=dtype, T=T, lam=1e-3)
+    dt = ctx.torch_dtype
+    ctx.set_phi((0.1 + _randn(1, H, m, 200, dtype=torch.float32).abs()).to(dt))
+    if T > 0:
+        S, Bm = ((0.01 + _randn(i, H, d, d, dtype=torch.float32).abs() / d).to(dt) for i in (2, 3))
+        ctx.set_lista_weights(S, Bm, torch.full((1, H), 0.01, device="cuda"))
+    Q, K, V = (0.05 * _randn(10 + i, 1, H, n, d, dtype=torch.float32) for i, n in enumerate((n_q, 200, 200)))
+    Q, K, V = Q.to(dt), K.to(dt), V.to(dt)
+    V2 = V.clone()
+    V2[0, 0, 17, 5] = sign * float("inf")
+    return ctx, Q, K, V, V2
+
+
+@pytest.mark.parametrize("sign", [1, -1])
+@pytest.mark.parametrize("T", [0, 1, 4])
+@pytest.mark.parametrize("d", [8, 24, 40, 64, 72, 96, 120, 128])
+def test_infinities_in_float32(d, T, sign):
+    """An infinity stays one through the float32 kernels, padded head sizes included, and is a decision in every layer."""
+    H, n_q = 2, 70
+    ctx, Q, K, V, V2 = _infinite_head(d, H, n_q, 50, T, "fp32", sign)
+    want = ctx.forward(Q, K, V).clone()
+    got = ctx.forward(Q, K, V2)
+    assert torch.isfinite(want).all() and torch.equal(got[:, 1:], want[:, 1:])
+    if T == 0:
+        assert (got[0, 0, :, 5] == sign * float("inf")).all()
+        got[0, 0, :, 5], want[0, 0, :, 5] = 0, 0
+        assert torch.equal(got, want)
+    else:
+        assert (got[0, 0] == sign * float("inf")).all()
+        binding.csat_set_i64(ctx.h, binding.CSAT_KEEP_MASKS, 1)
+        ctx.backward(Q, K, V2, _randn(4, 1, H, n_q, d, dtype=torch.float32))
+        assert (ctx.backward_masks()[0, 0] == (1 << T) - 1).all()
+    ctx.close()
