@@ -142,9 +142,66 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   lo = pack(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
 }
 
+// One row by one warp in float32 multiply-adds throughout, for rows whose output is not finite: the second part of an infinity
+// is NaN (and of a finite value that rounds to infinity in bf16, -inf), and so is an infinity times a part that is zero, where
+// the value itself has an infinite or even finite product.  A lane holds columns lane + 32 j.
+__device__ __noinline__ void plain_row(__nv_bfloat16* out, const __nv_bfloat16* q, const __nv_bfloat16* kvb, const FfmaAttend& p, int64_t hdd) {
+  constexpr int DC = kFfmaMaxD / 32;
+  const int lane = threadIdx.x & 31, d = p.d, m = (int)p.m;
+  // y (+)= x W, or x W^T
+  auto times = [&](float (&y)[DC], const float (&x)[DC], const float* W, int rs, int cs) {
+    for (int j = 0; j < DC; ++j) y[j] = 0.f;
+    for (int k = 0; k < d; ++k) {
+      const float xk = __shfl_sync(0xffffffffu, k < 32 ? x[0] : k < 64 ? x[1] : k < 96 ? x[2] : x[3], k & 31);
+      for (int j = 0; j < DC; ++j)
+        if (lane + 32 * j < d) y[j] = fmaf(xk, W[(int64_t)k * rs + (int64_t)(lane + 32 * j) * cs], y[j]);
+    }
+  };
+  float z[DC] = {}, run_max = -INFINITY, run_sum = 0.f;
+  for (int r0 = 0; r0 < m; r0 += 32) {
+    float s = -INFINITY;
+    if (r0 + lane < m) {
+      s = 0.f;
+      for (int c = 0; c < d; ++c) s = fmaf(__bfloat162float(q[c]), __bfloat162float(kvb[(int64_t)(r0 + lane) * 2 * d + c]), s);
+      s *= p.scale;
+    }
+    float mx = s, ps;
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float new_max = fmaxf(run_max, mx), corr = expf(run_max - new_max), pr = expf(s - new_max);
+    ps = pr;
+    for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+    run_sum = run_sum * corr + ps;
+    run_max = new_max;
+    for (int j = 0; j < DC; ++j) z[j] *= corr;
+    for (int r = 0; r < 32 && r0 + r < m; ++r) {
+      const float a = __shfl_sync(0xffffffffu, pr, r);
+      for (int j = 0; j < DC; ++j)
+        if (lane + 32 * j < d) z[j] = fmaf(a, __bfloat162float(kvb[(int64_t)(r0 + r) * 2 * d + d + lane + 32 * j]), z[j]);
+    }
+  }
+  for (int j = 0; j < DC; ++j) z[j] *= 1.f / run_sum;
+  if (p.T > 0) {
+    float c[DC], a[DC], y[DC] = {};
+    for (int it = 0; it < p.T; ++it) {
+      const float th = p.theta[(int64_t)it * p.theta_stride + hdd / ((int64_t)d * d)];
+      if (it == 0 || p.layer_stride != 0) times(c, z, p.B + it * p.layer_stride + hdd, d, 1);
+      if (it > 0) times(y, a, p.S + it * p.layer_stride + hdd, d, 1);
+      for (int j = 0; j < DC; ++j) {
+        const float x = y[j] + c[j];
+        a[j] = x - fminf(fmaxf(x, -th), th);
+      }
+    }
+    if (p.psi) times(z, a, p.psi + hdd, 1, d);
+    else
+      for (int j = 0; j < DC; ++j) z[j] = a[j];
+  }
+  for (int j = 0; j < DC; ++j)
+    if (lane + 32 * j < d) out[lane + 32 * j] = __float2bfloat16_rn(z[j]);
+}
+
 template <int DP, bool kUntied>                             // kUntied: one S_t, B_t per layer
 __global__ void __launch_bounds__(kW * 32) split_attend_kernel(__nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ Q,
-                                                               const __nv_bfloat16* __restrict__ kv, const FfmaAttend p, int tiles) {
+                                                               const __nv_bfloat16* __restrict__ kv, const __grid_constant__ FfmaAttend p, int tiles) {
   using L = AttSmem<DP>;
   constexpr int NT = DP / 8, KS = DP / 16, kLd = L::kLd;
   extern __shared__ __align__(16) __nv_bfloat16 smem[];
@@ -369,11 +426,20 @@ __global__ void __launch_bounds__(kW * 32) split_attend_kernel(__nv_bfloat16* __
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int row = row0 + g + 8 * u;
-    if (row >= nq) continue;
     __nv_bfloat16* o = out + ((int64_t)bh * nq + row) * d + 2 * t;
+    bool finite = true;
 #pragma unroll
     for (int j = 0; j < NT; ++j)
-      if (8 * j < d) *reinterpret_cast<uint32_t*>(o + 8 * j) = pack(a[j][2 * u], a[j][2 * u + 1]);
+      if (8 * j < d) {
+        finite = finite && fabsf(a[j][2 * u]) < INFINITY && fabsf(a[j][2 * u + 1]) < INFINITY;
+        if (row < nq) *reinterpret_cast<uint32_t*>(o + 8 * j) = pack(a[j][2 * u], a[j][2 * u + 1]);
+      }
+    uint32_t odd = __ballot_sync(0xffffffffu, !finite && row < nq);            // four lanes per row
+    for (odd = (odd | odd >> 1 | odd >> 2 | odd >> 3) & 0x11111111u; odd != 0; odd &= odd - 1) {
+      const int64_t at = ((int64_t)bh * nq + row0 + 8 * u + ((__ffs(odd) - 1) >> 2)) * d;
+      __syncwarp();                                            // after the stores above
+      plain_row(out + at, Q + at, kvb, p, hdd);
+    }
   }
 }
 

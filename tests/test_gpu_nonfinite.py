@@ -69,3 +69,44 @@ def test_infinities_in_float32(d, T, sign):
         ctx.backward(Q, K, V2, _randn(4, 1, H, n_q, d, dtype=torch.float32))
         assert (ctx.backward_masks()[0, 0] == (1 << T) - 1).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("sign", [1, -1])
+@pytest.mark.parametrize("T", [0, 1, 4])
+@pytest.mark.parametrize("d", [8, 24, 40, 72, 96, 120])
+def test_infinities_in_two_bf16_parts(d, T, sign):
+    """The same for bf16 storage at head sizes whose float32 values go through the matrix instructions in two parts (the second
+    part of an infinity is NaN)."""
+    H, n_q = 2, 70
+    ctx, Q, K, V, V2 = _infinite_head(d, H, n_q, 50, T, "bf16", sign)
+    want = ctx.forward(Q, K, V).clone()
+    got = ctx.forward(Q, K, V2)
+    assert torch.isfinite(want).all() and torch.equal(got[:, 1:], want[:, 1:])
+    if T == 0:
+        assert (got[0, 0, :, 5] == sign * float("inf")).all()
+        got[0, 0, :, 5], want[0, 0, :, 5] = 0, 0
+        # float32 throughout against two parts, rounded to bf16: at most one step (2^-7 of the value) apart
+        assert ((got - want).abs() <= 2 ** -7 * want.abs()).all()
+    else:
+        assert (got[0, 0] == sign * float("inf")).all()
+    ctx.close()
+
+
+@pytest.mark.parametrize("d", [8, 40, 96, 120])
+def test_where_two_bf16_parts_give_nan_and_infinity(d):
+    """NaN and infinities of either sign in queries, keys and values: each output is finite, NaN or an infinity where the float32
+    kernels' is (a few rows only: the rest of a head keeps what it had)."""
+    H, n_q, n, m, T = 4, 70, 200, 130, 3
+    ctx = binding.Csat(n, m, d, H, 3, n_q=n_q, dtype="bf16", T=T, lam=1e-3)
+    Q, K, V = _randn(1, 1, H, n_q, d), _randn(2, 1, H, n, d), _randn(3, 1, H, n, d)
+    Q[0, 0, 33, 1], Q[0, 0, 17, 2], Q[0, 0, 69, 0] = float("nan"), float("inf"), float("-inf")
+    V[0, 1, 5, 3], K[0, 2, 199, d - 1] = float("-inf"), float("inf")
+    for T in (0, 1, 3):
+        ctx.set(T=T, force_simt=0)
+        a = ctx.forward(Q, K, V).clone()
+        ctx.set(force_simt=1)
+        b = ctx.forward(Q, K, V)
+        assert torch.equal(torch.isnan(a), torch.isnan(b)) and torch.equal(torch.isposinf(a), torch.isposinf(b))
+        assert torch.equal(torch.isneginf(a), torch.isneginf(b))
+        assert torch.isnan(a[0, 0, 33]).all() and torch.isfinite(a[0, 0, :17]).all() and torch.isfinite(a[0, 3]).all()
+    ctx.close()
