@@ -771,7 +771,7 @@ static int ensure_backward_scratch(csat_ctx* c) {
   const csat::Params& p = c->p;
   const size_t bz = (size_t)(p.B * p.H * p.nq * p.d) * 4, bl = (size_t)(p.B * p.H * p.nq * 2) * 4 + 1024 /* read past the end by whole-tile copies */,
                bk = (size_t)(p.B * p.H * p.m * 2 * p.d) * 4,
-               bw = (size_t)(2 * (c->w_untied ? c->w_layers : 1) * p.H * p.d * p.d) * 4,
+               bw = p.d > csat::kFfmaMaxD ? (size_t)(2 * (c->w_untied ? c->w_layers : 1) * p.H * p.d * p.d) * 4 : 0,   // transposes
                b16 = c->tmap_phi_valid ? bk / 2 : 0, z16 = c->tmap_phi_valid ? bz / 2 : 0,
                bm = c->keep_masks && p.T > 0 ? bz : 0,
                bmb = c->tmap_phi_valid ? (size_t)(p.B * p.H * p.T * p.nq * (p.d / 32)) * 4 : 0,

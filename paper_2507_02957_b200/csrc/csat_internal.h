@@ -35,10 +35,13 @@ cudaError_t ensure_dynamic_smem(Kernel* kernel, int bytes, int device, DeviceFla
   return e;
 }
 
-// Programmatic dependent launch: the kernel may be scheduled while the one before it in the stream still runs.  Every kernel
-// launched this way (and every kernel before one) keeps to one order: set-up that touches nothing another kernel writes,
-// griddepcontrol.wait by every thread, then griddepcontrol.launch_dependents.  So whatever precedes the previous kernel is
-// complete when a kernel starts, and the previous one itself is after the wait.
+// Programmatic dependent launch: the kernel may be scheduled while the one before it in the stream still runs.  A kernel
+// that lets its successor start (griddepcontrol.launch_dependents) has by then waited for its own predecessor, or was launched
+// plainly and so started after it (the tcgen05 compression).  So whatever precedes the previous kernel is complete when a kernel
+// starts, and the previous one itself is after griddepcontrol.wait: before that a kernel touches only what the previous kernel
+// does not write, and stores nothing.  The backward kernels and the projection read nothing at all before their wait.  The
+// attention kernels do: their first queries (attend_recover_sm100), thresholds and decoder matrices are in place before this
+// call's own compression or fold starts.  Behind any other kernel they are launched with wait_first.
 template <typename... KP, typename... Args>
 cudaError_t launch_maybe_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -132,9 +135,11 @@ struct csat_ctx {
   // float32 scratch of csat_backward, allocated by its first call: dZ [B,H,n_q,d], (L, D) [B,H,n_q,2],
   // dK~|dV~ [B,H,m,2d]
   // and the float32 transposes of the decoder matrices [2][layers or 1][H][d][d]
+  // bw_dZ, bw_dKV (float32 dZ and dK~|dV~) belong to the float32 kernels; contexts with tensor-core stages hold them as well,
+  // because CSAT_FORCE_SIMT may change between two calls without a new allocation.  bw_WT: d > kFfmaMaxD only
   float* bw_dZ = nullptr; float* bw_LD = nullptr; float* bw_dKV = nullptr; float* bw_WT = nullptr;
-  __nv_bfloat16* bw_dKV16 = nullptr;     // bf16 copy of dK~|dV~ (operand of the tensor-core Phi^T product)
-  __nv_bfloat16* bw_dZ16 = nullptr;      // bf16 copy of dZ (operand of the tensor-core dK~|dV~ stage)
+  __nv_bfloat16* bw_dKV16 = nullptr;     // dK~|dV~ in bf16 (operand of the tensor-core Phi^T product)
+  __nv_bfloat16* bw_dZ16 = nullptr;      // dZ in bf16 (operand of the tensor-core dQ and dK~|dV~ stages)
   __nv_bfloat16* bw_Z16 = nullptr;       // Z = A~ V~ as the forward rounds it (tensor-core per-query stages)
   uint32_t* bw_maskbits = nullptr;       // the forward's decisions, one bit per (b, h, layer, query, column)
   size_t bw_bytes_Z16 = 0, bw_bytes_maskbits = 0;
@@ -291,7 +296,7 @@ cudaError_t launch_ffma_backward(csat_ctx* c, const void* Q, const void* G, void
                                  int* launches);
 
 // bwd_cols_sm100.cu : dK~ = scale dS^T Q, dV~ = P^T dZ on the tensor cores (bf16, d in {64, 128}); reads bw_dZ16,
-// bw_LD and the K~|V~ workspace, writes bw_dKV and bw_dKV16
+// bw_LD and the K~|V~ workspace, writes bw_dKV16
 cudaError_t launch_sm100_bwd_cols(csat_ctx* c, const void* Q, cudaStream_t s, int* launches);
 
 // phiT_sm100.cu : dK = Phi_K^T dK~, dV = Phi_V^T dV~ on the tensor cores (bf16, d in {64, 128}); g16 = dK~|dV~ as bf16
