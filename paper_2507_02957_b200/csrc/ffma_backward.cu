@@ -40,7 +40,7 @@ template <int DP, int TR> struct RowsSmem {                 // in floats
   static constexpr int kFloats = kM + (DP <= 64 ? kBuf : 0);
 };
 
-template <typename T, int DP, int TR>
+template <typename T, int DP, int TR, bool kPadded>         // kPadded: DP <= 64 and d < DP
 __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__ dQ, const T* __restrict__ Q, const T* __restrict__ G,
                                                                  const T* __restrict__ kv, const RowsArgs p) {
   using L = RowsSmem<DP, TR>;
@@ -127,26 +127,24 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
       {
         RegMatrix<kDR> S;
         if (p.T > 1) S.load(Ss, kLdB, d, tx, ty);
-        run_whole<kDR>(d, [&](auto whole) {
-          for (int it = 1; it < p.T; ++it) {
-            th = p.theta[(int64_t)it * p.theta_stride + h];
-            __syncwarp();
+        for (int it = 1; it < p.T; ++it) {
+          th = p.theta[(int64_t)it * p.theta_stride + h];
+          __syncwarp();
 #pragma unroll 1
-            for (int r = 0; r < kRW; r += kN) {
-              float y[kN][kNC];
-              S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+          for (int r = 0; r < kRW; r += kN) {
+            float y[kN][kNC];
+            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-              for (int u = 0; u < kN; ++u)
+            for (int u = 0; u < kN; ++u)
 #pragma unroll
-                for (int j = 0; j < kNC; ++j) {
-                  const int at = (r + u) * kLdA + col + 8 * j;
-                  const float x = whole.value || col + 8 * j < d ? y[u][j] + Drows[at] : 0.f;
-                  if (fabsf(x) > th) Mrows[at] |= 1u << it;
-                  Arows[at] = shrink(x, th);
-                }
-            }
+              for (int j = 0; j < kNC; ++j) {
+                const int at = (r + u) * kLdA + col + 8 * j;
+                const float x = kPadded && col + 8 * j >= d ? 0.f : y[u][j] + Drows[at];
+                if (fabsf(x) > th) Mrows[at] |= 1u << it;
+                Arows[at] = shrink(x, th);
+              }
           }
-        });
+        }
       }
       start_backward();
       for (int r = 0; r < kRW; ++r)
@@ -163,25 +161,23 @@ __global__ void __launch_bounds__(kThreads) ffma_bwd_rows_kernel(T* __restrict__
       {
         RegMatrix<kDR> S;
         if (p.T > 1) S.load_transposed(Ss, kLdB, d, tx, ty);
-        run_whole<kDR>(d, [&](auto whole) {
-          for (int it = p.T - 2; it >= 0; --it) {
-            __syncwarp();
+        for (int it = p.T - 2; it >= 0; --it) {
+          __syncwarp();
 #pragma unroll 1
-            for (int r = 0; r < kRW; r += kN) {
-              float y[kN][kNC];
-              S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+          for (int r = 0; r < kRW; r += kN) {
+            float y[kN][kNC];
+            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-              for (int u = 0; u < kN; ++u)
+            for (int u = 0; u < kN; ++u)
 #pragma unroll
-                for (int j = 0; j < kNC; ++j) {
-                  const int at = (r + u) * kLdA + col + 8 * j;
-                  const float dx = ((Mrows[at] >> it) & 1u) && (whole.value || col + 8 * j < d) ? y[u][j] : 0.f;
-                  Drows[at] += dx;
-                  Arows[at] = dx;
-                }
-            }
+              for (int j = 0; j < kNC; ++j) {
+                const int at = (r + u) * kLdA + col + 8 * j;
+                const float dx = ((Mrows[at] >> it) & 1u) && !(kPadded && col + 8 * j >= d) ? y[u][j] : 0.f;
+                Drows[at] += dx;
+                Arows[at] = dx;
+              }
           }
-        });
+        }
       }
       __syncwarp();
       times_transposed<TR>(Aw, Dw, kLdA, p.B + hdd, d, Ks, kLdB, tx, false);       // dZ = (sum_t dx_t) B^T
@@ -529,15 +525,15 @@ __global__ void __launch_bounds__(kThreads) ffma_phiT_kernel(T* __restrict__ dK,
   }
 }
 
-template <typename T, int DP, int TR>
+template <typename T, int DP, int TR, bool kPadded>
 cudaError_t launch_rows(csat_ctx* c, const void* Q, const void* G, void* dQ, cudaStream_t s, const RowsArgs& a) {
   using L = RowsSmem<DP, TR>;
   static_assert(L::kFloats * 4 <= 227 * 1024, "shared memory budget");
   static DeviceFlags opt_in;
-  cudaError_t e = ensure_dynamic_smem(ffma_bwd_rows_kernel<T, DP, TR>, L::kFloats * 4, c->device, opt_in);
+  cudaError_t e = ensure_dynamic_smem(ffma_bwd_rows_kernel<T, DP, TR, kPadded>, L::kFloats * 4, c->device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)(c->p.B * c->p.H));
-  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_bwd_rows_kernel<T, DP, TR>, grid, kThreads, L::kFloats * 4, s, (T*)dQ, (const T*)Q, (const T*)G,
+  return launch_maybe_pdl(small_grid(grid, c->sms), ffma_bwd_rows_kernel<T, DP, TR, kPadded>, grid, kThreads, L::kFloats * 4, s, (T*)dQ, (const T*)Q, (const T*)G,
                     (const T*)c->kv, a);
 }
 
@@ -571,8 +567,10 @@ cudaError_t run_d(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK,
   cudaError_t e;
   // rows per CTA: 16 where that fills no more than one wave, else 32 (d = 64, T = 10, us: 1024 rows 33 / 50, 4096 rows 52 / 51,
   // 8192 rows 98 / 73, 32768 rows 330 / 249; with 64 rows 78 / 78 / 79 / 311: two CTAs no longer fit an SM)
-  if ((p.nq + 15) / 16 * bh <= sms) e = launch_rows<T, DP, 1>(c, Q, G, dQ, s, a);
-  else e = launch_rows<T, DP, 2>(c, Q, G, dQ, s, a);
+  constexpr bool kMayPad = DP <= 64;
+  const bool padded = kMayPad && p.d < DP;
+  if ((p.nq + 15) / 16 * bh <= sms) e = padded ? launch_rows<T, DP, 1, kMayPad>(c, Q, G, dQ, s, a) : launch_rows<T, DP, 1, false>(c, Q, G, dQ, s, a);
+  else e = padded ? launch_rows<T, DP, 2, kMayPad>(c, Q, G, dQ, s, a) : launch_rows<T, DP, 2, false>(c, Q, G, dQ, s, a);
   if (e != cudaSuccess) return e;
   // measurements per CTA: the fewest of 4, 8 that fill no more than one wave, else 16 (d = 64, 512 queries, us with 4 / 8 /
   // 16: 192 measurements in all 25 / 26 / 32, 768 49 / 27 / 33, 1536 73 / 51 / 33, 3072 142 / 76 / 64)

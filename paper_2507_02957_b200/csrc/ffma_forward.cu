@@ -139,7 +139,7 @@ template <int DP, int TR> struct AttendSmem {               // in floats
   static constexpr int kFloats = kZ, kFloatsUntied = kZ + kRows * Ld<DP>::kA;
 };
 
-template <typename T, int DP, int TR>
+template <typename T, int DP, int TR, bool kPadded>         // kPadded: DP <= 64 and d < DP
 __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ out, const T* __restrict__ Q, const T* __restrict__ kv,
                                                                const FfmaAttend p) {
   using L = AttendSmem<DP, TR>;
@@ -205,24 +205,21 @@ __global__ void __launch_bounds__(kThreads) ffma_attend_kernel(T* __restrict__ o
       store_rows<TR, kTCQ>(Aw, kLdA, tx, a);
       const int col = RegMatrix<kDR>::col(tx, ty);
       constexpr int kN = 4;
-      run_whole<kDR>(d, [&](auto whole) {
-        for (int it = 1; it < p.T; ++it) {
-          th = p.theta[(int64_t)it * p.theta_stride + h];
-          __syncwarp();
+      for (int it = 1; it < p.T; ++it) {
+        th = p.theta[(int64_t)it * p.theta_stride + h];
+        __syncwarp();
 #pragma unroll 1
-          for (int r = 0; r < kRW; r += kN) {
-            float y[kN][kNC];
-            S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
+        for (int r = 0; r < kRW; r += kN) {
+          float y[kN][kNC];
+          S.template times<kN>(y, Arows + r * kLdA + 2 * ty, kLdA, ty);
 #pragma unroll
-            for (int u = 0; u < kN; ++u)
+          for (int u = 0; u < kN; ++u)
 #pragma unroll
-              for (int j = 0; j < kNC; ++j) {
-                const float a1 = shrink(y[u][j] + Crows[(r + u) * kLdA + col + 8 * j], th);
-                Arows[(r + u) * kLdA + col + 8 * j] = whole.value || col + 8 * j < d ? a1 : 0.f;
-              }
-          }
+            for (int j = 0; j < kNC; ++j)
+              Arows[(r + u) * kLdA + col + 8 * j] =
+                  kPadded && col + 8 * j >= d ? 0.f : shrink(y[u][j] + Crows[(r + u) * kLdA + col + 8 * j], th);
         }
-      });
+      }
       __syncwarp();
       load_rows<TR, kTCQ>(a, Aw, kLdA, tx);
     } else
@@ -316,32 +313,34 @@ cudaError_t compress_t(csat_ctx* c, TO* dst, const void* K, const void* V, cudaS
   return launch_compress<T, TO, 4, 1>(c, dst, K, V, s, phi_j0, n_len);
 }
 
-template <typename T, int DP, int TR>
+template <typename T, int DP, int TR, bool kPadded>
 cudaError_t launch_attend(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
   using L = AttendSmem<DP, TR>;
   static DeviceFlags opt_in;
-  cudaError_t e = ensure_dynamic_smem(ffma_attend_kernel<T, DP, TR>, L::kFloatsUntied * 4, a.device, opt_in);
+  cudaError_t e = ensure_dynamic_smem(ffma_attend_kernel<T, DP, TR, kPadded>, L::kFloatsUntied * 4, a.device, opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((a.nq + L::kRows - 1) / L::kRows), (unsigned)a.BH);
-  return launch_maybe_pdl(small_grid(grid, a.sms), ffma_attend_kernel<T, DP, TR>, grid, kThreads, (a.layer_stride ? L::kFloatsUntied : L::kFloats) * 4, s, (T*)out,
+  return launch_maybe_pdl(small_grid(grid, a.sms), ffma_attend_kernel<T, DP, TR, kPadded>, grid, kThreads, (a.layer_stride ? L::kFloatsUntied : L::kFloats) * 4, s, (T*)out,
                     (const T*)Q, (const T*)kv, a);
 }
 
-template <typename T, int DP>
+template <typename T, int DP, bool kPadded>
 cudaError_t attend_rows(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
   // the smallest tile that still gives every SM a CTA of its own: measured (d = 64, m = 96, T = 10; 16 / 32 / 64 rows per
   // CTA) at 1024 rows 15.9 / 21.2 / 31.9 us, at 4096 rows 25.2 / 22.3 / 32.9 us, at 16384 rows 80.9 / 65.9 / 55.0 us
-  if ((a.nq + 15) / 16 * a.BH <= a.sms) return launch_attend<T, DP, 1>(a, Q, kv, out, s);
-  if ((a.nq + 31) / 32 * a.BH <= a.sms) return launch_attend<T, DP, 2>(a, Q, kv, out, s);
-  return launch_attend<T, DP, 4>(a, Q, kv, out, s);
+  if ((a.nq + 15) / 16 * a.BH <= a.sms) return launch_attend<T, DP, 1, kPadded>(a, Q, kv, out, s);
+  if ((a.nq + 31) / 32 * a.BH <= a.sms) return launch_attend<T, DP, 2, kPadded>(a, Q, kv, out, s);
+  return launch_attend<T, DP, 4, kPadded>(a, Q, kv, out, s);
 }
 
 template <typename T>
 cudaError_t attend_t(const FfmaAttend& a, const void* Q, const void* kv, void* out, cudaStream_t s) {
-  if (a.d <= 32) return attend_rows<T, 32>(a, Q, kv, out, s);
-  if (a.d <= 64) return attend_rows<T, 64>(a, Q, kv, out, s);
-  if (a.d <= 96) return attend_rows<T, 96>(a, Q, kv, out, s);
-  return attend_rows<T, 128>(a, Q, kv, out, s);
+  if (a.d < 32) return attend_rows<T, 32, true>(a, Q, kv, out, s);
+  if (a.d == 32) return attend_rows<T, 32, false>(a, Q, kv, out, s);
+  if (a.d < 64) return attend_rows<T, 64, true>(a, Q, kv, out, s);
+  if (a.d == 64) return attend_rows<T, 64, false>(a, Q, kv, out, s);
+  if (a.d <= 96) return attend_rows<T, 96, false>(a, Q, kv, out, s);
+  return attend_rows<T, 128, false>(a, Q, kv, out, s);
 }
 
 }  // namespace
