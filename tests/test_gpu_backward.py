@@ -557,3 +557,23 @@ def test_saving_forward_without_recovery_layers():
     for a, b in zip(plain, saved):
         assert torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("d, nq", [(64, 1571), (64, 200), (128, 1571), (128, 65)])
+def test_queries_shared_out_between_the_ctas_of_a_cluster(d, nq):
+    """dK~ | dV~ with the queries of a block of measurements shared out: 8 blocks and 25, 4 or 2 tiles of 64 queries, the last one
+    partly filled and (25 tiles over four CTAs) the last CTA's share shorter; four CTAs at d = 64, two at d = 128.  lambda = 0:
+    every decision is |x| > 0 on both sides."""
+    w = wl.Workload("cluster", 1, 4, 300, nq, d, 200, "bf16", 2, 0.0, "iid", 800 + nq)
+    inp = wl.make_inputs(w)
+    Q, K, V, _ = device_inputs(w, inp)
+    ctx = make_ctx(w)
+    phi = to_np(ctx.get_phi())
+    G = wl.round_to_storage(np.random.default_rng(G_SEED).standard_normal(inp["Q"].shape).astype(np.float32), "bf16")
+    got = ctx.backward(Q, K, V, to_dev(G, "bf16"))
+    ref = orc.csat_backward(inp["Q"], inp["K"], inp["V"], phi, G, T=w.T, lam=0.0)
+    for nm, g, rf in zip(("dQ", "dK", "dV"), got, ref):
+        assert rel_err(to_np(g), rf) <= BWD_TOL["bf16"], (d, nq, nm, rel_err(to_np(g), rf))
+    again = ctx.backward(Q, K, V, to_dev(G, "bf16"))
+    assert all(torch.equal(a, b) for a, b in zip(got, again))
+    ctx.close()

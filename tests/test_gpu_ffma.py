@@ -105,3 +105,27 @@ def test_backward_at_the_edges_of_the_tiles(shape, untied):
         assert np.isfinite(g).all() and np.abs(rf).max() > 0
         assert rel_err(g, rf) <= 2e-5, (shape, nm, rel_err(g, rf))
     ctx.close()
+
+
+@pytest.mark.parametrize("d", [40, 96])
+def test_bf16_backward_at_other_head_sizes(d):
+    """bf16 storage without a tcgen05 kernel: compression in two bf16 parts, then the float32 backward kernels, which decide from
+    their own forward pass; oracle with the library's decisions, the bf16 bar."""
+    B, H, n, nq, m, T = 2, 3, 143, 90, 101, 4
+    w = wl.Workload("edges", B, H, n, nq, d, m, "bf16", T, 0.001, "iid", 970 + d)
+    inp = wl.make_inputs(w)
+    Q, K, V, _ = device_inputs(w, inp)
+    ctx = make_ctx(w)
+    binding.csat_set_i64(ctx.h, binding.CSAT_KEEP_MASKS, 1)
+    phi = to_np(ctx.get_phi())
+    G = wl.round_to_storage(np.random.default_rng(13).standard_normal(inp["Q"].shape).astype(np.float32), "bf16")
+    ctx.forward(Q, K, V)
+    got = ctx.backward(Q, K, V, to_dev(G, "bf16"))
+    words = ctx.backward_masks().cpu().numpy().astype(np.uint32)
+    masks = np.stack([(words >> t) & 1 for t in range(T)], axis=2).astype(bool)
+    ref = orc.csat_backward(inp["Q"], inp["K"], inp["V"], phi, G, T=T, lam=w.lam, masks=masks)
+    for nm, g, rf in zip(("dQ", "dK", "dV"), got, ref):
+        g = to_np(g)
+        assert np.isfinite(g).all() and np.abs(rf).max() > 0
+        assert rel_err(g, rf) <= TOL["bf16"], (d, nm, rel_err(g, rf))
+    ctx.close()
