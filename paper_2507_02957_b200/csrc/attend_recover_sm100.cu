@@ -108,28 +108,9 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= 512, "barrier block");
 
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&p);
-}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float y;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-  return y;
-}
-__device__ __forceinline__ float add_sat(float a, float b) {            // clamps the result to [0, 1]
-  float y;
-  asm("add.sat.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-  return y;
-}
-__device__ __forceinline__ float fma_sat(float a, float b, float c) {   // clamps the result to [0, 1]
-  float y;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
   return y;
 }
 // 32-byte store (the address is 32-byte aligned)
@@ -169,21 +150,6 @@ __device__ __forceinline__ void exp2_poly2(F2 x2, float& p0, float& p1) {
   p0 = __int_as_float(__float_as_int(q0) + (__float_as_int(t0) << 23));
   p1 = __int_as_float(__float_as_int(q1) + (__float_as_int(t1) << 23));
 }
-
-// warpgroup-wide change of the per-thread register allowance (every warp of the warpgroup executes it)
-template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
-
-// A wait that never blocks for more than the time-out and turns into a no-op once anything gave up.
-struct Waiter {
-  int* status;
-  int* cta_abort;
-  bool dead = false;
-  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, int code) {
-    if (dead) return;
-    if (!mbar_wait(bar, parity, status, code, cta_abort)) dead = true;
-  }
-};
 
 // kMasks (backward pass only, one S, B for all layers): besides the output the kernel leaves what the backward needs:
 // Z (bf16, as fed to the first product), every row's log sum exp, and the decision |x_t| > theta_t of every layer,
@@ -1215,24 +1181,14 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int T,
   if (n_items > (int64_t)1 << 30) return cudaErrorInvalidValue;
   const int sms = c->sms;
   const unsigned grid = (unsigned)(n_items < sms ? n_items : sms);
-  // programmatic dependent launch: the kernel may be scheduled while the compression kernel before it still runs
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, attend_recover_sm100_kernel<D, kUntied, kRec, kFold>, tq, c->tmap_kv,
-                            kUntied ? c->tmap_lmats : c->tmap_mats, to, c->tmap_vb, (__nv_bfloat16*)out, c->thr(), c->thr_stride(),
-                            (int)p.nq, (int)p.m, (int)p.H, T, c->psi ? 1 : 0, scale_log2, (int)items_x, (int)n_items,
-                            (int)c->bh0, c->status, lse_out, lse_stride, z_out, mask_out, alpha_out,
-                            (int64_t)(p.B * p.H * p.nq * p.d), alpha_out != nullptr ? c->bw_signbits : nullptr, wait_first ? 1 : 0,
-                            // S = I - mu G with mu at most 1 over G's largest eigenvalue
-                            !c->w_S && p.step == 0.0 ? 1 : 0);
+  // the kernel may be scheduled while the compression kernel before it still runs
+  return launch_pdl(attend_recover_sm100_kernel<D, kUntied, kRec, kFold>, dim3(grid), kThreads, C::kSmemBytes, s, tq, c->tmap_kv,
+                    kUntied ? c->tmap_lmats : c->tmap_mats, to, c->tmap_vb, (__nv_bfloat16*)out, c->thr(), c->thr_stride(), (int)p.nq,
+                    (int)p.m, (int)p.H, T, c->psi ? 1 : 0, scale_log2, (int)items_x, (int)n_items, (int)c->bh0, c->status, lse_out,
+                    lse_stride, z_out, mask_out, alpha_out, (int64_t)(p.B * p.H * p.nq * p.d),
+                    alpha_out != nullptr ? c->bw_signbits : nullptr, wait_first ? 1 : 0,
+                    // S = I - mu G with mu at most 1 over G's largest eigenvalue
+                    !c->w_S && p.step == 0.0 ? 1 : 0);
 }
 
 }  // namespace

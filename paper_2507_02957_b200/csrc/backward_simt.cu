@@ -22,6 +22,7 @@
 namespace csat {
 namespace {
 
+constexpr int kMaxD = 256;        // the largest head size
 constexpr int kRowWarps = 8;
 constexpr int kColWarps = 8;
 constexpr int kColRows = 16;      // query rows staged per step of bwd_cols_kernel
@@ -92,13 +93,14 @@ __global__ void expand_masks_kernel(uint32_t* __restrict__ out, const uint32_t* 
   out[i] = wv;
 }
 
-template <typename T, int DC>   // DC = ceil(d / 32)
+template <typename T>
 __global__ void __launch_bounds__(kRowWarps * 32) bwd_rows_kernel(
     T* __restrict__ dQ, float* __restrict__ ws_dZ, float* __restrict__ ws_LD,
     const T* __restrict__ Q,
     const T* __restrict__ G, const T* __restrict__ kv, const float* __restrict__ S_dec, const float* __restrict__ B_dec,
     const float* __restrict__ S_decT, const float* __restrict__ B_decT, int64_t layer_stride, const float* __restrict__ theta, int theta_stride, const float* __restrict__ psi_f32,
     int64_t nq, int64_t m, int d, int H, int T_iters, float scale, uint32_t* __restrict__ ws_masks) {
+  constexpr int DC = kMaxD / 32;                   // columns per lane
   extern __shared__ float smem[];
   const int d2 = 2 * d, ldk = d2 + 1;
   float* kvs = smem;                               // [32][2d+1]
@@ -268,10 +270,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) bwd_rows_kernel(
   }
 }
 
-template <typename T, int DC>
+template <typename T>
 __global__ void __launch_bounds__(kColWarps * 32) bwd_cols_kernel(
     float* __restrict__ ws_dKV, const T* __restrict__ Q, const T* __restrict__ kv, const float* __restrict__ ws_dZ,
     const float* __restrict__ ws_LD, int64_t nq, int64_t m, int d, float scale) {
+  constexpr int DC = kMaxD / 32;                   // columns per lane
   extern __shared__ float smem[];
   float* qt = smem;                                // [kColRows][d]
   float* dzt = qt + kColRows * d;                  // [kColRows][d]
@@ -440,28 +443,17 @@ cudaError_t run(csat_ctx* c, const void* Q, const void* G, void* dQ, void* dK, v
   {
     const dim3 grid((unsigned)((p.nq + kRowWarps - 1) / kRowWarps), BH);
     const size_t sm = (size_t)(32 * (2 * d + 1) + 2 * kRowWarps * d) * sizeof(float);
-#define CSAT_BWD_ROWS(DC)                                                                                            \
-  do {                                                                                                               \
-    if (sm > 48 * 1024)                                                                                              \
-      e = cudaFuncSetAttribute(bwd_rows_kernel<T, DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);        \
-    if (e == cudaSuccess)                                                                                            \
-      bwd_rows_kernel<T, DC><<<grid, kRowWarps * 32, sm, s>>>(                                                       \
-          (T*)dQ, c->bw_dZ, c->bw_LD, (const T*)Q, (const T*)G, (const T*)c->kv, Sd, Bd, SdT, BdT, lstride, c->thr(), \
-          c->thr_stride(), c->psi ? c->psi_f32 : nullptr, p.nq, p.m, d, (int)p.H, p.T, scale, c->bw_masks);          \
-  } while (0)
-    CSAT_BWD_ROWS(8);
-#undef CSAT_BWD_ROWS
+    if (sm > 48 * 1024) e = cudaFuncSetAttribute(bwd_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
+    bwd_rows_kernel<T><<<grid, kRowWarps * 32, sm, s>>>((T*)dQ, c->bw_dZ, c->bw_LD, (const T*)Q, (const T*)G, (const T*)c->kv, Sd, Bd, SdT,
+                                                        BdT, lstride, c->thr(), c->thr_stride(), c->psi ? c->psi_f32 : nullptr, p.nq,
+                                                        p.m, d, (int)p.H, p.T, scale, c->bw_masks);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
     const dim3 grid((unsigned)((p.m + kColWarps - 1) / kColWarps), BH);
     const size_t sm = (size_t)(2 * kColRows * d + 2 * kColRows) * sizeof(float);
-#define CSAT_BWD_COLS(DC)                                                                                            \
-  bwd_cols_kernel<T, DC><<<grid, kColWarps * 32, sm, s>>>(c->bw_dKV, (const T*)Q, (const T*)c->kv, c->bw_dZ, c->bw_LD, \
-                                                         p.nq, p.m, d, scale)
-    CSAT_BWD_COLS(8);
-#undef CSAT_BWD_COLS
+    bwd_cols_kernel<T><<<grid, kColWarps * 32, sm, s>>>(c->bw_dKV, (const T*)Q, (const T*)c->kv, c->bw_dZ, c->bw_LD, p.nq, p.m, d, scale);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {

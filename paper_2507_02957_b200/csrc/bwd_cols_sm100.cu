@@ -72,12 +72,6 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
 
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 __device__ __forceinline__ const float4* peer_smem(const float4* p, uint32_t rank) {   // the same place in a CTA of the cluster
   uint64_t a;
   asm("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
@@ -249,8 +243,8 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         uint32_t pw[8], dw[8];
 #pragma unroll
         for (int e = 0; e < 16; e += 2) {
-          const float p0 = ex2f(fmaf(__uint_as_float(s[e]), scale_log2, -ld[e].x * 1.4426950408889634f));
-          const float p1 = ex2f(fmaf(__uint_as_float(s[e + 1]), scale_log2, -ld[e + 1].x * 1.4426950408889634f));
+          const float p0 = ex2(fmaf(__uint_as_float(s[e]), scale_log2, -ld[e].x * 1.4426950408889634f));
+          const float p1 = ex2(fmaf(__uint_as_float(s[e + 1]), scale_log2, -ld[e + 1].x * 1.4426950408889634f));
           const float d0 = p0 * (__uint_as_float(a[e]) - ld[e].y) * scale;
           const float d1 = p1 * (__uint_as_float(a[e + 1]) - ld[e + 1].y) * scale;
           __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1), dd = __floats2bfloat162_rn(d0, d1);

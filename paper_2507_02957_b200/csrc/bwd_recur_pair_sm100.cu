@@ -39,25 +39,6 @@ struct Bars {
   int abort;
 };
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&p);
-}
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
-
-struct Waiter {
-  int* status;
-  int* cta_abort;
-  bool dead = false;
-  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, int code) {
-    if (dead) return;
-    if (!mbar_wait(bar, parity, status, code, cta_abort)) dead = true;
-  }
-};
-
 __global__ void __launch_bounds__(kThreads, 1)
 bwd_recur_pair_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __grid_constant__ CUtensorMap tmap_g,
                       const __grid_constant__ CUtensorMap tmap_dz, const __nv_bfloat16* __restrict__ Z16, float* __restrict__ ws_LD,

@@ -38,28 +38,6 @@ using namespace ptx;
 constexpr int kRows = 128;
 constexpr int kMC = 64;
 
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&p);
-}
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
-struct Waiter {
-  int* status;
-  int* cta_abort;
-  bool dead = false;
-  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, int code) {
-    if (dead) return;
-    if (!mbar_wait(bar, parity, status, code, cta_abort)) dead = true;
-  }
-};
-
 // ====================================================================================================================
 // recurrence backward
 // ====================================================================================================================
@@ -477,8 +455,8 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 32; e += 2) {
-          const float p0 = ex2f(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
-          const float p1 = ex2f(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
+          const float p0 = ex2(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
+          const float p1 = ex2(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
           const float d0 = live ? scale * p0 * (__uint_as_float(av[e]) - Dv) : 0.f;
           const float d1 = live ? scale * p1 * (__uint_as_float(av[e + 1]) - Dv) : 0.f;
           pk[e >> 1] = pack_bf16(d0, d1);

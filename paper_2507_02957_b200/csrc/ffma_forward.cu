@@ -296,19 +296,21 @@ cudaError_t launch_compress(csat_ctx* c, TO* dst, const void* K, const void* V, 
 
 // The tile: 32 measurements x all columns of K~ or V~ up to 96 (the operand reads of 8 rows per lane keep up with the
 // arithmetic) where that gives most SMs a CTA, otherwise 16 x 32, and 8 x 32 where even that fills less than one wave.
-// Measured (float32, d = 64, m = 96, n = 512; 8 x 32 / 16 x 32 / 32 x 64): 2 heads 4.7 / 5.3 / 10.7 us, 8 heads 9.9 / 8.6
-// / 10.9, 16 heads 17.6 / 12.2 / 11.1, 64 heads 55.6 / 38.3 / 30.7 us.
+// Measured (float32, m = 96, n = 512, calls back to back, us; 8 x 32 / 16 x 32 / 32 rows): d = 64: 1 head 4.6 / 5.2 / 10.0, 4
+// heads 8.4 / 6.3 / 10.1, 8 heads 11.5 / 10.4 / 10.3, 16 heads 18.6 / 14.4 / 12.5, 64 heads 57.3 / 39.1 / 31.1; d = 96: 1 head 4.6 /
+// 5.3 / 15.4, 8 heads 14.5 / 10.4 / 15.9, 16 heads 24.7 / 16.6 / 18.4, 24 heads 34.3 / 23.0 / 18.6, 64 heads 84.1 / 55.5 / 47.2; d =
+// 128 (two blocks of 64 columns): 4 heads 11.7 / 10.4 / 10.4, 8 heads 18.6 / 14.4 / 12.4, 64 heads 108.7 / 71.8 / 59.6.  (2 heads of
+// 64 or 96 take 6.3 / 5.3: a grid of 96 CTAs does not start under its predecessor, see small_grid; behind another kernel 4.7 /
+// 5.3.)  At d <= 32 the 32-row tile has a quarter of the columns to share its rows' reads with and is never ahead: 24 heads
+// 10.4 with 16 and with 32 rows, 64 heads 22.7 and 22.7, 128 heads 39.1 and 41.2.
 template <typename T, typename TO>
 cudaError_t compress_t(csat_ctx* c, TO* dst, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len) {
   const Params& p = c->p;
   const int tcq = p.d <= 32 ? 1 : p.d <= 64 ? 2 : p.d <= 96 ? 3 : 2;          // 128 columns: two blocks of 64
   const int64_t bh = p.B * p.H, sms = c->sms;
   const int64_t big = (p.m + 31) / 32 * bh * 2 * ((p.d + 32 * tcq - 1) / (32 * tcq));
-  if (5 * big >= (tcq == 1 ? 10 : 3) * sms) switch (tcq) {
-    case 1: return launch_compress<T, TO, 8, 1>(c, dst, K, V, s, phi_j0, n_len);
-    case 2: return launch_compress<T, TO, 8, 2>(c, dst, K, V, s, phi_j0, n_len);
-    default: return launch_compress<T, TO, 8, 3>(c, dst, K, V, s, phi_j0, n_len);
-  }
+  if (tcq > 1 && 5 * big >= 3 * sms)
+    return tcq == 2 ? launch_compress<T, TO, 8, 2>(c, dst, K, V, s, phi_j0, n_len) : launch_compress<T, TO, 8, 3>(c, dst, K, V, s, phi_j0, n_len);
   if ((p.m + 7) / 8 * bh * 2 * ((p.d + 31) / 32) <= sms) return launch_compress<T, TO, 2, 1>(c, dst, K, V, s, phi_j0, n_len);
   return launch_compress<T, TO, 4, 1>(c, dst, K, V, s, phi_j0, n_len);
 }

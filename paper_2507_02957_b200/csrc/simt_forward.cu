@@ -25,16 +25,18 @@ template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p,
 // block: 256 threads = 8 row groups x 32 column lanes; tile = 32 measurements x 2d columns;
 // the token axis is walked in chunks of 16 staged in shared memory.
 // ---------------------------------------------------------------------------------------------
+constexpr int kMaxD = 256;                         // the largest head size
 constexpr int kCmpRows = 32, kCmpChunk = 16;
 
 // Token-sharded use: K, V hold the n tokens [phi_j0, phi_j0 + n) of the sequence and the sums go out as float32
 // partials (TO = float) that are added over the shards before anything reads them.
-template <typename T, typename TO, int KC>   // KC = ceil(2d / 32) column slots per lane
+template <typename T, typename TO>
 __global__ void __launch_bounds__(256) compress_kernel(TO* __restrict__ kv, const T* __restrict__ phi,
                                                        const T* __restrict__ K, const T* __restrict__ V, int64_t n,
                                                        int64_t n_pad, int64_t m, int d, int H, int phi_v_head0,
                                                        int64_t phi_j0) {
   // phi_v_head0: index of the first Phi_V matrix in phi (0 when Phi_V = Phi_K, H when they are separate)
+  constexpr int KC = 2 * kMaxD / 32;               // column slots per lane
   extern __shared__ float smem[];
   float* phis = smem;                              // [2][32][17]: Phi_K tile, Phi_V tile
   float* phiv = smem + kCmpRows * (kCmpChunk + 1);
@@ -156,11 +158,12 @@ __device__ __forceinline__ void row_times_matrix(const float (&x)[DC], float (&y
   }
 }
 
-template <typename T, int DC>   // DC = ceil(d / 32)
+template <typename T>
 __global__ void __launch_bounds__(kAttWarps * 32) attend_recover_kernel(
     T* __restrict__ out, const T* __restrict__ Q, const T* __restrict__ kv, const float* __restrict__ S_dec,
     const float* __restrict__ B_dec, int64_t layer_stride, const float* __restrict__ theta, int theta_stride,
     const float* __restrict__ psi_f32, int64_t nq, int64_t m, int d, int H, int T_iters, float scale) {
+  constexpr int DC = kMaxD / 32;           // columns per lane
   extern __shared__ float smem[];
   const int d2 = 2 * d, ldk = d2 + 1;
   float* kvs = smem;                       // [32][2d+1]
@@ -283,19 +286,13 @@ cudaError_t compress_t(csat_ctx* c, const void* K, const void* V, cudaStream_t s
   const int d = (int)p.d;
   const dim3 grid((unsigned)((p.m + kCmpRows - 1) / kCmpRows), (unsigned)(p.B * p.H));
   const size_t sm = (size_t)(2 * kCmpRows * (kCmpChunk + 1) + kCmpChunk * 2 * d) * sizeof(float);
-#define CSAT_CMP(KC)                                                                                                  \
-  do {                                                                                                                \
-    if (partial)                                                                                                      \
-      compress_kernel<T, float, KC><<<grid, 256, sm, s>>>(partial, (const T*)c->phi, (const T*)K, (const T*)V, n_len, \
-                                                          p.n_pad, p.m, d, (int)p.H, p.separate_phi ? (int)p.H : 0,  \
-                                                          phi_j0);                                                    \
-    else                                                                                                              \
-      compress_kernel<T, T, KC><<<grid, 256, sm, s>>>((T*)c->kv, (const T*)c->phi, (const T*)K, (const T*)V, n_len,  \
-                                                      p.n_pad, p.m, d, (int)p.H, p.separate_phi ? (int)p.H : 0,      \
-                                                      phi_j0);                                                        \
-  } while (0)
-  CSAT_CMP(16);
-#undef CSAT_CMP
+  const int phi_v = p.separate_phi ? (int)p.H : 0;
+  if (partial)
+    compress_kernel<T, float><<<grid, 256, sm, s>>>(partial, (const T*)c->phi, (const T*)K, (const T*)V, n_len, p.n_pad, p.m, d, (int)p.H,
+                                                    phi_v, phi_j0);
+  else
+    compress_kernel<T, T><<<grid, 256, sm, s>>>((T*)c->kv, (const T*)c->phi, (const T*)K, (const T*)V, n_len, p.n_pad, p.m, d, (int)p.H,
+                                                phi_v, phi_j0);
   return cudaGetLastError();
 }
 
@@ -327,21 +324,13 @@ cudaError_t attend_t(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool
     return launch_ffma_attend(a, p.dtype, Q, c->kv, out, s);
   }
   cudaError_t e = cudaSuccess;
-#define CSAT_ATT(DC)                                                                                              \
-  do {                                                                                                            \
-    if (sm > 48 * 1024)                                                                                           \
-      e = cudaFuncSetAttribute(attend_recover_kernel<T, DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
-    if (e == cudaSuccess)                                                                                         \
-      attend_recover_kernel<T, DC><<<grid, kAttWarps * 32, sm, s>>>(                                              \
-          (T*)out, (const T*)Q, (const T*)c->kv, c->w_untied ? c->Sl_dec : c->S_dec,                             \
-          c->w_untied ? c->Bl_dec : c->B_dec, c->w_untied ? (int64_t)(p.H * p.d * p.d) : (int64_t)0, c->thr(),  \
-          c->thr_stride(),                                                                                       \
-          c->psi ? c->psi_f32 : nullptr,                                                                         \
-          p.nq, p.m, d, (int)p.H, p.T, scale);                                                                    \
-  } while (0)
-  CSAT_ATT(8);
-#undef CSAT_ATT
-  return e != cudaSuccess ? e : cudaGetLastError();
+  if (sm > 48 * 1024) e = cudaFuncSetAttribute(attend_recover_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  attend_recover_kernel<T><<<grid, kAttWarps * 32, sm, s>>>(
+      (T*)out, (const T*)Q, (const T*)c->kv, c->w_untied ? c->Sl_dec : c->S_dec, c->w_untied ? c->Bl_dec : c->B_dec,
+      c->w_untied ? (int64_t)(p.H * p.d * p.d) : (int64_t)0, c->thr(), c->thr_stride(), c->psi ? c->psi_f32 : nullptr, p.nq, p.m, d,
+      (int)p.H, p.T, scale);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -452,20 +441,13 @@ int attend_noalloc_t(const void* Q, const void* K, const void* V, const void* ph
       if (e == cudaSuccess)
         e = launch_ffma_attend(a, std::is_same<T, float>::value ? CSAT_DTYPE_FP32 : CSAT_DTYPE_BF16, Q, scratch, out, s);
     } else {
-    const dim3 grid((unsigned)((nq + kAttWarps - 1) / kAttWarps), (unsigned)(B * H));
-    const size_t sm = (size_t)(32 * (2 * d + 1) + kAttWarps * d) * sizeof(float);
-#define CSAT_NOALLOC_ATT(DC)                                                                                        \
-  do {                                                                                                              \
-    if (sm > 48 * 1024)                                                                                             \
-      e = cudaFuncSetAttribute(attend_recover_kernel<T, DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
-    if (e == cudaSuccess)                                                                                           \
-      attend_recover_kernel<T, DC><<<grid, kAttWarps * 32, sm, s>>>((T*)out, (const T*)Q, (const T*)scratch,        \
-                                                                    nullptr, nullptr, (int64_t)0, nullptr, 0,       \
-                                                                    nullptr, nq, m, d,                              \
-                                                                    (int)H, /*T_iters=*/0, scale);                  \
-  } while (0)
-    CSAT_NOALLOC_ATT(8);
-#undef CSAT_NOALLOC_ATT
+      const dim3 grid((unsigned)((nq + kAttWarps - 1) / kAttWarps), (unsigned)(B * H));
+      const size_t sm = (size_t)(32 * (2 * d + 1) + kAttWarps * d) * sizeof(float);
+      if (sm > 48 * 1024 && e == cudaSuccess)
+        e = cudaFuncSetAttribute(attend_recover_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e == cudaSuccess)
+        attend_recover_kernel<T><<<grid, kAttWarps * 32, sm, s>>>((T*)out, (const T*)Q, (const T*)scratch, nullptr, nullptr, (int64_t)0,
+                                                                  nullptr, 0, nullptr, nq, m, d, (int)H, /*T_iters=*/0, scale);
     }
     if (e == cudaSuccess) e = cudaGetLastError();
   }

@@ -31,6 +31,35 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// ---- arithmetic ------------------------------------------------------------------------------------
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float add_sat(float a, float b) {            // clamps the result to [0, 1]
+  float y;
+  asm("add.sat.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {   // clamps the result to [0, 1]
+  float y;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+// two values as bf16 in one register, the first in the low half; the halves of such a register
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&p);
+}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// ---- registers ------------------------------------------------------------------------------------
+// warpgroup-wide change of the per-thread register allowance (every warp of the warpgroup executes it)
+template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // ---- programmatic dependent launch ------------------------------------------------------------------
 // A kernel launched with the programmatic-stream-serialization attribute may start while the kernel before it in the
 // stream is still running; it must not touch that kernel's results before pdl_wait() (which returns once the earlier
@@ -92,6 +121,17 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity) 
     if ((++spins & 0x3ff) == 0 && globaltimer() - t0 > kWaitTimeoutNs) return false;
   return true;
 }
+
+// A wait that never blocks for more than the time-out and turns into a no-op once anything gave up.
+struct Waiter {
+  int* status;
+  int* cta_abort;
+  bool dead = false;
+  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, int code) {
+    if (dead) return;
+    if (!mbar_wait(bar, parity, status, code, cta_abort)) dead = true;
+  }
+};
 
 // ---- TMA (tiled bulk tensor copies global -> shared, completion on an mbarrier) -------------
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {

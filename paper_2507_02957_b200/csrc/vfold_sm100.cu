@@ -142,18 +142,9 @@ cudaError_t launch(csat_ctx* c, cudaStream_t s) {
   static DeviceFlags smem_opt_in;
   cudaError_t e = ensure_dynamic_smem(vfold_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(c->bh_cnt ? c->bh_cnt : p.B * p.H));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, vfold_sm100_kernel<D>, c->tmap_kv, c->tmap_mats, c->tmap_vb_st, (int)p.H, (int)c->bh0,
-                            c->status);
+  const dim3 grid((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(c->bh_cnt ? c->bh_cnt : p.B * p.H));
+  return launch_pdl(vfold_sm100_kernel<D>, grid, kThreads, C::kSmemBytes, s, c->tmap_kv, c->tmap_mats, c->tmap_vb_st, (int)p.H,
+                    (int)c->bh0, c->status);
 }
 
 }  // namespace

@@ -351,18 +351,9 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   a.lse = lse; a.lse_stride = lse_stride; a.z = z; a.masks = masks;
   const int64_t grid = (int64_t)a.tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
   if (grid > (int64_t)1 << 30) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kWarps * 32);
-  // one CTA per SM: without that, CTAs that start early would pile up on the SMs the compression leaves free
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;    // the prologue may run under the compression's tail
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, warp_attend_kernel<kRec>, a);
+  // The prologue may run under the compression's tail.  One CTA per SM: without that (kSmemBytes), CTAs that start early would
+  // pile up on the SMs the compression leaves free
+  return launch_pdl(warp_attend_kernel<kRec>, dim3((unsigned)grid), kWarps * 32, kSmemBytes, s, a);
 }
 
 }  // namespace

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sm100_ptx.cuh"
+
 namespace csat {
 namespace wmma16 {
 
@@ -35,25 +37,10 @@ __device__ __forceinline__ void cp16(__nv_bfloat16* s, const void* g, bool in) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ uint32_t pack(float a, float b) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&p);
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float add_sat(float a, float b) {            // clamps the result to [0, 1]
-  float y;
-  asm("add.sat.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-  return y;
-}
-__device__ __forceinline__ float fma_sat(float a, float b, float c) {
-  float y;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-  return y;
-}
+__device__ __forceinline__ uint32_t pack(float a, float b) { return ptx::pack_bf16(a, b); }
+using ptx::add_sat;
+using ptx::ex2;
+using ptx::fma_sat;
 
 // the 16 x D float32 rows x (accumulator layout, NT = D / 8 tiles of 8 columns) as bf16 A operands of D / 16 steps
 template <int NT> __device__ __forceinline__ void to_operand(uint32_t (&a)[NT / 2][4], const float (&x)[NT][4]) {
