@@ -199,7 +199,7 @@ int csat_set_lista_layer_weights(csat_ctx* ctx, const void* S, const void* Bm, c
  *   dQ [B,H,n_q,d], dK, dV [B,H,n,d]  outputs (context dtype)
  * Unless the last csat_forward ran with CSAT_SAVE_FOR_BACKWARD, nothing of an earlier csat_forward is reused: the
  * call compresses K, V again and recomputes what it needs.  Its
- * first call allocates scratch (B H (n_q (d + 2) + 2 m d) floats and transposed copies of the decoder matrices;
+ * first call allocates scratch (B H (n_q (d + 2) + 2 m d) floats; transposed copies of the decoder matrices for d > 128;
  * bf16 copies of Z, dZ and dK~|dV~ and B H T n_q d / 32 decision words on the tensor-core path; B H n_q d words
  * more with CSAT_KEEP_MASKS; all counted by csat_workspace_bytes).
  * Two paths.  bf16 contexts with d in {64, 128} run every stage on the tensor cores (one S, B for all layers, or one

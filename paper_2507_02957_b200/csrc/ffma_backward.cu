@@ -7,7 +7,9 @@
 //   ffma_bwd_cols : a few measurements per CTA, the queries shared out between its warps (a fixed order, no atomics):
 //                   dK~ = scale dS^T Q, dV~ = P^T dZ.
 //   ffma_phiT     : dK = Phi^T dK~, dV = Phi_V^T dV~.
-// Bound: shared-memory reads and the FMA pipe (ffma_tile.cuh); for small jobs the chain of waits of one warp.  Measured
+// Bound: shared-memory reads and the FMA pipe (ffma_tile.cuh), neither of them full at the sizes measured (rows 64 % and 42 % of
+// the active cycles, columns 38 % and 30 %, Phi^T 25 % and 42 %: two warps per sub-core and less than a wave); for small jobs the
+// chain of waits of one warp.  Measured
 // against kernels with one warp per row (one B200, 16 heads of 512 x 64, m = 96, T = 10, float32): rows 344 -> 73,
 // columns 158 -> 33, Phi^T 16.6 -> 8.0 us.
 #include "csat_internal.h"
