@@ -71,7 +71,7 @@ def test_attend_behind_attend_and_forward(d, T, H, n):
     second.close()
 
 
-@pytest.mark.parametrize("weights", [False, True], ids=["derived", "supplied"])
+@pytest.mark.parametrize("weights", ["derived", "supplied", "per_layer"])
 @pytest.mark.parametrize("dtype, d, H, n", [("bf16", 64, 4, 1024), ("bf16", 64, 6, 1600), ("bf16", 128, 6, 1600), ("bf16", 96, 2, 300),
                                             ("fp32", 64, 1, 300), ("fp32", 128, 1, 300)])
 def test_attend_behind_the_decoder_set_up(dtype, d, H, n, weights):
@@ -86,7 +86,10 @@ def test_attend_behind_the_decoder_set_up(dtype, d, H, n, weights):
     th = [torch.full((1, H), x, device="cuda") for x in (0.01, 0.03)]
 
     def change(i):
-        if weights:
+        if weights == "per_layer":
+            ctx.set_lista_layer_weights(S[i].expand(10, H, d, d).contiguous(), Bm[i].expand(10, H, d, d).contiguous(),
+                                        th[i].expand(10, H).contiguous())
+        elif weights == "supplied":
             ctx.set_lista_weights(S[i], Bm[i], th[i])
         else:
             ctx.set(step=(0.05, 0.1)[i])
