@@ -1,4 +1,5 @@
-// Compressed attention and sparse recovery for two tiles of 128 queries per CTA, on the sm_100a tensor cores.
+// Compressed attention and sparse recovery for two tiles of 128 queries per CTA, on the sm_100a tensor cores (d = 128; d = 64 has
+// attend_tile_sm100.cu, with three tiles in flight per SM).
 //
 // Paper, in order: A~ = softmax(Q K~^T / sqrt(d_k)) over the m measurements; Z = A~ V~;
 // alpha^{t+1} = eta_theta(S alpha^t + B Z_i) (LISTA recurrence with S = I - mu G, B = mu M); C^_i = Psi alpha^_i.
@@ -51,6 +52,7 @@
 // item's chunks (S_t - I in the K~ slots, B_t in the V~ slots), so layer t + 1 is loaded while layer t is computed.
 // The registers hold alpha^t + theta_t, which turns the shrinkage into y - 2 theta sat(y / (2 theta)).
 #include "csat_internal.h"
+#include "row_math.cuh"
 #include "sm100_ptx.cuh"
 #include "tma_host.h"
 
@@ -60,6 +62,7 @@ namespace csat {
 namespace {
 
 using namespace ptx;
+using namespace rowmath;
 
 constexpr int kRows = 128;            // queries per tile
 constexpr int kTiles = 2;             // tiles per CTA
@@ -67,15 +70,14 @@ constexpr int kMC = 64;               // measurements per chunk
 constexpr int kTileThreads = 128;
 constexpr int kThreads = 384;          // three warpgroups: tile A, tile B, control
 constexpr int kMmaWarp = 8, kTmaWarp = 9, kMmaWarpB = 10;   // tile A's MMA issuer, TMA producer, tile B's MMA issuer
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 4;
 constexpr int kComputeRegs = 224, kControlRegs = 56;   // registers per thread after setmaxnreg (checked on the host)
-constexpr int kPolyEvery = 4;          // every 4th pair of scores takes the polynomial exp2 (measured best of 1, 2, 3, 4, none)
 
 // kStaged: the output leaves through shared-memory boxes and TMA stores (the plain forward); the recording variants
 // store directly (they spill more, and the 32 KB of boxes would take the L1 those spills live in)
 template <int D, bool kStaged> struct Cfg {
   static constexpr int kDBoxes = D / 64;                          // 64-column boxes across the head dimension
-  static constexpr int kStages = (D == 64) ? 6 : 4;               // K~ / V~ chunks in flight
+  static constexpr int kStages = 4;                               // K~ / V~ chunks in flight
   static constexpr uint32_t kQBytes = kDBoxes * kRows * 128;      // one Q tile; tile A's buffer later holds B
   static constexpr uint32_t kBoxBytes = kMC * 128;                // one 64-column box of a K~ or V~ chunk
   static constexpr uint32_t kSlotBytes = kDBoxes * kBoxBytes;     // K~ chunk (= V~ chunk)
@@ -91,7 +93,7 @@ template <int D, bool kStaged> struct Cfg {
   // TMEM columns per tile (tile t starts at column 256 t): S[0] | S[1] | accumulator (Zacc, then r_t).
   // P_j overlays S[j&1]; the recovery operand overlays S[0].
   static constexpr uint32_t kTileCols = 256, kColS = 0, kColAcc = 2 * kMC, kTmemCols = 512;
-  static_assert(2 * kMC + D <= 256, "TMEM budget");
+  static_assert(D == 128 && 2 * kMC + D <= 256, "TMEM budget");
   static_assert(D <= 2 * kMC, "recovery operands (z and alpha, D / 2 packed columns each) fit in the S columns");
   static_assert(kStages >= kDBoxes && kStages <= kMaxStages, "mu G and Psi are staged box by box in ring slots");
   static_assert(kMatBoxBytes <= kSlotBytes && kMatBytes <= kQBytes, "decoder matrices fit where they are staged");
@@ -107,49 +109,6 @@ struct Bars {
   int abort;
 };
 static_assert(sizeof(Bars) <= 512, "barrier block");
-
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float y;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-  return y;
-}
-// 32-byte store (the address is 32-byte aligned)
-__device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&r)[8]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
-               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-// two-element packed fp32 arithmetic (one instruction for both halves of a register pair): the compiler's float2
-// builtins, so that it sees the register pairs (inline assembly on 64-bit registers cost extra moves and spills)
-using F2 = float2;
-__device__ __forceinline__ F2 pack2(float lo, float hi) { return make_float2(lo, hi); }
-__device__ __forceinline__ F2 pack2u(uint32_t lo, uint32_t hi) { return make_float2(__uint_as_float(lo), __uint_as_float(hi)); }
-__device__ __forceinline__ void unpack2(F2 v, float& lo, float& hi) { lo = v.x; hi = v.y; }
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ F2 add2(F2 a, F2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) { return __fmul2_rn(a, b); }
-
-// exp2 of both halves on the FMA pipe (the MUFU unit is the bottleneck of the softmax: 4 lanes per clock and
-// sub-core).  x <= ~9; anything below -120 (masked columns are -inf) gives 2^-120.  Round-to-nearest split
-// x = i + f, f in [-1/2, 1/2]; 2^f by a cubic fitted to 7.5e-5 relative error (P is rounded to bf16, 3.9e-3,
-// and the row sum tolerates far more); 2^i by adding i to the exponent field.
-__device__ __forceinline__ void exp2_poly2(F2 x2, float& p0, float& p1) {
-  float x0, x1;
-  unpack2(x2, x0, x1);
-  x2 = pack2(fmaxf(x0, -120.f), fmaxf(x1, -120.f));
-  const F2 magic = pack2(12582912.f, 12582912.f);          // 1.5 * 2^23: the sum's low mantissa bits hold i
-  const F2 t2 = add2(x2, magic);
-  const F2 f2 = sub2(x2, sub2(t2, magic));
-  F2 q2 = fma2(f2, pack2(0.055171459913253784f, 0.055171459913253784f), pack2(0.2426108568906784f, 0.2426108568906784f));
-  q2 = fma2(q2, f2, pack2(0.6932609677314758f, 0.6932609677314758f));
-  q2 = fma2(q2, f2, pack2(0.9999281167984009f, 0.9999281167984009f));
-  float t0, t1, q0, q1;
-  unpack2(t2, t0, t1);
-  unpack2(q2, q0, q1);
-  p0 = __int_as_float(__float_as_int(q0) + (__float_as_int(t0) << 23));
-  p1 = __int_as_float(__float_as_int(q1) + (__float_as_int(t1) << 23));
-}
 
 // kMasks (backward pass only, one S, B for all layers): besides the output the kernel leaves what the backward needs:
 // Z (bf16, as fed to the first product), every row's log sum exp, and the decision |x_t| > theta_t of every layer,
@@ -267,7 +226,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
         // launch this kernel may have started (and loaded its first Q tiles) before that one finished.  What else is read
         // (Q, theta, the matrices) was complete before that kernel let this one start, unless wait_first says otherwise;
         // every store follows from what is loaded below.
-        if (items_done == 0) {
+        if (items_done == 0 && !kFold) {
           pdl_wait();
           pdl_launch_dependents();
         }
@@ -280,6 +239,10 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
             tma_load_3d(k_slot(s) + gx * C::kBoxBytes, &tmap_kv, &bars->k_full[s], gx * 64, j * kMC, bh);
           k_hist = (k_hist << 1) | 1u;
           v_hist <<= 1;
+          if (kFold && items_done == 0 && j == 0) {     // K~ was complete before the fold let this kernel start, V~ B was not
+            pdl_wait();
+            pdl_launch_dependents();
+          }
           ring_wait_v(g, 202);
           if (w.dead) { ++g; break; }
           mbar_arrive_expect_tx(&bars->v_full[s], C::kSlotBytes);
@@ -687,13 +650,11 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
       auto store_masks = [&](int layer) {
         if (signs && grow_m < nq) {
           uint32_t* so = sign_out + (((int64_t)bh * T + layer) * nq + grow_m) * (D / 32);
-          if (D == 128) *reinterpret_cast<uint4*>(so) = make_uint4(sw[0], sw[1], sw[2], sw[D / 32 - 1]);
-          else *reinterpret_cast<uint2*>(so) = make_uint2(sw[0], sw[1]);
+          *reinterpret_cast<uint4*>(so) = make_uint4(sw[0], sw[1], sw[2], sw[3]);
         }
         if (kMasks && mask_out != nullptr && grow_m < nq) {
           uint32_t* mo = mask_out + (((int64_t)bh * T + layer) * nq + grow_m) * (D / 32);
-          if (D == 128) *reinterpret_cast<uint4*>(mo) = make_uint4(mw[0], mw[1], mw[2], mw[D / 32 - 1]);
-          else *reinterpret_cast<uint2*>(mo) = make_uint2(mw[0], mw[1]);
+          *reinterpret_cast<uint4*>(mo) = make_uint4(mw[0], mw[1], mw[2], mw[3]);
         }
       };
       auto publish = [&](uint32_t col) {                        // v2 as a bf16 A operand, from column col of S on
@@ -1227,26 +1188,25 @@ cudaError_t make_layer_weights_tmap(csat_ctx* c) {
 
 cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first) {
   *launches += 1;
-#define CSAT_ATTEND(DD, UU) launch<DD, UU>(c, Q, out, s, c->p.T, nullptr, 0, nullptr, nullptr, nullptr, wait_first)
-  // with untied layers and T > 0 the per-layer kernel; the set-up has then built its operands for exactly T layers
-  if (c->w_S && c->w_untied && c->p.T > 0)
-    return c->p.d == 64 ? CSAT_ATTEND(64, true) : CSAT_ATTEND(128, true);
-  if (warp_attend_better(c)) return launch_warp_attend(c, Q, out, s, wait_first);
+  const Params& p = c->p;
+  const bool untied = c->w_S && c->w_untied && p.T > 0;         // the set-up has then built the operands of exactly T layers
+  if (p.d == 64) {
+    if (!untied && warp_attend_better(c)) return launch_warp_attend(c, Q, out, s, wait_first);
+    return launch_attend_tile(c, Q, out, s, launches, wait_first);
+  }
+  if (untied) return launch<128, true>(c, Q, out, s, p.T, nullptr, 0, nullptr, nullptr, nullptr, wait_first);
   // Long jobs with the ISTA-derived decoder (one S, B and one positive threshold for all layers) fold B into the
   // values first: one more small launch, which only pays where the attention kernel walks several items per SM
-  // (measured: from ~2 tiles of 128 queries per SM at d = 128, where a layer's hand-over chain is long, from ~8 at
-  // d = 64).  The choice looks at the context's whole job, not at the launch's range of (batch, head) pairs, so that
-  // a forward cut into sub-range launches returns the same bits as one launch.
-  const int64_t tiles = ((c->p.nq + kRows - 1) / kRows) * c->p.B * c->p.H;
-  if (!c->w_S && c->p.T >= 2 && c->p.lambda > 0.0 && tiles >= (c->p.d == 128 ? 2 : 8) * (int64_t)c->sms) {
+  // (measured: from ~2 tiles of 128 queries per SM).  The choice looks at the context's whole job, not at the launch's
+  // range of (batch, head) pairs, so that a forward cut into sub-range launches returns the same bits as one launch.
+  const int64_t tiles = ((p.nq + kRows - 1) / kRows) * p.B * p.H;
+  if (!c->w_S && p.T >= 2 && p.lambda > 0.0 && tiles >= 2 * (int64_t)c->sms) {
     cudaError_t e = launch_sm100_vfold(c, s, launches);
     if (e != cudaSuccess) return e;
     // the fold waits for whatever is before it: nothing to wait for but the fold itself
-    return c->p.d == 64 ? launch<64, false, 0, true>(c, Q, out, s, c->p.T, nullptr, 0)
-                        : launch<128, false, 0, true>(c, Q, out, s, c->p.T, nullptr, 0);
+    return launch<128, false, 0, true>(c, Q, out, s, p.T, nullptr, 0);
   }
-  return c->p.d == 64 ? CSAT_ATTEND(64, false) : CSAT_ATTEND(128, false);
-#undef CSAT_ATTEND
+  return launch<128, false>(c, Q, out, s, p.T, nullptr, 0, nullptr, nullptr, nullptr, wait_first);
 }
 
 // The forward with what the backward pass needs as its only outputs: Z (bf16), the rows' log sum exp and the layers'
@@ -1256,16 +1216,15 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
                                              cudaStream_t s, int* launches, void* out) {
   *launches += 1;
   const bool untied = c->w_S && c->w_untied && c->p.T > 0;      // one S_t, B_t per layer
-  const bool d64 = c->p.d == 64;
-#define CSAT_REC_LAUNCH(DD, UU, RR) \
-  launch<DD, UU, RR>(c, Q, out, s, c->p.T, lse_out, lse_stride, z_out, mask_out, alpha_out)
-  if (alpha_out != nullptr) {                   // with the iterates and the sign bits
-    if (untied) return d64 ? CSAT_REC_LAUNCH(64, true, 2) : CSAT_REC_LAUNCH(128, true, 2);
-    return d64 ? CSAT_REC_LAUNCH(64, false, 2) : CSAT_REC_LAUNCH(128, false, 2);
+  if (c->p.d == 64) {
+    if (alpha_out == nullptr && !untied && warp_attend_better(c))
+      return launch_warp_attend_recording(c, Q, out, s, lse_out, lse_stride, z_out, mask_out);
+    return launch_attend_tile_recording(c, Q, out, s, lse_out, lse_stride, z_out, mask_out, alpha_out);
   }
-  if (!untied && warp_attend_better(c)) return launch_warp_attend_recording(c, Q, out, s, lse_out, lse_stride, z_out, mask_out);
-  if (untied) return d64 ? CSAT_REC_LAUNCH(64, true, 1) : CSAT_REC_LAUNCH(128, true, 1);
-  return d64 ? CSAT_REC_LAUNCH(64, false, 1) : CSAT_REC_LAUNCH(128, false, 1);
+#define CSAT_REC_LAUNCH(UU, RR) \
+  launch<128, UU, RR>(c, Q, out, s, c->p.T, lse_out, lse_stride, z_out, mask_out, alpha_out)
+  if (alpha_out != nullptr) return untied ? CSAT_REC_LAUNCH(true, 2) : CSAT_REC_LAUNCH(false, 2);   // with the iterates and the sign bits
+  return untied ? CSAT_REC_LAUNCH(true, 1) : CSAT_REC_LAUNCH(false, 1);
 #undef CSAT_REC_LAUNCH
 }
 

@@ -41,7 +41,8 @@ cudaError_t ensure_dynamic_smem(Kernel* kernel, int bytes, int device, DeviceFla
 // starts, and the previous one itself is after griddepcontrol.wait: before that a kernel touches only what the previous kernel
 // does not write, and stores nothing.  The backward kernels and the projection read nothing at all before their wait.  The
 // attention kernels do: their first queries (attend_recover_sm100), thresholds and decoder matrices are in place before this
-// call's own compression or fold starts.  Behind any other kernel they are launched with wait_first.
+// call's own compression or fold starts, and behind the fold K~ as well, which the compression in front of that has written.
+// Behind any other kernel they are launched with wait_first.
 template <typename... KP, typename... Args>
 cudaError_t launch_maybe_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -262,6 +263,11 @@ cudaError_t launch_sm100_attend_recover(csat_ctx* c, const void* Q, void* out, c
 cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bfloat16* z_out, float* lse_out,
                                              int lse_stride, uint32_t* mask_out, __nv_bfloat16* alpha_out,
                                              cudaStream_t s, int* launches, void* out = nullptr);
+
+// attend_tile_sm100.cu : the same with one tile of 128 queries per CTA and several CTAs per SM
+cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first);
+cudaError_t launch_attend_tile_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
+                                         __nv_bfloat16* z, uint32_t* masks, __nv_bfloat16* alpha);
 
 // warp_attend.cu : the same two for d = 64 with 16 queries per warp (one S, B for all layers; no iterates)
 bool warp_attend_better(const csat_ctx* c);      // by the context's shape alone
