@@ -39,12 +39,15 @@ constexpr uint32_t kBoxBytes = 64 * kChunk * 2;       // 8 KB: 64 columns x 64 t
 // what an SM can load; two elements (N = 256) halve the operand bytes per flop and the L2 reads of Phi.
 // MT: measurement tiles per CTA (1 or 2; 2 only without SEP).  Two tiles of the same (batch, head) share every K, V
 // chunk: a second A tile per stage and a second accumulator, so the B operand is loaded once for twice the products.
-template <int D, bool SEP, int BG, int MT = 1> struct Cfg {
-  static constexpr int kN = 2 * D * BG;               // accumulator columns (per measurement tile)
+// HALF: the K and the V columns in CTAs of their own (blockIdx.z), for grids that leave at least half of the SMs idle.
+template <int D, bool SEP, int BG, int MT = 1, bool HALF = false> struct Cfg {
+  static constexpr int kHalfN = D * BG;               // accumulator columns of K (or V)
+  static constexpr int kN = (HALF ? 1 : 2) * kHalfN;  // accumulator columns (per measurement tile)
   static constexpr int kBoxes = kN / 64;              // B boxes per stage
   static constexpr int kATiles = SEP ? 2 : MT;
-  static constexpr int kStages = (D == 64 && BG == 1) ? ((SEP || MT == 2) ? 4 : 6) : ((SEP || MT == 2) ? 3 : 4);
+  static constexpr int kStages = (kN == 128) ? ((SEP || MT == 2) ? 4 : 6) : ((SEP || MT == 2) ? 3 : 4);
   static_assert(kN <= 256, "one MMA covers the accumulator");
+  static_assert(kN >= 128 && !(HALF && (SEP || MT == 2)), "built variants");
   static_assert(!(SEP && MT == 2) && MT * kN <= 512, "tensor memory");
   static constexpr uint32_t kStageBytes = kATiles * kABytes + kBoxes * kBoxBytes;
   static constexpr uint32_t kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
@@ -52,13 +55,13 @@ template <int D, bool SEP, int BG, int MT = 1> struct Cfg {
   static_assert(4 * MT * (kN / 64) * kOutBoxBytes <= kStages * kStageBytes, "the epilogue's boxes fit in the ring");
 };
 
-template <int D, bool SEP, int BG, int MT>
+template <int D, bool SEP, int BG, int MT, bool HALF>
 __global__ void __launch_bounds__(kThreads, 1)
 compress_sm100_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_constant__ CUtensorMap tmap_k,
                       const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_out,
                       __nv_bfloat16* __restrict__ kv, int m, int n, int H,
                       int B, int bh0, int* status, int phi_j0, float* __restrict__ partial) {
-  using C = Cfg<D, SEP, BG, MT>;
+  using C = Cfg<D, SEP, BG, MT, HALF>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* a_buf = smem;                                      // [stages][A tiles][16 KB]
@@ -122,8 +125,8 @@ compress_sm100_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid
           tma_load_3d(a_buf + (s * C::kATiles + 1) * kABytes, &tmap_phi, &full[s], phi_j0 + i * kChunk, (mtile + 1) * kTileM, hphi);
 #pragma unroll
         for (int g = 0; g < C::kBoxes; ++g) {
-          const bool is_v = g >= C::kBoxes / 2;
-          const int gg = g % (C::kBoxes / 2);               // box within the K (or V) half: element, then 64-column box
+          const bool is_v = HALF ? blockIdx.z != 0 : g >= C::kHalfN / 64;
+          const int gg = g % (C::kHalfN / 64);              // box within the K (or V) half: element, then 64-column box
           tma_load_3d(b_buf + (s * C::kBoxes + g) * kBoxBytes, is_v ? &tmap_v : &tmap_k, &full[s],
                       (gg % (D / 64)) * 64, i * kChunk, bh_of(gg / (D / 64)));
         }
@@ -173,7 +176,7 @@ compress_sm100_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid
         tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(mt * C::kN + c0), r);
         tmem_wait_ld();
         // accumulator column c0: K half or V half, batch element e of the group, feature column
-        const int half = c0 / (C::kN / 2), e = (c0 % (C::kN / 2)) / D, col = c0 % D;
+        const int half = HALF ? (int)blockIdx.z : c0 / C::kHalfN, e = (c0 % C::kHalfN) / D, col = c0 % D;
         if (row < m && b0 + e < B && partial != nullptr) {
           float4* o = reinterpret_cast<float4*>(partial + ((int64_t)bh_of(e) * m + row) * (2 * D) + half * D + col);
 #pragma unroll
@@ -231,10 +234,10 @@ __global__ void wait_timeout_selftest_kernel(int* status, unsigned long long lim
 
 // n_len tokens of K, V (a shard that starts at token phi_j0 of the sequence, or the whole sequence); partial: float32
 // destination of a shard's sums, null = the workspace
-template <int D, bool SEP, int BG, int MT = 1>
+template <int D, bool SEP, int BG, int MT = 1, bool HALF = false>
 cudaError_t launch(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len,
                    float* partial) {
-  using C = Cfg<D, SEP, BG, MT>;
+  using C = Cfg<D, SEP, BG, MT, HALF>;
   const Params& p = c->p;
   CUtensorMap tk, tv;
   const uint64_t kd[3] = {(uint64_t)D, (uint64_t)n_len, (uint64_t)(p.B * p.H)};
@@ -244,13 +247,13 @@ cudaError_t launch(csat_ctx* c, const void* K, const void* V, cudaStream_t s, in
   if ((e = make_tmap_bf16_3d(&tk, K, kd, ks, kb)) != cudaSuccess) return e;
   if ((e = make_tmap_bf16_3d(&tv, V, kd, ks, kb)) != cudaSuccess) return e;
   static DeviceFlags smem_opt_in;
-  if ((e = ensure_dynamic_smem(compress_sm100_kernel<D, SEP, BG, MT>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess)
+  if ((e = ensure_dynamic_smem(compress_sm100_kernel<D, SEP, BG, MT, HALF>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess)
     return e;
   // whole batch, or a range of heads of one batch element
   const int64_t Bl = c->bh_cnt ? 1 : p.B, Hl = c->bh_cnt ? c->bh_cnt : p.H;
   const int64_t mtiles = (p.m + kTileM - 1) / kTileM;
-  const dim3 grid((unsigned)((mtiles + MT - 1) / MT), (unsigned)(((Bl + BG - 1) / BG) * Hl));
-  compress_sm100_kernel<D, SEP, BG, MT><<<grid, kThreads, C::kSmemBytes, s>>>(c->tmap_phi, tk, tv, c->tmap_kv_st, (__nv_bfloat16*)c->kv, (int)p.m,
+  const dim3 grid((unsigned)((mtiles + MT - 1) / MT), (unsigned)(((Bl + BG - 1) / BG) * Hl), HALF ? 2 : 1);
+  compress_sm100_kernel<D, SEP, BG, MT, HALF><<<grid, kThreads, C::kSmemBytes, s>>>(c->tmap_phi, tk, tv, c->tmap_kv_st, (__nv_bfloat16*)c->kv, (int)p.m,
                                                                  (int)n_len, (int)p.H, (int)Bl, (int)c->bh0, c->status,
                                                                  (int)phi_j0, partial);
   return cudaGetLastError();
@@ -278,15 +281,22 @@ cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cud
   // two measurement tiles per CTA where that still leaves at least ~0.8 CTAs per SM
   const int64_t mtiles = (c->p.m + kTileM - 1) / kTileM;
   auto pairs_fill = [&](int64_t columns_of_ctas) { return mtiles >= 2 && ((mtiles + 1) / 2) * columns_of_ctas * 5 >= (int64_t)c->sms * 4; };
+  // the K and the V columns in CTAs of their own where those fit the SMs in one wave: a CTA then loads 32 instead of 48 KB per chunk
+  // of tokens, and what an SM can load (~49 bytes per clock) is what these grids wait for: 32 heads of 3001 x 128, m = 187 (64
+  // CTAs) 24.9 -> 18.0 us, 48 of 1568 x 64, m = 256 (48 CTAs) 14.3 -> 10.0, 16 of 8192 x 128, m = 512 (64) 58 -> 44
+  auto halves_fit = [&](int64_t columns_of_ctas) { return 2 * mtiles * columns_of_ctas <= (int64_t)c->sms; };
   // d = 64: two batch elements per CTA where the batch has them (N = 256 MMAs)
   if (c->p.d == 64 && c->p.B >= 2 && c->bh_cnt == 0) {
     if (c->p.separate_phi) return launch<64, true, 2>(c, K, V, s, phi_j0, n_len, partial);
+    if (halves_fit(((c->p.B + 1) / 2) * c->p.H)) return launch<64, false, 2, 1, true>(c, K, V, s, phi_j0, n_len, partial);
     return pairs_fill(((c->p.B + 1) / 2) * c->p.H) ? launch<64, false, 2, 2>(c, K, V, s, phi_j0, n_len, partial)
                                                   : launch<64, false, 2>(c, K, V, s, phi_j0, n_len, partial);
   }
   if (c->p.separate_phi)
     return c->p.d == 64 ? launch<64, true, 1>(c, K, V, s, phi_j0, n_len, partial)
                         : launch<128, true, 1>(c, K, V, s, phi_j0, n_len, partial);
+  if (c->p.d == 128 && halves_fit(c->bh_cnt ? c->bh_cnt : c->p.B * c->p.H))
+    return launch<128, false, 1, 1, true>(c, K, V, s, phi_j0, n_len, partial);
   if (c->p.d == 128 && pairs_fill(c->bh_cnt ? c->bh_cnt : c->p.B * c->p.H))
     return launch<128, false, 1, 2>(c, K, V, s, phi_j0, n_len, partial);
   return c->p.d == 64 ? launch<64, false, 1>(c, K, V, s, phi_j0, n_len, partial)
