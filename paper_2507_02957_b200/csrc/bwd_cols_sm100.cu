@@ -18,7 +18,8 @@
 //                dK~ += dS^T Q    (A = dS^T in tensor memory; B = the Q tile,  MN-major)
 //              The Q and dZ tiles are read twice without being moved: a tile of 64 rows x d with 128-byte rows is a
 //              K-major operand when its rows are the N index and an MN-major operand when they are the K index.
-//              Two sets of S^T | dA^T: the products of tile i + 1 run while the threads work on tile i.  The MMAs of
+//              Two sets of S^T | dA^T (SETS): the products of tile i + 1 run while the threads work on tile i; or one
+//              set in half of the tensor memory, and a second CTA on the SM does the overlapping.  The MMAs of
 //              one thread execute in issue order, so tile i + 2's scores overwrite set[i & 1] only after tile i's
 //              second pair of products has read it.
 //   warps 2-9: TMEM lane = measurement; warps 2-5 take the tile's queries [0, 32), warps 6-9 the queries [32, 64):
@@ -44,7 +45,8 @@ constexpr int kStages = 4;       // Q | dZ tiles in flight
 constexpr int kSimtWarps = 8;
 constexpr int kThreads = (2 + kSimtWarps) * 32;
 
-template <int D> struct Cfg {
+template <int D, int SETS> struct Cfg {
+  static constexpr int kCtas = SETS == 1 ? 2 : 1;                     // per SM
   static constexpr int kDBoxes = D / 64;
   static constexpr uint32_t kKvBoxBytes = kRows * 128;                // 128 rows x 64 columns
   static constexpr uint32_t kKvBytes = kDBoxes * kKvBoxBytes;         // K~ block (= V~ block)
@@ -57,12 +59,12 @@ template <int D> struct Cfg {
   static constexpr uint32_t kOffBar = kOffLd + kStages * kLdStride;
   static constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024 /*alignment slack*/;
   // TMEM columns: set s at 128 s: S^T (64) | dA^T (64); then the accumulators
-  static constexpr uint32_t kSetCols = 2 * kQT, kColA = kQT, kColV = 2 * kSetCols, kColK = kColV + D, kTmemCols = 512;
+  static constexpr uint32_t kSetCols = 2 * kQT, kColA = kQT, kColV = SETS * kSetCols, kColK = kColV + D, kTmemCols = 512 / kCtas;
   // at the end, over K~, V~ and the ring: the accumulators dK~ | dV~, four columns of row r at 16 (c4 kRedLd + r) bytes
   static constexpr uint32_t kRedLd = kRows + 1;
   static_assert((2 * D / 4) * kRedLd * 16 <= kOffBar, "accumulators in shared memory");
-  static_assert(2 * kSetCols + 2 * D <= 512, "TMEM budget");
-  static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+  static_assert(SETS * kSetCols + 2 * D <= kTmemCols, "TMEM budget");
+  static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "shared memory budget");
 };
 
 struct Bars {
@@ -85,12 +87,12 @@ __device__ __forceinline__ void cluster_sync_all() {
 // half write over the first 16 columns of their own 32 scores, the second half over columns [32, 48)
 __device__ __forceinline__ constexpr uint32_t pcol(int k) { return (uint32_t)((k >> 1) * 32 + (k & 1) * 8); }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int D, int SETS>
+__global__ void __launch_bounds__(kThreads, Cfg<D, SETS>::kCtas)
 bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_z,
                       const __grid_constant__ CUtensorMap tmap_kv, __nv_bfloat16* __restrict__ ws_dKV16,
                       const float* __restrict__ ws_LD, int nq, int m, float scale, int* status) {
-  using C = Cfg<D>;
+  using C = Cfg<D, SETS>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Bars* bars = reinterpret_cast<Bars*>(smem + C::kOffBar);
@@ -107,7 +109,7 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     prefetch_tmap(&tmap_kv);
     mbar_init(&bars->kv_full, 1);
     for (int s = 0; s < kStages; ++s) { mbar_init(&bars->in_full[s], 1); mbar_init(&bars->in_free[s], 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(&bars->sd_full[s], 1); mbar_init(&bars->pd_full[s], kSimtWarps * 32); }
+    for (int s = 0; s < SETS; ++s) { mbar_init(&bars->sd_full[s], 1); mbar_init(&bars->pd_full[s], kSimtWarps * 32); }
     mbar_init(&bars->acc_done, 1);
     bars->abort = 0;
     fence_mbar_init();
@@ -180,7 +182,7 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         ok = mbar_wait(&bars->in_full[s], (i / kStages) & 1, status, 503, &bars->abort);
         if (!ok) return;
         tc_fence_after();
-        const uint32_t ts = tmem + (uint32_t)(i & 1) * C::kSetCols;
+        const uint32_t ts = tmem + (uint32_t)(i % SETS) * C::kSetCols;
         const uint64_t st = (uint64_t)s * kStageStep;
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
@@ -188,15 +190,15 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
           mma_f16_ss(ts + C::kColA, vd + kstep(k, C::kKvBoxBytes), zk0 + st + kstep(k, C::kInBoxBytes), idesc_s, k != 0);
-        mma_commit(&bars->sd_full[i & 1]);
+        mma_commit(&bars->sd_full[i % SETS]);
       };
       if (ok) issue_scores(0);
-      if (ok && ntiles > 1) issue_scores(1);
+      if (SETS == 2 && ok && ntiles > 1) issue_scores(1);
       for (int i = 0; i < ntiles && ok; ++i) {
-        ok = mbar_wait(&bars->pd_full[i & 1], (i >> 1) & 1, status, 504, &bars->abort);   // P^T and dS^T are written
+        ok = mbar_wait(&bars->pd_full[i % SETS], (i / SETS) & 1, status, 504, &bars->abort);   // P^T and dS^T are written
         if (!ok) break;
         tc_fence_after();
-        const uint32_t ts = tmem + (uint32_t)(i & 1) * C::kSetCols;
+        const uint32_t ts = tmem + (uint32_t)(i % SETS) * C::kSetCols;
         const uint64_t st = (uint64_t)(i % kStages) * kStageStep;
 #pragma unroll
         for (int k = 0; k < kQT / 16; ++k) {
@@ -204,7 +206,7 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
           mma_f16_ts(tmem + C::kColK, ts + C::kColA + pcol(k), qn0 + st + (uint64_t)(k * 128), idesc_g, (i | k) != 0);
         }
         mma_commit(&bars->in_free[i % kStages]);  // the stage may be overwritten
-        if (i + 2 < ntiles) issue_scores(i + 2);
+        if (i + SETS < ntiles) issue_scores(i + SETS);
       }
       if (ok) mma_commit(&bars->acc_done);
     }
@@ -217,9 +219,9 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     const int ld_off = (int)((reinterpret_cast<uintptr_t>(reinterpret_cast<const float2*>(ws_LD) + (int64_t)bh * nq) >> 3) & 1);
     bool ok = true;
     for (int i = 0; i < ntiles && ok; ++i) {
-      const uint32_t ts = tbase + (uint32_t)(i & 1) * C::kSetCols;
+      const uint32_t ts = tbase + (uint32_t)(i % SETS) * C::kSetCols;
       // the TMEM loads and stores below are warp-wide: the whole warp gives up together
-      ok = __all_sync(0xffffffffu, mbar_wait(&bars->sd_full[i & 1], (i >> 1) & 1, status, 505, &bars->abort));
+      ok = __all_sync(0xffffffffu, mbar_wait(&bars->sd_full[i % SETS], (i / SETS) & 1, status, 505, &bars->abort));
       if (!ok) break;
       // The scores' commit follows the stage's arrival in the MMA thread's program order, but this thread reads the
       // staged L, D itself, so it observes the stage's barrier too (complete by now: no waiting).
@@ -257,7 +259,7 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&bars->pd_full[i & 1]);
+      mbar_arrive(&bars->pd_full[i % SETS]);
     }
     if (__all_sync(0xffffffffu, ok && mbar_wait(&bars->acc_done, 0, status, 506, &bars->abort) &&
                                     *(volatile int*)&bars->abort == 0)) {
@@ -306,9 +308,9 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
   if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
 }
 
-template <int D>
+template <int D, int SETS>
 cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
-  using C = Cfg<D>;
+  using C = Cfg<D, SETS>;
   const Params& p = c->p;
   CUtensorMap tq, tz;
   const uint64_t qd[3] = {(uint64_t)D, (uint64_t)p.nq, (uint64_t)(p.B * p.H)};
@@ -318,7 +320,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   if ((e = make_tmap_bf16_3d(&tq, Q, qd, qs, qb)) != cudaSuccess) return e;
   if ((e = make_tmap_bf16_3d(&tz, c->bw_dZ16, qd, qs, qb)) != cudaSuccess) return e;
   static DeviceFlags smem_opt_in;
-  if ((e = ensure_dynamic_smem(bwd_cols_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
+  if ((e = ensure_dynamic_smem(bwd_cols_sm100_kernel<D, SETS>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   // Queries per block shared out between 1, 2 or (d = 64) 4 CTAs: the fewest rounds of CTAs (one per SM) weighted with their
   // length, a CTA's start and end counted as kFixed query tiles.  Measured, us with 1 / 2 / 4: d = 64, 25 query tiles: 24
@@ -328,7 +330,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   constexpr int kFixed = 12;
   int splits = 1;
   int64_t best = 0;
-  for (int k = 1; k <= (D == 64 ? 4 : 2); k *= 2) {
+  for (int k = 1; k <= (SETS == 1 ? 1 : D == 64 ? 4 : 2); k *= 2) {
     const int64_t per = (tiles + k - 1) / k;
     if (k > 1 && (k - 1) * per >= tiles) break;   // every CTA has a tile
     const int64_t cost = (blocks * k + c->sms - 1) / c->sms * (per + kFixed);
@@ -346,7 +348,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   attr[0].val.clusterDim.z = (unsigned)splits;
   cfg.attrs = attr;
   cfg.numAttrs = splits > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, bwd_cols_sm100_kernel<D>, tq, tz, c->tmap_kv, c->bw_dKV16, (const float*)c->bw_LD, (int)p.nq, (int)p.m,
+  return cudaLaunchKernelEx(&cfg, bwd_cols_sm100_kernel<D, SETS>, tq, tz, c->tmap_kv, c->bw_dKV16, (const float*)c->bw_LD, (int)p.nq, (int)p.m,
                             scale, c->status);
 }
 
@@ -355,7 +357,10 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
 // needs dZ as bf16 (bw_dZ16), L and D (bw_LD) from the per-row stage, and K~|V~ in the workspace
 cudaError_t launch_sm100_bwd_cols(csat_ctx* c, const void* Q, cudaStream_t s, int* launches) {
   *launches += 1;
-  return c->p.d == 64 ? launch<64>(c, Q, s) : launch<128>(c, Q, s);
+  const int64_t blocks = (c->p.m + kRows - 1) / kRows * c->p.B * c->p.H;
+  // d = 64 with more blocks than SMs: one score set and two CTAs per SM (192 blocks of 25 query tiles: 61 -> 50 us)
+  if (c->p.d == 64 && blocks > c->sms) return launch<64, 1>(c, Q, s);
+  return c->p.d == 64 ? launch<64, 2>(c, Q, s) : launch<128, 2>(c, Q, s);
 }
 
 }  // namespace csat
