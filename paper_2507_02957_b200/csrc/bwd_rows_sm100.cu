@@ -19,7 +19,7 @@
 //   no transposed copy); the identity part of S^T stays exact in float32 registers;
 //   at the end dZ (bf16, the operand of the stages that follow) and D = <dZ, Z>.
 //
-// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 64 measurements:
+// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 32 measurements:
 //        S_j = Q K~_j^T,  dA_j = dZ V~_j^T                        (two SS MMAs into tensor memory)
 //        dS_j = scale * exp(scale S_j - L) o (dA_j - D)           (one thread per row; bf16 back into tensor memory)
 //        dQ  += dS_j K~_j                                         (TS MMA, K~_j read as an MN-major operand)
@@ -36,7 +36,7 @@ namespace {
 using namespace ptx;
 
 constexpr int kRows = 128;
-constexpr int kMC = 64;
+constexpr int kQC = 32;        // measurements per chunk of the dQ kernel
 
 // ====================================================================================================================
 // recurrence backward
@@ -50,23 +50,28 @@ template <int D, bool kUntied = false> struct RCfg {
   static constexpr int kMats = kUntied ? 5 : 3;                   // untied: [stage 0: S_t - I | B_t][stage 1: ...][Psi]
   static constexpr uint32_t kOffBar = kMats * kMatBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + 128 + 1024 /*alignment slack*/;
-  // TMEM columns: accumulator | dZ accumulator | two bf16 operand buffers (two values per column)
-  static constexpr uint32_t kColAcc = 0, kColDz = D, kColOp = 2 * D, kOpCols = D / 2;
-  static constexpr uint32_t kTmemCols = (D == 64) ? 256 : 512;
-  static_assert(2 * D + 2 * kOpCols <= kTmemCols, "TMEM budget");
+  // TMEM columns: accumulator | dZ accumulator, and in an allocation of their own the bf16 operand buffers (two values per
+  // column).  d = 64 has one buffer, 160 columns in all, so that three CTAs share an SM: a layer is a chain thread -> MMA issuer ->
+  // tensor pipe -> thread that uses neither the tensor pipe nor the issue slots for long (96 heads of 1568 queries, T = 20: 109 -> 84
+  // us, with the accumulator's additions, the decisions and the operand in one pass over the row instead of two).
+  static constexpr int kCtas = D == 64 ? 3 : 1, kOps = D == 64 ? 1 : 2;
+  static constexpr uint32_t kColAcc = 0, kColDz = D, kOpCols = D / 2;
+  static constexpr uint32_t kTmemCols = 2 * D, kTmemOpCols = D == 64 ? 32 : 128;
+  static_assert(kOps * kOpCols <= kTmemOpCols && kCtas * (kTmemCols + kTmemOpCols) <= 512, "TMEM budget");
+  static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
 };
 
 struct RBars {
-  uint64_t mats_full, a_full, r_full, op_free[2];
+  uint64_t mats_full, a_full, r_full, op_free[2];      // op_free: by operand buffer
   uint64_t lm_full[2], lm_free[2];   // untied layers: a stage's pair of matrices has landed / has been read
-  uint32_t tmem_slot;
+  uint32_t tmem_slot, tmem_op_slot;
   int abort;
 };
 
 constexpr int kRThreads = 160;      // warps 0-3: one thread per query row; warp 4: TMA and MMA issue
 
 template <int D, bool kUntied>
-__global__ void __launch_bounds__(kRThreads, 1)
+__global__ void __launch_bounds__(kRThreads, RCfg<D, kUntied>::kCtas)
 bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv_bfloat16* __restrict__ Z16,
                        const __nv_bfloat16* __restrict__ G, __nv_bfloat16* __restrict__ dZ16, float* __restrict__ ws_LD,
                        const uint32_t* __restrict__ maskbits, int nq, int H, int T, int has_psi, int* status,
@@ -92,12 +97,13 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
   }
   if (warp == 4) {
     tmem_alloc(&bars->tmem_slot, C::kTmemCols);
+    tmem_alloc(&bars->tmem_op_slot, C::kTmemOpCols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_slot;
+  const uint32_t tmem = bars->tmem_slot, tmem_op = bars->tmem_op_slot;
   pdl_wait();
   pdl_launch_dependents();
 
@@ -133,8 +139,8 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
       constexpr uint32_t idesc_t = make_idesc_bf16(kRows, D, false, true);    // transposed products: B MN-major
       const uint32_t acc = tmem + C::kColAcc, dz = tmem + C::kColDz;
       // product with the transpose of a matrix the forward stores [output column][k]: the tile's rows are now the
-      // reduction index, 16 rows (2048 bytes) per K step, the next 64 output columns one box further.  The operands
-      // alternate between two buffers (publication n uses buffer n & 1).
+      // reduction index, 16 rows (2048 bytes) per K step, the next 64 output columns one box further.  Publication
+      // n uses operand buffer n % kOps.
       auto mma_tr = [&](uint32_t d_t, uint32_t op, int slot, uint32_t accumulate) {
         const uint64_t bd = make_smem_desc(smem_u32(smem + C::kOffMat + slot * C::kMatBytes), C::kMatBoxBytes, 1024);
 #pragma unroll
@@ -150,14 +156,14 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
       // The threads only wait for the product they need next (r_full); the dZ product trails it and releases the
       // operand buffer (op_free) when it has read it.
       if (has_psi) {                                           // d alpha_T = G Psi
-        const uint32_t op = tmem + C::kColOp + (n_ops & 1) * C::kOpCols;
+        const uint32_t op = tmem_op + (n_ops % C::kOps) * C::kOpCols;
         operand_ready();
         mma_tr(acc, op, kUntied ? 4 : 2, 0u);
         mma_commit(&bars->r_full);
-        mma_commit(&bars->op_free[(n_ops - 1) & 1]);
+        mma_commit(&bars->op_free[(n_ops - 1) % C::kOps]);
       }
       for (int t = T - 1; t >= 0; --t) {
-        const uint32_t op = tmem + C::kColOp + (n_ops & 1) * C::kOpCols;
+        const uint32_t op = tmem_op + (n_ops % C::kOps) * C::kOpCols;
         const int li = T - 1 - t, st = li & 1;                 // untied: this layer's stage
         operand_ready();
         if (kUntied) {
@@ -171,7 +177,7 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
         }
         mma_tr(dz, op, sB, t == T - 1 ? 0u : 1u);              // dZ += dx_t B_t^T
         if (t == 0) mma_commit(&bars->r_full);                 // the last result the threads wait for is dZ itself
-        mma_commit(&bars->op_free[(n_ops - 1) & 1]);
+        mma_commit(&bars->op_free[(n_ops - 1) % C::kOps]);
         if (kUntied && t >= 2) {                               // the stage is free once these products have read it
           mma_commit(&bars->lm_free[st]);
           w.wait(&bars->lm_free[st], (li >> 1) & 1, 603);
@@ -193,26 +199,27 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
     const uint32_t acc_addr = tbase + C::kColAcc, dz_addr = tbase + C::kColDz;
     const int64_t goff = ((int64_t)bh * nq + (live ? grow : 0)) * D;
     int phase = 0;
-    uint32_t n_pub = 0;                           // operands published so far (buffer n_pub & 1)
+    uint32_t n_pub = 0;                           // operands published so far (buffer n_pub % kOps)
     float v[D];                                   // d alpha_{t+1}, then dx_t
-    // v as the bf16 A operand; with `keep` also to global memory (dx_t, for the gradients of the decoder's weights)
-    auto publish_bf16 = [&](__nv_bfloat16* keep = nullptr) {
-      const uint32_t op_addr = tbase + C::kColOp + (n_pub & 1) * C::kOpCols;
-      // the buffer's previous operand (two publications ago) has been read by its trailing product
-      if (n_pub >= 2) w.wait(&bars->op_free[n_pub & 1], ((n_pub >> 1) - 1) & 1, 613);
+    // the operand buffer of the next publication, once its previous operand has been read by the trailing product
+    auto next_operand = [&]() -> uint32_t {
+      const uint32_t buf = n_pub % C::kOps;
+      if (n_pub >= (uint32_t)C::kOps) w.wait(&bars->op_free[buf], (n_pub / C::kOps - 1) & 1, 613);
       ++n_pub;
+      return tmem_op + ((uint32_t)(warp * 32) << 16) + buf * C::kOpCols;
+    };
+    auto publish16 = [&](uint32_t op_addr, int c0, __nv_bfloat16* keep) {      // v[c0 .. c0 + 15], with `keep` also to global memory
+      uint32_t pk[8];
 #pragma unroll
-      for (int c0 = 0; c0 < D; c0 += 16) {
-        uint32_t pk[8];
-#pragma unroll
-        for (int e = 0; e < 16; e += 2) pk[e >> 1] = pack_bf16(v[c0 + e], v[c0 + e + 1]);
-        tmem_st_32x32b_x8(op_addr + c0 / 2, pk);
-        if (keep != nullptr) {
-          uint4* kp = reinterpret_cast<uint4*>(keep + c0);
-          kp[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          kp[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        }
+      for (int e = 0; e < 16; e += 2) pk[e >> 1] = pack_bf16(v[c0 + e], v[c0 + e + 1]);
+      tmem_st_32x32b_x8(op_addr + c0 / 2, pk);
+      if (keep != nullptr) {
+        uint4* kp = reinterpret_cast<uint4*>(keep + c0);
+        kp[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        kp[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
       }
+    };
+    auto published = [&]() {
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->a_full);
@@ -230,7 +237,10 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
     }
     if (T > 0) {
       if (has_psi) {
-        publish_bf16();                                         // G is bf16 already: nothing is lost
+        const uint32_t op_addr = next_operand();
+#pragma unroll
+        for (int c0 = 0; c0 < D; c0 += 16) publish16(op_addr, c0, nullptr);      // G is bf16 already: nothing is lost
+        published();
         w.wait(&bars->r_full, phase & 1, 611); ++phase;
         tc_fence_after();
 #pragma unroll
@@ -248,30 +258,50 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
 #pragma unroll
         for (int q = 0; q < D / 32; ++q) m[q] = live ? mp[q] : 0u;
       };
-      uint32_t mwd[D / 32], mnext[D / 32];
+      uint32_t mwd[D / 32];
       load_masks(T - 1, mwd);
       for (int t = T - 1; t >= 0; --t) {
-        // dx_t = d alpha_{t+1} o mask_t
+        // d alpha_{t+1} = dx_{t+1} + dx_{t+1} (S - I)^T, then dx_t = d alpha_{t+1} o mask_t, 16 columns at a time with the next
+        // ones' load in flight
+        __nv_bfloat16* keep = dx_out != nullptr && live && !w.dead ? dx_out + (int64_t)t * dx_slot + goff : nullptr;
+        auto mask16 = [&](int c0) {
 #pragma unroll
-        for (int c = 0; c < D; ++c)
-          v[c] = ((mwd[c >> 5] >> (31 - (c & 31))) & 1u) ? v[c] : 0.f;
-        publish_bf16(dx_out != nullptr && live && !w.dead ? dx_out + (int64_t)t * dx_slot + goff : nullptr);
-        if (t > 0) load_masks(t - 1, mnext);
-        w.wait(&bars->r_full, phase & 1, 612); ++phase;
-        tc_fence_after();
+          for (int e = 0; e < 16; ++e) {
+            const int c = c0 + e;
+            v[c] = ((mwd[c >> 5] >> (31 - (c & 31))) & 1u) ? v[c] : 0.f;
+          }
+        };
+        if (t == T - 1) {
+          const uint32_t op_addr = next_operand();
 #pragma unroll
-        for (int q = 0; q < D / 32; ++q) mwd[q] = mnext[q];
-        if (t > 0) {
+          for (int c0 = 0; c0 < D; c0 += 16) { mask16(c0); publish16(op_addr, c0, keep); }
+        } else {
+          w.wait(&bars->r_full, phase & 1, 612); ++phase;
+          tc_fence_after();
+          uint32_t r0[16], r1[16];
+          tmem_ld_32x32b_x16(acc_addr, r0);
+          const uint32_t op_addr = next_operand();
+          auto piece = [&](const uint32_t (&r)[16], int c0) {
 #pragma unroll
-          for (int c0 = 0; c0 < D; c0 += 16) {
-            uint32_t r[16];
-            tmem_ld_32x32b_x16(acc_addr + c0, r);
+            for (int e = 0; e < 16; ++e) v[c0 + e] += __uint_as_float(r[e]);
+            mask16(c0);
+            publish16(op_addr, c0, keep);
+          };
+#pragma unroll
+          for (int c0 = 0; c0 < D; c0 += 32) {
             tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 16; ++e) v[c0 + e] += __uint_as_float(r[e]);        // d alpha_t = dx_t + dx_t (S - I)^T
+            tmem_ld_32x32b_x16(acc_addr + c0 + 16, r1);
+            piece(r0, c0);
+            tmem_wait_ld();
+            if (c0 + 32 < D) tmem_ld_32x32b_x16(acc_addr + c0 + 32, r0);
+            piece(r1, c0 + 16);
           }
         }
+        published();
+        if (t > 0) load_masks(t - 1, mwd);
       }
+      w.wait(&bars->r_full, phase & 1, 614); ++phase;           // the last result is dZ itself
+      tc_fence_after();
     }
     // ---- dZ (the accumulated products; G itself without a decoder) and D = <dZ, Z> ----
     float dsum = 0.f;
@@ -304,25 +334,33 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) tmem_dealloc(tmem, C::kTmemCols);
+  if (warp == 4) {
+    tmem_dealloc(tmem, C::kTmemCols);
+    tmem_dealloc(tmem_op, C::kTmemOpCols);
+  }
 }
 
 // ====================================================================================================================
 // dQ
 // ====================================================================================================================
+// Chunks of 32 measurements: with 64, S and dA in two buffers each and dQ took 512 columns of tensor memory and held one tile of
+// 128 queries per SM.  d = 64: 128 columns (one buffer), three tiles per SM: 47 -> 38 us for 96 heads of 1568
+// queries, m = 256; d = 128: 256 columns (two buffers), two tiles.
 template <int D> struct QCfg {
   static constexpr int kDBoxes = D / 64;
-  static constexpr int kStages = 3;
+  static constexpr int kCtas = D == 64 ? 3 : 2;                     // per SM
+  static constexpr int kStages = 3, kBufs = D == 64 ? 1 : 2;
   static constexpr uint32_t kTileBoxBytes = kRows * 128;            // 128 rows x 64 columns
   static constexpr uint32_t kTileBytes = kDBoxes * kTileBoxBytes;   // Q tile, dZ tile
-  static constexpr uint32_t kBoxBytes = kMC * 128;                  // one 64-column box of a K~ or V~ chunk
+  static constexpr uint32_t kBoxBytes = kQC * 128;                  // one 64-column box of a K~ or V~ chunk
   static constexpr uint32_t kSlotBytes = kDBoxes * kBoxBytes;
   static constexpr uint32_t kOffQ = 0, kOffZ = kTileBytes, kOffRing = 2 * kTileBytes;   // ring: [stage][K~ slot | V~ slot]
   static constexpr uint32_t kOffBar = kOffRing + kStages * 2 * kSlotBytes;
-  static constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024 /*alignment slack*/;
-  // TMEM columns: S[2] | dA[2] | dQ accumulator; dS_j (bf16) overlays the first half of S[j & 1]
-  static constexpr uint32_t kColS = 0, kColA = 2 * kMC, kColQ = 4 * kMC, kTmemCols = 512;
-  static_assert(4 * kMC + D <= 512, "TMEM budget");
+  static constexpr uint32_t kSmemBytes = kOffBar + 256;             // base must be 1024-byte aligned (checked)
+  // TMEM columns: S[bufs] | dA[bufs] | dQ accumulator; dS_j (bf16) overlays the first half of S[j % bufs]
+  static constexpr uint32_t kColS = 0, kColA = kBufs * kQC, kColQ = 2 * kBufs * kQC, kTmemCols = D == 64 ? 128 : 256;
+  static_assert(kColQ + D <= kTmemCols && kCtas * kTmemCols <= 512, "TMEM budget");
+  static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
 };
 
 struct QBars {
@@ -334,17 +372,20 @@ struct QBars {
 constexpr int kQThreads = 192;      // warps 0-3: one thread per query row; warp 4: TMA; warp 5: MMA issue
 
 template <int D>
-__global__ void __launch_bounds__(kQThreads, 1)
+__global__ void __launch_bounds__(kQThreads, QCfg<D>::kCtas)
 bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_z,
                     const __grid_constant__ CUtensorMap tmap_kv, __nv_bfloat16* __restrict__ dQ,
                     const float* __restrict__ ws_LD, int nq, int m, float scale, int* status) {
   using C = QCfg<D>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];
+  if ((smem_u32(smem) & 1023u) != 0) {          // swizzled tiles need 1024-byte alignment; never seen to fail
+    if (threadIdx.x == 0) atomicCAS(status, 0, 700);
+    return;
+  }
   QBars* bars = reinterpret_cast<QBars*>(smem + C::kOffBar);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.y, row0 = blockIdx.x * kRows;
-  const int nchunks = (m + kMC - 1) / kMC;
+  const int nchunks = (m + kQC - 1) / kQC;
   Waiter w{status, &bars->abort};
   auto k_slot = [&](int s) { return smem + C::kOffRing + (2 * s) * C::kSlotBytes; };
   auto v_slot = [&](int s) { return smem + C::kOffRing + (2 * s + 1) * C::kSlotBytes; };
@@ -355,7 +396,7 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
     prefetch_tmap(&tmap_kv);
     mbar_init(&bars->qz_full, 1);
     for (int s = 0; s < C::kStages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&bars->s_full[b], 1); mbar_init(&bars->p_full[b], kRows); }
+    for (int b = 0; b < C::kBufs; ++b) { mbar_init(&bars->s_full[b], 1); mbar_init(&bars->p_full[b], kRows); }
     mbar_init(&bars->acc_done, 1);
     bars->abort = 0;
     fence_mbar_init();
@@ -385,8 +426,8 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
         if (w.dead) break;
         mbar_arrive_expect_tx(&bars->full[s], 2 * C::kSlotBytes);
         for (int gx = 0; gx < C::kDBoxes; ++gx) {
-          tma_load_3d(k_slot(s) + gx * C::kBoxBytes, &tmap_kv, &bars->full[s], gx * 64, j * kMC, bh);
-          tma_load_3d(v_slot(s) + gx * C::kBoxBytes, &tmap_kv, &bars->full[s], D + gx * 64, j * kMC, bh);
+          tma_load_3d(k_slot(s) + gx * C::kBoxBytes, &tmap_kv, &bars->full[s], gx * 64, j * kQC, bh);
+          tma_load_3d(v_slot(s) + gx * C::kBoxBytes, &tmap_kv, &bars->full[s], D + gx * 64, j * kQC, bh);
         }
         ++issued;
       }
@@ -398,39 +439,40 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
     }
   } else if (warp == 5) {
     if (elect_one()) {
-      constexpr uint32_t idesc_s = make_idesc_bf16(kRows, kMC, false, false);   // S, dA: both operands K-major
+      constexpr uint32_t idesc_s = make_idesc_bf16(kRows, kQC, false, false);   // S, dA: both operands K-major
       constexpr uint32_t idesc_q = make_idesc_bf16(kRows, D, false, true);      // dQ += dS K~: K~ is MN-major
       auto kstep = [](int k, uint32_t box_bytes) { return (uint64_t)((k / 4) * (box_bytes >> 4) + (k % 4) * 2); };
       const uint64_t qd = make_smem_desc(smem_u32(smem + C::kOffQ), 16, 1024);
       const uint64_t zd = make_smem_desc(smem_u32(smem + C::kOffZ), 16, 1024);
       auto issue_sd = [&](int j) {
-        const int s = j % C::kStages, b = j & 1;
+        const int s = j % C::kStages, b = j % C::kBufs;
         w.wait(&bars->full[s], (j / C::kStages) & 1, 711);
         tc_fence_after();
         const uint64_t kd = make_smem_desc(smem_u32(k_slot(s)), 16, 1024);
         const uint64_t vd = make_smem_desc(smem_u32(v_slot(s)), 16, 1024);
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
-          mma_f16_ss(tmem + C::kColS + b * kMC, qd + kstep(k, C::kTileBoxBytes), kd + kstep(k, C::kBoxBytes), idesc_s, k != 0);
+          mma_f16_ss(tmem + C::kColS + b * kQC, qd + kstep(k, C::kTileBoxBytes), kd + kstep(k, C::kBoxBytes), idesc_s, k != 0);
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
-          mma_f16_ss(tmem + C::kColA + b * kMC, zd + kstep(k, C::kTileBoxBytes), vd + kstep(k, C::kBoxBytes), idesc_s, k != 0);
+          mma_f16_ss(tmem + C::kColA + b * kQC, zd + kstep(k, C::kTileBoxBytes), vd + kstep(k, C::kBoxBytes), idesc_s, k != 0);
         mma_commit(&bars->s_full[b]);
       };
       w.wait(&bars->qz_full, 0, 710);
       issue_sd(0);
       for (int j = 0; j < nchunks; ++j) {
-        // S_{j+1}, dA_{j+1} run while the threads work on chunk j; they overwrite the buffers dS_{j-1} was read from
-        // by the dQ product of chunk j-1, which was issued earlier and therefore executes first
-        if (j + 1 < nchunks) issue_sd(j + 1);
-        const int s = j % C::kStages, b = j & 1;
-        w.wait(&bars->p_full[b], (j >> 1) & 1, 712);
+        // Two buffers: S_{j+1}, dA_{j+1} run while the threads work on chunk j; they overwrite what the dQ product of chunk j - 1
+        // read dS_{j-1} from, which was issued earlier and therefore executes first.  One buffer: they follow chunk j's.
+        if (C::kBufs == 2 && j + 1 < nchunks) issue_sd(j + 1);
+        const int s = j % C::kStages, b = j % C::kBufs;
+        w.wait(&bars->p_full[b], (j / C::kBufs) & 1, 712);
         tc_fence_after();
         const uint64_t kd = make_smem_desc(smem_u32(k_slot(s)), C::kBoxBytes, 1024);      // MN-major: rows = reduction
 #pragma unroll
-        for (int k = 0; k < kMC / 16; ++k)
-          mma_f16_ts(tmem + C::kColQ, tmem + C::kColS + b * kMC + k * 8, kd + (uint64_t)(k * 128), idesc_q, (uint32_t)((j | k) != 0));
+        for (int k = 0; k < kQC / 16; ++k)
+          mma_f16_ts(tmem + C::kColQ, tmem + C::kColS + b * kQC + k * 8, kd + (uint64_t)(k * 128), idesc_q, (uint32_t)((j | k) != 0));
         mma_commit(&bars->empty[s]);
+        if (C::kBufs == 1 && j + 1 < nchunks) issue_sd(j + 1);
       }
       mma_commit(&bars->acc_done);
     }
@@ -443,33 +485,23 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
     const float Dv = live ? ws_LD[((int64_t)bh * nq + grow) * 2 + 1] : 0.f;
     const float scale_log2 = scale * l2e;
     for (int j = 0; j < nchunks; ++j) {
-      const int b = j & 1;
-      w.wait(&bars->s_full[b], (j >> 1) & 1, 720);
+      const int b = j % C::kBufs;
+      w.wait(&bars->s_full[b], (j / C::kBufs) & 1, 720);
       tc_fence_after();
+      uint32_t sv[32], av[32];
+      tmem_ld_32x32b_x32(tbase + C::kColS + b * kQC, sv);
+      tmem_ld_32x32b_x32(tbase + C::kColA + b * kQC, av);
+      tmem_wait_ld();
+      uint32_t pk[16];
 #pragma unroll
-      for (int hlf = 0; hlf < 2; ++hlf) {
-        uint32_t sv[32], av[32];
-        tmem_ld_32x32b_x32(tbase + C::kColS + b * kMC + hlf * 32, sv);
-        tmem_ld_32x32b_x32(tbase + C::kColA + b * kMC + hlf * 32, av);
-        tmem_wait_ld();
-        uint32_t pk[16];
-#pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          const float p0 = ex2(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
-          const float p1 = ex2(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
-          const float d0 = live ? scale * p0 * (__uint_as_float(av[e]) - Dv) : 0.f;
-          const float d1 = live ? scale * p1 * (__uint_as_float(av[e + 1]) - Dv) : 0.f;
-          pk[e >> 1] = pack_bf16(d0, d1);
-        }
-        // dS over the first 32 columns of S[b]: the first half's 16 packed columns are written after both of its
-        // S columns groups ... the second half's S columns (32..63) are read before columns 16..31 are overwritten
-        if (hlf == 0) {
-          // columns 0..15 of S[b] hold scores this thread has already read (they are in sv)
-          tmem_st_32x32b_x16(tbase + C::kColS + b * kMC, pk);
-        } else {
-          tmem_st_32x32b_x16(tbase + C::kColS + b * kMC + 16, pk);
-        }
+      for (int e = 0; e < 32; e += 2) {
+        const float p0 = ex2(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
+        const float p1 = ex2(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
+        const float d0 = live ? scale * p0 * (__uint_as_float(av[e]) - Dv) : 0.f;
+        const float d1 = live ? scale * p1 * (__uint_as_float(av[e + 1]) - Dv) : 0.f;
+        pk[e >> 1] = pack_bf16(d0, d1);
       }
+      tmem_st_32x32b_x16(tbase + C::kColS + b * kQC, pk);       // dS over the first half of S[b]
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->p_full[b]);
@@ -527,7 +559,7 @@ cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
   if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD,
+  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, c->tmap_kv_st, (__nv_bfloat16*)dQ, c->bw_LD,
                     (int)p.nq, (int)p.m, scale, c->status);
 }
 
