@@ -88,7 +88,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                    const __grid_constant__ CUtensorMap tmap_mats, const __grid_constant__ CUtensorMap tmap_out,
                    const __grid_constant__ CUtensorMap tmap_vb, const Args p) {
   constexpr bool kUnit = kDec == kUnits || kDec == kFolded, kUntied = kDec == kPerLayer, kFold = kDec == kFolded;
-  constexpr bool kMasks = kRec >= 1, kKeep = kRec >= 2, kStaged = kRec == 0;
+  constexpr bool kMasks = kRec >= 1, kKeep = kRec >= 2, kStaged = kDec != kPerLayer;     // kStaged: Z's way out, through a stage of the ring
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {          // swizzled tiles need 1024-byte alignment; never seen to fail
     if (threadIdx.x == 0) atomicCAS(p.status, 0, 240);
@@ -106,7 +106,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     prefetch_tmap(&tmap_q);
     prefetch_tmap(&tmap_kv);
     prefetch_tmap(&tmap_mats);
-    if (kStaged) prefetch_tmap(&tmap_out);
+    prefetch_tmap(&tmap_out);
     mbar_init(&bars->q_full, 1);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->k_full[s], 1);
@@ -401,14 +401,38 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
       for (int e = 0; e < 16; e += 2) v2[(c0 + e) >> 1] = mul2(pack2u(a[e], a[e + 1]), inv2);
     }
   }
-  if (kMasks && p.z != nullptr && grow < nq) {
-    uint4* zo = reinterpret_cast<uint4*>(p.z + ((int64_t)bh * nq + grow) * kD);
+  // v2 as bf16 into one box of the warp's 32 rows (128-byte swizzle), from where one TMA store takes it: 16-byte stores of 32
+  // different rows would keep the threads at the stores
+  auto stage_rows = [&](uint8_t* buf, const CUtensorMap* map) {
+    uint8_t* box = buf + warp * kOutBytes;
 #pragma unroll
-    for (int c = 0; c < kD / 8; ++c) {
+    for (int c = 0; c < 8; ++c) {
       float x[8];
 #pragma unroll
       for (int u = 0; u < 4; ++u) unpack2(v2[c * 4 + u], x[2 * u], x[2 * u + 1]);
-      zo[c] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+      *reinterpret_cast<uint4*>(box + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+          make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+    }
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0 && live && !w.dead && *(volatile int*)&bars->abort == 0) {
+      tma_store_3d(map, box, 0, grow, bh);
+      bulk_commit_group();
+    }
+  };
+  if (kMasks && p.z != nullptr) {
+    if (kStaged) {
+      // every chunk has been read: the ring is free
+      stage_rows(ring, &tmap_vb);
+    } else if (grow < nq) {
+      uint4* zo = reinterpret_cast<uint4*>(p.z + ((int64_t)bh * nq + grow) * kD);
+#pragma unroll
+      for (int c = 0; c < kD / 8; ++c) {
+        float x[8];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) unpack2(v2[c * 4 + u], x[2 * u], x[2 * u + 1]);
+        zo[c] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+      }
     }
   }
   __nv_bfloat16* arow = (kKeep && p.alpha != nullptr && grow < nq) ? p.alpha + ((int64_t)bh * nq + grow) * kD : nullptr;
@@ -693,36 +717,9 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
       });
     }
   }
-  const bool ok = !w.dead && *(volatile int*)&bars->abort == 0;
-  if (kStaged && p.out != nullptr) {
-    // every MMA of the tile is done: Q's buffer (-mu G's) takes the output, the warp's 32 rows as one box
-    uint8_t* box = smem + warp * kOutBytes;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      float x[8];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) unpack2(v2[c * 4 + u], x[2 * u], x[2 * u + 1]);
-      *reinterpret_cast<uint4*>(box + lane * 128 + ((c ^ (lane & 7)) << 4)) =
-          make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-    }
-    fence_proxy_async();
-    __syncwarp();
-    if (lane == 0 && live && ok) {
-      tma_store_3d(&tmap_out, box, 0, grow, bh);
-      bulk_commit_group();
-      bulk_wait_group0();
-    }
-  }
-  if (!kStaged && p.out != nullptr && grow < nq && ok) {
-    uint4* o = reinterpret_cast<uint4*>(p.out + ((int64_t)bh * nq + grow) * kD);
-#pragma unroll
-    for (int c = 0; c < kD / 8; ++c) {
-      float x[8];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) unpack2(v2[c * 4 + u], x[2 * u], x[2 * u + 1]);
-      o[c] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-    }
-  }
+  // every MMA of the tile is done: Q's place (or Psi's) takes the output
+  if (p.out != nullptr) stage_rows(smem, &tmap_out);
+  if (lane == 0) bulk_wait_group0();                          // the stores are done before the kernel ends
   }
   tc_fence_before();
   __syncthreads();
@@ -740,7 +737,9 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   cudaError_t e;
   if ((e = make_tmap_bf16_3d(&tq, Q, qd, qs, qb)) != cudaSuccess) return e;
   CUtensorMap to = tq;
-  if (kRec == 0 && out != nullptr && (e = make_tmap_bf16_3d(&to, out, qd, qs, ob)) != cudaSuccess) return e;
+  if (out != nullptr && (e = make_tmap_bf16_3d(&to, out, qd, qs, ob)) != cudaSuccess) return e;
+  CUtensorMap tv = c->tmap_vb;                                  // V~ B, or with kRec where Z goes
+  if (kRec != 0 && z != nullptr && (e = make_tmap_bf16_3d(&tv, z, qd, qs, ob)) != cudaSuccess) return e;
   // Up to one or two tiles per SM the CTAs ask for so much shared memory that no more share an SM: started early, they would
   // pile up on the SMs that the kernel before leaves free.
   const int64_t tiles = (p.nq + kRows - 1) / kRows, n = tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
@@ -761,7 +760,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
          (int64_t)(p.B * p.H * p.nq * p.d), alpha != nullptr ? c->bw_signbits : nullptr, wait_first,
          !c->w_S && p.step == 0.0 && p.T <= 1024};
   return launch_pdl(attend_tile_kernel<kRec, kDec, kBufs>, dim3((unsigned)n), kThreads, smem, s, tq, c->tmap_kv,
-                    kDec == kPerLayer ? c->tmap_lmats : c->tmap_mats, to, c->tmap_vb, a);
+                    kDec == kPerLayer ? c->tmap_lmats : c->tmap_mats, to, tv, a);
 }
 
 }  // namespace

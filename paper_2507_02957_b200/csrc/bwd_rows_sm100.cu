@@ -283,7 +283,11 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
           const uint32_t op_addr = next_operand();
           auto piece = [&](const uint32_t (&r)[16], int c0) {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) v[c0 + e] += __uint_as_float(r[e]);
+            for (int e = 0; e < 16; e += 2) {
+              const float2 x = __fadd2_rn(make_float2(v[c0 + e], v[c0 + e + 1]), make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])));
+              v[c0 + e] = x.x;
+              v[c0 + e + 1] = x.y;
+            }
             mask16(c0);
             publish16(op_addr, c0, keep);
           };
