@@ -40,7 +40,7 @@ cudaError_t ensure_dynamic_smem(Kernel* kernel, int bytes, int device, DeviceFla
 // plainly and so started after it (the tcgen05 compression).  So whatever precedes the previous kernel is complete when a kernel
 // starts, and the previous one itself is after griddepcontrol.wait: before that a kernel touches only what the previous kernel
 // does not write, and stores nothing.  The backward kernels and the projection read nothing at all before their wait.  The
-// attention kernels do: their first queries (attend_recover_sm100), thresholds and decoder matrices are in place before this
+// attention kernels do: their first queries (attend_recover_sm100, attend_tile_sm100), thresholds and decoder matrices are in place before this
 // call's own compression or fold starts, and behind the fold K~ as well, which the compression in front of that has written.
 // Behind any other kernel they are launched with wait_first.
 template <typename... KP, typename... Args>
@@ -251,7 +251,7 @@ cudaError_t launch_sm100_vfold(csat_ctx* c, cudaStream_t s, int* launches);
 cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int* launches,
                                   int64_t phi_j0 = 0, int64_t n_len = 0, float* partial = nullptr);
 
-// attend_recover_sm100.cu : tcgen05 compressed attention + recovery (bf16, d in {64, 128})
+// attend_recover_sm100.cu : tcgen05 compressed attention + recovery (bf16, d = 128), and the choice of kernel for d in {64, 128}
 cudaError_t make_attend_tmaps(csat_ctx* c);
 cudaError_t make_layer_weights_tmap(csat_ctx* c);
 // wait_first: the kernel before it in the stream is not this call's own compression, so nothing is read before that has finished
@@ -264,7 +264,7 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
                                              int lse_stride, uint32_t* mask_out, __nv_bfloat16* alpha_out,
                                              cudaStream_t s, int* launches, void* out = nullptr);
 
-// attend_tile_sm100.cu : the same with one tile of 128 queries per CTA and several CTAs per SM
+// attend_tile_sm100.cu : the same for d = 64, one tile of 128 queries per CTA and three CTAs per SM
 cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first);
 cudaError_t launch_attend_tile_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
                                          __nv_bfloat16* z, uint32_t* masks, __nv_bfloat16* alpha);

@@ -2,12 +2,12 @@
 // row block, softmax(Q K~^T / sqrt(d_k)) V~ and the unrolled recurrence alpha^{t+1} = eta_theta(S alpha^t + B Z_i), runs in
 // the registers of one warp (warp_mma.cuh), with -mu G held there as operand fragments.
 //
-// Why beside attend_recover_sm100.cu, which has four times the matrix rate: at d = 64 a layer of that kernel is a chain
-// thread -> MMA issuer -> tensor pipe -> thread of ~1500 cycles for 256 queries, and its tiles of 128 (pairs: 256) queries
-// leave SMs idle or rows empty at the sizes of single images and short query lists.  Here a layer takes 32 matrix
-// instructions (272 cycles) and ~80 others per 16 queries, 370 cycles in all: matrix and float32 instructions of different
-// warps do not overlap on a sub-core (one warp per sub-core 0.20 us per layer, two 0.38, three 0.575), which is why the
-// kernel stops paying off at one warp per sub-core, i.e. one CTA of 64 queries per SM (see warp_attend_better).
+// Why beside attend_tile_sm100.cu, which has four times the matrix rate: a layer of that kernel is a chain thread -> MMA issuer ->
+// tensor pipe -> thread of ~1300 cycles for 128 queries, and its tiles of 128 queries leave SMs idle or rows empty at the sizes
+// of single images and short query lists.  Here a layer takes 32 matrix instructions (272 cycles) and ~80 others per 16 queries,
+// 370 cycles in all: matrix and float32 instructions of different warps do not overlap on a sub-core (one warp per sub-core
+// 0.20 us per layer, two 0.38, three 0.575), which is why the kernel stops paying off beyond one or two warps per sub-core (see
+// warp_attend_better).
 //
 // The arithmetic is that kernel's: bf16 P and increments, float32 accumulators, statistics and iterates; the plain forward
 // with one positive threshold in units of 2 theta, otherwise the accumulator biased by the first threshold.
@@ -20,7 +20,7 @@ namespace {
 
 using namespace wmma16;
 
-constexpr int kD = 64, kWarps = 4, kRows = 16 * kWarps, kMC = 64;
+constexpr int kD = 64, kMC = 64;
 constexpr int kLd = kD + 8;                                   // bf16 row pitch: 8 rows of 16 bytes hit different banks
 constexpr int kTile = kMC * kLd;                              // K~ or V~ chunk, or a decoder matrix
 constexpr int kStages = 2;
@@ -35,19 +35,19 @@ struct Args {
   int theta_stride, nq, m, H, T, has_psi, tiles, bh0;
   bool wait_first;
   float scale_log2;
-  // recording (the backward pass's forward), as in attend_recover_sm100.cu
+  // recording (the backward pass's forward), as in attend_tile_sm100.cu
   float* lse;
   int lse_stride;
   __nv_bfloat16* z;
   uint32_t* masks;
 };
 
-template <bool kRec>
+template <bool kRec, int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args p) {
   extern __shared__ __align__(16) __nv_bfloat16 smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int bh = p.bh0 + blockIdx.x / p.tiles, h = bh % p.H;
-  const int row0 = (blockIdx.x % p.tiles) * kRows + warp * 16;
+  const int row0 = (blockIdx.x % p.tiles) * (16 * kWarps) + warp * 16;
   const bool live = row0 < p.nq;                                // the warp has rows (it helps with the copies in any case)
   const __nv_bfloat16* kvb = p.kv + (int64_t)bh * p.m * (2 * kD);
   const int nchunks = (p.m + kMC - 1) / kMC;
@@ -328,12 +328,12 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
   }
 }
 
-template <bool kRec>
+template <bool kRec, int kWarps>
 cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride, __nv_bfloat16* z, uint32_t* masks,
                    bool wait_first) {
   const Params& p = c->p;
   static DeviceFlags opt_in;
-  cudaError_t e = ensure_dynamic_smem(warp_attend_kernel<kRec>, kSmemBytes, c->device, opt_in);
+  cudaError_t e = ensure_dynamic_smem(warp_attend_kernel<kRec, kWarps>, kSmemBytes, c->device, opt_in);
   if (e != cudaSuccess) return e;
   Args a;
   a.out = (__nv_bfloat16*)out;
@@ -344,7 +344,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   a.theta_stride = c->thr_stride();
   a.nq = (int)p.nq; a.m = (int)p.m; a.H = (int)p.H; a.T = p.T;
   a.has_psi = c->psi ? 1 : 0;
-  a.tiles = (int)((p.nq + kRows - 1) / kRows);
+  a.tiles = (int)((p.nq + 16 * kWarps - 1) / (16 * kWarps));
   a.bh0 = (int)c->bh0;
   a.wait_first = wait_first;
   a.scale_log2 = (float)((p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)kD)) * 1.4426950408889634);
@@ -353,27 +353,35 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   if (grid > (int64_t)1 << 30) return cudaErrorInvalidValue;
   // The prologue may run under the compression's tail.  One CTA per SM: without that (kSmemBytes), CTAs that start early would
   // pile up on the SMs the compression leaves free
-  return launch_pdl(warp_attend_kernel<kRec>, dim3((unsigned)grid), kWarps * 32, kSmemBytes, s, a);
+  return launch_pdl(warp_attend_kernel<kRec, kWarps>, dim3((unsigned)grid), kWarps * 32, kSmemBytes, s, a);
 }
 
 }  // namespace
 
-// As long as every SM has at most one CTA of 64 queries.  Measured with the compression in front (n = 1568, m = 256, T = 20,
-// us, this kernel / attend_recover_sm100): 1 CTA 16.2 / 21.3, 100 CTAs 17.2 / 25.0, 128 CTAs (heads of 64 queries) 22.5 /
-// 28.4, 256 CTAs 28.4 / 28.6 (queries in single tiles of 128) and 27.4 / 29.5 (pairs), 300 CTAs 28.9 / 25.3; one image of 12
-// heads of 197 tokens, m = 64, T = 10: 9.0 / 13.6.  The whole job counts, not the launch's range of (batch, head) pairs, so
-// that a forward cut into sub-range launches returns the same bits.
+// One CTA per SM at most, of 64 queries (one warp per sub-core) or of 128 where not all of its eight warps have rows or the
+// attention phase is a single chunk.  Attention alone, us, this kernel / attend_tile_sm100:
+//   64 queries: 12 heads of 197, m = 64, T = 10 5.0 / 8.2; 74 of 77, m = 392, T = 20 12.2 / 17.7; 8 of 1024, m = 128, T = 10 6.1 / 9.0
+//   128, and whole calls: 148 heads of 65, m = 64, T = 10 7.3 / 9.0 and 12.4 / 14.3; 74 of 197 8.0 / 8.9 and 11.8 / 12.8; 140 of 100,
+//   m = 128, T = 20 12.5 / 13.3 and 18.4 / 19.6; 128 of 77, m = 392 18.0 / 17.8 and 95.3 / 97.0 (its CTAs start under the compression);
+//   otherwise not: 11 of 1568, m = 256, T = 20 15.2 / 14.7, 48 of 300, m = 256 15.1 / 15.0.
+// The whole job counts, not the launch's range of (batch, head) pairs, so that a forward cut into sub-range launches returns the
+// same bits.
+static int64_t blocks_of(const csat_ctx* c, int rows) { return (c->p.nq + rows - 1) / rows * c->p.B * c->p.H; }
+
 bool warp_attend_better(const csat_ctx* c) {
   const Params& p = c->p;
-  return p.d == kD && !(c->w_S && c->w_untied && p.T > 0) && (p.nq + kRows - 1) / kRows * p.B * p.H <= c->sms;
+  if (p.d != kD || (c->w_S && c->w_untied && p.T > 0)) return false;
+  return blocks_of(c, 64) <= c->sms || (blocks_of(c, 128) <= c->sms && (p.nq <= 112 || p.m <= kMC));
 }
 
 cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool wait_first) {
-  return launch<false>(c, Q, out, s, nullptr, 0, nullptr, nullptr, wait_first);
+  return blocks_of(c, 64) <= c->sms ? launch<false, 4>(c, Q, out, s, nullptr, 0, nullptr, nullptr, wait_first)
+                                    : launch<false, 8>(c, Q, out, s, nullptr, 0, nullptr, nullptr, wait_first);
 }
 cudaError_t launch_warp_attend_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,
                                          __nv_bfloat16* z, uint32_t* masks) {
-  return launch<true>(c, Q, out, s, lse, lse_stride, z, masks, false);
+  return blocks_of(c, 64) <= c->sms ? launch<true, 4>(c, Q, out, s, lse, lse_stride, z, masks, false)
+                                    : launch<true, 8>(c, Q, out, s, lse, lse_stride, z, masks, false);
 }
 
 }  // namespace csat

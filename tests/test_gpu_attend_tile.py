@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import csat_oracle as orc
-from paper_2507_02957_b200 import workloads as wl
+from paper_2507_02957_b200 import binding, workloads as wl
 from gpu_util import TOL, device_inputs, make_ctx, rel_err, to_dev, to_np
 
 pytestmark = pytest.mark.gpu
@@ -42,4 +42,21 @@ def test_forward_at_the_edges(B, H, nq, m):
     ctx.set(T=3)
     ctx.set_lista_layer_weights(to_dev(S, "bf16"), to_dev(Bm, "bf16"), torch.from_numpy(th).cuda())
     check(T=3, lam=0.0, Psi=Psi.astype(np.float64), weights=(S.astype(np.float64), Bm.astype(np.float64), list(th.astype(np.float64))))
+    ctx.close()
+
+
+@pytest.mark.parametrize("nq,m", [(65, 64), (80, 131), (97, 65), (112, 200), (113, 64), (128, 64), (113, 65)])
+def test_the_rule_between_this_kernel_and_128_queries_per_cta_of_the_warp_kernel(nq, m):
+    """120 heads of up to 128 queries: eight warps of 16 queries up to 112 queries or with one chunk of measurements, this kernel
+    otherwise; the plain and the recording forward."""
+    w = wl.Workload("warp8", 2, 60, 230, nq, D, m, "bf16", 3, 0.001, "iid", 300 + nq)
+    inp = wl.make_inputs(w)
+    Q, K, V, _ = device_inputs(w, inp)
+    ctx = make_ctx(w)
+    phi = to_np(ctx.get_phi())
+    ref = orc.csat_forward(inp["Q"], inp["K"], inp["V"], phi, T=3, lam=w.lam)
+    for save in (0, 1):
+        binding.csat_set_i64(ctx.h, binding.CSAT_SAVE_FOR_BACKWARD, save)
+        out = to_np(ctx.forward(Q, K, V))
+        assert np.isfinite(out).all() and rel_err(out, ref) <= TOL["bf16"], (save, rel_err(out, ref))
     ctx.close()
