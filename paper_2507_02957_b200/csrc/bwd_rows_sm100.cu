@@ -19,7 +19,7 @@
 //   no transposed copy); the identity part of S^T stays exact in float32 registers;
 //   at the end dZ (bf16, the operand of the stages that follow) and D = <dZ, Z>.
 //
-// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 32 measurements:
+// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 32 (d = 64) or 64 measurements:
 //        S_j = Q K~_j^T,  dA_j = dZ V~_j^T                        (two SS MMAs into tensor memory)
 //        dS_j = scale * exp(scale S_j - L) o (dA_j - D)           (one thread per row; bf16 back into tensor memory)
 //        dQ  += dS_j K~_j                                         (TS MMA, K~_j read as an MN-major operand)
@@ -36,7 +36,6 @@ namespace {
 using namespace ptx;
 
 constexpr int kRows = 128;
-constexpr int kQC = 32;        // measurements per chunk of the dQ kernel
 
 // ====================================================================================================================
 // recurrence backward
@@ -347,12 +346,14 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
 // ====================================================================================================================
 // dQ
 // ====================================================================================================================
-// Chunks of 32 measurements: with 64, S and dA in two buffers each and dQ took 512 columns of tensor memory and held one tile of
-// 128 queries per SM.  d = 64: 128 columns (one buffer), three tiles per SM: 47 -> 38 us for 96 heads of 1568
-// queries, m = 256; d = 128: 256 columns (two buffers), two tiles.
+// d = 64: chunks of 32 measurements, so that S, dA (one buffer each) and dQ take 128 columns of tensor memory and three tiles of 128
+// queries share an SM, where chunks of 64 in two buffers (512 columns allocated) left room for one: 47 -> 38 us for 96 heads of 1568
+// queries, m = 256.  d = 128: chunks of 64, two buffers, one tile (with chunks of 32 and two tiles per SM 16 heads of 8192, m = 512
+// take 82 us instead of 79).
 template <int D> struct QCfg {
   static constexpr int kDBoxes = D / 64;
-  static constexpr int kCtas = D == 64 ? 3 : 2;                     // per SM
+  static constexpr int kQC = D == 64 ? 32 : 64;                     // measurements per chunk
+  static constexpr int kCtas = D == 64 ? 3 : 1;                     // per SM
   static constexpr int kStages = 3, kBufs = D == 64 ? 1 : 2;
   static constexpr uint32_t kTileBoxBytes = kRows * 128;            // 128 rows x 64 columns
   static constexpr uint32_t kTileBytes = kDBoxes * kTileBoxBytes;   // Q tile, dZ tile
@@ -362,7 +363,7 @@ template <int D> struct QCfg {
   static constexpr uint32_t kOffBar = kOffRing + kStages * 2 * kSlotBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + 256;             // base must be 1024-byte aligned (checked)
   // TMEM columns: S[bufs] | dA[bufs] | dQ accumulator; dS_j (bf16) overlays the first half of S[j % bufs]
-  static constexpr uint32_t kColS = 0, kColA = kBufs * kQC, kColQ = 2 * kBufs * kQC, kTmemCols = D == 64 ? 128 : 256;
+  static constexpr uint32_t kColS = 0, kColA = kBufs * kQC, kColQ = 2 * kBufs * kQC, kTmemCols = D == 64 ? 128 : 512;
   static_assert(kColQ + D <= kTmemCols && kCtas * kTmemCols <= 512, "TMEM budget");
   static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
 };
@@ -381,6 +382,7 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
                     const __grid_constant__ CUtensorMap tmap_kv, __nv_bfloat16* __restrict__ dQ,
                     const float* __restrict__ ws_LD, int nq, int m, float scale, int* status) {
   using C = QCfg<D>;
+  constexpr int kQC = C::kQC;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {          // swizzled tiles need 1024-byte alignment; never seen to fail
     if (threadIdx.x == 0) atomicCAS(status, 0, 700);
@@ -492,20 +494,23 @@ bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_con
       const int b = j % C::kBufs;
       w.wait(&bars->s_full[b], (j / C::kBufs) & 1, 720);
       tc_fence_after();
-      uint32_t sv[32], av[32];
-      tmem_ld_32x32b_x32(tbase + C::kColS + b * kQC, sv);
-      tmem_ld_32x32b_x32(tbase + C::kColA + b * kQC, av);
-      tmem_wait_ld();
-      uint32_t pk[16];
 #pragma unroll
-      for (int e = 0; e < 32; e += 2) {
-        const float p0 = ex2(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
-        const float p1 = ex2(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
-        const float d0 = live ? scale * p0 * (__uint_as_float(av[e]) - Dv) : 0.f;
-        const float d1 = live ? scale * p1 * (__uint_as_float(av[e + 1]) - Dv) : 0.f;
-        pk[e >> 1] = pack_bf16(d0, d1);
+      for (int c0 = 0; c0 < kQC; c0 += 32) {
+        uint32_t sv[32], av[32];
+        tmem_ld_32x32b_x32(tbase + C::kColS + b * kQC + c0, sv);
+        tmem_ld_32x32b_x32(tbase + C::kColA + b * kQC + c0, av);
+        tmem_wait_ld();
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          const float p0 = ex2(fmaf(__uint_as_float(sv[e]), scale_log2, -L2));
+          const float p1 = ex2(fmaf(__uint_as_float(sv[e + 1]), scale_log2, -L2));
+          const float d0 = live ? scale * p0 * (__uint_as_float(av[e]) - Dv) : 0.f;
+          const float d1 = live ? scale * p1 * (__uint_as_float(av[e + 1]) - Dv) : 0.f;
+          pk[e >> 1] = pack_bf16(d0, d1);
+        }
+        tmem_st_32x32b_x16(tbase + C::kColS + b * kQC + c0 / 2, pk);      // dS over scores that have been read
       }
-      tmem_st_32x32b_x16(tbase + C::kColS + b * kQC, pk);       // dS over the first half of S[b]
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->p_full[b]);
@@ -563,7 +568,7 @@ cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
   if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, c->tmap_kv_st, (__nv_bfloat16*)dQ, c->bw_LD,
+  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, C::kQC == 32 ? c->tmap_kv_st : c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD,
                     (int)p.nq, (int)p.m, scale, c->status);
 }
 
