@@ -592,6 +592,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
       w.wait(&bars->zc_full[t], (cb + nchunks - 1) & 1, 222);   // every P V~ product has been added
       cb += nchunks;
       tc_fence_after();
+      const float unit = kFold ? unit_threshold<D>(kappa, acc_addr, inv) : kappa;
       // v2 holds, in turn: Z, b_t = alpha^t - theta, alpha^T, Psi alpha^T  (pairs of adjacent columns)
       F2 v2[D / 2];
       {
@@ -795,7 +796,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
       // in units of 2 theta, which saves one instruction per pair of elements.  Registers c = alpha / (2 theta),
       // accumulator r' = 1/2 + (z B - a^ mu G) / (2 theta) (the threads store 1/2, z is published divided by 2 theta):
       //   s = sat(c + r') (= sat(x / (2 theta) + 1/2), one saturating add);  increment = r' - s;  c += increment.
-      bool scaled_units = kFold || (!kUntied && !kKeep && T > 0 && theta_stride == 0 && kappa > 0.f);
+      bool scaled_units = kFold || (!kUntied && !kKeep && T > 0 && theta_stride == 0 && threshold_is_a_unit(kappa));
       if (kMasks && scaled_units) {
         // The saturating add turns NaN into 0, which would be recorded as a decision like any other.  So a warp records in these
         // units only where no iterate can leave the finite numbers: finite rows far from overflow, in a recurrence that does
@@ -814,7 +815,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
         if (kFold) {
           // the accumulator held z B (unnormalised): r'_0 = 1/2 + z B / (2 theta) goes back into it, and the first
           // pass below reads it from there like every later one
-          const float inv2th = 0.5f / kappa;
+          const float inv2th = 0.5f / unit;
           const F2 i2 = pack2(inv2th, inv2th), hf = pack2(0.5f, 0.5f);
 #pragma unroll
           for (int c0 = 0; c0 < D; c0 += 16) {
@@ -835,7 +836,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
           for (int e = 0; e < 16; ++e) tb[e] = __float_as_uint(0.5f);
 #pragma unroll
           for (int c0 = 0; c0 < D; c0 += 16) tmem_st_32x32b_x16(acc_addr + c0, tb);
-          const float inv2th = 0.5f / kappa;
+          const float inv2th = 0.5f / unit;
           const F2 i2 = pack2(inv2th, inv2th);
 #pragma unroll
           for (int i = 0; i < D / 2; ++i) v2[i] = mul2(v2[i], i2);
@@ -889,7 +890,7 @@ attend_recover_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __
         // last iteration, exact shrinkage, back in the data's units: alpha^T = 2 theta eta_{1/2}(c + r' - 1/2)
         w.wait(&bars->r_full[t], phase & 1, 231); ++phase;
         tc_fence_after();
-        const F2 tt2 = pack2(2.f * kappa, 2.f * kappa), mh2 = pack2(-0.5f, -0.5f);
+        const F2 tt2 = pack2(2.f * unit, 2.f * unit), mh2 = pack2(-0.5f, -0.5f);
         auto last16 = [&](const uint32_t (&r)[16], int c0) {
 #pragma unroll
           for (int e = 0; e < 16; e += 2) {

@@ -389,6 +389,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     if (p.lse != nullptr && grow < nq) p.lse[((int64_t)bh * nq + grow) * p.lse_stride] = (ref + __log2f(s0 + s1)) * 0.69314718056f;
   }
   for (int i = 0; i < kBufs; ++i) wait_done(244);             // every P V~ product has been added
+  const float unit = kUnit ? unit_threshold<kD>(kappa, acc_addr, inv) : kappa;
   F2 v2[kD / 2];                                               // in turn: Z, the iterate, alpha^T, Psi alpha^T
   {
     const F2 inv2 = pack2(inv, inv);
@@ -512,7 +513,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     }
   };
 
-  bool scaled_units = kUnit || (!kUntied && !kKeep && T > 0 && p.theta_stride == 0 && kappa > 0.f);
+  bool scaled_units = kUnit || (!kUntied && !kKeep && T > 0 && p.theta_stride == 0 && threshold_is_a_unit(kappa));
   if (kMasks && scaled_units) {
     F2 q2 = pack2(0.f, 0.f);
 #pragma unroll
@@ -585,7 +586,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
   if (!kUntied && (kUnit || T > 0)) {
     if (kFold) {
       // the accumulator held z B: r'_0 = 1/2 + z B / (2 theta) goes back into it, and the first pass below reads it from there
-      const float inv2th = 0.5f / kappa;
+      const float inv2th = 0.5f / unit;
       const F2 i2 = pack2(inv2th, inv2th), hf = pack2(0.5f, 0.5f);
 #pragma unroll
       for (int c0 = 0; c0 < kD; c0 += 16) {
@@ -609,7 +610,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
 #pragma unroll
       for (int c0 = 0; c0 < kD; c0 += 16) tmem_st_32x32b_x16(acc_addr + c0, tb);
       if (scaled_units) {
-        const float inv2th = 0.5f / kappa;
+        const float inv2th = 0.5f / unit;
         const F2 i2 = pack2(inv2th, inv2th);
 #pragma unroll
         for (int i = 0; i < kD / 2; ++i) v2[i] = mul2(v2[i], i2);
@@ -689,7 +690,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
     // last iteration, exact shrinkage
     wait_done(247);
     if (scaled_units) {
-      const F2 tt2 = pack2(2.f * kappa, 2.f * kappa), mh2 = pack2(-0.5f, -0.5f);
+      const F2 tt2 = pack2(2.f * unit, 2.f * unit), mh2 = pack2(-0.5f, -0.5f);
       pieces([&](const uint32_t (&r)[16], int c0) {
 #pragma unroll
         for (int e = 0; e < 16; e += 2) {

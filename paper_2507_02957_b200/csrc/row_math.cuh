@@ -1,6 +1,8 @@
-// Arithmetic on a query's row that the two attention / recovery kernels share: packed float32, the exponential on the FMA
-// pipe, 32-byte stores.
+// Arithmetic on a query's row that the attention / recovery kernels share: packed float32, the exponential on the FMA pipe,
+// 32-byte stores, the unit of the recurrence.
 #pragma once
+#include "sm100_ptx.cuh"
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -48,6 +50,26 @@ __device__ __forceinline__ void exp2_poly2(F2 x2, float& p0, float& p1) {
   unpack2(q2, q0, q1);
   p0 = __int_as_float(__float_as_int(q0) + (__float_as_int(t0) << 23));
   p1 = __int_as_float(__float_as_int(q1) + (__float_as_int(t1) << 23));
+}
+
+// The recurrence in units of 2 theta needs z / (2 theta) far from overflow.  theta = mu lambda may be so small, or zero in float32,
+// that it is not: kernels with both forms then keep the data's units, the others take a unit of 2^-70 of the row's largest
+// magnitude: as a threshold that is less than a rounding of what is above 2^-46 of that magnitude, and little of the rest.
+__device__ __forceinline__ bool threshold_is_a_unit(float theta) { return theta >= 0x1p-50f; }
+// The row is `scale` times the N columns of tensor memory from addr on.  (To be called before the row is read into registers: a
+// branch between that and their first use cost 1 % of both kernels, with thresholds that never took it.)
+template <int N> __device__ __forceinline__ float unit_threshold(float theta, uint32_t addr, float scale) {
+  if (threshold_is_a_unit(theta)) return theta;
+  float mx = 0x1p-56f;                                        // a normal number after the scaling below
+#pragma unroll 1
+  for (int c0 = 0; c0 < N; c0 += 16) {
+    uint32_t a[16];
+    ptx::tmem_ld_32x32b_x16(addr + c0, a);
+    ptx::tmem_wait_ld();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) mx = fmaxf(mx, fabsf(__uint_as_float(a[e]) * scale));
+  }
+  return fmaxf(theta, fminf(mx, 3.402823466e38f) * 0x1p-70f);  // (an infinity in the row stays one)
 }
 
 constexpr int kPolyEvery = 4;          // every 4th pair of scores takes the polynomial exp2 (measured best of 1, 2, 3, 4, none)

@@ -12,6 +12,7 @@
 // The arithmetic is that kernel's: bf16 P and increments, float32 accumulators, statistics and iterates; the plain forward
 // with one positive threshold in units of 2 theta, otherwise the accumulator biased by the first threshold.
 #include "csat_internal.h"
+#include "row_math.cuh"
 #include "sm100_ptx.cuh"
 #include "warp_mma.cuh"
 
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) warp_attend_kernel(const Args 
     const float kappa = p.theta[h];
     uint32_t a[4][4];
     float r[8][4], v[8][4];                                     // accumulator; iterate
-    if (!kRec && p.theta_stride == 0 && kappa > 0.f) {
+    if (!kRec && p.theta_stride == 0 && rowmath::threshold_is_a_unit(kappa)) {
       // v = alpha / (2 theta), r = 1/2 + (z B - a^ mu G) / (2 theta): s = sat(v + r), increment = r - s
       const float i2 = 0.5f / kappa;
 #pragma unroll
