@@ -48,16 +48,22 @@ template <int D, bool kUntied = false> struct RCfg {
   static constexpr uint32_t kOffMat = 0;                          // [3]: S - I | B | Psi, as the forward stages them
   static constexpr int kMats = kUntied ? 5 : 3;                   // untied: [stage 0: S_t - I | B_t][stage 1: ...][Psi]
   static constexpr uint32_t kOffBar = kMats * kMatBytes;
-  static constexpr uint32_t kSmemBytes = kOffBar + 128 + 1024 /*alignment slack*/;
-  // TMEM columns: accumulator | dZ accumulator, and in an allocation of their own the bf16 operand buffers (two values per
-  // column).  d = 64 has one buffer, 160 columns in all, so that three CTAs share an SM: a layer is a chain thread -> MMA issuer ->
+  static constexpr uint32_t kSmemUsed = kOffBar + 128 + 1024 /*alignment slack*/;
+  // d = 64: a CTA holds its first allocation of tensor memory (128 columns) while it waits for the second (32).  Four on an SM
+  // would hold all 512 columns and wait for ever, so every CTA asks for so much shared memory that no fourth is resident.
+  // (d = 128: one allocation.)
+  static constexpr uint32_t kSmemBytes = D == 64 ? 58 * 1024 : kSmemUsed;
+  // TMEM columns: accumulator | dZ accumulator | the bf16 operand buffers (two values per column; in an allocation of their own
+  // at d = 64).  d = 64 has one buffer, 160 columns in all, so that three CTAs share an SM: a layer is a chain thread -> MMA issuer ->
   // tensor pipe -> thread that uses neither the tensor pipe nor the issue slots for long (96 heads of 1568 queries, T = 20: 109 -> 84
   // us, with the accumulator's additions, the decisions and the operand in one pass over the row instead of two).
   static constexpr int kCtas = D == 64 ? 3 : 1, kOps = D == 64 ? 1 : 2;
   static constexpr uint32_t kColAcc = 0, kColDz = D, kOpCols = D / 2;
-  static constexpr uint32_t kTmemCols = 2 * D, kTmemOpCols = D == 64 ? 32 : 128;
-  static_assert(kOps * kOpCols <= kTmemOpCols && kCtas * (kTmemCols + kTmemOpCols) <= 512, "TMEM budget");
-  static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
+  static constexpr uint32_t kTmemCols = D == 64 ? 2 * D : 512, kTmemOpCols = D == 64 ? 32 : 0;
+  static_assert(2 * D + kOps * kOpCols <= kTmemCols + kTmemOpCols && kCtas * (kTmemCols + kTmemOpCols) <= 512, "TMEM budget");
+  static_assert(kSmemUsed <= kSmemBytes && kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
+  static_assert(kTmemOpCols == 0 || 512 / kTmemCols * (kSmemBytes + 1024) > 228 * 1024,
+                "CTAs on one SM must not hold all of tensor memory with their first allocations");
 };
 
 struct RBars {
@@ -96,13 +102,13 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
   }
   if (warp == 4) {
     tmem_alloc(&bars->tmem_slot, C::kTmemCols);
-    tmem_alloc(&bars->tmem_op_slot, C::kTmemOpCols);
+    if (C::kTmemOpCols != 0) tmem_alloc(&bars->tmem_op_slot, C::kTmemOpCols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_slot, tmem_op = bars->tmem_op_slot;
+  const uint32_t tmem = bars->tmem_slot, tmem_op = C::kTmemOpCols != 0 ? bars->tmem_op_slot : tmem + 2 * D;
   pdl_wait();
   pdl_launch_dependents();
 
@@ -339,7 +345,7 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
   __syncthreads();
   if (warp == 4) {
     tmem_dealloc(tmem, C::kTmemCols);
-    tmem_dealloc(tmem_op, C::kTmemOpCols);
+    if (C::kTmemOpCols != 0) tmem_dealloc(tmem_op, C::kTmemOpCols);
   }
 }
 
