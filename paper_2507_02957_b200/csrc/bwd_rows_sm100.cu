@@ -52,7 +52,7 @@ template <int D, bool kUntied = false> struct RCfg {
   // d = 64: a CTA holds its first allocation of tensor memory (128 columns) while it waits for the second (32).  Four on an SM
   // would hold all 512 columns and wait for ever, so every CTA asks for so much shared memory that no fourth is resident.
   // (d = 128: one allocation.)
-  static constexpr uint32_t kSmemBytes = D == 64 ? 58 * 1024 : kSmemUsed;
+  static constexpr uint32_t kSmemBytes = D == 64 ? 58 * 1024 : kSmemUsed, kSmemTwo = 80 * 1024;
   // TMEM columns: accumulator | dZ accumulator | the bf16 operand buffers (two values per column; in an allocation of their own
   // at d = 64).  d = 64 has one buffer, 160 columns in all, so that three CTAs share an SM: a layer is a chain thread -> MMA issuer ->
   // tensor pipe -> thread that uses neither the tensor pipe nor the issue slots for long (96 heads of 1568 queries, T = 20: 109 -> 84
@@ -62,6 +62,7 @@ template <int D, bool kUntied = false> struct RCfg {
   static constexpr uint32_t kTmemCols = D == 64 ? 2 * D : 512, kTmemOpCols = D == 64 ? 32 : 0;
   static_assert(2 * D + kOps * kOpCols <= kTmemCols + kTmemOpCols && kCtas * (kTmemCols + kTmemOpCols) <= 512, "TMEM budget");
   static_assert(kSmemUsed <= kSmemBytes && kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
+  static_assert(D != 64 || (2 * (kSmemTwo + 1024) <= 228 * 1024 && 3 * kSmemTwo > 228 * 1024), "two CTAs per SM");
   static_assert(kTmemOpCols == 0 || 512 / kTmemCols * (kSmemBytes + 1024) > 228 * 1024,
                 "CTAs on one SM must not hold all of tensor memory with their first allocations");
 };
@@ -549,12 +550,17 @@ template <int D, bool kUntied>
 cudaError_t launch_recur(csat_ctx* c, const void* G, cudaStream_t s) {
   using C = RCfg<D, kUntied>;
   const Params& p = c->p;
+  constexpr uint32_t kMost = D == 64 ? C::kSmemTwo : C::kSmemBytes;
   static DeviceFlags smem_opt_in;
-  cudaError_t e = ensure_dynamic_smem(bwd_recur_sm100_kernel<D, kUntied>, (int)C::kSmemBytes, c->device, smem_opt_in);
+  cudaError_t e = ensure_dynamic_smem(bwd_recur_sm100_kernel<D, kUntied>, (int)kMost, c->device, smem_opt_in);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
+  // Up to two tiles per SM no three share one: started early, CTAs pile up on the SMs that the kernel before leaves free.  Whole
+  // training steps, us, with three per SM / two: 256 tiles, T = 20, m = 512 138 / 123; 128, T = 20, m = 256 86 / 78; 296, T = 5
+  // 55.6 / 53.2.  512 tiles 182 either way, 312 with two 7 % slower.
+  const uint32_t smem = (int64_t)grid.x * grid.y <= 2 * (int64_t)c->sms ? kMost : C::kSmemBytes;
   return launch_pdl(
-      bwd_recur_sm100_kernel<D, kUntied>, grid, kRThreads, C::kSmemBytes, s,
+      bwd_recur_sm100_kernel<D, kUntied>, grid, kRThreads, smem, s,
       kUntied ? c->tmap_lmats : c->tmap_mats, c->bw_Z16, (const __nv_bfloat16*)G, c->bw_dZ16, c->bw_LD, c->bw_maskbits, (int)p.nq, (int)p.H, p.T,
       c->psi ? 1 : 0, c->status, c->weight_grads ? c->bw_dx16 : nullptr, (int64_t)(p.B * p.H * p.nq * p.d));
 }

@@ -1,0 +1,32 @@
+"""bf16, d = 64: the backward on both sides of the rules that choose its kernels by the size of the job (148 SMs): tiles per SM for the
+recurrence.  Sampled (batch, head) pairs against the float64 oracle within the
+parity bar; the threshold is so low that no iterate lies near it."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import csat_oracle as orc
+from paper_2507_02957_b200 import binding
+from gpu_util import TOL, rel_err, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,nq,m", [
+    (4, 37, 129, 70),       # 296 tiles: two of the recurrence per SM
+    (2, 99, 150, 64),       # 396: three
+])
+def test_gradients_of_sampled_heads(B, H, nq, m):
+    n, d, T, lam = 200, 64, 3, 1e-9
+    g = torch.Generator(device="cuda").manual_seed(nq + m)
+    Q, K, V, G = (torch.randn(B, H, r, d, generator=g, device="cuda").bfloat16() for r in (nq, n, n, nq))
+    ctx = binding.Csat(n, m, d, H, 3, B=B, n_q=nq, dtype="bf16", T=T, lam=lam)
+    phi = ctx.get_phi()
+    got = ctx.backward(Q, K, V, G)
+    again = ctx.backward(Q, K, V, G)
+    assert all(torch.isfinite(x).all() and torch.equal(x, y) for x, y in zip(got, again))
+    for b, h in ((0, 0), (B // 2, H // 2), (B - 1, H - 1)):
+        ref = orc.csat_backward_head(*(to_np(x[b, h]) for x in (Q, K, V)), to_np(phi[h]), to_np(G[b, h]), T=T, lam=lam)
+        for name, x, r in zip(("dQ", "dK", "dV"), got, ref):
+            assert np.abs(r).max() > 0 and rel_err(to_np(x[b, h]), r) <= TOL["bf16"], (b, h, name, rel_err(to_np(x[b, h]), r))
+    ctx.close()
