@@ -19,7 +19,7 @@
 //   no transposed copy); the identity part of S^T stays exact in float32 registers;
 //   at the end dZ (bf16, the operand of the stages that follow) and D = <dZ, Z>.
 //
-// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 32 (d = 64) or 64 measurements:
+// bwd_dq_sm100_kernel, one CTA per tile of 128 queries, K~|V~ streamed in chunks of 32 (d = 64, many tiles) or 64 measurements:
 //        S_j = Q K~_j^T,  dA_j = dZ V~_j^T                        (two SS MMAs into tensor memory)
 //        dS_j = scale * exp(scale S_j - L) o (dA_j - D)           (one thread per row; bf16 back into tensor memory)
 //        dQ  += dS_j K~_j                                         (TS MMA, K~_j read as an MN-major operand)
@@ -355,12 +355,13 @@ bwd_recur_sm100_kernel(const __grid_constant__ CUtensorMap tmap_mats, const __nv
 // ====================================================================================================================
 // d = 64: chunks of 32 measurements, so that S, dA (one buffer each) and dQ take 128 columns of tensor memory and three tiles of 128
 // queries share an SM, where chunks of 64 in two buffers (512 columns allocated) left room for one: 47 -> 38 us for 96 heads of 1568
-// queries, m = 256.  d = 128: chunks of 64, two buffers, one tile (with chunks of 32 and two tiles per SM 16 heads of 8192, m = 512
-// take 82 us instead of 79).
-template <int D> struct QCfg {
+// queries, m = 256.  Few tiles (kFew): chunks of 64, half as many hand-overs, and two tiles per SM (see launch_sm100_bwd_dq).  d = 128:
+// chunks of 64, two buffers, one tile (with chunks of 32 and two tiles per SM 16 heads of 8192, m = 512 take 82 us instead of 79).
+template <int D, bool kFew> struct QCfg {
+  static_assert(!kFew || D == 64, "built variants");
   static constexpr int kDBoxes = D / 64;
-  static constexpr int kQC = D == 64 ? 32 : 64;                     // measurements per chunk
-  static constexpr int kCtas = D == 64 ? 3 : 1;                     // per SM
+  static constexpr int kQC = D == 64 && !kFew ? 32 : 64;            // measurements per chunk
+  static constexpr int kCtas = D == 64 ? (kFew ? 2 : 3) : 1;        // per SM
   static constexpr int kStages = 3, kBufs = D == 64 ? 1 : 2;
   static constexpr uint32_t kTileBoxBytes = kRows * 128;            // 128 rows x 64 columns
   static constexpr uint32_t kTileBytes = kDBoxes * kTileBoxBytes;   // Q tile, dZ tile
@@ -370,7 +371,7 @@ template <int D> struct QCfg {
   static constexpr uint32_t kOffBar = kOffRing + kStages * 2 * kSlotBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + 256;             // base must be 1024-byte aligned (checked)
   // TMEM columns: S[bufs] | dA[bufs] | dQ accumulator; dS_j (bf16) overlays the first half of S[j % bufs]
-  static constexpr uint32_t kColS = 0, kColA = kBufs * kQC, kColQ = 2 * kBufs * kQC, kTmemCols = D == 64 ? 128 : 512;
+  static constexpr uint32_t kColS = 0, kColA = kBufs * kQC, kColQ = 2 * kBufs * kQC, kTmemCols = D == 128 ? 512 : kFew ? 256 : 128;
   static_assert(kColQ + D <= kTmemCols && kCtas * kTmemCols <= 512, "TMEM budget");
   static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024, "CTAs per SM");
 };
@@ -383,12 +384,12 @@ struct QBars {
 
 constexpr int kQThreads = 192;      // warps 0-3: one thread per query row; warp 4: TMA; warp 5: MMA issue
 
-template <int D>
-__global__ void __launch_bounds__(kQThreads, QCfg<D>::kCtas)
+template <int D, bool kFew>
+__global__ void __launch_bounds__(kQThreads, QCfg<D, kFew>::kCtas)
 bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_z,
                     const __grid_constant__ CUtensorMap tmap_kv, __nv_bfloat16* __restrict__ dQ,
                     const float* __restrict__ ws_LD, int nq, int m, float scale, int* status) {
-  using C = QCfg<D>;
+  using C = QCfg<D, kFew>;
   constexpr int kQC = C::kQC;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {          // swizzled tiles need 1024-byte alignment; never seen to fail
@@ -565,9 +566,9 @@ cudaError_t launch_recur(csat_ctx* c, const void* G, cudaStream_t s) {
       c->psi ? 1 : 0, c->status, c->weight_grads ? c->bw_dx16 : nullptr, (int64_t)(p.B * p.H * p.nq * p.d));
 }
 
-template <int D>
+template <int D, bool kFew = false>
 cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
-  using C = QCfg<D>;
+  using C = QCfg<D, kFew>;
   const Params& p = c->p;
   CUtensorMap tq, tz;
   const uint64_t qd[3] = {(uint64_t)D, (uint64_t)p.nq, (uint64_t)(p.B * p.H)};
@@ -577,10 +578,10 @@ cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
   if ((e = make_tmap_bf16_3d(&tq, Q, qd, qs, qb)) != cudaSuccess) return e;
   if ((e = make_tmap_bf16_3d(&tz, c->bw_dZ16, qd, qs, qb)) != cudaSuccess) return e;
   static DeviceFlags smem_opt_in;
-  if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
+  if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D, kFew>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  return launch_pdl(bwd_dq_sm100_kernel<D>, grid, kQThreads, C::kSmemBytes, s, tq, tz, C::kQC == 32 ? c->tmap_kv_st : c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD,
+  return launch_pdl(bwd_dq_sm100_kernel<D, kFew>, grid, kQThreads, C::kSmemBytes, s, tq, tz, C::kQC == 32 ? c->tmap_kv_st : c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD,
                     (int)p.nq, (int)p.m, scale, c->status);
 }
 
@@ -596,7 +597,12 @@ cudaError_t launch_sm100_bwd_recur(csat_ctx* c, const void* G, cudaStream_t s, i
 
 cudaError_t launch_sm100_bwd_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s, int* launches) {
   *launches += 1;
-  return c->p.d == 64 ? launch_dq<64>(c, Q, dQ, s) : launch_dq<128>(c, Q, dQ, s);
+  if (c->p.d == 128) return launch_dq<128>(c, Q, dQ, s);
+  // Two tiles per SM where that takes as many rounds as three.  Whole training steps, us, chunks of 64 and two per SM / of 32 and three:
+  // 128 tiles, m = 512 66.5 / 74.7, m = 256 77.5 / 83.2; 256, m = 512 120 / 126; 512, m = 512 183 / 190; 592, m = 128 87.4 / 89.7;
+  // 312, m = 256 109.7 / 107.7; 624, m = 256 174 / 171; 1248, m = 256 273 / 269.  The same bits.
+  const int64_t tiles = (c->p.nq + kRows - 1) / kRows * c->p.B * c->p.H;
+  return two_tiles_per_sm(tiles, c->sms) ? launch_dq<64, true>(c, Q, dQ, s) : launch_dq<64>(c, Q, dQ, s);
 }
 
 }  // namespace csat

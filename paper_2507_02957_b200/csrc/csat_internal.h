@@ -264,6 +264,9 @@ cudaError_t launch_sm100_attend_for_backward(csat_ctx* c, const void* Q, __nv_bf
                                              int lse_stride, uint32_t* mask_out, __nv_bfloat16* alpha_out,
                                              cudaStream_t s, int* launches, void* out = nullptr);
 
+// d = 64: two tiles of 128 queries per SM take as many rounds as three would, and each has half an SM instead of a third
+inline bool two_tiles_per_sm(int64_t tiles, int sms) { return tiles <= 2 * (int64_t)sms || (tiles > 3 * (int64_t)sms && tiles <= 4 * (int64_t)sms); }
+
 // attend_tile_sm100.cu : the same for d = 64, one tile of 128 queries per CTA and three CTAs per SM
 cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first);
 cudaError_t launch_attend_tile_recording(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float* lse, int lse_stride,

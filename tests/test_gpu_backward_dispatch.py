@@ -1,5 +1,5 @@
 """bf16, d = 64: the backward on both sides of the rules that choose its kernels by the size of the job (148 SMs): tiles per SM for the
-recurrence.  Sampled (batch, head) pairs against the float64 oracle within the
+recurrence and dQ.  Sampled (batch, head) pairs against the float64 oracle within the
 parity bar; the threshold is so low that no iterate lies near it."""
 import numpy as np
 import pytest
@@ -13,8 +13,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,H,nq,m", [
-    (4, 37, 129, 70),       # 296 tiles: two of the recurrence per SM
-    (2, 99, 150, 64),       # 396: three
+    (4, 37, 129, 70),       # 296 tiles: two of the recurrence per SM, dQ in chunks of 64
+    (2, 99, 150, 64),       # 396: three, and dQ in chunks of 32
+    (16, 37, 33, 129),      # 592 tiles: dQ in chunks of 64
+    (2, 297, 31, 193),      # 594: in chunks of 32
 ])
 def test_gradients_of_sampled_heads(B, H, nq, m):
     n, d, T, lam = 200, 64, 3, 1e-9
