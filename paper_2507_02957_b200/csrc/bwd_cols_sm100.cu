@@ -29,7 +29,7 @@
 //              operand of the product with Phi^T.
 // A cluster of 2 (d = 64: or 4) CTAs shares out the queries of a block where that fills the SMs better (16 heads with m = 512 are 64
 // blocks); each CTA then adds up its share of the rows from all CTAs' shared memory, in rank order (bit-identical reruns).
-// 16 heads of 8192 x 128, m = 512: 131 -> 77 us; 96 heads of 1568 x 64, m = 256 (192 blocks, not shared out): 65 -> 61 us.
+// 16 heads of 8192 x 128, m = 512: 131 -> 77 us.
 #include "csat_internal.h"
 #include "sm100_ptx.cuh"
 #include "tma_host.h"
@@ -308,6 +308,38 @@ bwd_cols_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
   if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
 }
 
+int64_t blocks_of(const Params& p) { return (p.m + kRows - 1) / kRows * p.B * p.H; }
+int64_t tiles_of(const Params& p) { return (p.nq + kQT - 1) / kQT; }
+
+// Two score sets.  Queries per block shared out between 1, 2 or (d = 64) 4 CTAs: the fewest rounds of CTAs (one per SM) weighted with
+// their length, a CTA's start and end counted as kFixed query tiles.  Measured, us with 1 / 2 / 4: d = 64, 25 query tiles: 24 blocks
+// 31 / 22 / 17, 72 blocks 31 / 23 / 48; d = 128: 64 blocks of 128 tiles 126 / 77 / 100, 16 blocks of 32 tiles 38 / 31 / 54.
+constexpr int kFixed = 12;
+int best_splits(const csat_ctx* c, int most, int64_t* cost_out = nullptr) {
+  const int64_t blocks = blocks_of(c->p), tiles = tiles_of(c->p);
+  int splits = 1;
+  int64_t best = 0;
+  for (int k = 1; k <= most; k *= 2) {
+    const int64_t per = (tiles + k - 1) / k;
+    if (k > 1 && (k - 1) * per >= tiles) break;   // every CTA has a tile
+    const int64_t cost = (blocks * k + c->sms - 1) / c->sms * (per + kFixed);
+    if (k == 1 || cost < best) { best = cost; splits = k; }
+  }
+  if (cost_out) *cost_out = best;
+  return splits;
+}
+
+// One score set and two CTAs per SM (d = 64), by the same measure: a round of 2 SMs' worth of blocks takes 1.7 of those tiles' time
+// per tile and 18 for its start and end, a further round 0.65 of that.  Fitted to the kernel's times, us, two sets / one: 192 blocks of
+// 25 tiles 61 / 50; 297 of 25 91 / 85, of 64 204 / 201, of 128 366 / 392; 370 of 128 377 / 398; 444 of 128 416 / 402; 592 of 64
+// 289 / 245; whole backward calls: 149 blocks of 64 355 / 346, of 128 654 / 666; 222 of 128 880 / 890; 224 of 128 931 / 896.
+bool one_set_better(const csat_ctx* c) {
+  const int64_t blocks = blocks_of(c->p), rounds = (blocks + 2 * c->sms - 1) / (2 * c->sms);
+  int64_t two;
+  best_splits(c, 4, &two);
+  return blocks > c->sms && (17 * tiles_of(c->p) + 180) * (7 + 13 * rounds) <= 200 * two;
+}
+
 template <int D, int SETS>
 cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   using C = Cfg<D, SETS>;
@@ -322,20 +354,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
   static DeviceFlags smem_opt_in;
   if ((e = ensure_dynamic_smem(bwd_cols_sm100_kernel<D, SETS>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
-  // Queries per block shared out between 1, 2 or (d = 64) 4 CTAs: the fewest rounds of CTAs (one per SM) weighted with their
-  // length, a CTA's start and end counted as kFixed query tiles.  Measured, us with 1 / 2 / 4: d = 64, 25 query tiles: 24
-  // blocks 31 / 22 / 17, 72 blocks 31 / 23 / 48, 192 blocks 61 / 65 / 98; d = 128: 64 blocks of 128 tiles 126 / 77 / 100, 16
-  // blocks of 32 tiles 38 / 31 / 54.
-  const int64_t blocks = (p.m + kRows - 1) / kRows * p.B * p.H, tiles = (p.nq + kQT - 1) / kQT;
-  constexpr int kFixed = 12;
-  int splits = 1;
-  int64_t best = 0;
-  for (int k = 1; k <= (SETS == 1 ? 1 : D == 64 ? 4 : 2); k *= 2) {
-    const int64_t per = (tiles + k - 1) / k;
-    if (k > 1 && (k - 1) * per >= tiles) break;   // every CTA has a tile
-    const int64_t cost = (blocks * k + c->sms - 1) / c->sms * (per + kFixed);
-    if (k == 1 || cost < best) { best = cost; splits = k; }
-  }
+  const int splits = SETS == 1 ? 1 : best_splits(c, D == 64 ? 4 : 2);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((p.m + kRows - 1) / kRows), (unsigned)(p.B * p.H), (unsigned)splits);
   cfg.blockDim = dim3(kThreads);
@@ -357,9 +376,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, cudaStream_t s) {
 // needs dZ as bf16 (bw_dZ16), L and D (bw_LD) from the per-row stage, and K~|V~ in the workspace
 cudaError_t launch_sm100_bwd_cols(csat_ctx* c, const void* Q, cudaStream_t s, int* launches) {
   *launches += 1;
-  const int64_t blocks = (c->p.m + kRows - 1) / kRows * c->p.B * c->p.H;
-  // d = 64 with more blocks than SMs: one score set and two CTAs per SM (192 blocks of 25 query tiles: 61 -> 50 us)
-  if (c->p.d == 64 && blocks > c->sms) return launch<64, 1>(c, Q, s);
+  if (c->p.d == 64 && one_set_better(c)) return launch<64, 1>(c, Q, s);
   return c->p.d == 64 ? launch<64, 2>(c, Q, s) : launch<128, 2>(c, Q, s);
 }
 

@@ -1,5 +1,5 @@
 """bf16, d = 64: the backward on both sides of the rules that choose its kernels by the size of the job (148 SMs): tiles per SM for the
-recurrence and dQ.  Sampled (batch, head) pairs against the float64 oracle within the
+recurrence and dQ, measurement blocks and queries for dK~ | dV~.  Sampled (batch, head) pairs against the float64 oracle within the
 parity bar; the threshold is so low that no iterate lies near it."""
 import numpy as np
 import pytest
@@ -17,6 +17,11 @@ pytestmark = pytest.mark.gpu
     (2, 99, 150, 64),       # 396: three, and dQ in chunks of 32
     (16, 37, 33, 129),      # 592 tiles: dQ in chunks of 64
     (2, 297, 31, 193),      # 594: in chunks of 32
+    (1, 150, 4096, 65),     # 150 blocks of measurements: one score set for 4096 queries
+    (1, 150, 8200, 65),     # two, and the queries shared out, for 8200
+    (1, 300, 4000, 64),     # 300 blocks: the same two
+    (1, 300, 8192, 64),
+    (1, 297, 70, 100),
 ])
 def test_gradients_of_sampled_heads(B, H, nq, m):
     n, d, T, lam = 200, 64, 3, 1e-9
