@@ -31,7 +31,6 @@ using namespace rowmath;
 constexpr int kD = 64;
 constexpr int kRows = 128;             // queries per CTA: one thread per query, TMEM lane = query
 constexpr int kMC = 64;                // measurements per chunk
-constexpr int kStages = 2;             // K~|V~ chunks in flight
 constexpr int kRowWarps = 4, kMmaWarp = 4, kTmaWarp = 5;
 constexpr int kThreads = 256;          // the rows' warps, then one warpgroup of control
 constexpr int kCtas = 3;               // per SM
@@ -41,24 +40,32 @@ constexpr uint32_t kQBytes = kRows * 128;                         // Q; later Ps
 constexpr uint32_t kSlotBytes = kMC * 128;                        // K~ chunk (= V~ chunk)
 constexpr uint32_t kStageBytes = 2 * kSlotBytes;
 constexpr uint32_t kMatBytes = kD * 128;                          // a d x d bf16 matrix
-constexpr uint32_t kOffRing = kQBytes, kOffG = kOffRing + kStages * kStageBytes, kOffB = kOffG + kMatBytes;
-constexpr uint32_t kOffBar = kOffB + kMatBytes, kSmemBytes = kOffBar + 256;
-constexpr uint32_t kSmemTwo = 80 * 1024, kSmemOne = 120 * 1024;   // no more than two, one CTA per SM
+constexpr uint32_t kOffRing = kQBytes, kBarBytes = 256;
+// Shared memory: Q | ring | -mu G | B | barriers.  K~|V~ chunks in flight: two where three CTAs share an SM; four with two score buffers
+// (kBufs), where few CTAs wait for their own copies: 76 heads of 77 queries, m = 392 23.6 -> 21.0 us, 96 of 112, m = 512, T = 5 18.1 ->
+// 15.8, one chunk 10.1 either way.
+template <int kBufs> struct Layout {
+  static constexpr int kStages = 2 * kBufs;
+  static constexpr uint32_t kOffG = kOffRing + kStages * kStageBytes, kOffB = kOffG + kMatBytes, kOffBar = kOffB + kMatBytes;
+  static constexpr uint32_t kSmemBytes = kOffBar + kBarBytes;
+};
+constexpr uint32_t kSmemTwo = 100 * 1024, kSmemOne = 120 * 1024;  // no more than two, one CTA per SM
 constexpr uint32_t kOutBytes = 32 * 128;                          // one warp's rows of the output
 // TMEM columns: accumulator (Zacc, then r_t) | S (P_j overlays its first half; later the recovery operand)
 constexpr uint32_t kColAcc = 0, kColS = kD, kTmemCols = 2 * kD;   // (kBufs = 2: another S behind it)
-static_assert(kSmemBytes <= kSmemTwo && 3 * kSmemTwo > 228 * 1024 && 2 * kSmemOne > 228 * 1024, "fewer CTAs per SM");
+static_assert(Layout<2>::kSmemBytes <= kSmemTwo && 2 * (kSmemTwo + 1024) <= 228 * 1024 && 3 * kSmemTwo > 228 * 1024 &&
+              2 * kSmemOne > 228 * 1024, "fewer CTAs per SM");
 static_assert(kMatBytes <= kQBytes && 4 * kOutBytes <= kQBytes, "overlays");
-static_assert(kCtas * (kSmemBytes + 1024) <= 228 * 1024 && kCtas * kTmemCols <= 512, "CTAs per SM");
+static_assert(kCtas * (Layout<1>::kSmemBytes + 1024) <= 228 * 1024 && kCtas * kTmemCols <= 512, "CTAs per SM");
 
 struct Bars {
-  uint64_t q_full, k_full[kStages], k_free[kStages], v_full[kStages], v_free[kStages], mats_full[3];
+  uint64_t q_full, k_full[4], k_free[4], v_full[4], v_free[4], mats_full[3];
   uint64_t rows[2], done[2];  // by publication and by step modulo kBufs, since with two score buffers either may be one ahead:
                               // the rows' operand is in tensor memory; the products issued on it are finished
   uint32_t tmem_slot;
   int abort;
 };
-static_assert(sizeof(Bars) <= 256, "barrier block");
+static_assert(sizeof(Bars) <= kBarBytes, "barrier block");
 
 struct Args {
   __nv_bfloat16* out;
@@ -89,13 +96,17 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
                    const __grid_constant__ CUtensorMap tmap_vb, const Args p) {
   constexpr bool kUnit = kDec == kUnits || kDec == kFolded, kUntied = kDec == kPerLayer, kFold = kDec == kFolded;
   constexpr bool kMasks = kRec >= 1, kKeep = kRec >= 2, kStaged = kDec != kPerLayer;     // kStaged: Z's way out, through a stage of the ring
+  using L = Layout<kBufs>;
+  constexpr int kStages = L::kStages;
+  auto slot = [](int j) { return j & (kStages - 1); };          // ring position j: its stage, and the parity of that stage's phase
+  auto phase = [](int j) { return (uint32_t)(j / kStages) & 1u; };
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {          // swizzled tiles need 1024-byte alignment; never seen to fail
     if (threadIdx.x == 0) atomicCAS(p.status, 0, 240);
     return;
   }
   uint8_t* ring = smem + kOffRing;
-  Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
+  Bars* bars = reinterpret_cast<Bars*>(smem + L::kOffBar);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = p.bh0 + blockIdx.x / p.tiles, row0 = (blockIdx.x % p.tiles) * kRows, h = bh % p.H;
   const int nq = p.nq, m = p.m, T = p.T;
@@ -162,27 +173,27 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
       // K~'s says that S_j is done, and with it P_i V~_i.
       for (int j = 0; j < nchunks + kBufs; ++j, ++step) {
         const int i = j - kBufs;
-        if (j < nchunks) w.wait(&bars->k_full[j & 1], (j >> 1) & 1, 241);
+        if (j < nchunks) w.wait(&bars->k_full[slot(j)], phase(j), 241);
         if (i >= 0) {
-          w.wait(&bars->v_full[i & 1], (i >> 1) & 1, 242);
+          w.wait(&bars->v_full[slot(i)], phase(i), 242);
           rows_wait();
         }
         tc_fence_after();
         if (elect_one()) {
           const uint32_t sp = op_col + (kBufs == 1 ? 0 : (uint32_t)(j & 1) * kMC);
           if (i >= 0) {
-            const uint64_t vd = rv + (uint64_t)(i & 1) * kStageStep;
+            const uint64_t vd = rv + (uint64_t)slot(i) * kStageStep;
 #pragma unroll
             for (int k = 0; k < kMC / 16; ++k) mma_f16_ts(acc, sp + k * 8, vd + (uint64_t)(k * 128), idesc_z, (uint32_t)((i > 0) | (k != 0)));
           }
           if (j < nchunks) {
-            const uint64_t kd = rk + (uint64_t)(j & 1) * kStageStep;
+            const uint64_t kd = rk + (uint64_t)slot(j) * kStageStep;
 #pragma unroll
             for (int k = 0; k < kD / 16; ++k) mma_f16_ss(sp, qd + kstep(k), kd + kstep(k), idesc_s, k != 0);
           }
           finish_step();
-          if (j < nchunks && (j + kStages < n_ring || (!kUntied && j + 1 == nchunks))) mma_commit(&bars->k_free[j & 1]);
-          if (i >= 0 && i + kStages < n_ring) mma_commit(&bars->v_free[i & 1]);
+          if (j < nchunks && (j + kStages < n_ring || (!kUntied && j + 1 == nchunks))) mma_commit(&bars->k_free[slot(j)]);
+          if (i >= 0 && i + kStages < n_ring) mma_commit(&bars->v_free[slot(i)]);
         }
         __syncwarp();
       }
@@ -190,11 +201,11 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
         // layer l: r = z^ B_l (+ a^_l (S_l - I) from the second layer on), its matrices in ring position nchunks + l; then Psi
         for (int l = 0; l < n_mma; ++l, ++step) {
           const int q = nchunks + l;
-          w.wait(&bars->k_full[q & 1], (q >> 1) & 1, 251);
-          w.wait(&bars->v_full[q & 1], (q >> 1) & 1, 252);
+          w.wait(&bars->k_full[slot(q)], phase(q), 251);
+          w.wait(&bars->v_full[slot(q)], phase(q), 252);
           rows_wait();
           tc_fence_after();
-          const uint64_t sd = rk + (uint64_t)(q & 1) * kStageStep, bd = sd + (uint64_t)(kSlotBytes >> 4);
+          const uint64_t sd = rk + (uint64_t)slot(q) * kStageStep, bd = sd + (uint64_t)(kSlotBytes >> 4);
           if (elect_one()) {
 #pragma unroll
             for (int k = 0; k < kD / 16; ++k)
@@ -205,8 +216,8 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             }
             finish_step();
             if (q + kStages < n_ring) {
-              mma_commit(&bars->k_free[q & 1]);
-              mma_commit(&bars->v_free[q & 1]);
+              mma_commit(&bars->k_free[slot(q)]);
+              mma_commit(&bars->v_free[slot(q)]);
             }
           }
           __syncwarp();
@@ -217,7 +228,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
           if (i <= first || which == 2) w.wait(&bars->mats_full[which], 0, 245);
           rows_wait();
           tc_fence_after();
-          const uint64_t wd = qd + (which == 0 ? (uint64_t)(kOffG >> 4) : which == 1 ? (uint64_t)(kOffB >> 4) : 0);
+          const uint64_t wd = qd + (which == 0 ? (uint64_t)(L::kOffG >> 4) : which == 1 ? (uint64_t)(L::kOffB >> 4) : 0);
           const uint32_t accum = which != 2;
           if (elect_one()) {
 #pragma unroll
@@ -232,9 +243,9 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
       if (elect_one()) {
         int nk = 0, nv = 0, nm = 0;           // ring positions, and matrices (bit i: mats_full[i]), whose copies were issued
         auto load_slot = [&](int j, int half, const CUtensorMap* map, int x, int y, int z) {
-          uint64_t* full = half ? &bars->v_full[j & 1] : &bars->k_full[j & 1];
+          uint64_t* full = half ? &bars->v_full[slot(j)] : &bars->k_full[slot(j)];
           mbar_arrive_expect_tx(full, kSlotBytes);
-          tma_load_3d(ring + (j & 1) * kStageBytes + half * kSlotBytes, map, full, x, y, z);
+          tma_load_3d(ring + slot(j) * kStageBytes + half * kSlotBytes, map, full, x, y, z);
         };
         auto load_mat = [&](uint8_t* dst, int i) {
           nm |= 1 << i;
@@ -243,24 +254,24 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
         };
         mbar_arrive_expect_tx(&bars->q_full, kQBytes);
         tma_load_3d(smem, &tmap_q, &bars->q_full, 0, row0, bh);
-        if (!kUntied && T > 1) load_mat(smem + kOffG, 0);
-        if (!kUntied && !kFold && T > 0) load_mat(smem + kOffB, 1);
+        if (!kUntied && T > 1) load_mat(smem + L::kOffG, 0);
+        if (!kUntied && !kFold && T > 0) load_mat(smem + L::kOffB, 1);
         if (!kFold) {
           pdl_wait();
           pdl_launch_dependents();
         }
         for (int j = 0; j < n_ring; ++j) {
           const int l = j - nchunks, mat0 = h * (2 * T + 1);
-          if (j >= kStages) w.wait(&bars->k_free[j & 1], ((j >> 1) - 1) & 1, 247);
+          if (j >= kStages) w.wait(&bars->k_free[slot(j)], phase(j - kStages), 247);
           if (w.dead) break;
           if (l < 0) load_slot(j, 0, &tmap_kv, 0, j * kMC, bh);
           else if (l > 0 && l < T) load_slot(j, 0, &tmap_mats, 0, 0, mat0 + 2 * l);
-          else mbar_arrive(&bars->k_full[j & 1]);             // alpha^0 = 0, Psi: nothing to load, the phases stay in step
+          else mbar_arrive(&bars->k_full[slot(j)]);             // alpha^0 = 0, Psi: nothing to load, the phases stay in step
           if (kFold && j == 0) {              // K~ was complete before the fold let this kernel start, V~ B was not
             pdl_wait();
             pdl_launch_dependents();
           }
-          if (j >= kStages) w.wait(&bars->v_free[j & 1], ((j >> 1) - 1) & 1, 248);
+          if (j >= kStages) w.wait(&bars->v_free[slot(j)], phase(j - kStages), 248);
           if (w.dead) { ++nk; break; }
           if (l < 0) load_slot(j, 1, kFold ? &tmap_vb : &tmap_kv, kFold ? 0 : kD, j * kMC, bh);
           else load_slot(j, 1, &tmap_mats, 0, 0, mat0 + (l == T ? 2 * T : 2 * l + 1));
@@ -268,7 +279,7 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
           ++nv;
         }
         if (!kUntied && T > 0 && p.has_psi && !w.dead) {
-          w.wait(&bars->k_free[(nchunks - 1) & 1], ((nchunks - 1) >> 1) & 1, 249);      // the last S: Q's place is free
+          w.wait(&bars->k_free[slot(nchunks - 1)], phase(nchunks - 1), 249);      // the last S: Q's place is free
           if (!w.dead) load_mat(smem, 2);
         }
         if (w.dead) {
@@ -276,8 +287,8 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
           mbar_wait_drain(&bars->q_full, 0);
           for (int i = 0; i < 3; ++i)
             if ((nm >> i) & 1) mbar_wait_drain(&bars->mats_full[i], 0);
-          for (int j = nk > 2 ? nk - 2 : 0; j < nk; ++j) mbar_wait_drain(&bars->k_full[j & 1], (j >> 1) & 1);
-          for (int j = nv > 2 ? nv - 2 : 0; j < nv; ++j) mbar_wait_drain(&bars->v_full[j & 1], (j >> 1) & 1);
+          for (int j = nk > kStages ? nk - kStages : 0; j < nk; ++j) mbar_wait_drain(&bars->k_full[slot(j)], phase(j));
+          for (int j = nv > kStages ? nv - kStages : 0; j < nv; ++j) mbar_wait_drain(&bars->v_full[slot(j)], phase(j));
         }
       }
     }
@@ -745,7 +756,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   // pile up on the SMs that the kernel before leaves free.
   const int64_t tiles = (p.nq + kRows - 1) / kRows, n = tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
   if (n > (int64_t)1 << 30) return cudaErrorInvalidValue;
-  const uint32_t smem = n <= c->sms ? kSmemOne : n <= 2 * (int64_t)c->sms || kBufs == 2 ? kSmemTwo : kSmemBytes;
+  const uint32_t smem = n <= c->sms ? kSmemOne : n <= 2 * (int64_t)c->sms || kBufs == 2 ? kSmemTwo : Layout<kBufs>::kSmemBytes;
   static DeviceFlags smem_opt_in;
   if (!smem_opt_in.test(c->device)) {
     // setmaxnreg moves registers inside the pool the CTA is launched with (threads x the compiled register count); a request
