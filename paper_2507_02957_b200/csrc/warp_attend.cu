@@ -359,12 +359,13 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
 
 }  // namespace
 
-// One CTA per SM at most, of 64 queries (one warp per sub-core) or of 128 where not all of its eight warps have rows or the
-// attention phase is a single chunk.  Attention alone, us, this kernel / attend_tile_sm100:
+// One CTA per SM at most, of 64 queries (one warp per sub-core), or of 128 where the attention phase has few chunks: up to three where not
+// all of its eight warps have rows, else one.  Beyond, the tensor cores' products pay off.  Attention alone, us, this kernel /
+// attend_tile_sm100:
 //   64 queries: 12 heads of 197, m = 64, T = 10 5.0 / 8.2; 74 of 77, m = 392, T = 20 12.2 / 17.7; 8 of 1024, m = 128, T = 10 6.1 / 9.0
-//   128, and whole calls: 148 heads of 65, m = 64, T = 10 7.3 / 9.0 and 12.4 / 14.3; 74 of 197 8.0 / 8.9 and 11.8 / 12.8; 140 of 100,
-//   m = 128, T = 20 12.5 / 13.3 and 18.4 / 19.6; 128 of 77, m = 392 18.0 / 17.8 and 95.3 / 97.0 (its CTAs start under the compression);
-//   otherwise not: 11 of 1568, m = 256, T = 20 15.2 / 14.7, 48 of 300, m = 256 15.1 / 15.0.
+//   128, whole calls, T = 20: 128 heads of 77, m = 128 18.9 / 21.3, m = 192 20.5 / 21.7, m = 256 21.7 / 22.4, m = 392 29.1 / 27.6; 148 of
+//   112, m = 128 19.9 / 21.5, m = 192 25.5 / 25.8, m = 256 26.9 / 26.4; 80 of 100, T = 5, m = 256 18.6 / 17.5; 96 of 112, m = 512 27.1 / 23.5
+//   one chunk, T = 10: 148 heads of 65 12.4 / 14.3, 74 of 197 11.8 / 12.8; otherwise not: 11 of 1568, m = 256, T = 20 15.2 / 14.7
 // The whole job counts, not the launch's range of (batch, head) pairs, so that a forward cut into sub-range launches returns the
 // same bits.
 static int64_t blocks_of(const csat_ctx* c, int rows) { return (c->p.nq + rows - 1) / rows * c->p.B * c->p.H; }
@@ -372,7 +373,7 @@ static int64_t blocks_of(const csat_ctx* c, int rows) { return (c->p.nq + rows -
 bool warp_attend_better(const csat_ctx* c) {
   const Params& p = c->p;
   if (p.d != kD || (c->w_S && c->w_untied && p.T > 0)) return false;
-  return blocks_of(c, 64) <= c->sms || (blocks_of(c, 128) <= c->sms && (p.nq <= 112 || p.m <= kMC));
+  return blocks_of(c, 64) <= c->sms || (blocks_of(c, 128) <= c->sms && p.m <= (p.nq <= 112 ? 3 * kMC : kMC));
 }
 
 cudaError_t launch_warp_attend(csat_ctx* c, const void* Q, void* out, cudaStream_t s, bool wait_first) {

@@ -34,6 +34,8 @@ def _check(ctx, Q, K, V, what, **kw):
 
 
 @pytest.mark.parametrize("B,H,nq,m", [
+    (2, 64, 77, 192),       # 128 queries per CTA of the warp kernel, up to three chunks
+    (2, 64, 77, 193),       # two score buffers, four chunks in flight
     (1, 60, 150, 257),
     (1, 60, 150, 520),
     (2, 70, 129, 64),       # 280 tiles, the second of a head has one row
