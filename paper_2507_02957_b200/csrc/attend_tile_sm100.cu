@@ -777,9 +777,14 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
 
 }  // namespace
 
-// Two score buffers where an SM holds at most two tiles: S_{j+1} is formed under chunk j's exponentials.  By the context's whole
-// job, not the launch's range of (batch, head) pairs.
-static bool few_tiles(const csat_ctx* c) { return (c->p.nq + kRows - 1) / kRows * c->p.B * c->p.H <= 2 * (int64_t)c->sms; }
+// Two score buffers where an SM holds at most two tiles: S_{j+1} is formed under chunk j's exponentials.  Between three and four tiles per
+// SM two rounds of two take the place of two of three, unless there is a single chunk.  us, two buffers / one: 592 tiles, m = 256, T =
+// 20 37.8 / 38.3; 512 36.6 / 37.8, T = 10 25.9 / 27.1; 512, m = 64 21.2 / 20.8; 300, m = 256, T = 20 38 / 27.  By the context's whole job,
+// not the launch's range of (batch, head) pairs.
+static bool few_tiles(const csat_ctx* c) {
+  const int64_t tiles = (c->p.nq + kRows - 1) / kRows * c->p.B * c->p.H;
+  return tiles <= 2 * (int64_t)c->sms || (c->p.m > kMC && two_tiles_per_sm(tiles, c->sms));
+}
 
 cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first) {
 #define CSAT_TILE(DEC, BUFS) launch<0, DEC, BUFS>(c, Q, out, s, nullptr, 0, nullptr, nullptr, nullptr, wait_first)

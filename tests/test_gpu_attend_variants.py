@@ -40,6 +40,10 @@ def _check(ctx, Q, K, V, what, **kw):
     (1, 60, 150, 520),
     (2, 70, 129, 64),       # 280 tiles, the second of a head has one row
     (2, 70, 129, 131),
+    (2, 99, 150, 64),       # 396 tiles: one buffer
+    (2, 140, 250, 64),      # 560: one buffer for a single chunk
+    (2, 140, 250, 131),     # two for more
+    (2, 149, 250, 131),     # 596: one
 ])
 def test_thresholds_and_sizes(B, H, nq, m):
     n, T = 530, 4
