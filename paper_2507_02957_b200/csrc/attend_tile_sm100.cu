@@ -84,9 +84,9 @@ struct Args {
   bool wait_first, contracting;
 };
 
-// kTied: one S, B, thresholds as they are; kUnits: the same with one positive threshold (units of 2 theta); kFolded: the same with
-// V~ B in the place of V~ (vfold_sm100_kernel); kPerLayer: one S_t, B_t per layer
-enum Decoder { kTied, kUnits, kFolded, kPerLayer };
+// kTied: one S, B, one threshold (in a recording forward: or one per layer); kThresholds: one threshold per layer; kUnits: one positive
+// threshold (units of 2 theta); kFolded: the same with V~ B in the place of V~ (vfold_sm100_kernel); kPerLayer: one S_t, B_t per layer
+enum Decoder { kTied, kThresholds, kUnits, kFolded, kPerLayer };
 
 // kRec: 0 = the plain forward; 1 = also Z, log sum exp and the decisions; 2 = also the iterates and the sign bits of x_t
 template <int kRec, Decoder kDec, int kBufs>
@@ -660,7 +660,9 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             tmem_st_32x32b_x8(op_addr + c0 / 2, pk);
           });
         } else {
-          const float th = p.theta[(int64_t)it * p.theta_stride + h];
+          // the add of theta_t - kappa and the loads of thresholds cost 0.1 us a layer: only where thresholds differ
+          constexpr bool kDiffer = kDec == kThresholds || kMasks;
+          const float th = kDiffer ? p.theta[(int64_t)it * p.theta_stride + h] : kappa;
           const float inv2th = th > 0.f ? 0.5f / th : 0.f;        // theta = 0: sat(1/2) = 1/2 and eta(x) = x
           const F2 m2th2 = pack2(-2.f * th, -2.f * th);
           const F2 dk2 = pack2(th - kappa, th - kappa);
@@ -674,8 +676,8 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
               unpack2(x2, x0, x1);
               if (kMasks) push_x(th, x0, x1, c0);
               const F2 t2 = pack2(fma_sat(x0, inv2th, 0.5f), fma_sat(x1, inv2th, 0.5f));
-              const F2 bn = add2(fma2(t2, m2th2, x2), dk2);            // eta_theta(x) - kappa
-              const F2 dn = add2(fma2(t2, m2th2, r2), dk2);            // alpha^{t+1} - alpha^t
+              F2 bn = fma2(t2, m2th2, x2), dn = fma2(t2, m2th2, r2);   // eta_theta(x) - theta; alpha^{t+1} - alpha^t
+              if (kDiffer) { bn = add2(bn, dk2); dn = add2(dn, dk2); }   // ... - kappa
               v2[(c0 + e) >> 1] = bn;
               float d0, d1;
               unpack2(dn, d0, d1);
@@ -790,6 +792,7 @@ cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream
 #define CSAT_TILE(DEC, BUFS) launch<0, DEC, BUFS>(c, Q, out, s, nullptr, 0, nullptr, nullptr, nullptr, wait_first)
   const Params& p = c->p;
   if (c->w_S && c->w_untied && p.T > 0) return CSAT_TILE(kPerLayer, 1);
+  if (c->thr_stride() != 0) return CSAT_TILE(kThresholds, 1);
   if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return CSAT_TILE(kTied, 1);
   // one positive threshold for all layers
   if (few_tiles(c)) return CSAT_TILE(kUnits, 2);

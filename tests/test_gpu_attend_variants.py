@@ -51,4 +51,14 @@ def test_thresholds_and_sizes(B, H, nq, m):
     Q, K, V = (_randn(g, B, H, r, D).bfloat16() for r in (nq, n, n))
     ctx = binding.Csat(n, m, D, H, 3, B=B, n_q=nq, dtype="bf16", T=T, lam=0.001)
     _check(ctx, Q, K, V, "one threshold", T=T, lam=0.001)
+    ctx.set(lam=0.0)
+    _check(ctx, Q, K, V, "no threshold", T=T, lam=0.0)
+    S = (0.6 * torch.eye(D, device="cuda") + 0.05 * _randn(g, H, D, D)).bfloat16()
+    Bm = (0.125 * _randn(g, H, D, D)).bfloat16()
+    theta = 0.02 * (0.2 + 1.3 * torch.rand(T, H, generator=g, device="cuda"))
+    for th in (theta, theta[:1]):
+        ctx.set_lista_weights(S, Bm, th.contiguous())
+        each = th.expand(T, H)
+        _check(ctx, Q, K, V, ("weights", len(th)), T=T, lam=0.0,
+               weights=lambda h: (to_np(S[h]), to_np(Bm[h]), [float(x) for x in each[:, h]]))
     ctx.close()
