@@ -62,3 +62,44 @@ def test_thresholds_and_sizes(B, H, nq, m):
         _check(ctx, Q, K, V, ("weights", len(th)), T=T, lam=0.0,
                weights=lambda h: (to_np(S[h]), to_np(Bm[h]), [float(x) for x in each[:, h]]))
     ctx.close()
+
+
+@pytest.mark.parametrize("B,H,nq,m", [
+    (1, 12, 100, 200),      # 64 queries per CTA of the warp kernel
+    (2, 50, 90, 190),       # 128
+    (2, 80, 128, 250),      # two score buffers
+    (2, 140, 250, 200),
+    (2, 120, 160, 200),     # one
+    (8, 152, 31, 200),      # B folded into the values
+])
+def test_scores_that_rise_from_chunk_to_chunk(B, H, nq, m):
+    """Row r of K~ is near u r / 64: a row's scores rise (or fall, by the sign of its query) by about 7 = 10 log2 units a chunk of 64, more
+    than the 8 that a reference may lag behind, so that every chunk rescales what half of a warp's rows have summed up.  K~ is rounded to
+    2^-9 of its values, which moves a score of at most 36 by 36 2^-9 / sqrt(64) = 0.9 %."""
+    n, T, lam = 256, 3, 1e-3
+    g = torch.Generator(device="cuda").manual_seed(m)
+    u = (2 * torch.randint(0, 2, (D,), generator=g, device="cuda") - 1).float()
+    sign = (2 * torch.randint(0, 2, (B, H, nq, 1), generator=g, device="cuda") - 1).float()
+    Q = (sign * u + 0.1 * _randn(g, B, H, nq, D)).bfloat16()
+    K = (u + 0.2 * _randn(g, B, H, n, D)).bfloat16()
+    V = _randn(g, B, H, n, D).bfloat16()
+    ramp = 0.875 * torch.arange(m, device="cuda") / 64 / n
+    phi = (ramp[None, :, None] + 0.04 / n ** 0.5 * _randn(g, H, m, n)).bfloat16()
+    ctx = binding.Csat(n, m, D, H, 3, B=B, n_q=nq, dtype="bf16", T=T, lam=lam)
+    ctx.set_phi(phi)
+    st = {}
+    orc.csat_forward_head(to_np(Q[0, 0]), to_np(K[0, 0]), to_np(V[0, 0]), to_np(phi[0]), T=0, lam=0.0, stages=st)
+    s = np.sign(to_np(sign[0, 0])) * (to_np(Q[0, 0]) @ st["Kt"].T) / 8 / np.log(2)
+    tops = [s[:, c:c + 64].max(1) for c in range(0, m - m % 64, 64)]
+    assert all((b - a > 8).mean() > 0.8 for a, b in zip(tops, tops[1:]))
+    eye = (torch.eye(D, device="cuda") + 0.03 * _randn(g, H, D, D)).bfloat16()
+    ctx.set(T=0)
+    _check(ctx, Q, K, V, "no decoder", T=0, lam=0.0)
+    ctx.set(T=T)
+    ctx.set_decoder_matrix(eye)
+    _check(ctx, Q, K, V, "derived", T=T, lam=lam, D=lambda h: to_np(eye[h]))
+    th = torch.full((T, H), 1e-3, device="cuda")
+    Sl, Bl = (x[None].expand(T, H, D, D).contiguous() for x in (0.1 * eye, eye))
+    ctx.set_lista_layer_weights(Sl, Bl, th)
+    _check(ctx, Q, K, V, "per layer", T=T, lam=0.0, weights=lambda h: (to_np(Sl[:, h]), to_np(Bl[:, h]), [1e-3] * T))
+    ctx.close()

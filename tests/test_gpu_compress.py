@@ -1,8 +1,10 @@
 """bf16 compression on the tensor cores, one shape or more for every way a measurement tile is dealt out (K and V columns together
-or in CTAs of their own, one or two tiles per CTA), with ragged token and measurement counts and an odd batch: K~ and V~ against float64 products with the matrix the library exports.
+or in CTAs of their own, one or two tiles per CTA, a batch element alone, a matrix of its own for the values), with ragged token and
+measurement counts and an odd batch: K~ and V~ against float64 products with the matrix the library exports.
 
-Bound: the products of bf16 numbers are exact in float32 and their sums lose at most n 2^-24 of the sum of magnitudes (n <= 1100:
-7e-5 of it, and that is at most sqrt(n) = 33 times the typical result: 2e-3 of the largest); the result is rounded once, 2^-8."""
+Bound: the result is rounded to bf16 once, 2^-8 of itself.  The products of bf16 numbers are exact in float32; the roundings of their sum
+act like n random ones of 2^-24 of partial sums that grow to the result's typical size: sqrt(n) 2^-24 <= 2e-6 of the largest (n <= 1100),
+and four times that is allowed (2e-3 2^-8 = 7.8e-6)."""
 import numpy as np
 import pytest
 import torch
@@ -20,6 +22,7 @@ pytestmark = pytest.mark.gpu
     (5, 40, 200, 130, 64),      # two tiles per CTA
     (7, 20, 1100, 511, 64),     # the same, odd batch, ragged in everything
     (8, 30, 400, 300, 64),      # three tiles
+    (1, 20, 700, 190, 64),      # a batch of one
     (2, 8, 777, 187, 128),      # d = 128, K and V apart
     (3, 25, 515, 135, 128),     # one tile per CTA, K and V together
     (4, 32, 300, 256, 128),     # two tiles per CTA
@@ -34,6 +37,23 @@ def test_compression_of_every_kind(B, H, n, m, d):
     phi = torch.from_numpy(to_np(ctx.get_phi())).cuda()
     for got, x in zip(ctx.get_compressed(), (K, V)):
         ref = phi @ x.double()
+        bound = 2.0 ** -8 * ref.abs() + 2e-3 * 2.0 ** -8 * ref.abs().max()
+        assert got.shape == ref.shape and bool(((got.double() - ref).abs() <= bound).all()), (got.double() - ref).abs().max().item()
+    ctx.close()
+
+
+@pytest.mark.parametrize("B,H,n,m,d", [(3, 5, 331, 200, 64), (1, 9, 515, 129, 64), (2, 6, 777, 187, 128)])
+def test_compression_with_a_matrix_of_its_own_for_the_values(B, H, n, m, d):
+    ctx = binding.Csat(n, m, d, H, 3, B=B, n_q=16, dtype="bf16", T=1, lam=0.05)
+    ctx.set(separate_phi=True)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + m)
+    K, V = (torch.randn(B, H, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    ctx.forward(torch.randn(B, H, 16, d, generator=g, device="cuda").bfloat16(), K, V)
+    phi = torch.from_numpy(to_np(ctx.get_phi())).cuda()
+    assert not torch.equal(phi[:H], phi[H:])
+    for got, x, p in zip(ctx.get_compressed(), (K, V), (phi[:H], phi[H:])):
+        ref = p @ x.double()
         bound = 2.0 ** -8 * ref.abs() + 2e-3 * 2.0 ** -8 * ref.abs().max()
         assert got.shape == ref.shape and bool(((got.double() - ref).abs() <= bound).all()), (got.double() - ref).abs().max().item()
     ctx.close()

@@ -12,7 +12,7 @@ def _randn(seed, *shape, dtype=torch.bfloat16):
     return torch.randn(*shape, generator=g, device="cuda").to(dtype)
 
 
-@pytest.mark.parametrize("d, H, n_q", [(64, 2, 70), (64, 40, 300), (128, 2, 70), (128, 3, 300)])
+@pytest.mark.parametrize("d, H, n_q", [(64, 2, 70), (64, 40, 300), (64, 110, 300), (128, 2, 70), (128, 3, 300)])
 def test_decisions_of_rows_that_are_not_finite(d, H, n_q):
     """|NaN| > theta is false: a NaN in the values of head 0 makes every pre-activation of that head NaN, and none of its
     decisions is recorded as taken; the other heads' decisions and gradients keep their bits."""
