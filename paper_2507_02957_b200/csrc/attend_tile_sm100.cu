@@ -781,8 +781,9 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
 
 // Two score buffers where an SM holds at most two tiles: S_{j+1} is formed under chunk j's exponentials.  Between three and four tiles per
 // SM two rounds of two take the place of two of three, unless there is a single chunk.  us, two buffers / one: 592 tiles, m = 256, T =
-// 20 37.8 / 38.3; 512 36.6 / 37.8, T = 10 25.9 / 27.1; 512, m = 64 21.2 / 20.8; 300, m = 256, T = 20 38 / 27.  By the context's whole job,
-// not the launch's range of (batch, head) pairs.
+// 20 37.8 / 38.3; 512 36.6 / 37.8, T = 10 25.9 / 27.1; 512, m = 64 21.2 / 20.8; 300, m = 256, T = 20 38 / 27; 128, m = 392, T = 0 11.8 / 13.7; one
+// S_t, B_t per layer: 128, m = 392, T = 10 20.7 / 22.9; 592, m = 256, T = 20 45.6 / 47.9.  By the context's whole job, not the launch's range
+// of (batch, head) pairs.
 static bool few_tiles(const csat_ctx* c) {
   const int64_t tiles = (c->p.nq + kRows - 1) / kRows * c->p.B * c->p.H;
   return tiles <= 2 * (int64_t)c->sms || (c->p.m > kMC && two_tiles_per_sm(tiles, c->sms));
@@ -791,9 +792,9 @@ static bool few_tiles(const csat_ctx* c) {
 cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream_t s, int* launches, bool wait_first) {
 #define CSAT_TILE(DEC, BUFS) launch<0, DEC, BUFS>(c, Q, out, s, nullptr, 0, nullptr, nullptr, nullptr, wait_first)
   const Params& p = c->p;
-  if (c->w_S && c->w_untied && p.T > 0) return CSAT_TILE(kPerLayer, 1);
-  if (c->thr_stride() != 0) return CSAT_TILE(kThresholds, 1);
-  if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return CSAT_TILE(kTied, 1);
+  if (c->w_S && c->w_untied && p.T > 0) return few_tiles(c) ? CSAT_TILE(kPerLayer, 2) : CSAT_TILE(kPerLayer, 1);
+  if (c->thr_stride() != 0) return CSAT_TILE(kThresholds, 1);       // (156 tiles, m = 128, T = 10: 22.8 us with two buffers as well)
+  if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return few_tiles(c) ? CSAT_TILE(kTied, 2) : CSAT_TILE(kTied, 1);
   // one positive threshold for all layers
   if (few_tiles(c)) return CSAT_TILE(kUnits, 2);
   if (p.T >= 2 && (p.nq + kRows - 1) / kRows * p.B * p.H >= 8 * (int64_t)c->sms) {

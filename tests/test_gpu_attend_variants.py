@@ -53,6 +53,9 @@ def test_thresholds_and_sizes(B, H, nq, m):
     _check(ctx, Q, K, V, "one threshold", T=T, lam=0.001)
     ctx.set(lam=0.0)
     _check(ctx, Q, K, V, "no threshold", T=T, lam=0.0)
+    ctx.set(T=0)
+    _check(ctx, Q, K, V, "no decoder", T=0, lam=0.0)
+    ctx.set(T=T)
     S = (0.6 * torch.eye(D, device="cuda") + 0.05 * _randn(g, H, D, D)).bfloat16()
     Bm = (0.125 * _randn(g, H, D, D)).bfloat16()
     theta = 0.02 * (0.2 + 1.3 * torch.rand(T, H, generator=g, device="cuda"))
@@ -61,6 +64,13 @@ def test_thresholds_and_sizes(B, H, nq, m):
         each = th.expand(T, H)
         _check(ctx, Q, K, V, ("weights", len(th)), T=T, lam=0.0,
                weights=lambda h: (to_np(S[h]), to_np(Bm[h]), [float(x) for x in each[:, h]]))
+    for L in (1, T):                                            # one S_t, B_t per layer
+        Sl, Bl = (x[None] + 0.02 * _randn(g, L, H, D, D) for x in (S.float(), Bm.float()))
+        Sl, Bl = Sl.bfloat16(), Bl.bfloat16()
+        ctx.set(T=L)
+        ctx.set_lista_layer_weights(Sl, Bl, theta[:L].contiguous())
+        _check(ctx, Q, K, V, ("layers", L), T=L, lam=0.0,
+               weights=lambda h: (to_np(Sl[:, h]), to_np(Bl[:, h]), [float(x) for x in theta[:L, h]]))
     ctx.close()
 
 
