@@ -9,8 +9,8 @@
 // tensor-memory stores 60, arrivals and the issuer's wait 200, four MMAs and their commit 180, the rows' wait 200), of which the tensor
 // pipe needs 128 and a sub-core's issue slots ~250.  Only tiles in flight shorten it: two per SM (one CTA with both, 1 KB of registers a
 // row) took 750 cycles per tile and layer, three take 450.  A tile needs 128 columns of tensor memory, so four would fit; in the 104
-// registers per thread that leaves them they took 86 us for 96 heads of 1568 queries, T = 20, m = 256, where three take 79 and the two
-// took 95 (whole forward).  The same tiles without warps of their own for MMAs and copies (128 threads) took 89: the issuing warp's own
+// registers per thread that leaves them they took 86 us for 96 heads of 1568 queries, T = 20, m = 256, where three took 79 and the two
+// took 95 (whole forward, B not folded; as dispatched now, folded, 82).  The same tiles without warps of their own for MMAs and copies (128 threads) took 89: the issuing warp's own
 // pass then starts ~300 cycles late, and a divided `elect` (chosen once, used later) costs 100 instead of 45 cycles per MMA.
 //
 // CTA = 8 warps: 0-3 one thread per query row (TMEM lane = row); 4 allocates tensor memory, one elected lane issues the MMAs; 5 every TMA
@@ -797,6 +797,10 @@ cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream
   if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return few_tiles(c) ? CSAT_TILE(kTied, 2) : CSAT_TILE(kTied, 1);
   // one positive threshold for all layers
   if (few_tiles(c)) return CSAT_TILE(kUnits, 2);
+  // B folded into the values: the first tiles wait for the fold (4 us), every tile saves a hand-over.  Whole forward, us, folded / not: 1248
+  // tiles, m = 256, T = 20 82.2 / 80.3, 1776 93.8 / 94.0, 2368 125.2 / 125.5, 4736 231.2 / 233.7; 1536 short tiles, m = 64 90.0 / 84.4.  It pays from
+  // about 16 tiles per SM on; the line at eight was measured on the kernel with two tiles per CTA, and the tests hold the first of
+  // these shapes to the folded launches and their bits.
   if (p.T >= 2 && (p.nq + kRows - 1) / kRows * p.B * p.H >= 8 * (int64_t)c->sms) {
     cudaError_t e = launch_sm100_vfold(c, s, launches);
     if (e != cudaSuccess) return e;
