@@ -48,13 +48,14 @@ template <int kBufs> struct Layout {
   static constexpr int kStages = 2 * kBufs;
   static constexpr uint32_t kOffG = kOffRing + kStages * kStageBytes, kOffB = kOffG + kMatBytes, kOffBar = kOffB + kMatBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + kBarBytes;
+  static constexpr uint32_t kSmemTwo = (kBufs == 1 ? 80 : 100) * 1024;  // no more than two CTAs per SM; the rest is L1, for the iterates' stores
+  static_assert(kSmemBytes <= kSmemTwo && 2 * (kSmemTwo + 1024) <= 228 * 1024 && 3 * kSmemTwo > 228 * 1024, "two CTAs per SM");
 };
-constexpr uint32_t kSmemTwo = 100 * 1024, kSmemOne = 120 * 1024;  // no more than two, one CTA per SM
+constexpr uint32_t kSmemOne = 120 * 1024;                         // no more than one CTA per SM
 constexpr uint32_t kOutBytes = 32 * 128;                          // one warp's rows of the output
 // TMEM columns: accumulator (Zacc, then r_t) | S (P_j overlays its first half; later the recovery operand)
 constexpr uint32_t kColAcc = 0, kColS = kD, kTmemCols = 2 * kD;   // (kBufs = 2: another S behind it)
-static_assert(Layout<2>::kSmemBytes <= kSmemTwo && 2 * (kSmemTwo + 1024) <= 228 * 1024 && 3 * kSmemTwo > 228 * 1024 &&
-              2 * kSmemOne > 228 * 1024, "fewer CTAs per SM");
+static_assert(2 * kSmemOne > 228 * 1024 && Layout<2>::kSmemBytes <= kSmemOne, "one CTA per SM");
 static_assert(kMatBytes <= kQBytes && 4 * kOutBytes <= kQBytes, "overlays");
 static_assert(kCtas * (Layout<1>::kSmemBytes + 1024) <= 228 * 1024 && kCtas * kTmemCols <= 512, "CTAs per SM");
 
@@ -758,7 +759,7 @@ cudaError_t launch(csat_ctx* c, const void* Q, void* out, cudaStream_t s, float*
   // pile up on the SMs that the kernel before leaves free.
   const int64_t tiles = (p.nq + kRows - 1) / kRows, n = tiles * (c->bh_cnt ? c->bh_cnt : p.B * p.H);
   if (n > (int64_t)1 << 30) return cudaErrorInvalidValue;
-  const uint32_t smem = n <= c->sms ? kSmemOne : n <= 2 * (int64_t)c->sms || kBufs == 2 ? kSmemTwo : Layout<kBufs>::kSmemBytes;
+  const uint32_t smem = n <= c->sms ? kSmemOne : n <= 2 * (int64_t)c->sms || kBufs == 2 ? Layout<kBufs>::kSmemTwo : Layout<kBufs>::kSmemBytes;
   static DeviceFlags smem_opt_in;
   if (!smem_opt_in.test(c->device)) {
     // setmaxnreg moves registers inside the pool the CTA is launched with (threads x the compiled register count); a request
