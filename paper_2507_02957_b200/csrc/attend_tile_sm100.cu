@@ -641,6 +641,9 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
 #pragma unroll
     for (int i = 0; i < kD / 2; ++i) v2[i] = pack2(off, off);
     for (int it = 0; it + 1 < T; ++it) {
+      // thresholds that differ are loaded while the products run (156 tiles, T = 10: 21.0 -> 19.0 us)
+      const float th_it = kDec == kThresholds ? p.theta[(int64_t)it * p.theta_stride + h] : kappa;
+      const float inv_it = th_it > 0.f ? 0.5f / th_it : 0.f;
       if (!kFold || it > 0) wait_done(246);
       if (live) {
         if (scaled_units) {
@@ -661,10 +664,9 @@ attend_tile_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_cons
             tmem_st_32x32b_x8(op_addr + c0 / 2, pk);
           });
         } else {
-          // the add of theta_t - kappa and the loads of thresholds cost 0.1 us a layer: only where thresholds differ
-          constexpr bool kDiffer = kDec == kThresholds || kMasks;
-          const float th = kDiffer ? p.theta[(int64_t)it * p.theta_stride + h] : kappa;
-          const float inv2th = th > 0.f ? 0.5f / th : 0.f;        // theta = 0: sat(1/2) = 1/2 and eta(x) = x
+          constexpr bool kDiffer = kDec == kThresholds || kMasks;      // (the add costs 0.1 us a layer)
+          const float th = kMasks ? p.theta[(int64_t)it * p.theta_stride + h] : th_it;
+          const float inv2th = kMasks ? (th > 0.f ? 0.5f / th : 0.f) : inv_it;    // theta = 0: sat(1/2) = 1/2 and eta(x) = x
           const F2 m2th2 = pack2(-2.f * th, -2.f * th);
           const F2 dk2 = pack2(th - kappa, th - kappa);
           pieces([&](const uint32_t (&r)[16], int c0) {
@@ -794,7 +796,7 @@ cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream
 #define CSAT_TILE(DEC, BUFS) launch<0, DEC, BUFS>(c, Q, out, s, nullptr, 0, nullptr, nullptr, nullptr, wait_first)
   const Params& p = c->p;
   if (c->w_S && c->w_untied && p.T > 0) return few_tiles(c) ? CSAT_TILE(kPerLayer, 2) : CSAT_TILE(kPerLayer, 1);
-  if (c->thr_stride() != 0) return CSAT_TILE(kThresholds, 1);       // (156 tiles, m = 128, T = 10: 22.8 us with two buffers as well)
+  if (c->thr_stride() != 0) return few_tiles(c) ? CSAT_TILE(kThresholds, 2) : CSAT_TILE(kThresholds, 1);
   if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return few_tiles(c) ? CSAT_TILE(kTied, 2) : CSAT_TILE(kTied, 1);
   // one positive threshold for all layers
   if (few_tiles(c)) return CSAT_TILE(kUnits, 2);
