@@ -655,6 +655,7 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
     return fail(c, CSAT_ERR_TIMEOUT, "a bounded device-side wait of an earlier launch gave up; its output is invalid");
   cudaStream_t s = (cudaStream_t)stream;
   int launches = 0;
+  c->saved_valid = false;                  // from here on K~|V~ may be overwritten
   prof_mark(c, s, -1);
   if (c->p.T > 0 && c->w_S && (c->w_layers != 1 || c->w_untied) && c->w_layers != c->p.T)
     return fail(c, CSAT_ERR_STATE, "the supplied LISTA weights are for a number of layers other than CSAT_T");
@@ -676,7 +677,6 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
     e = tc_compress ? csat::launch_sm100_compress(c, K, V, s, &launches) : csat::launch_simt_compress(c, K, V, s, &launches);
   if (e != cudaSuccess) return fail_cuda(c, e, "compress launch");
   prof_mark(c, s, CSAT_KERNEL_COMPRESS);
-  c->saved_valid = false;
   if (c->save_for_backward && tc_attend && c->p.B * c->p.H <= 32767) {
     // the recording variant of the same kernel: the output, and Z, the rows' log sum exp, the layers' decisions (and
     // the iterates with CSAT_WEIGHT_GRADS) where csat_backward will look for them
@@ -875,6 +875,7 @@ int csat_backward(csat_ctx* c, const void* Q, const void* K, const void* V, cons
                    (fp32_can_save(c) || (c->tmap_phi_valid && c->force_simt == 0 && (!c->weight_grads || c->saved_alpha)));
   cudaError_t e = cudaSuccess;
   if (!c->reuse_saved) {
+    c->saved_valid = false;                // this call's own forward pass overwrites it
     e = c->debug_canary ? cudaMemsetAsync(c->kv, 0xFF, kv_bytes(p), s) : cudaSuccess;
     if (e != cudaSuccess) return fail_cuda(c, e, "canary fill");
     e = tc_compress ? csat::launch_sm100_compress(c, K, V, s, &launches) : csat::launch_simt_compress(c, K, V, s, &launches);
@@ -931,7 +932,11 @@ int csat_forward_host(csat_ctx* c, const void* Qh, const void* Kh, const void* V
         (e = cudaMemcpyAsync(c->stage_k, Kh, bkv, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(c->stage_v, Vh, bkv, cudaMemcpyHostToDevice, s)) != cudaSuccess)
       return fail_cuda(c, e, "host->device copy");
+    // No state of the staged tensors for a backward: the next csat_backward is on others
+    const bool save = c->save_for_backward;
+    c->save_for_backward = false;
     int rc = csat_forward(c, c->stage_q, c->stage_k, c->stage_v, c->stage_o, stream);
+    c->save_for_backward = save;
     if (rc != CSAT_OK) return rc;
     if ((e = cudaMemcpyAsync(outh, c->stage_o, bq, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
       return fail_cuda(c, e, "device->host copy");

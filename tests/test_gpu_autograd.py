@@ -44,3 +44,27 @@ def test_module_owns_a_context():
     assert out.shape == (1, 2, 256, 64) and torch.isfinite(out).all()
     out.float().sum().backward()
     assert all(t.grad is not None and torch.isfinite(t.grad).all() for t in (Q, K, V))
+
+
+@pytest.mark.parametrize("dtype,d,profile", [("fp32", 32, 0), ("fp32", 64, 0), ("bf16", 64, 4), ("bf16", 128, 4), ("bf16", 64, 0), ("bf16", 96, 0)])
+def test_other_calls_between_a_forward_and_its_backward(dtype, d, profile):
+    """Whatever else the context computes in between, on other data, the gradients are those of the forward's own tensors, bit for
+    bit as without saved state."""
+    from paper_2507_02957_b200.autograd import csat_attention
+    B, H, n, nq, m, T = 2, 3, 143, 90, 72 if d < 96 else 130, 4
+    g = torch.Generator(device="cuda").manual_seed(d)
+    ctx = binding.Csat(n, m, d, H, 3, B=B, n_q=nq, dtype=dtype, T=T, lam=0.02)
+    binding.csat_set_i64(ctx.h, binding.CSAT_PROFILE, profile)
+    Q, K, V, G, Q2, K2, V2 = (torch.randn(B, H, r, d, generator=g, device="cuda").to(ctx.torch_dtype) for r in (nq, n, n, nq, nq, n, n))
+    want = ctx.backward(Q, K, V, G)
+    host = [t.cpu() for t in (Q2, K2, V2, Q2)]
+    between = {"forward_host": lambda: ctx.forward_host(*host), "forward": lambda: ctx.forward(Q2, K2, V2), "attend": lambda: ctx.attend(Q2),
+               "compress": lambda: ctx.reduce_partials(torch.stack([ctx.compress_partial(K2[:, :, :80].contiguous(), V2[:, :, :80].contiguous(), 0)])),
+               "none": lambda: None}
+    for name, call in between.items():
+        leaves = [t.clone().requires_grad_(True) for t in (Q, K, V)]
+        out = csat_attention(ctx, *leaves)
+        call()
+        grads = torch.autograd.grad(out, leaves, G)
+        assert all(torch.equal(a, b) for a, b in zip(grads, want)), name
+    ctx.close()
