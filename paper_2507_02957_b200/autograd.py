@@ -2,8 +2,8 @@
 
 `csat_attention(ctx, Q, K, V)` runs `csat_forward` through a `binding.Csat` context and, under autograd, registers
 `csat_backward` as its backward, so that the compressed-sensing attention can sit inside a torch model.  With
-`save_for_backward=True` (the default) the forward keeps what the backward needs (CSAT_SAVE_FOR_BACKWARD), and the
-backward starts from it instead of recomputing.  Every step of the path runs in the library's kernels; nothing here
+`save_for_backward=True` (the default) the forward of inputs that require gradients keeps what the backward needs
+(CSAT_SAVE_FOR_BACKWARD), and the backward starts from it instead of recomputing.  Every step of the path runs in the library's kernels; nothing here
 computes.
 
 The gradients with respect to the decoder's parameters and to the measurement matrices are not torch leaves of this
@@ -38,7 +38,9 @@ def csat_attention(csat, Q, K, V, save_for_backward=True):
     """Compressed-sensing attention of Q [B,H,n_q,d], K, V [B,H,n,d] through the context `csat` (a binding.Csat of that
     shape and dtype), differentiable with respect to Q, K, V.  The context holds the saved state of its last forward; the
     backward of an earlier one recomputes."""
-    return _CsatFunction.apply(csat, Q, K, V, save_for_backward)
+    # decided here: inside the function gradients are always off
+    save = save_for_backward and torch.is_grad_enabled() and (Q.requires_grad or K.requires_grad or V.requires_grad)
+    return _CsatFunction.apply(csat, Q, K, V, save)
 
 
 class CsatAttention(torch.nn.Module):

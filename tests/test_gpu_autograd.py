@@ -68,3 +68,25 @@ def test_other_calls_between_a_forward_and_its_backward(dtype, d, profile):
         grads = torch.autograd.grad(out, leaves, G)
         assert all(torch.equal(a, b) for a, b in zip(grads, want)), name
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("fp32", 32), ("bf16", 64), ("bf16", 128)])
+def test_nothing_is_recorded_where_no_gradient_can_be_asked_for(dtype, d):
+    """Without gradients (or inputs that require none) csat_attention is Csat.forward: the same bits, no scratch of the backward."""
+    from paper_2507_02957_b200.autograd import CsatAttention
+    mod = CsatAttention(256, 130, d, 2, B=2, n_q=70, T=4, lam=0.01, seed=5, dtype=dtype)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    Q, K, V = (torch.randn(2, 2, r, d, device="cuda", generator=g).to(mod.csat.torch_dtype) for r in (70, 256, 256))
+    want, before = mod.csat.forward(Q, K, V), mod.csat.workspace_bytes
+    leaves = [t.clone().requires_grad_(True) for t in (Q, K, V)]
+    with torch.no_grad():
+        assert torch.equal(mod(*leaves), want)
+    assert torch.equal(mod(Q, K, V), want) and mod.csat.workspace_bytes == before
+    out = mod(Q, leaves[1], V)                              # one of them is enough
+    assert mod.csat.workspace_bytes > before
+    with torch.no_grad():                                   # and a call without gradients takes nothing from it
+        mod(Q, K, V)
+    G = torch.randn(out.shape, device="cuda", generator=g).to(out.dtype)
+    dK, = torch.autograd.grad(out, leaves[1:2], G)
+    binding.csat_set_i64(mod.csat.h, binding.CSAT_SAVE_FOR_BACKWARD, 0)
+    assert torch.equal(dK, mod.csat.backward(Q, K, V, G)[1])
