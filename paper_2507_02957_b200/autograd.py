@@ -19,8 +19,11 @@ class _CsatFunction(torch.autograd.Function):
     @staticmethod
     def forward(fn_ctx, csat, Q, K, V, save):
         Q, K, V = Q.contiguous(), K.contiguous(), V.contiguous()
-        binding.csat_set_i64(csat.h, binding.CSAT_SAVE_FOR_BACKWARD, 1 if save else 0)
-        out = csat.forward(Q, K, V)
+        user = binding._set_saving(csat.h, save)
+        try:
+            out = csat.forward(Q, K, V)
+        finally:
+            csat.h.user_saves = user
         fn_ctx.csat, fn_ctx.forward_no = csat, csat.forwards
         fn_ctx.save_for_backward(Q, K, V)
         return out
@@ -28,9 +31,16 @@ class _CsatFunction(torch.autograd.Function):
     @staticmethod
     def backward(fn_ctx, dOut):
         Q, K, V = fn_ctx.saved_tensors
-        if fn_ctx.csat.forwards != fn_ctx.forward_no:      # another forward has been here: its state is not this one's
-            binding.csat_set_i64(fn_ctx.csat.h, binding.CSAT_SAVE_FOR_BACKWARD, 0)
-        dQ, dK, dV = fn_ctx.csat.backward(Q, K, V, dOut.contiguous())
+        csat = fn_ctx.csat
+        if csat.forwards != fn_ctx.forward_no or csat.h.user_saves is None:
+            # another forward has been here, or another setting: what state there is is not this forward's
+            user = binding._set_saving(csat.h, False)
+        else:
+            user, csat.h.user_saves = csat.h.user_saves, None
+        try:
+            dQ, dK, dV = csat.backward(Q, K, V, dOut.contiguous())
+        finally:
+            csat.h.user_saves = user
         return None, dQ, dK, dV, None
 
 

@@ -117,6 +117,25 @@ def _check(handle, rc):
         raise CsatError(rc, (load().csat_last_error(handle) or b"").decode())
 
 
+class _Handle(C.c_void_p):
+    """A context's handle.  user_saves: CSAT_SAVE_FOR_BACKWARD as it was when csat_attention set it for its own forward;
+    None: the key is the user's.  csat_attention's setting, and the state its forward has left, are for its own backward
+    alone: direct calls of csat_forward and csat_backward, which may be on other tensors, put the user's setting back first
+    (which drops the state)."""
+    user_saves = None
+
+
+def _restore_saving(h):
+    csat_set_i64(h, CSAT_SAVE_FOR_BACKWARD, h.user_saves)
+
+
+def _set_saving(h, save):
+    """Sets the key for csat_attention, which then calls the library and stores what this returns in h.user_saves."""
+    user = h.user_saves if h.user_saves is not None else csat_get_i64(h, CSAT_SAVE_FOR_BACKWARD)
+    csat_set_i64(h, CSAT_SAVE_FOR_BACKWARD, int(save))
+    return user
+
+
 # ---- thin functions, one per C entry point -------------------------------------------------
 def csat_version() -> int:
     return load().csat_version()
@@ -126,7 +145,7 @@ def csat_create(n, m, d, H, seed):
     h = load().csat_create(n, m, d, H, seed)
     if not h:
         raise CsatError(0, (load().csat_last_error(None) or b"").decode())
-    return C.c_void_p(h)
+    return _Handle(h)
 
 
 def csat_destroy(h):
@@ -134,6 +153,8 @@ def csat_destroy(h):
 
 
 def csat_set_i64(h, key, v):
+    if key == CSAT_SAVE_FOR_BACKWARD and isinstance(h, _Handle):
+        h.user_saves = None
     _check(h, load().csat_set_i64(h, key, int(v)))
 
 
@@ -183,6 +204,8 @@ def csat_project_qkv(h, Xq, Xkv, W, d_model, Q, K, V, stream=None):
 
 
 def csat_forward(h, Q, K, V, out, stream=None):
+    if getattr(h, "user_saves", None) is not None:
+        _restore_saving(h)
     _check(h, load().csat_forward(h, _ptr(Q), _ptr(K), _ptr(V), _ptr(out), _stream(stream)))
 
 
@@ -200,6 +223,8 @@ def csat_attend(h, Q, out, stream=None):
 
 
 def csat_backward(h, Q, K, V, dOut, dQ, dK, dV, stream=None):
+    if getattr(h, "user_saves", None) is not None:
+        _restore_saving(h)
     _check(h, load().csat_backward(h, _ptr(Q), _ptr(K), _ptr(V), _ptr(dOut), _ptr(dQ), _ptr(dK), _ptr(dV),
                                    _stream(stream)))
 

@@ -90,3 +90,46 @@ def test_nothing_is_recorded_where_no_gradient_can_be_asked_for(dtype, d):
     dK, = torch.autograd.grad(out, leaves[1:2], G)
     binding.csat_set_i64(mod.csat.h, binding.CSAT_SAVE_FOR_BACKWARD, 0)
     assert torch.equal(dK, mod.csat.backward(Q, K, V, G)[1])
+
+
+@pytest.mark.parametrize("dtype,d", [("fp32", 64), ("bf16", 64), ("bf16", 128)])
+def test_direct_calls_beside_csat_attention(dtype, d):
+    """The key that csat_attention sets is its own: a direct backward on other tensors does not start from its forward's state, a
+    direct forward does not record, and a key set by hand stays as it was set."""
+    from paper_2507_02957_b200.autograd import csat_attention
+    KEY = binding.CSAT_SAVE_FOR_BACKWARD
+    B, H, n, nq, m, T = 2, 3, 143, 90, 130, 4
+    g = torch.Generator(device="cuda").manual_seed(d)
+    ctx = binding.Csat(n, m, d, H, 3, B=B, n_q=nq, dtype=dtype, T=T, lam=0.02)
+    x, y = ([torch.randn(B, H, r, d, generator=g, device="cuda").to(ctx.torch_dtype) for r in (nq, n, n, nq)] for _ in range(2))
+    out_y, want_x, want_y = ctx.forward(*y[:3]), ctx.backward(*x), ctx.backward(*y)
+    same = lambda got, want: all(torch.equal(a, b) for a, b in zip(got, want))
+    leaves = [t.clone().requires_grad_(True) for t in x[:3]]
+    for by_hand in (None, 1, 0):
+        if by_hand is not None:
+            binding.csat_set_i64(ctx.h, KEY, by_hand)
+        out = csat_attention(ctx, *leaves)
+        assert same(ctx.backward(*y), want_y)
+        assert same(torch.autograd.grad(out, leaves, x[3]), want_x)
+        out = csat_attention(ctx, *leaves)
+        if not by_hand:
+            assert torch.equal(ctx.forward(*y[:3]), out_y)
+        else:
+            ctx.forward(*y[:3])
+            assert same(ctx.backward(*y), want_y)
+        assert binding.csat_get_i64(ctx.h, KEY) == (by_hand or 0)
+        assert same(torch.autograd.grad(out, leaves, x[3]), want_x)
+        out = csat_attention(ctx, *leaves)
+        binding.csat_set_i64(ctx.h, KEY, 1)
+        res = torch.empty_like(y[0])
+        binding.csat_forward(ctx.h, *y[:3], res)
+        assert same(torch.autograd.grad(out, leaves, x[3]), want_x)
+        out = csat_attention(ctx, *leaves)                   # and it still saves: both backwards start from the state
+        launches = []
+        for _ in range(2):
+            assert same(torch.autograd.grad(out, leaves, x[3], retain_graph=True), want_x)
+            launches.append(ctx.launches)
+        binding.csat_set_i64(ctx.h, KEY, 0)
+        ctx.backward(*x)
+        assert max(launches) < ctx.launches
+    ctx.close()
