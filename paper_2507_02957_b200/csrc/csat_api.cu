@@ -129,9 +129,10 @@ void free_backward(csat_ctx* c) {
   dev_free(c, &c->bw_thpart, c->bw_bytes_thpart);
   dev_free(c, &c->bw_wgrad, c->bw_bytes_wgrad);
   dev_free(c, &c->bw_signbits, c->bw_bytes_signbits);
-  c->bw_Z32 = nullptr;                                      // both in the allocation of bw_dZ
+  dev_free(c, &c->bw_save, c->bw_bytes_save);
+  c->bw_Z32 = nullptr;
   c->bw_words = nullptr;
-  c->bw_bytes_Z32 = 0;
+  c->bw_bytes_save = c->bw_bytes_tail = 0;
   c->bw_bytes_signbits = 0;
   c->bw_bytes_alpha16 = c->bw_bytes_dx16 = c->bw_bytes_wpart = c->bw_bytes_thpart = c->bw_bytes_wgrad = 0;
   c->have_wgrads = false;
@@ -334,6 +335,7 @@ int csat_destroy(csat_ctx* c) {
 int csat_set_i64(csat_ctx* c, int key, int64_t v) {
   if (!c) return CSAT_ERR_INVALID_ARG;
   c->saved_valid = false;
+  if (key != CSAT_SAVE_FOR_BACKWARD || (v != 0) != c->save_for_backward) c->save_denied = false;
   csat::Params& p = c->p;
   switch (key) {
     case CSAT_BATCH: {
@@ -628,7 +630,7 @@ static int ensure_decoder(csat_ctx* c, cudaStream_t s, int* launches) {
   return CSAT_OK;
 }
 
-static int ensure_backward_scratch(csat_ctx* c, bool may_allocate = true);
+static int ensure_backward_scratch(csat_ctx* c, bool save = false, bool may_allocate = true);
 
 // float32 contexts whose forward can leave what their backward needs
 static bool fp32_can_save(const csat_ctx* c) {
@@ -690,8 +692,11 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
     // csat_backward recomputes, as without the key
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
-    const bool record = ensure_backward_scratch(c, cap == cudaStreamCaptureStatusNone) == CSAT_OK;
-    if (!record) c->err.clear();
+    bool record = false;
+    if (c->bw_Z32 != nullptr || !c->save_denied) {
+      record = ensure_backward_scratch(c, true, cap == cudaStreamCaptureStatusNone) == CSAT_OK && c->bw_Z32 != nullptr;
+      if (!record) c->err.clear();
+    }
     e = csat::launch_simt_attend_recover(c, Q, out, s, &launches, false, record);
     c->saved_valid = e == cudaSuccess && record;
   } else {
@@ -785,10 +790,10 @@ int csat_attend(csat_ctx* c, const void* Q, void* out, void* stream) {
   return CSAT_OK;
 }
 
-// scratch of csat_backward (and of a csat_forward that saves for it), (re)allocated when a size has changed
-static int ensure_backward_scratch(csat_ctx* c, bool may_allocate) {
+// scratch of csat_backward (and of a csat_forward that saves for it), (re)allocated when a size has changed.  save: with room for
+// what a saving float32 forward leaves, if that can be had (bw_Z32 says so); if not, that is remembered until a size or the key changes
+static int ensure_backward_scratch(csat_ctx* c, bool save, bool may_allocate) {
   const csat::Params& p = c->p;
-  const bool save32 = (c->save_for_backward && fp32_can_save(c)) || c->bw_bytes_Z32 != 0;   // kept once it is there
   const size_t bz = (size_t)(p.B * p.H * p.nq * p.d) * 4, bl = (size_t)(p.B * p.H * c->ld_pitch() * 2) * 4 + 1024 /* read past the end by whole-tile copies */,
                bk = (size_t)(p.B * p.H * p.m * 2 * p.d) * 4,
                bw = p.d > csat::kFfmaMaxD ? (size_t)(2 * (c->w_untied ? c->w_layers : 1) * p.H * p.d * p.d) * 4 : 0,   // transposes
@@ -799,39 +804,58 @@ static int ensure_backward_scratch(csat_ctx* c, bool may_allocate) {
                bdx = c->weight_grads ? (size_t)(p.T * p.B * p.H * p.nq * p.d) * 2 : 0,
                wz = (size_t)(c->w_untied && p.T > 0 ? p.T : 1),      // one dS, dB per layer with per-layer weights
                bwp = c->weight_grads ? (size_t)(csat::wgrad_splits(c) * p.H * 2 * p.d * p.d) * wz * 4 : 0,
-               bz32 = save32 ? bz : 0, bw32 = save32 ? (size_t)(p.B * p.H * p.nq * csat::saved_words_per_row(p.d)) * 4 : 0,
+               bsv = bz + (size_t)(p.B * p.H * p.nq * csat::saved_words_per_row(p.d)) * 4,      // Z, the decisions
                bsg = c->weight_grads ? bmb : 0,
                bth = c->weight_grads ? (size_t)((csat::wgrad_splits(c) > 64 ? csat::wgrad_splits(c) : 64) * p.T * p.H) * 4 : 0,
                bwg = c->weight_grads ? ((size_t)(2 * p.H * p.d * p.d) * wz + (size_t)(p.d * p.d + p.T * p.H)) * 4 : 0;
-  if (c->bw_bytes_Z32 != bz32 || c->bw_bytes_signbits != bsg || c->bw_bytes_alpha16 != bal || c->bw_bytes_dx16 != bdx || c->bw_bytes_wpart != bwp || c->bw_bytes_thpart != bth ||
-      c->bw_bytes_wgrad != bwg || c->bw_bytes_maskbits != bmb || c->bw_bytes_Z16 != z16 || c->bw_bytes_masks != bm || c->bw_bytes_dZ != bz + bz32 + bw32 || c->bw_bytes_LD != bl || c->bw_bytes_dKV != bk || c->bw_bytes_WT != bw ||
-      c->bw_bytes_dKV16 != b16 || c->bw_bytes_dZ16 != z16) {
-    if (!may_allocate) return CSAT_ERR_ALLOC;
-    cudaDeviceSynchronize();
+  auto saved_at = [&](float* at) {
+    c->bw_Z32 = at;
+    c->bw_words = reinterpret_cast<uint32_t*>(at + bz / 4);
+  };
+  if (c->bw_bytes_signbits == bsg && c->bw_bytes_alpha16 == bal && c->bw_bytes_dx16 == bdx && c->bw_bytes_wpart == bwp && c->bw_bytes_thpart == bth &&
+      c->bw_bytes_wgrad == bwg && c->bw_bytes_maskbits == bmb && c->bw_bytes_Z16 == z16 && c->bw_bytes_masks == bm && c->bw_bytes_dZ == bz + c->bw_bytes_tail && c->bw_bytes_LD == bl &&
+      c->bw_bytes_dKV == bk && c->bw_bytes_WT == bw && c->bw_bytes_dKV16 == b16 && c->bw_bytes_dZ16 == z16) {
+    if (save && c->bw_Z32 == nullptr && !c->save_denied && may_allocate) {       // the rest, and the last backward's decisions, stay
+      c->save_denied = dev_alloc(c, &c->bw_save, bsv) != cudaSuccess;
+      if (c->save_denied) {
+        cudaGetLastError();
+      } else {
+        c->bw_bytes_save = bsv;
+        saved_at(c->bw_save);
+      }
+    }
+    return CSAT_OK;
+  }
+  if (!may_allocate) return CSAT_ERR_ALLOC;
+  cudaDeviceSynchronize();
+  auto allocate = [&](size_t tail) {
     free_backward(c);
-    c->bw_bytes_dZ = bz + bz32 + bw32; c->bw_bytes_LD = bl; c->bw_bytes_dKV = bk; c->bw_bytes_WT = bw; c->bw_bytes_dKV16 = b16;
+    c->bw_bytes_dZ = bz + tail; c->bw_bytes_LD = bl; c->bw_bytes_dKV = bk; c->bw_bytes_WT = bw; c->bw_bytes_dKV16 = b16;
     c->bw_bytes_dZ16 = z16;
     c->bw_bytes_masks = bm;
     c->bw_bytes_Z16 = z16;
     c->bw_bytes_maskbits = bmb;
     c->bw_bytes_alpha16 = bal; c->bw_bytes_dx16 = bdx; c->bw_bytes_wpart = bwp; c->bw_bytes_thpart = bth; c->bw_bytes_wgrad = bwg;
     c->bw_bytes_signbits = bsg;
-    c->bw_bytes_Z32 = bz32;
-    if (dev_alloc(c, &c->bw_signbits, bsg) != cudaSuccess || dev_alloc(c, &c->bw_alpha16, bal) != cudaSuccess || dev_alloc(c, &c->bw_dx16, bdx) != cudaSuccess ||
-        dev_alloc(c, &c->bw_wpart, bwp) != cudaSuccess || dev_alloc(c, &c->bw_thpart, bth) != cudaSuccess ||
-        dev_alloc(c, &c->bw_wgrad, bwg) != cudaSuccess || dev_alloc(c, &c->bw_maskbits, bmb) != cudaSuccess || dev_alloc(c, &c->bw_Z16, z16) != cudaSuccess || dev_alloc(c, &c->bw_masks, bm) != cudaSuccess || dev_alloc(c, &c->bw_dZ, c->bw_bytes_dZ) != cudaSuccess || dev_alloc(c, &c->bw_LD, bl) != cudaSuccess ||
-        dev_alloc(c, &c->bw_dKV, bk) != cudaSuccess || dev_alloc(c, &c->bw_WT, bw) != cudaSuccess ||
-        dev_alloc(c, &c->bw_dKV16, b16) != cudaSuccess || dev_alloc(c, &c->bw_dZ16, z16) != cudaSuccess) {
-      cudaGetLastError();
-      free_backward(c);
-      return fail(c, CSAT_ERR_ALLOC, "cudaMalloc(backward scratch) failed");
+    c->bw_bytes_tail = tail;
+    if (dev_alloc(c, &c->bw_signbits, bsg) == cudaSuccess && dev_alloc(c, &c->bw_alpha16, bal) == cudaSuccess && dev_alloc(c, &c->bw_dx16, bdx) == cudaSuccess &&
+        dev_alloc(c, &c->bw_wpart, bwp) == cudaSuccess && dev_alloc(c, &c->bw_thpart, bth) == cudaSuccess &&
+        dev_alloc(c, &c->bw_wgrad, bwg) == cudaSuccess && dev_alloc(c, &c->bw_maskbits, bmb) == cudaSuccess && dev_alloc(c, &c->bw_Z16, z16) == cudaSuccess && dev_alloc(c, &c->bw_masks, bm) == cudaSuccess && dev_alloc(c, &c->bw_dZ, c->bw_bytes_dZ) == cudaSuccess && dev_alloc(c, &c->bw_LD, bl) == cudaSuccess &&
+        dev_alloc(c, &c->bw_dKV, bk) == cudaSuccess && dev_alloc(c, &c->bw_WT, bw) == cudaSuccess &&
+        dev_alloc(c, &c->bw_dKV16, b16) == cudaSuccess && dev_alloc(c, &c->bw_dZ16, z16) == cudaSuccess)
+      return true;
+    cudaGetLastError();
+    free_backward(c);
+    return false;
+  };
+  if (save && !c->save_denied) {                            // no allocation of its own: 0.1 ms in a context's first training step
+    if (allocate(bsv)) {
+      saved_at(c->bw_dZ + bz / 4);
+      return CSAT_OK;
     }
-    if (save32) {                                           // no allocations of their own: 0.1 ms each in a context's first training step
-      c->bw_Z32 = c->bw_dZ + bz / 4;
-      c->bw_words = reinterpret_cast<uint32_t*>(c->bw_Z32 + bz32 / 4);
-    }
+    c->save_denied = true;
   }
-  return CSAT_OK;
+  return allocate(0) ? CSAT_OK : fail(c, CSAT_ERR_ALLOC, "cudaMalloc(backward scratch) failed");
 }
 
 int csat_backward(csat_ctx* c, const void* Q, const void* K, const void* V, const void* dOut, void* dQ, void* dK,

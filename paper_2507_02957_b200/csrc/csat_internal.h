@@ -151,9 +151,12 @@ struct csat_ctx {
   uint32_t* bw_maskbits = nullptr;       // the forward's decisions, one bit per (b, h, layer, query, column)
   size_t bw_bytes_Z16 = 0, bw_bytes_maskbits = 0;
   size_t bw_bytes_dZ = 0, bw_bytes_LD = 0, bw_bytes_dKV = 0, bw_bytes_WT = 0, bw_bytes_dKV16 = 0, bw_bytes_dZ16 = 0;
-  // float32 contexts that save for the backward: Z, and the decisions (saved_words_per_row)
+  // float32 contexts that save for the backward: Z, and the decisions (saved_words_per_row).  At the end of bw_dZ's allocation
+  // (bw_bytes_tail), or, where the scratch was there before the first saving forward, in one of their own (bw_save)
   float* bw_Z32 = nullptr; uint32_t* bw_words = nullptr;
-  size_t bw_bytes_Z32 = 0;
+  float* bw_save = nullptr;
+  size_t bw_bytes_tail = 0, bw_bytes_save = 0;
+  bool save_denied = false;      // there was no memory for them
   // CSAT_KEEP_MASKS: the shrinkage decisions of the most recent csat_backward, one word per (b, h, query, column),
   // bit t = |x_t| > theta_t
   bool keep_masks = false;

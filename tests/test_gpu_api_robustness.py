@@ -80,3 +80,40 @@ def test_workspace_canary_finds_no_unwritten_row(shape, dtype):
     for a, b in zip(ctx.backward(Q, K, V, G), gref):
         assert torch.isfinite(a).all() and torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("first", ["saving_forward", "backward"])
+def test_a_saving_float32_forward_without_memory_for_its_state(first):
+    """The allocation fails (on the host) where the state is asked for with the rest of the scratch, or for itself behind an earlier
+    backward: the forward returns what it returns, the backward recomputes, nothing is asked for again until the key changes, and
+    the earlier backward's decisions stay."""
+    B, H, n, nq, d, m, T = 2, 3, 140, 70, 40, 60, 4
+    g = torch.Generator(device="cuda").manual_seed(4)
+    Q, K, V, G = (torch.randn(B, H, r, d, generator=g, device="cuda") for r in (nq, n, n, nq))
+    SAVE = binding.CSAT_SAVE_FOR_BACKWARD
+    plain, ctx = (binding.Csat(n, m, d, H, 3, B=B, n_q=nq, dtype="fp32", T=T, lam=0.02) for _ in range(2))
+    for c in (plain, ctx):
+        binding.csat_set_i64(c.h, binding.CSAT_KEEP_MASKS, 1)
+    out, want = plain.forward(Q, K, V), plain.backward(Q, K, V, G)
+    masks = plain.backward_masks()
+    if first == "backward":
+        ctx.backward(Q, K, V, G)
+    binding.csat_set_i64(ctx.h, SAVE, 1)
+    # (with CSAT_KEEP_MASKS the scratch begins with the decisions: its second allocation is the one the state is in)
+    binding.csat_debug_fail_alloc(2 if first == "saving_forward" else 1)
+    for _ in range(2):                                       # the second one would succeed if it asked
+        assert torch.equal(ctx.forward(Q, K, V), out)
+        binding.csat_debug_fail_alloc(0)
+        assert ctx.workspace_bytes == plain.workspace_bytes
+        if first == "backward":
+            assert torch.equal(ctx.backward_masks(), masks)
+        assert all(torch.equal(a, b) for a, b in zip(ctx.backward(Q, K, V, G), want)) and ctx.launches > 3
+    binding.csat_set_i64(ctx.h, SAVE, 0)
+    binding.csat_set_i64(ctx.h, SAVE, 1)
+    ctx.forward(Q, K, V)
+    assert torch.equal(ctx.backward_masks(), masks)
+    assert ctx.workspace_bytes > plain.workspace_bytes
+    assert all(torch.equal(a, b) for a, b in zip(ctx.backward(Q, K, V, G), want)) and ctx.launches == 3
+    assert torch.equal(ctx.backward_masks(), masks)
+    for c in (plain, ctx):
+        c.close()
