@@ -637,6 +637,25 @@ static bool fp32_can_save(const csat_ctx* c) {
   return c->p.dtype == CSAT_DTYPE_FP32 && c->p.d <= csat::kFfmaMaxD && c->p.T <= 32 && c->p.B * c->p.H <= 32767;
 }
 
+// The capture that a float32 context's call is part of (0: none).  A replay of it writes K~|V~ and the saved state unseen by the
+// host, so what a forward saves serves a backward of the same capture, or, while no call of the context has been captured, one
+// that runs at once like itself; every other backward recomputes.
+static constexpr unsigned long long kUnknownCapture = ~0ull;
+static unsigned long long note_capture(csat_ctx* c, cudaStream_t s) {
+  if (c->p.dtype != CSAT_DTYPE_FP32) return 0;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &status, &id) != cudaSuccess) {
+    cudaGetLastError();
+    id = kUnknownCapture;
+  } else if (status != cudaStreamCaptureStatusActive) {
+    id = status == cudaStreamCaptureStatusNone ? 0 : kUnknownCapture;
+  }
+  if (id != 0) c->captured = true;
+  return id;
+}
+static bool can_reuse(const csat_ctx* c, unsigned long long capture) { return capture != 0 ? capture != kUnknownCapture : !c->captured; }
+
 int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void* out, void* stream) {
   if (!c) return CSAT_ERR_INVALID_ARG;
   if (!Q || !K || !V || !out) return fail(c, CSAT_ERR_INVALID_ARG, "csat_forward: NULL tensor pointer");
@@ -658,6 +677,7 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
   cudaStream_t s = (cudaStream_t)stream;
   int launches = 0;
   c->saved_valid = false;                  // from here on K~|V~ may be overwritten
+  const unsigned long long capture = note_capture(c, s);
   prof_mark(c, s, -1);
   if (c->p.T > 0 && c->w_S && (c->w_layers != 1 || c->w_untied) && c->w_layers != c->p.T)
     return fail(c, CSAT_ERR_STATE, "the supplied LISTA weights are for a number of layers other than CSAT_T");
@@ -687,18 +707,17 @@ int csat_forward(csat_ctx* c, const void* Q, const void* K, const void* V, void*
     e = csat::launch_sm100_attend_for_backward(c, Q, c->bw_Z16, c->bw_LD, c->bw_maskbits, wg ? c->bw_alpha16 : nullptr, s,
                                                &launches, out);
     if (e == cudaSuccess) { c->saved_valid = true; c->saved_alpha = wg; }
-  } else if (c->save_for_backward && fp32_can_save(c)) {
+  } else if (c->save_for_backward && fp32_can_save(c) && can_reuse(c, capture)) {
     // Where the scratch is missing and cannot be had (a stream that is being captured, no memory left) the forward saves nothing and
     // csat_backward recomputes, as without the key
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
     bool record = false;
     if (c->bw_Z32 != nullptr || !c->save_denied) {
-      record = ensure_backward_scratch(c, true, cap == cudaStreamCaptureStatusNone) == CSAT_OK && c->bw_Z32 != nullptr;
+      record = ensure_backward_scratch(c, true, capture == 0) == CSAT_OK && c->bw_Z32 != nullptr;
       if (!record) c->err.clear();
     }
     e = csat::launch_simt_attend_recover(c, Q, out, s, &launches, false, record);
     c->saved_valid = e == cudaSuccess && record;
+    c->saved_capture = capture;
   } else {
     e = tc_attend ? csat::launch_sm100_attend_recover(c, Q, out, s, &launches)
                   : csat::launch_simt_attend_recover(c, Q, out, s, &launches);
@@ -748,6 +767,7 @@ int csat_reduce_partials(csat_ctx* c, const float* partials, int count, void* st
   std::string why;
   if (!on_device(c, &why)) return fail(c, CSAT_ERR_STATE, why);
   int launches = 0;
+  note_capture(c, (cudaStream_t)stream);
   cudaError_t e = csat::launch_reduce_partials(c, partials, count, (cudaStream_t)stream, &launches);
   if (e != cudaSuccess) return fail_cuda(c, e, "csat_reduce_partials launch");
   c->have_forward = true;                 // the workspace now holds K~|V~
@@ -887,6 +907,7 @@ int csat_backward(csat_ctx* c, const void* Q, const void* K, const void* V, cons
     return fail(c, CSAT_ERR_STATE, "the supplied LISTA weights are for a number of layers other than CSAT_T");
   cudaStream_t s = (cudaStream_t)stream;
   int launches = 0;
+  const unsigned long long capture = note_capture(c, s);
   if (p.T > 0) {
     int rc = ensure_decoder(c, s, &launches);
     if (rc != CSAT_OK) return rc;
@@ -896,7 +917,8 @@ int csat_backward(csat_ctx* c, const void* Q, const void* K, const void* V, cons
   // what a csat_forward with CSAT_SAVE_FOR_BACKWARD left (K~|V~, Z, the softmax statistics, the decisions, the iterates
   // if asked for) replaces the compression and the forward pass of this call
   c->reuse_saved = c->save_for_backward && c->saved_valid &&
-                   (fp32_can_save(c) || (c->tmap_phi_valid && c->force_simt == 0 && (!c->weight_grads || c->saved_alpha)));
+                   ((fp32_can_save(c) && c->saved_capture == capture && can_reuse(c, capture)) ||
+                    (c->tmap_phi_valid && c->force_simt == 0 && (!c->weight_grads || c->saved_alpha)));
   cudaError_t e = cudaSuccess;
   if (!c->reuse_saved) {
     c->saved_valid = false;                // this call's own forward pass overwrites it

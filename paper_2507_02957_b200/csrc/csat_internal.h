@@ -157,6 +157,8 @@ struct csat_ctx {
   float* bw_save = nullptr;
   size_t bw_bytes_tail = 0, bw_bytes_save = 0;
   bool save_denied = false;      // there was no memory for them
+  bool captured = false;         // float32 contexts: a call that writes K~|V~ or the state has been captured into a graph
+  unsigned long long saved_capture = 0;                      // the capture in which the state was saved, 0: none
   // CSAT_KEEP_MASKS: the shrinkage decisions of the most recent csat_backward, one word per (b, h, query, column),
   // bit t = |x_t| > theta_t
   bool keep_masks = false;
