@@ -55,7 +55,8 @@ compress_pair_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_
   uint64_t* empty = full + kMaxStages;
   uint64_t* acc_done = empty + kMaxStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_done + 1);
-  int* cta_abort = reinterpret_cast<int*>(tmem_slot + 1);
+  PairEnd* end = reinterpret_cast<PairEnd*>(tmem_slot + 1);
+  int* cta_abort = &end->abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   // blockIdx.x walks the batch fastest (CTAs that stream the same rows of Phi run together), then come the measurement groups of a head
@@ -76,7 +77,7 @@ compress_pair_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_
       mbar_init(&empty[s], 1);
     }
     mbar_init(acc_done, 1);
-    *cta_abort = 0;
+    end->init();
     fence_mbar_init();
   }
   if (warp == 1) tmem_alloc_pair(tmem_slot, a.cols);
@@ -110,8 +111,8 @@ compress_pair_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_
           tma_load_3d_pair(st + kABytes + p * a.nhalf * 128, &tmap_phi, bar, i * kChunk, r0 + p * N + (int)rank * a.nhalf, h);
         ++issued;
       }
-      if (!ok && rank == 0)                              // gave up: let the copies in flight land (rank 1's land before rank 0's barrier)
-        for (int i = issued > a.stages ? issued - a.stages : 0; i < issued; ++i) mbar_wait_drain(&full[i % a.stages], (i / a.stages) & 1);
+      if (!ok) end->give_up();
+      end->producer_done(rank, issued);
     }
   } else if (warp == 1) {
     if (rank == 0 && elect_one()) {
@@ -131,13 +132,15 @@ compress_pair_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_
         }
         mma_commit_pair(&empty[s]);
       }
+      if (!ok) end->give_up();                           // before both epilogues wake
       mma_commit_pair(acc_done);
     }
   } else {
     const int q = warp & 3, half = (warp - 2) >> 2;      // lanes [32q, 32q+32) = features; which groups of 32 measurements
     const int box = q >> 1;                              // features [0, 64) or [64, 128) of the CTA's 128
-    const bool ok = mbar_wait(acc_done, 0, a.status, 154, cta_abort) && *(volatile int*)cta_abort == 0;
-    if (__all_sync(0xffffffffu, ok)) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_done, 0, a.status, 154, cta_abort) && *(volatile int*)cta_abort == 0);
+    if (!ok && lane == 0) end->give_up();
+    if (ok) {
       tc_fence_after();
       const int f = (q & 1) * 32 + lane, odd = lane & 1; // feature within the box
       const int x = (D == 64 ? 0 : (int)rank * 128) + box * 64;
@@ -176,6 +179,8 @@ compress_pair_kernel(const __grid_constant__ CUtensorMap tmap_phi, const __grid_
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && rank == 0 && *(volatile int*)cta_abort != 0) end->drain(full, a.stages, [&](int) { return sb; });
+  __syncwarp();
   cluster_sync();                                        // the peer's shared memory is read, and its barriers arrived at, until here
   if (warp == 1) tmem_dealloc_pair(tmem, a.cols);
 }

@@ -238,6 +238,47 @@ __global__ void wait_timeout_selftest_kernel(int* status, unsigned long long lim
   }
 }
 
+// The same for a pair of CTAs, by the functions its kernels end with: cluster k's wait runs out in rank k % 2, the producers have then
+// requested 1 and kSelfStages stages, the other way round for k >= 2 (their copies, here a late complete_tx, on rank 0's barriers).
+// Both CTAs' waits have to end, and every requested stage to be complete when the pair does.
+constexpr int kSelfStages = 4;
+__global__ void __cluster_dims__(2, 1, 1) pair_give_up_selftest_kernel(int* status, unsigned long long limit_ns) {
+  __shared__ uint64_t full[kSelfStages], never;
+  __shared__ PairEnd end;
+  const uint32_t rank = cluster_ctarank();
+  const int k = blockIdx.x >> 1, n = ((k >> 1) ^ (int)rank) ? kSelfStages : 1;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSelfStages; ++s) mbar_init(&full[s], 1);
+    mbar_init(&never, 1);
+    end.init();
+    fence_mbar_init();
+  }
+  __syncthreads();
+  cluster_sync();
+  if (threadIdx.x == 0) {
+    if (rank == 0)
+      for (int s = 0; s < n; ++s) mbar_arrive_expect_tx(&full[s], 2 * 16);
+    const bool ok = mbar_wait(&never, 0, status, 999, &end.abort, rank == (uint32_t)(k & 1) ? limit_ns : kWaitTimeoutNs);
+    if (!ok) end.give_up();
+    end.producer_done(rank, n);
+  } else if (threadIdx.x == 32) {
+    for (const unsigned long long t0 = globaltimer(); globaltimer() - t0 < 2 * limit_ns;) {}
+    for (int s = 0; s < n; ++s)
+      asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cluster.b64 [%0], 16;" ::"r"(cluster_smem_u32(&full[s], 0)) : "memory");
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bool good = *(volatile int*)&end.abort != 0;
+    if (rank == 0) {
+      end.drain(full, kSelfStages, [](int) { return 16; });
+      for (int s = 0; s < kSelfStages; ++s) good = good && mbar_try_wait(&full[s], 0);
+    }
+    if (!good) *(volatile int*)status = 998;
+  }
+  __syncwarp();
+  cluster_sync();
+}
+
 // n_len tokens of K, V (a shard that starts at token phi_j0 of the sequence, or the whole sequence); partial: float32
 // destination of a shard's sums, null = the workspace
 template <int D, bool SEP, int BG, int MT = 1, bool HALF = false, bool TWO = false>
@@ -276,6 +317,7 @@ cudaError_t launch(csat_ctx* c, const void* K, const void* V, cudaStream_t s, in
 
 cudaError_t launch_wait_timeout_selftest(csat_ctx* c, unsigned long long limit_ns, cudaStream_t s) {
   wait_timeout_selftest_kernel<<<1, 32, 0, s>>>(c->status, limit_ns);
+  pair_give_up_selftest_kernel<<<8, 64, 0, s>>>(c->status, limit_ns);
   return cudaGetLastError();
 }
 

@@ -1185,6 +1185,7 @@ int csat_selftest_wait_timeout(csat_ctx* c, int64_t limit_us, void* stream) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail_cuda(c, e, "csat_selftest_wait_timeout");
   if (*(volatile int*)c->status == 0) return fail(c, CSAT_ERR_STATE, "the bounded wait did not report its time-out");
+  if (*(volatile int*)c->status == 998) return fail(c, CSAT_ERR_STATE, "a pair of CTAs did not give up together");
   return fail(c, CSAT_ERR_TIMEOUT, "a bounded device-side wait gave up (self-test)");
 }
 

@@ -69,7 +69,7 @@ struct Unit {
 
 // The epilogue warps' walk over a CTA's units (q: TMEM lanes [32q, 32q+32); rank: the CTA's half of a pair's rows, -1: no pair)
 template <int D, typename Release>
-__device__ __forceinline__ void epilogue(const ProjArgs& a, const OutMaps& maps, uint32_t tmem_base, uint8_t* o_buf, int q, int lane, int first, int step, int rank,
+__device__ __forceinline__ bool epilogue(const ProjArgs& a, const OutMaps& maps, uint32_t tmem_base, uint8_t* o_buf, int q, int lane, int first, int step, int rank,
                                          uint64_t* acc_full, int* status, int* cta_abort, Release release) {
   const int HD = a.H * D;
   uint32_t tc = 0;
@@ -135,6 +135,7 @@ __device__ __forceinline__ void epilogue(const ProjArgs& a, const OutMaps& maps,
     release(buf);
   }
   if (lane == 0) bulk_wait_group0();                      // the stores are done before the kernel ends
+  return ok;                                              // (the same in every lane)
 }
 
 template <int D>
@@ -256,7 +257,8 @@ project_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
   uint64_t* acc_full = empty + kPairStages;               // [2]
   uint64_t* acc_empty = acc_full + 2;                     // [2], rank 0's count
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
-  int* cta_abort = reinterpret_cast<int*>(tmem_slot + 1);
+  PairEnd* end = reinterpret_cast<PairEnd*>(tmem_slot + 1);
+  int* cta_abort = &end->abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int first = blockIdx.x >> 1, step = gridDim.x >> 1, nk = (a.dm + kChunkK - 1) / kChunkK;
@@ -266,7 +268,7 @@ project_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     prefetch_tmap(&tmap_w);
     for (int s = 0; s < kPairStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int u = 0; u < 2; ++u) { mbar_init(&acc_full[u], 1); mbar_init(&acc_empty[u], 2 * 4); }
-    *cta_abort = 0;
+    end->init();
     fence_mbar_init();
   }
   if (warp == 1) tmem_alloc_pair(tmem_slot, 2 * kTileN);
@@ -297,9 +299,8 @@ project_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             tma_load_3d_pair(st + kABytes + g * kBoxBytes, &tmap_w, bar, a.col0 + t.col + ((int)rank * half + g) * 64, k * kChunkK, 0);
         }
       }
-      if (!ok && rank == 0)                               // gave up: let the copies in flight land (rank 1's on rank 0's barriers)
-        for (uint32_t i = it > (uint32_t)kPairStages ? it - kPairStages : 0; i < it; ++i)
-          mbar_wait_drain(&full[i % kPairStages], (i / kPairStages) & 1);
+      if (!ok) end->give_up();
+      end->producer_done(rank, (int)it);
     }
   } else if (warp == 1) {
     if (rank == 0 && elect_one()) {
@@ -325,17 +326,24 @@ project_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             mma_f16_ss_pair(acc, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 128), idesc, (k | kk) != 0);
           mma_commit_pair(&empty[s]);
         }
+        if (!ok) end->give_up();                          // before both epilogues wake
         mma_commit_pair(&acc_full[buf]);
       }
+      if (!ok) end->give_up();
     }
   } else {
-    epilogue<D>(a, OutMaps{{&tmap_oq, &tmap_ok, &tmap_ov}}, tmem_base, o_buf, warp & 3, lane, first, step, (int)rank, acc_full, status, cta_abort, [&](uint32_t buf) {
+    const bool ok = epilogue<D>(a, OutMaps{{&tmap_oq, &tmap_ok, &tmap_ov}}, tmem_base, o_buf, warp & 3, lane, first, step, (int)rank, acc_full, status, cta_abort,
+                                [&](uint32_t buf) {
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_smem_u32(&acc_empty[buf], 0));
     });
+    if (!ok && lane == 0) end->give_up();
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && rank == 0 && *(volatile int*)cta_abort != 0)
+    end->drain(full, kPairStages, [&](int i) { return kABytes + Unit(a, first + i / nk * step).boxes / 2 * kBoxBytes; });
+  __syncwarp();
   cluster_sync();                                         // the peer's shared memory is read, and its barriers arrived at, until here
   if (warp == 1) tmem_dealloc_pair(tmem_base, 2 * kTileN);
 }

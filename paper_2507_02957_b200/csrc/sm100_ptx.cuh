@@ -312,6 +312,36 @@ __device__ __forceinline__ void mma_f16_ss_pair(uint32_t d_tmem, uint64_t a_desc
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
+// What a pair needs when a bounded wait gives up.  Either CTA ends the waits of both, and before they leave rank 0 lets land whatever
+// either producer has requested (all of a stage's copies complete on its barriers, which count 2 x bytes).
+struct PairEnd {
+  int abort;                 // this CTA's waits have ended
+  int issued[2];             // rank 0's: stages that the producer of rank 0 or 1 has requested; -1 while it is at work
+  __device__ __forceinline__ void init() { abort = 0; issued[0] = issued[1] = -1; }
+  // by the thread whose wait has failed, before it commits or arrives anywhere: whoever that wakes finds the flag
+  __device__ __forceinline__ void give_up() {
+    uint32_t old;
+    for (uint32_t r = 0; r < 2; ++r)
+      asm volatile("atom.relaxed.cluster.shared::cluster.exch.b32 %0, [%1], 1;" : "=r"(old) : "r"(cluster_smem_u32(&abort, r)) : "memory");
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
+  }
+  __device__ __forceinline__ void producer_done(uint32_t rank, int n) {
+    asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_smem_u32(&issued[rank], 0)), "r"(n) : "memory");
+  }
+  // by one thread of rank 0 behind its CTA's last wait; bytes(i): of stage i in each CTA
+  template <typename Bytes> __device__ __forceinline__ void drain(uint64_t* full, int stages, Bytes bytes) {
+    const unsigned long long t0 = globaltimer();
+    while (*(volatile int*)&issued[1] < 0 && globaltimer() - t0 < kWaitTimeoutNs) {}
+    const int n0 = *(volatile int*)&issued[0], n1 = *(volatile int*)&issued[1] < 0 ? n0 : *(volatile int*)&issued[1], n = n0 > n1 ? n0 : n1;
+    for (int i = n > stages ? n - stages : 0; i < n; ++i) {
+      uint64_t* bar = &full[i % stages];
+      if (i >= n0) mbar_arrive_expect_tx(bar, bytes(i));     // requested by rank 1 alone
+      if (i >= n1)                                           // by rank 0 alone, for both
+        asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"((uint32_t)bytes(i)) : "memory");
+      mbar_wait_drain(bar, (i / stages) & 1);
+    }
+  }
+};
 // one arrival at this place in both CTAs once every MMA issued so far by this thread has finished
 __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),

@@ -112,3 +112,15 @@ def test_compression_with_two_ctas_per_sm(B, H, n, m, d):
     ctx.forward_host(Q.cpu(), K.cpu(), V.cpu(), host)
     assert torch.equal(host, out.cpu()) and all(torch.equal(a, b) for a, b in zip(got, ctx.get_compressed()))
     ctx.close()
+
+
+@pytest.mark.parametrize("limit_us", [200, 3000])
+def test_a_pair_of_ctas_gives_up_together(limit_us):
+    """The functions that the kernels on pairs of CTAs end with after a wait that ran out: both CTAs' waits end (long before their own
+    limit), and what only one of the producers had requested is complete when the pair ends.  998: it was not."""
+    ctx = binding.Csat(64, 64, 64, 1, 3, dtype="bf16", T=1, lam=0.05)
+    for _ in range(3):
+        assert binding.csat_selftest_wait_timeout(ctx.h, limit_us) == 7
+        assert "self-test" in binding.csat_last_error(ctx.h)
+        assert binding.csat_clear_status(ctx.h) == 999
+    ctx.close()
