@@ -401,6 +401,8 @@ cudaError_t compress_t(csat_ctx* c, TO* dst, const void* K, const void* V, cudaS
   if constexpr (sizeof(TO) == 4) {                            // whole launches of larger heads: compress_sm100.cu
     if (c->p.d > 96) return launch_compress<TO, 128>(c, dst, K, V, s, phi_j0, n_len);
     if (c->p.d > 64) return launch_compress<TO, 96>(c, dst, K, V, s, phi_j0, n_len);
+  } else if (c->p.d > 64) {
+    return cudaErrorInvalidValue;
   }
   return launch_compress<TO, 64>(c, dst, K, V, s, phi_j0, n_len);
 }
