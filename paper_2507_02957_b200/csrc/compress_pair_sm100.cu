@@ -7,7 +7,8 @@
 // m = 392, 42 KB here), and were no faster than tiles of 128.  us, tiles / pairs: 128 heads of 3136 x 64, m = 392 41.6 / 35.2 (tensor
 // pipe 72 % of the active cycles; the rest is the ring's start and the epilogue); 64 of 4096 x 128, m = 400 55.5 / 43.3-46; 64 of 5000 x 64,
 // m = 600 68.8 / 41.5; 32 of 4000 x 128, m = 300 31.0 / 26.5; 4 of 16384 x 128, m = 3000 102 / 87.  The start of a cluster, the allocation by
-// both CTAs and their barrier at the end cost 1 to 2 us more than a single CTA: short token axes and multiples of 128 stay there.
+// both CTAs and their barrier at the end cost 1 to 2 us more than a single CTA: short token axes, multiples of 128 and grids of few CTAs stay
+// there.
 //
 // The pair: d = 64 two batch elements of one head (an odd batch repeats the last one and does not store it), d = 128 the K and the V
 // features of one (batch, head).  A CTA takes one or two parts of N measurements (accumulators side by side in tensor memory).
@@ -252,18 +253,38 @@ cudaError_t launch(csat_ctx* c, const void* K, const void* V, cudaStream_t s, co
 
 }  // namespace
 
-// other_cycles: the tensor-pipe cycles of an SM in compress_sm100.cu.  The difference is for the longer start and end (8 x 12 heads of 3000 x 64, m = 260
-// 26.7 / 25.3 us with tiles and 3 x 16 of 3339, m = 385 32.6 / 31.3 stay with tiles).  The ratio at d = 64: 11 x 16 heads of 5814, m = 1633 (0.894) 365 /
-// 337 with tiles, 12 x 16 of 6186, m = 1317 (0.875) 263 / 294, 13 x 16 of 10745, m = 1652 (0.86) 787 / 927.  d = 128 in several rounds: up to m = 1000 all
-// ten shapes measured gain (14 x 8 of 8320, m = 908 322 / 424; 7 x 8 of 2553, m = 192 20.4 / 23.7), beyond the operands' way in counts as much as the
-// tensor pipe: 7 x 8 of 6318, m = 1190 192 / 155, 4 x 16 of 4855, m = 1433 184 / 171, 15 x 4 of 6455, m = 1283 193 / 266.
-bool compress_pair_better(const csat_ctx* c, double other_cycles) {
+// Cycles of an SM, on the scale of compress_sm100.cu's tensor-pipe cycles (1.4 to 1.5 clocks each, there and here).  A stage takes a pair no
+// less than 480 of them where it has the SM to itself and 300 where two share one, however few its measurements: 590 to 630 clocks at N =
+// 112 to 192 (8 heads of 11129 x 128, m = 210; of 11925, m = 1334), 1017 for two of N = 144 (48 of 9459, m = 423).
+static double pair_time(const csat_ctx* c, const Plan& pl) {
+  const Params& p = c->p;
+  const int64_t units = p.d == 64 ? (p.B + 1) / 2 * p.H : p.B * p.H, ctas = 2 * units * pl.groups, sms = c->sms;
+  const double chunks = (double)((p.n + kChunk - 1) / kChunk), tensor = 4.0 * pl.parts * pl.nhalf;
+  const double alone = chunks * (tensor > 480.0 ? tensor : 480.0) + 9000.0, both = chunks * 2.0 * (tensor > 300.0 ? tensor : 300.0) + 10000.0;
+  if (ctas <= sms || 2 * pl.parts * pl.nhalf > 256) return (double)((ctas + sms - 1) / sms) * alone;
+  const int64_t rest = ctas % (2 * sms);
+  return (double)(ctas / (2 * sms)) * both + (rest > sms ? both : rest > 0 ? alone : 0.0);
+}
+
+// tile_cycles: the tensor-pipe cycles of an SM in compress_sm100.cu; tile_rounds: of CTAs there, whose start and end take 6000 each; one_tile:
+// no SM has more than one tile of 128 measurements.  Of 334 drawn shapes that the first conditions let through (1 to 32 batch elements, 1 to
+// 16 heads, 600 to 16384 tokens, m = 192 to 2000) pairs are slower on 51, by up to 79 % (8 heads of 11129 x 128, m = 210 30 / 54 us); of those
+// taken now 12 are slower, and 15 that would gain (13 of them less than 8 %) are not taken.
+//   one_tile: pairs gain 8 to 20 % a stage whatever N and need some 60 stages for what they cost: 24 heads of 3200 x 64, m = 625 21.9 / 23.3, 42 of
+//             5759, m = 512 39.1 / 32.2; the worst taken 19 of 5569 x 128, m = 635 37 / 48.
+//   else    : by the times; the worst taken 24 heads of 2949 x 128, m = 1134 40 / 49 and 32 of 4747, m = 960 55 / 61.
+// The first conditions: 11 x 16 heads of 5814 x 64, m = 1633 (0.894) 337 / 365, 12 x 16 of 6186, m = 1317 (0.875) 294 / 263; d = 128 in several
+// rounds with m > 1000 is slower as often as not (7 x 8 of 6318, m = 1190 155 / 192, 15 x 4 of 6455, m = 1283 266 / 193).
+bool compress_pair_better(const csat_ctx* c, double tile_cycles, double tile_rounds, bool one_tile) {
   const Params& p = c->p;
   if (p.separate_phi || p.m < 192 || (p.d == 64 ? p.B < 2 : p.d != 128) || p.H * ((p.m + 511) / 512) > 65535 || p.B > (1 << 29)) return false;
   const Plan pl = plan(c);
   if (pl.groups == 0) return false;
-  if (p.d == 64) return pl.cycles + 5200.0 < other_cycles && pl.cycles < 0.88 * other_cycles;
-  return pl.cycles + 4000.0 < other_cycles && (p.m <= 1000 || 2 * p.B * p.H * pl.groups <= c->sms);
+  if (p.d == 64 ? pl.cycles + 5200.0 >= tile_cycles || pl.cycles >= 0.88 * tile_cycles
+                : pl.cycles + 4000.0 >= tile_cycles || (p.m > 1000 && 2 * p.B * p.H * pl.groups > c->sms))
+    return false;
+  if (one_tile) return p.n > 63 * kChunk;
+  return pair_time(c, pl) < tile_cycles + 6000.0 * tile_rounds;
 }
 
 cudaError_t launch_compress_pair(csat_ctx* c, const void* K, const void* V, cudaStream_t s) {

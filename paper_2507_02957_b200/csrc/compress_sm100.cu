@@ -357,12 +357,15 @@ cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cud
   // more CTAs than SMs: two on each (whole compression, us, one / two CTAs per SM: 384 heads of 197 x 64, m = 64 (192 CTAs) 10.4 / 7.5; 384 of 300 12.9 /
   // 9.6; 320 of 1000, m = 100 26.5 / 22.1; 384 of 2000 45.9 / 41.3; 160 of 6000 x 128 104.5 / 90.7; 256 of 400 x 128 18.9 / 14.9)
   auto two = [&](int64_t columns_of_ctas) { return mtiles * columns_of_ctas > (int64_t)c->sms; };
-  // pairs of CTAs with the measurements in N where those waste less of the tensor pipe on rows beyond m
-  if (whole) {
-    const int64_t units = c->p.d == 64 ? (c->p.B + 1) / 2 * c->p.H : c->p.B * c->p.H, mt = pairs_fill(units) ? 2 : 1;
-    const double chunks = (double)((n_len + kChunk - 1) / kChunk);
-    const double cycles = halves_fit(units) ? chunks * 256.0 : (double)(((mtiles + mt - 1) / mt * units + c->sms - 1) / c->sms) * chunks * 512.0 * (double)mt;
-    if (compress_pair_better(c, cycles)) return launch_compress_pair(c, K, V, s);
+  // pairs of CTAs with the measurements in N where those waste less of the tensor pipe on rows beyond m; not in the place of CTAs for K
+  // and V, whose 256 cycles a stage a pair does not reach (8 heads of 11237 x 128, m = 222 38 / 55 us)
+  const int64_t units = c->p.d == 64 ? (c->p.B + 1) / 2 * c->p.H : c->p.B * c->p.H;
+  if (whole && !halves_fit(units)) {
+    const int64_t mt = pairs_fill(units) ? 2 : 1, tiles = (mtiles + mt - 1) / mt * units, sms = c->sms;
+    const double cycles = (double)((tiles + sms - 1) / sms) * (double)((n_len + kChunk - 1) / kChunk) * 512.0 * (double)mt;
+    const int64_t per_round = mt == 1 ? 2 * sms : sms;
+    if (compress_pair_better(c, cycles, (double)((tiles + per_round - 1) / per_round), mt == 1 && tiles <= sms))
+      return launch_compress_pair(c, K, V, s);
   }
   // d = 64: two batch elements per CTA where the batch has them (N = 256 MMAs)
   if (c->p.d == 64 && c->p.B >= 2 && c->bh_cnt == 0) {

@@ -286,7 +286,7 @@ cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cud
 cudaError_t launch_sm100_compress_padded(csat_ctx* c, const void* K, const void* V, cudaStream_t s);
 
 // compress_pair_sm100.cu : the same for a whole batch with shared Phi, features in M, on pairs of CTAs
-bool compress_pair_better(const csat_ctx* c, double other_cycles);
+bool compress_pair_better(const csat_ctx* c, double tile_cycles, double tile_rounds, bool one_tile);
 cudaError_t launch_compress_pair(csat_ctx* c, const void* K, const void* V, cudaStream_t s);
 
 // attend_recover_sm100.cu : tcgen05 compressed attention + recovery (bf16, d = 128), and the choice of kernel for d in {64, 128}

@@ -114,6 +114,17 @@ def test_compression_with_two_ctas_per_sm(B, H, n, m, d):
     ctx.close()
 
 
+@pytest.mark.parametrize("B,H,n,m,d", [
+    (13, 4, 1517, 361, 128),    # one group of two parts
+    (6, 8, 3000, 423, 128),     # three groups of one part, two CTAs per SM
+    (2, 12, 3300, 927, 128),    # three groups of two parts
+    (7, 16, 1600, 260, 128),    # more CTAs than SMs, one on each
+    (11, 6, 3400, 460, 64),     # (64 x 64: three groups)
+])
+def test_compression_on_pairs_of_ctas_where_it_is_chosen(B, H, n, m, d):
+    test_compression_on_pairs_of_ctas(B, H, n, m, d)
+
+
 @pytest.mark.parametrize("limit_us", [200, 3000])
 def test_a_pair_of_ctas_gives_up_together(limit_us):
     """The functions that the kernels on pairs of CTAs end with after a wait that ran out: both CTAs' waits end (long before their own
