@@ -1187,8 +1187,11 @@ cudaError_t make_attend_tmaps(csat_ctx* c) {
   const uint32_t kb[3] = {64, (uint32_t)kMC, 1};
   cudaError_t e = make_tmap_bf16_3d(&c->tmap_kv, c->kv, kd, ks, kb);
   if (e != cudaSuccess) return e;
-  const uint32_t sb[3] = {64, 32, 1};                           // the compression kernel's stores: one warp's rows
-  if ((e = make_tmap_bf16_3d(&c->tmap_kv_st, c->kv, kd, ks, sb)) != cudaSuccess) return e;
+  const uint32_t sb[3] = {64, 32, 1};
+  if ((e = make_tmap_bf16_3d(&c->tmap_kv32, c->kv, kd, ks, sb)) != cudaSuccess) return e;
+  const uint64_t hd[3] = {(uint64_t)p.d, (uint64_t)p.m, (uint64_t)(p.B * p.H)};      // K~ and V~ by themselves: the compression's stores
+  if ((e = make_tmap_bf16_3d(&c->tmap_kt_st, c->kv, hd, ks, sb)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16_3d(&c->tmap_vt_st, (const __nv_bfloat16*)c->kv + p.d, hd, ks, sb)) != cudaSuccess) return e;
   // V~ B behind K~|V~: [B H, m, d]
   const __nv_bfloat16* vb = (const __nv_bfloat16*)c->kv + (size_t)(p.B * p.H * p.m * 2 * p.d);
   const uint64_t vd[3] = {(uint64_t)p.d, (uint64_t)p.m, (uint64_t)(p.B * p.H)};

@@ -685,7 +685,7 @@ cudaError_t launch_dq(csat_ctx* c, const void* Q, void* dQ, cudaStream_t s) {
   if ((e = ensure_dynamic_smem(bwd_dq_sm100_kernel<D, kFew>, (int)C::kSmemBytes, c->device, smem_opt_in)) != cudaSuccess) return e;
   const float scale = (float)(p.scale > 0.0 ? p.scale : 1.0 / sqrt((double)D));
   const dim3 grid((unsigned)((p.nq + kRows - 1) / kRows), (unsigned)(p.B * p.H));
-  return launch_pdl(bwd_dq_sm100_kernel<D, kFew>, grid, kQThreads, C::kSmemBytes, s, tq, tz, C::kQC == 32 ? c->tmap_kv_st : c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD, c->bw_negD(),
+  return launch_pdl(bwd_dq_sm100_kernel<D, kFew>, grid, kQThreads, C::kSmemBytes, s, tq, tz, C::kQC == 32 ? c->tmap_kv32 : c->tmap_kv, (__nv_bfloat16*)dQ, c->bw_LD, c->bw_negD(),
                     (int)c->ld_pitch(), (int)p.nq, (int)p.m, scale, c->status);
 }
 

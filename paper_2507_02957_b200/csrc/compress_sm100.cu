@@ -290,14 +290,21 @@ cudaError_t launch(csat_ctx* c, const void* K, const void* V, cudaStream_t s, in
   const uint64_t d = (uint64_t)p.d, BH = (uint64_t)(p.B * p.H), heads = (uint64_t)c->phi_heads();
   const uint64_t kd[3] = {d, (uint64_t)n_len, BH}, ks[2] = {d * 2, (uint64_t)n_len * d * 2};
   const uint32_t kb[3] = {64, (uint32_t)kChunk, 1};
-  const uint64_t fd[3] = {(uint64_t)p.n_pad, (uint64_t)p.m, heads}, fs[2] = {(uint64_t)p.n_pad * 2, (uint64_t)p.m * p.n_pad * 2};
-  const uint32_t fb[3] = {(uint32_t)kChunk, (uint32_t)kTileM, 1};
-  const uint64_t od[3] = {d, (uint64_t)p.m, BH}, os[2] = {d * 4, (uint64_t)p.m * d * 4};
-  const uint32_t ob[3] = {64, 32, 1};                           // one warp's rows
   cudaError_t e;
-  if ((e = make_tmap_bf16_3d(&tphi, c->phi, fd, fs, fb)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16_3d(&tok, c->kv, od, os, ob)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16_3d(&tov, (const __nv_bfloat16*)c->kv + d, od, os, ob)) != cudaSuccess) return e;
+  if (c->tmap_phi_valid) {
+    // Phi's and the workspace's maps are the context's (d = 64 and 128): three look-ups of five per call, 0.2 us of the host's 10 for a small one
+    tphi = c->tmap_phi;
+    tok = c->tmap_kt_st;
+    tov = c->tmap_vt_st;
+  } else {
+    const uint64_t fd[3] = {(uint64_t)p.n_pad, (uint64_t)p.m, heads}, fs[2] = {(uint64_t)p.n_pad * 2, (uint64_t)p.m * p.n_pad * 2};
+    const uint32_t fb[3] = {(uint32_t)kChunk, (uint32_t)kTileM, 1};
+    const uint64_t od[3] = {d, (uint64_t)p.m, BH}, os[2] = {d * 4, (uint64_t)p.m * d * 4};
+    const uint32_t ob[3] = {64, 32, 1};                         // one warp's rows
+    if ((e = make_tmap_bf16_3d(&tphi, c->phi, fd, fs, fb)) != cudaSuccess) return e;
+    if ((e = make_tmap_bf16_3d(&tok, c->kv, od, os, ob)) != cudaSuccess) return e;
+    if ((e = make_tmap_bf16_3d(&tov, (const __nv_bfloat16*)c->kv + d, od, os, ob)) != cudaSuccess) return e;
+  }
   if ((e = make_tmap_bf16_3d(&tk, K, kd, ks, kb)) != cudaSuccess) return e;
   if ((e = make_tmap_bf16_3d(&tv, V, kd, ks, kb)) != cudaSuccess) return e;
   static DeviceFlags smem_opt_in;

@@ -102,10 +102,11 @@ struct csat_ctx {
   size_t had_bytes_signs = 0, had_bytes_ab = 0;
   int hadamard_transform = 0; // CSAT_HADAMARD_TRANSFORM
   int debug_canary = 0;       // CSAT_DEBUG_CANARY: the K~|V~ workspace is filled with NaN bit patterns before every compression
-  CUtensorMap tmap_phi;       // TMA view of phi for the tensor-core compress kernel (bf16, d in {64,128})
+  CUtensorMap tmap_phi;       // TMA view of phi for compress_sm100.cu (bf16, d in {64, 128}; the other tensor maps with it)
   bool tmap_phi_valid = false;
   CUtensorMap tmap_kv;        // TMA view of the K~|V~ workspace
-  CUtensorMap tmap_kv_st;     // the same workspace in boxes of 32 rows (the compression kernel's stores)
+  CUtensorMap tmap_kv32;      // the same workspace in boxes of 32 rows (dQ's chunks)
+  CUtensorMap tmap_kt_st, tmap_vt_st;   // K~ and V~ in boxes of 32 rows (the stores of compress_sm100.cu)
   CUtensorMap tmap_vb;        // V~ B [B H, m, d] behind K~|V~ in the same allocation (bf16 contexts), as the attention phase loads it
   CUtensorMap tmap_vb_st;     // the same in boxes of 32 rows (the stores of the kernel that forms it)
   CUtensorMap tmap_mats;      // TMA view of mats_bf16
