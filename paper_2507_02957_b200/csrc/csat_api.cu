@@ -370,6 +370,13 @@ int csat_set_i64(csat_ctx* c, int key, int64_t v) {
       free_lista(c);
       free_staging(c);
       p.dtype = (int)v;
+      if (csat::split_tile_head(p) != (c->mats_split != nullptr)) {
+        dev_free(c, &c->mats_split, 6 * dd_bytes(p, 2));
+        if (csat::split_tile_head(p) && dev_alloc(c, &c->mats_split, 6 * dd_bytes(p, 2)) != cudaSuccess) {
+          c->broken = true;
+          return fail(c, CSAT_ERR_ALLOC, "cudaMalloc(decoder matrices) failed");
+        }
+      }
       return allocate_and_generate(c);   // user-set Phi, Psi, D are dropped with the old dtype
     }
     case CSAT_ENSEMBLE: {

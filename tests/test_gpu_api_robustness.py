@@ -117,3 +117,35 @@ def test_a_saving_float32_forward_without_memory_for_its_state(first):
     assert torch.equal(ctx.backward_masks(), masks)
     for c in (plain, ctx):
         c.close()
+
+
+@pytest.mark.parametrize("d", [40, 64, 96, 120])
+def test_a_context_holds_what_its_storage_type_needs(d):
+    """Phi, K~|V~ (bf16 with V~ B behind it), the decoder in float32 and float64 and its bf16 operands; the operands in two parts
+    only where a kernel reads them, also after the storage type has changed."""
+    B, H, n, m = 2, 3, 200, 130
+    n_pad = -(-n // 64) * 64
+    Q, K, V = (torch.randn(B, H, n, d, generator=torch.Generator(device="cuda").manual_seed(i), device="cuda") for i in range(3))
+    ctx = binding.Csat(n, m, d, H, 3, B=B, dtype="fp32", T=3, lam=0.02)
+    outs = {}
+    for dtype, es, code in (("fp32", 4, binding.CSAT_DTYPE_FP32), ("bf16", 2, binding.CSAT_DTYPE_BF16)) * 2:
+        binding.csat_set_i64(ctx.h, binding.CSAT_DTYPE, code)
+        two_parts = dtype == "bf16" and d <= 96 and d != 64
+        decoder = H * d * d * (2 * 8 + 3 * 4 + (3 + (6 if two_parts else 0)) * 2) + 2 * H * 4
+        assert ctx.workspace_bytes == H * m * n_pad * es + B * H * m * (3 if dtype == "bf16" else 2) * d * es + decoder
+        ctx.torch_dtype = torch.bfloat16 if dtype == "bf16" else torch.float32
+        out = ctx.forward(*(t.to(ctx.torch_dtype) for t in (Q, K, V)))
+        assert torch.equal(out, outs.setdefault(dtype, out)) and torch.isfinite(out).all()
+    ctx.close()
+    if d in (40, 96):                                        # the added allocation fails: refused until it succeeds
+        ctx = binding.Csat(n, m, d, H, 3, B=B, dtype="fp32", T=3, lam=0.02)
+        binding.csat_debug_fail_alloc(1)
+        with pytest.raises(binding.CsatError):
+            binding.csat_set_i64(ctx.h, binding.CSAT_DTYPE, binding.CSAT_DTYPE_BF16)
+        binding.csat_debug_fail_alloc(0)
+        ctx.torch_dtype = torch.bfloat16
+        with pytest.raises(binding.CsatError):
+            ctx.forward(*(t.bfloat16() for t in (Q, K, V)))
+        binding.csat_set_i64(ctx.h, binding.CSAT_DTYPE, binding.CSAT_DTYPE_BF16)
+        assert torch.equal(ctx.forward(*(t.bfloat16() for t in (Q, K, V))), outs["bf16"])
+        ctx.close()
