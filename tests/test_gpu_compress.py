@@ -65,9 +65,9 @@ def test_compression_with_a_matrix_of_its_own_for_the_values(B, H, n, m, d):
     (16, 8, 2000, 392, 64),     # two parts of 208
     (5, 16, 2000, 600, 64),     # three groups of one part of 208
     (7, 10, 1030, 513, 64),     # the last group ends at its 161st row
-    (2, 16, 2100, 300, 128),    # K and V features in the two CTAs
-    (2, 12, 3001, 530, 128),
-    (1, 4, 4100, 3000, 128),    # sixteen groups
+    (2, 16, 2100, 300, 128),    # (tiles: one per SM, too few stages)
+    (2, 12, 3001, 530, 128),    # (tiles)
+    (1, 4, 4100, 3000, 128),    # sixteen groups of one part, K and V features in the two CTAs
 ])
 def test_compression_on_pairs_of_ctas(B, H, n, m, d):
     """Features in M, measurements in N; the host-buffer forward compresses a head at a time on single CTAs: the same bits."""
@@ -90,7 +90,8 @@ def test_compression_on_pairs_of_ctas(B, H, n, m, d):
 
 @pytest.mark.parametrize("B,H,n,m,d", [
     (32, 12, 197, 64, 64),      # one tile of measurements, a ragged token count
-    (5, 30, 333, 65, 64),       # two groups of columns a little above one per SM
+    (5, 30, 333, 65, 64),       # (90 tiles: one CTA per SM)
+    (5, 60, 333, 65, 64),       # two batch elements per CTA, the last one alone; 180 tiles
     (1, 160, 500, 100, 64),     # a lone batch: K and V of one (batch, head) per tile
     (7, 16, 400, 140, 128),     # an odd batch
     (1, 160, 203, 128, 128),
@@ -119,7 +120,7 @@ def test_compression_with_two_ctas_per_sm(B, H, n, m, d):
     (6, 8, 3000, 423, 128),     # three groups of one part, two CTAs per SM
     (2, 12, 3300, 927, 128),    # three groups of two parts
     (7, 16, 1600, 260, 128),    # more CTAs than SMs, one on each
-    (11, 6, 3400, 460, 64),     # (64 x 64: three groups)
+    (11, 8, 2600, 441, 64),     # an odd batch, three groups of one part
 ])
 def test_compression_on_pairs_of_ctas_where_it_is_chosen(B, H, n, m, d):
     test_compression_on_pairs_of_ctas(B, H, n, m, d)
