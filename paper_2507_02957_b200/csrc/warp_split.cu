@@ -425,10 +425,21 @@ template <int DP> cudaError_t attend_d(const FfmaAttend& a, const void* Q, const
 }  // namespace
 
 // Whole launches: these kernels or compress_sm100.cu's, us: d > 64 4.9 / 3.8 (4 heads of 128 x 96, m = 96) to 18.8 / 7.0: always the latter.  Up to
-// 64, by CTAs x tokens: 16 x 200 3.0 / 4.6, 192 x 300 5.1 / 6.3, 256 x 256 4.4 / 6.0, 288 x 300 (d = 48) 7.4 / 6.7, 512 x 400 9.5 / 7.1, 768 x 500 14.3 / 7.4.
+// 64, by CTAs x tokens: 16 x 200 3.0 / 4.6, 192 x 300 5.1 / 6.3, 256 x 256 4.4 / 6.0; beyond, by what bounds each: the tiles a stage of 64
+// tokens, 0.28 us with one batch element and 0.42 with two per CTA (half as much again where rows do not start on 32 bytes), and whole
+// rounds of them beyond a tile per SM; these kernels a CTA's walk over the tokens, or the matrix pipes.  16 heads of 1715 x 40, m = 113 11.7
+// / 22.9, 12 of 2762 x 24, m = 289 18.0 / 32.4, 36 of 1753 x 8, m = 111 10.9 / 17.8; 27 of 3134 x 48, m = 272 50.5 / 25.9, 176 of 3576 x 32, m = 384 259
+// / 52.  Of 79 drawn shapes (d = 8 to 56, 64 to 4000 tokens) the rule takes the slower one once, by 2 %; CTAs x tokens alone did 25 times.
 bool split_compress_better(const csat_ctx* c) {
   const Params& p = c->p;
-  return p.d <= 64 && (p.m + kCRows - 1) / kCRows * p.B * p.H * 2 * p.n <= 72000;
+  if (p.d > 64) return false;
+  const int64_t ctas = (p.m + kCRows - 1) / kCRows * p.B * p.H * 2;
+  if (ctas * p.n <= 72000) return true;
+  const bool two = p.B >= 2 && !p.separate_phi;
+  const int64_t tiles = (p.m + 127) / 128 * (two ? (p.B + 1) / 2 : p.B) * p.H;
+  const double stage = (two ? 420.0 : 280.0) * (p.d % 16 != 0 ? 1.5 : 1.0), rounds = tiles > c->sms ? (double)tiles / c->sms : 1.0;
+  const double token = p.d <= 32 ? (0.028 * ctas > 2.9 ? 0.028 * ctas : 2.9) : (0.034 * ctas > 4.2 ? 0.034 * ctas : 4.2);
+  return (double)p.n * token < (double)((p.n + 63) / 64) * stage * rounds;             // ns
 }
 
 cudaError_t launch_split_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int64_t phi_j0, int64_t n_len, float* partial) {

@@ -126,6 +126,37 @@ def test_compression_on_pairs_of_ctas_where_it_is_chosen(B, H, n, m, d):
     test_compression_on_pairs_of_ctas(B, H, n, m, d)
 
 
+@pytest.mark.parametrize("B,H,n,m,d,separate", [
+    (3, 8, 636, 116, 32, False),       # the warp kernel: few tiles
+    (6, 6, 1053, 111, 8, False),
+    (2, 6, 700, 157, 56, False),
+    (2, 5, 900, 150, 40, True),
+    (3, 50, 140, 129, 32, False),      # the kernel of 64 columns: two batch elements per CTA, an odd batch
+    (17, 24, 100, 40, 40, False),      # two CTAs per SM
+    (5, 60, 130, 70, 48, False),
+    (1, 16, 800, 540, 8, False),       # a lone batch
+    (1, 160, 300, 100, 56, False),     # with two CTAs per SM
+    (3, 50, 140, 129, 32, True),       # a matrix of their own for the values
+    (1, 6, 300, 129, 72, False),       # the kernel of 128 columns: K and V apart
+    (4, 32, 150, 100, 96, False),      # together
+    (3, 60, 150, 120, 120, False),     # two CTAs per SM
+    (2, 9, 333, 130, 88, True),
+])
+def test_compression_of_other_head_sizes(B, H, n, m, d, separate):
+    """Both kernels that whole launches go to, either side of the choice between them."""
+    ctx = binding.Csat(n, m, d, H, 3, B=B, n_q=16, dtype="bf16", T=0, lam=0.05)
+    ctx.set(separate_phi=separate)
+    g = torch.Generator(device="cuda").manual_seed(n + m)
+    K, V = (torch.randn(B, H, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    ctx.forward(torch.randn(B, H, 16, d, generator=g, device="cuda").bfloat16(), K, V)
+    phi = torch.from_numpy(to_np(ctx.get_phi())).cuda()
+    for got, x, p in zip(ctx.get_compressed(), (K, V), (phi[:H], phi[-H:])):
+        ref = p @ x.double()
+        bound = 2.0 ** -8 * ref.abs() + 2e-3 * 2.0 ** -8 * ref.abs().max()
+        assert got.shape == ref.shape and bool(((got.double() - ref).abs() <= bound).all()), (got.double() - ref).abs().max().item()
+    ctx.close()
+
+
 @pytest.mark.parametrize("limit_us", [200, 3000])
 def test_a_pair_of_ctas_gives_up_together(limit_us):
     """The functions that the kernels on pairs of CTAs end with after a wait that ran out: both CTAs' waits end (long before their own
