@@ -464,17 +464,24 @@ cudaError_t launch(csat_ctx* c, const FfmaAttend& a, const void* Q, void* out, c
 
 }  // namespace
 
-// Against warp_split.cu, us, warps / tiles of 128 queries: d > 64 from 27.4 / 21.5 (4 heads of 128 x 96, T = 10) to 75 / 25 (32 of 1024 x 96): always.
-// d = 48, T = 10: 8 heads of 256 12.9 / 14.9, 72 of 300 22.4 / 18.4: from a tile for every other SM on.  d <= 32, where a warp's layer is short and
-// a tile's chain is not: up to a tile per SM 7.5 / 10.5 to 9.2 / 9.4; beyond, the attention phase is faster (96 heads of 500, m = 100, T = 10
-// 22.6 / 16.9; 128 of 1000, m = 64, T = 5 30.1 / 22.9), the layers are not (128 of 400, m = 64, T = 20 35.1 / 37.9; 256 of 250 x 16, m = 40, T = 20
-// 25.6 / 32.8): up to ten layers per chunk of measurements.  By the context's whole job.
+// Against warp_split.cu, us, warps / tiles of 128 queries: d > 64 from 27.4 / 21.5 (4 heads of 128 x 96, T = 10) to 75 / 25 (32 of 1024 x 96): always
+// (behind, by 1.3 us of 12.7, in whole forwards of up to 12 tiles with T = 1 alone).  d = 48, T = 10: 8 heads of 256 12.9 / 14.9, 72 of 300 22.4 /
+// 18.4: from a tile for every other SM on.  d <= 32, where a warp's layer is short and a tile's chain is not: up to a tile per SM 7.5 / 10.5 to
+// 9.2 / 9.4; beyond, the attention phase is faster (96 heads of 500, m = 100, T = 10 22.6 / 16.9; 128 of 1000, m = 64, T = 5 30.1 / 22.9), the layers
+// are not (128 of 400, m = 64, T = 20 35.1 / 37.9; 12 of 2139 x 24, m = 92, T = 20 20.7 / 23.4): up to ten layers per chunk of measurements,
+// six up to two tiles per SM, and less by 0.6 and by the rows that a tile lacks for d <= 16, whose products take a warp half the steps (10 of
+// 2113 x 8, m = 16, T = 5 8.5 / 11.4; 32 of 593 x 8, m = 159, T = 20 14.8 / 21.4; 556 tiles of 70 x 16, m = 69, T = 10 22.4 / 25.8).  Of 129 drawn jobs
+// with d <= 32 three are slower by more than 4 % (at most 11), with ten layers alone 13 were (up to 35).  By the context's whole job.
 bool split_tile_better(const csat_ctx* c) {
   const Params& p = c->p;
   if (c->mats_split == nullptr || !split_tile_head(p) || (c->w_S && c->w_untied && p.T > 0)) return false;
   const int64_t tiles = (p.nq + kRows - 1) / kRows * p.B * p.H;
   if (p.d > 64) return true;
-  return p.d > 32 ? 2 * tiles > c->sms : tiles > c->sms && p.T <= 10 * ((p.m + kMC - 1) / kMC);
+  if (p.d > 32) return 2 * tiles > c->sms;
+  double layers = 10.0 * (double)((p.m + kMC - 1) / kMC);
+  if (tiles <= 2 * (int64_t)c->sms) layers *= 0.6;
+  if (p.d <= 16) layers *= 0.6 * (double)(p.B * p.H * p.nq) / (double)(tiles * kRows);
+  return tiles > c->sms && p.T <= layers;
 }
 
 cudaError_t launch_split_tile(csat_ctx* c, const FfmaAttend& a, const void* Q, void* out, cudaStream_t s) {

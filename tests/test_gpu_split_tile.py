@@ -65,3 +65,9 @@ def test_tile_kernel_against_float64(B, H, n, nq, m, d, T, variant):
     bound = 2.0 ** -8 * ref.abs() + 3 * (T + 4) * 2.0 ** -15 * big
     assert bool(((out - ref).abs() <= bound).all()), ((out - ref).abs() / bound).max().item()
     ctx.close()
+
+
+@pytest.mark.parametrize("B,H,n,nq,m,d,T", [(1, 300, 80, 128, 63, 24, 10), (1, 150, 80, 128, 63, 24, 6), (2, 160, 40, 128, 40, 16, 5), (1, 152, 30, 127, 20, 8, 3)])
+def test_tile_kernel_of_small_heads(B, H, n, nq, m, d, T):
+    """Jobs at the ends of the choice: the tile kernel's."""
+    test_tile_kernel_against_float64(B, H, n, nq, m, d, T, "psi_thresholds_per_layer")
