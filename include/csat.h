@@ -205,7 +205,8 @@ int csat_set_lista_layer_weights(csat_ctx* ctx, const void* S, const void* Bm, c
  * call compresses K, V again and recomputes what it needs.  Its
  * first call allocates scratch (B H (n_q (d + 2) + 2 m d) floats; transposed copies of the decoder matrices for d > 128;
  * bf16 copies of Z, dZ and dK~|dV~ and B H T n_q d / 32 decision words on the tensor-core path; B H n_q d words
- * more with CSAT_KEEP_MASKS, twice as many for float32 contexts with CSAT_SAVE_FOR_BACKWARD; all counted by csat_workspace_bytes).
+ * more with CSAT_KEEP_MASKS; float32 contexts with CSAT_SAVE_FOR_BACKWARD B H n_q (d + w) more, w = 32 up to d = 32, 64 up to d = 64 and
+ * d beyond, if there is memory for them; all counted by csat_workspace_bytes).
  * Two paths.  bf16 contexts with d in {64, 128} run every stage on the tensor cores (one S, B for all layers, or one
  * pair per layer streamed through shared memory from the last layer to the first): the forward
  * kernel once more (it keeps Z, the softmax statistics and one decision bit per layer, query and column), the

@@ -800,10 +800,10 @@ cudaError_t launch_attend_tile(csat_ctx* c, const void* Q, void* out, cudaStream
   if (c->w_S || p.T == 0 || !(p.lambda > 0.0)) return few_tiles(c) ? CSAT_TILE(kTied, 2) : CSAT_TILE(kTied, 1);
   // one positive threshold for all layers
   if (few_tiles(c)) return CSAT_TILE(kUnits, 2);
-  // B folded into the values: the first tiles wait for the fold (4 us), every tile saves a hand-over.  Whole forward, us, folded / not: 1248
-  // tiles, m = 256, T = 20 82.2 / 80.3, 1776 93.8 / 94.0, 2368 125.2 / 125.5, 4736 231.2 / 233.7; 1536 short tiles, m = 64 90.0 / 84.4.  It pays from
-  // about 16 tiles per SM on; the line at eight was measured on the kernel with two tiles per CTA, and the tests hold the first of
-  // these shapes to the folded launches and their bits.
+  // B folded into the values: the first tiles wait for the fold (4 us), every tile saves a hand-over.  The line at eight tiles per SM was
+  // measured on the kernel with two tiles per CTA, and the tests hold the first of these shapes to the folded launches and their bits;
+  // since the rows hand over through named barriers the saved hand-over no longer pays for the wait.  Whole forward, us, folded / not: 1248
+  // tiles, m = 256, T = 20 80.3 / 78.2, 1776 126.4 / 122.7, 2368 153.7 / 151.3, 4736 288.8 / 285.6; 1536 short tiles, m = 64 82.4 / 76.2.
   if (p.T >= 2 && (p.nq + kRows - 1) / kRows * p.B * p.H >= 8 * (int64_t)c->sms) {
     cudaError_t e = launch_sm100_vfold(c, s, launches);
     if (e != cudaSuccess) return e;

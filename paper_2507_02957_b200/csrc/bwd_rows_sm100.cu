@@ -5,8 +5,8 @@
 // where |x| > theta and 0 elsewhere.
 //
 // Before these kernels the forward's own kernels have left K~|V~ in the workspace, Z (bf16, as the forward rounds it
-// for its first product) in bw_Z16, every row's log sum exp L in bw_LD and the layers' shrinkage decisions in
-// bw_maskbits.
+// for its first product) in bw_Z16, minus every row's log sum exp L in bw_LD (in units of log 2, as it enters the exponentials) and the
+// layers' shrinkage decisions in bw_maskbits.
 //
 // bwd_recur_sm100_kernel, one CTA per tile of 128 queries (TMEM lane = query row, one thread per row): the recurrence
 // run backwards.  The decisions |x_t| > theta_t are the forward kernel's own (it records them, one bit per column and

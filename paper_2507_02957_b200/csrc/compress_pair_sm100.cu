@@ -5,7 +5,7 @@
 // as the A operand and the pair shares the rows of Phi as the B operand, half of them in each CTA's shared memory: N is the measurements
 // rounded up to 16 per part of at most 256.  Single CTAs with the features in M would load all rows of Phi each (65 KB per 64 tokens at
 // m = 392, 42 KB here), and were no faster than tiles of 128.  us, tiles / pairs: 128 heads of 3136 x 64, m = 392 41.6 / 35.2 (tensor
-// pipe 72 % of the active cycles; the rest is the ring's start and the epilogue); 64 of 4096 x 128, m = 400 55.5 / 43.3-46; 64 of 5000 x 64,
+// pipe 74 % of the active cycles; the rest is the ring's start and the epilogue); 64 of 4096 x 128, m = 400 55.5 / 43.3-46; 64 of 5000 x 64,
 // m = 600 68.8 / 41.5; 32 of 4000 x 128, m = 300 31.0 / 26.5; 4 of 16384 x 128, m = 3000 102 / 87.  The start of a cluster, the allocation by
 // both CTAs and their barrier at the end cost 1 to 2 us more than a single CTA: short token axes, multiples of 128 and grids of few CTAs stay
 // there.

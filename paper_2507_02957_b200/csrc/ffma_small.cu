@@ -175,6 +175,8 @@ template <int DP> cudaError_t launch(const FfmaAttend& a, const float* Q, const 
 
 // While all CTAs fit at once.  The whole call in a replayed graph, here / ffma_attend_kernel (us): d = 64 on 64 CTAs 8.2 / 15.2, 152
 // 11.6 / 15.4, 256 with T = 20 16.6 / 21.0; 128 with m = 400 19.6 / 37.4; 32 heads of 8 batches with 4 queries each (256) 148 / 195.
+// Attention and recovery alone, every four rows reading all of K~|V~: 16 CTAs with m = 400 13.4 / 30.5, m = 10000 220 / 569; 296 22 / 33 and 381 / 574;
+// d = 32, 584 (T = 5) 20.3 / 24.9 and 387 / 444.
 // d <= 32: 300 with T = 20 11.4 / 14.0, 512 with T = 5 11.5 / 12.7, with T = 20 13.0 / 12.8 (every warp of the SM in every layer).  d = 64
 // with a second round of CTAs (441): 14.6 / 15.0 with T = 5 but 25.3 / 22.6 with T = 20.
 bool ffma_small_better(const FfmaAttend& a) {
