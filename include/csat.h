@@ -90,8 +90,9 @@ enum {
                           and the next csat_backward on the same Q, K, V skips its own compression and forward pass
                           (about a third of its time).  The saved state is dropped by any setter and by any other
                           compute call in between; it is the caller's contract that Q, K, V are unchanged.  (A replayed
-                          graph is not seen: float32 contexts use the state within one capture, or outside of any while
-                          no call of the context has been captured, and recompute otherwise.)  The
+                          graph is not seen: bf16 contexts take the state as it is then; float32 contexts use it within
+                          one capture, or outside of any while no call of the context has been captured, and recompute
+                          otherwise.)  The
                           forward then costs about a third more.  0 (default): csat_backward recomputes  */
   CSAT_WEIGHT_GRADS = 12, /* 1: csat_backward also forms the gradients with respect to the decoder's parameters (S, B,
                           the thresholds, the dictionary) for csat_get_weight_grads; tensor-core path only (bf16, d in

@@ -32,7 +32,7 @@ class _CsatFunction(torch.autograd.Function):
     def backward(fn_ctx, dOut):
         Q, K, V = fn_ctx.saved_tensors
         csat = fn_ctx.csat
-        if csat.forwards != fn_ctx.forward_no or csat.h.user_saves is None:
+        if csat.forwards != fn_ctx.forward_no or getattr(csat.h, "user_saves", None) is None:
             # another forward has been here, or another setting: what state there is is not this forward's
             user = binding._set_saving(csat.h, False)
         else:

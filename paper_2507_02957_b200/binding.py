@@ -131,7 +131,9 @@ def _restore_saving(h):
 
 def _set_saving(h, save):
     """Sets the key for csat_attention, which then calls the library and stores what this returns in h.user_saves."""
-    user = h.user_saves if h.user_saves is not None else csat_get_i64(h, CSAT_SAVE_FOR_BACKWARD)
+    user = getattr(h, "user_saves", None)                    # (a closed context's handle is None: the call below refuses it)
+    if user is None:
+        user = csat_get_i64(h, CSAT_SAVE_FOR_BACKWARD)
     csat_set_i64(h, CSAT_SAVE_FOR_BACKWARD, int(save))
     return user
 

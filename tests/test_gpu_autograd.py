@@ -133,3 +133,14 @@ def test_direct_calls_beside_csat_attention(dtype, d):
         ctx.backward(*x)
         assert max(launches) < ctx.launches
     ctx.close()
+
+
+def test_a_closed_context_is_refused():
+    from paper_2507_02957_b200.autograd import csat_attention
+    ctx = binding.Csat(140, 70, 64, 2, 3, dtype="fp32", T=2, lam=0.02)
+    Q, K, V = (torch.randn(1, 2, 140, 64, device="cuda").requires_grad_(True) for _ in range(3))
+    out = csat_attention(ctx, Q, K, V)
+    ctx.close()
+    for call in (lambda: torch.autograd.grad(out.sum(), (Q, K, V)), lambda: csat_attention(ctx, Q, K, V), lambda: ctx.forward(Q, K, V)):
+        with pytest.raises(binding.CsatError):
+            call()
