@@ -49,7 +49,7 @@ def csat_attention(csat, Q, K, V, save_for_backward=True):
     shape and dtype), differentiable with respect to Q, K, V.  The context holds the saved state of its last forward; the
     backward of an earlier one recomputes."""
     # decided here: inside the function gradients are always off
-    save = save_for_backward and torch.is_grad_enabled() and (Q.requires_grad or K.requires_grad or V.requires_grad)
+    save = bool(save_for_backward) and torch.is_grad_enabled() and (Q.requires_grad or K.requires_grad or V.requires_grad)
     return _CsatFunction.apply(csat, Q, K, V, save)
 
 
