@@ -336,17 +336,27 @@ cudaError_t make_phi_tmap(csat_ctx* c) {
   return make_tmap_bf16_3d(&c->tmap_phi, c->phi, d, st, b);
 }
 
+// More CTAs than SMs: two on each.  A stage takes 0.9 of its time alone then (beside another's), and a round of two has one start and end
+// where two rounds have two of some ten stages each; but an odd number of rounds of one becomes an even one.  Whole compression, us, one / two
+// per SM: 384 heads of 197 x 64, m = 64 (192 CTAs) 10.4 / 7.5; 384 of 300 12.9 / 9.6; 320 of 1000, m = 100 26.5 / 22.1; 384 of 2000 45.9 / 41.3; 160 of 6000 x
+// 128 104.5 / 90.7; 256 of 400 x 128 18.9 / 14.9; 448 CTAs 36.7 / 30.2 (500 tokens) to 344 / 324 (9000); three rounds for four: 320 CTAs of 500 x 128 27.1 /
+// 25.0, of 1500 57.5 / 60.3, of 9000 258 / 299; 384 of 8225 x 64, m = 4009 (12 heads, a lone batch) 143 / 159.
+static bool two_per_sm(const csat_ctx* c, int64_t ctas, int64_t tokens) {
+  const int64_t sms = c->sms, ones = (ctas + sms - 1) / sms, twos = (ctas + 2 * sms - 1) / (2 * sms);
+  return ctas > sms && (1.8 * (double)twos - (double)ones) * (double)((tokens + kChunk - 1) / kChunk) < 10.0 * (double)(ones - twos);
+}
+
 // Head sizes without a kernel of their own: the same choice of CTAs as below for d = 64 or 128 (one Phi for keys and values or two)
 cudaError_t launch_sm100_compress_padded(csat_ctx* c, const void* K, const void* V, cudaStream_t s) {
   const Params& p = c->p;
   if (p.separate_phi) return p.d <= 64 ? launch<64, true, 1>(c, K, V, s, 0, p.n, nullptr) : launch<128, true, 1>(c, K, V, s, 0, p.n, nullptr);
   const int64_t mtiles = (p.m + kTileM - 1) / kTileM, ctas = mtiles * p.B * p.H;
   if (p.d <= 64 && p.B >= 2)
-    return mtiles * ((p.B + 1) / 2) * p.H > c->sms ? launch<64, false, 2, 1, false, true>(c, K, V, s, 0, p.n, nullptr)
-                                                   : launch<64, false, 2>(c, K, V, s, 0, p.n, nullptr);
-  if (p.d <= 64) return ctas > c->sms ? launch<64, false, 1, 1, false, true>(c, K, V, s, 0, p.n, nullptr) : launch<64, false, 1>(c, K, V, s, 0, p.n, nullptr);
+    return two_per_sm(c, mtiles * ((p.B + 1) / 2) * p.H, p.n) ? launch<64, false, 2, 1, false, true>(c, K, V, s, 0, p.n, nullptr)
+                                                              : launch<64, false, 2>(c, K, V, s, 0, p.n, nullptr);
+  if (p.d <= 64) return two_per_sm(c, ctas, p.n) ? launch<64, false, 1, 1, false, true>(c, K, V, s, 0, p.n, nullptr) : launch<64, false, 1>(c, K, V, s, 0, p.n, nullptr);
   if (2 * ctas <= c->sms) return launch<128, false, 1, 1, true>(c, K, V, s, 0, p.n, nullptr);
-  return ctas > c->sms ? launch<128, false, 1, 1, false, true>(c, K, V, s, 0, p.n, nullptr) : launch<128, false, 1>(c, K, V, s, 0, p.n, nullptr);
+  return two_per_sm(c, ctas, p.n) ? launch<128, false, 1, 1, false, true>(c, K, V, s, 0, p.n, nullptr) : launch<128, false, 1>(c, K, V, s, 0, p.n, nullptr);
 }
 
 cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cudaStream_t s, int* launches,
@@ -361,9 +371,7 @@ cudaError_t launch_sm100_compress(csat_ctx* c, const void* K, const void* V, cud
   // of tokens, and what one CTA has in flight is what these grids wait for: 32 heads of 3001 x 128, m = 187 (64
   // CTAs) 24.9 -> 18.0 us, 48 of 1568 x 64, m = 256 (48 CTAs) 14.3 -> 10.0, 16 of 8192 x 128, m = 512 (64) 58 -> 44
   auto halves_fit = [&](int64_t columns_of_ctas) { return 2 * mtiles * columns_of_ctas <= (int64_t)c->sms; };
-  // more CTAs than SMs: two on each (whole compression, us, one / two CTAs per SM: 384 heads of 197 x 64, m = 64 (192 CTAs) 10.4 / 7.5; 384 of 300 12.9 /
-  // 9.6; 320 of 1000, m = 100 26.5 / 22.1; 384 of 2000 45.9 / 41.3; 160 of 6000 x 128 104.5 / 90.7; 256 of 400 x 128 18.9 / 14.9)
-  auto two = [&](int64_t columns_of_ctas) { return mtiles * columns_of_ctas > (int64_t)c->sms; };
+  auto two = [&](int64_t columns_of_ctas) { return two_per_sm(c, mtiles * columns_of_ctas, n_len); };
   // pairs of CTAs with the measurements in N where those waste less of the tensor pipe on rows beyond m; not in the place of CTAs for K
   // and V, whose 256 cycles a stage a pair does not reach (8 heads of 11237 x 128, m = 222 38 / 55 us)
   const int64_t units = c->p.d == 64 ? (c->p.B + 1) / 2 * c->p.H : c->p.B * c->p.H;

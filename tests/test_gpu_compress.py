@@ -95,6 +95,8 @@ def test_compression_on_pairs_of_ctas(B, H, n, m, d):
     (1, 160, 500, 100, 64),     # a lone batch: K and V of one (batch, head) per tile
     (7, 16, 400, 140, 128),     # an odd batch
     (1, 160, 203, 128, 128),
+    (5, 100, 260, 70, 64),      # 300 tiles: three rounds of one for two of two, a short token axis
+    (2, 150, 1200, 128, 128),   # (a longer one: one CTA per SM)
 ])
 def test_compression_with_two_ctas_per_sm(B, H, n, m, d):
     """More tiles than SMs; a head at a time (the host-buffer forward) has fewer, with one CTA per SM: the same bits."""
