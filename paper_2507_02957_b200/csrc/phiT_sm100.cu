@@ -212,8 +212,10 @@ cudaError_t launch_sm100_phiT(csat_ctx* c, const void* g16, void* dK, void* dV, 
   if (p.separate_phi) return p.d == 64 ? launch<64, true, 1>(c, g16, dK, dV, s) : launch<128, true, 1>(c, g16, dK, dV, s);
   if (p.d == 128) return launch<128, false, 2>(c, g16, dK, dV, s);
   // d = 64: three CTAs per SM where there are more than two for each (1248 tiles, m = 256 22.2 -> 18.5 us, 624 13.4 -> 12.0), else the deeper
-  // ring (64 tiles, m = 1024 7.7, with two stages 9.5)
-  return (p.n + kTileM - 1) / kTileM * p.B * p.H > 2 * (int64_t)c->sms ? launch<64, false, 3>(c, g16, dK, dV, s) : launch<64, false, 2>(c, g16, dK, dV, s);
+  // ring (64 tiles, m = 1024 7.7, with two stages 9.5).  Between three and four tiles per SM two rounds of three stand against two of two,
+  // which only a single chunk of rows pays for, being mostly start and end (480 tiles, m = 64 7.4 / 7.0, m = 512 14.6 / 15.5, m = 1200 29.1 / 32.2)
+  const int64_t tiles = (p.n + kTileM - 1) / kTileM * p.B * p.H;
+  return (p.m > kChunk ? !two_tiles_per_sm(tiles, c->sms) : tiles > 2 * (int64_t)c->sms) ? launch<64, false, 3>(c, g16, dK, dV, s) : launch<64, false, 2>(c, g16, dK, dV, s);
 }
 
 }  // namespace csat
