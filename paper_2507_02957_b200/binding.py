@@ -213,7 +213,10 @@ def csat_project_qkv(h, Xq, Xkv, W, d_model, Q, K, V, stream=None):
 def csat_forward(h, Q, K, V, out, stream=None):
     if getattr(h, "user_saves", None) is not None:
         _restore_saving(h)
-    _check(h, load().csat_forward(h, _ptr(Q), _ptr(K), _ptr(V), _ptr(out), _stream(stream)))
+    # (the host bounds the smallest calls: the look at the key above is paid for by two Python calls less)
+    rc = (_lib or load()).csat_forward(h, _ptr(Q), _ptr(K), _ptr(V), _ptr(out), _stream(stream))
+    if rc != CSAT_OK:
+        _check(h, rc)
 
 
 def csat_compress_partial(h, K_shard, V_shard, n0, n_len, partial_out, stream=None):
